@@ -11,19 +11,47 @@ using namespace psb;
 
 namespace {
 
+// Lines between the CUDA-core and the tensor path under PSB_PATH_AUTO, in multiply-accumulates of the call.
+// Padded layers of full-range unsigned bytes: the calls of the tensor path take 15-18 us in a stream of such calls
+// whatever the size, conv_direct_kernel 118 us at 10.6 M, 264 us at 19 M (3x3, 64 -> 64 channels) but 34 us at 11 M
+// with 40 output channels: the line stands where the tensor path has won for every shape measured.
+constexpr uint64_t kPaddedOffsetMinMacs = 16u << 20;
+// Layers whose activation rows have to be repacked first (one launch more): a fully connected layer of 333 features,
+// batch 37, 13 outputs (0.16 M) took 27.5 us with its sampling on CUDA cores, 30.5 us on the tensor path; a 1x1 layer of
+// 52 channels (3.6 M) 25.6 and 22.6 us.
+constexpr uint64_t kRepackMinMacs = 1u << 20;
+
 bool pow2_level_ok(uint32_t log2k) { return log2k < (uint32_t)kMaxLevels; }
 
-psb_status ensure_scratch(psb_ctx* ctx, int slot, size_t bytes) {
-  if (ctx->scratch_bytes[slot] >= bytes) return PSB_OK;
-  if (ctx->scratch[slot]) cudaFree(ctx->scratch[slot]);
-  ctx->scratch[slot] = nullptr;
-  ctx->scratch_bytes[slot] = 0;
+// The work buffers of a stream.  A stream not met before takes a free set, or the one unused longest once the device
+// has finished with it.
+ScratchSet& scratch_for(psb_ctx* ctx, cudaStream_t s) {
+  ScratchSet* pick = nullptr;
+  for (ScratchSet& c : ctx->scratch) {
+    if (c.used && c.stream == s) { pick = &c; break; }
+    if (!pick || (pick->used && (!c.used || c.last_use < pick->last_use))) pick = &c;
+  }
+  if (!pick->used || pick->stream != s) {
+    if (pick->used) cudaDeviceSynchronize();
+    pick->used = true;
+    pick->stream = s;
+    pick->sorted_rows = 0;
+  }
+  pick->last_use = ++ctx->scratch_clock;
+  return *pick;
+}
+
+psb_status ensure_scratch(ScratchSet& sc, int slot, size_t bytes) {
+  if (sc.bytes[slot] >= bytes) return PSB_OK;
+  if (sc.buf[slot]) cudaFree(sc.buf[slot]);
+  sc.buf[slot] = nullptr;
+  sc.bytes[slot] = 0;
   size_t want = bytes + bytes / 4;
-  if (cudaMalloc(&ctx->scratch[slot], want) != cudaSuccess) {
+  if (cudaMalloc(&sc.buf[slot], want) != cudaSuccess) {
     cudaGetLastError();
     return PSB_ERR_ALLOC;
   }
-  ctx->scratch_bytes[slot] = want;
+  sc.bytes[slot] = want;
   return PSB_OK;
 }
 
@@ -107,37 +135,54 @@ psb_status run_layer(psb_ctx* ctx, const psb_weights* wt, const void* x_dev, uin
   a.out_nchw = (layout == PSB_LAYOUT_NCHW && sh.out_ch > 1 && (uint64_t)oh * ow > 1) ? 1u : 0u;
 
   // largest activation magnitude the caller vouches for
-  uint32_t amax = in_max ? in_max : (in_dtype == PSB_DT_U8 ? 255u : 128u);
+  const uint32_t amax = in_max ? in_max : (in_dtype == PSB_DT_U8 ? 255u : 128u);
   const uint64_t M = (uint64_t)n * oh * ow;
-  bool tensor_ok = false, range_checked = false;
+  // The MMA takes signed bytes.  Unsigned data above 127 is fed as x - 128 (top bit flipped, by the gather or in
+  // shared memory) and corrected by 128 * sum(W).
+  const bool needs_offset = in_dtype == PSB_DT_U8 && amax > 127u;
+  bool tensor_ok = false;
   if (path != PSB_PATH_SHIFT_ADD) {
-    // the MMA takes signed bytes: unsigned data above 127 qualifies only where the activation
-    // matrix is gathered explicitly (packed-K filters), which stores x - 128
-    // the MMA takes signed bytes.  Unsigned data above 127 still qualifies where it can be fed as
-    // x - 128 and corrected by 128 * sum(W): packed-K filters (the gathered matrix is built with
-    // the offset) and layers without padding (one pass flips the top bit of the whole input)
-    const bool needs_offset = in_dtype == PSB_DT_U8 && amax > 127u;
-    tensor_ok = (!needs_offset || wt->packed_k || pad == 0) && tensor_supported(ctx, wt, a) == PSB_OK;
+    tensor_ok = tensor_supported(ctx, wt, a) == PSB_OK;
+    const bool padded_offset = needs_offset && !wt->packed_k && pad > 0;
+    if (padded_offset && M < 128u) tensor_ok = false;
     if (path == PSB_PATH_TENSOR && !tensor_ok) return PSB_ERR_UNSUPPORTED;
-    if (path == PSB_PATH_AUTO && M < (wt->packed_k ? 128u : 32u)) tensor_ok = false;
+    if (path == PSB_PATH_AUTO && (M < (wt->packed_k ? 128u : 32u) ||
+                                  (padded_offset && M * sh.out_ch * wt->d < kPaddedOffsetMinMacs) ||
+                                  (!wt->packed_k && c % 16u && M * sh.out_ch * wt->d < kRepackMinMacs)))
+      tensor_ok = false;
   }
+  // Channel pitch of the matrix the copy engine reads: its rows must be 16-byte multiples, and with taps as wide as
+  // a K block.
+  const bool direct = tensor_ok && !wt->packed_k;
+  uint32_t pitch = c;
+  if (direct) pitch = sh.kh * sh.kw > 1u || stride > 1u ? round_up(c < wt->bk ? wt->bk : c, 16u) : round_up(c, 16u);
 
+  ScratchSet& sc = scratch_for(ctx, s);
+  bool range_checked = false;
   if (in_conv) {
-    size_t bytes = (size_t)n * c * h * w;
-    st = ensure_scratch(ctx, 0, bytes);
+    st = ensure_scratch(sc, 0, (size_t)n * h * w * pitch);
     if (st != PSB_OK) return st;
-    if (launch_nchw_to_nhwc(x_dev, ctx->scratch[0], n, c, h * w, 1, in_dtype == PSB_DT_S8, amax, ctx->err_dev, s) !=
+    if (launch_nchw_to_nhwc(x_dev, sc.buf[0], n, c, h * w, pitch, in_dtype == PSB_DT_S8, amax, ctx->err_dev, s) !=
         cudaSuccess)
       return PSB_ERR_CUDA;
-    a.x = ctx->scratch[0];
+    a.x = sc.buf[0];
     range_checked = true;     // the conversion pass has looked at every byte
+  } else if (direct && (pitch != c || ((uintptr_t)x_dev & 15u))) {
+    st = ensure_scratch(sc, 0, (size_t)n * h * w * pitch);
+    if (st != PSB_OK) return st;
+    if (launch_repack_rows(x_dev, sc.buf[0], (size_t)n * h * w, c, pitch, in_dtype == PSB_DT_S8, amax, ctx->err_dev, s) !=
+        cudaSuccess)
+      return PSB_ERR_CUDA;
+    a.x = sc.buf[0];
+    range_checked = true;
   }
   // in_max is a promise the kernels rely on (bytes above 127 would read as negative on the tensor path):
   // passes that touch every input byte anyway verify it for free; the routes that hand the tensor
-  // straight to the copy engine verify it only on request (PSB_CHECK_RANGE)
+  // straight to the copy engine verify it only on request (PSB_CHECK_RANGE) or where it is between the two natural
+  // limits of unsigned bytes
   const uint32_t no_limit = in_dtype == PSB_DT_U8 ? 255u : 128u;
-  const bool gathers = tensor_ok && (wt->packed_k || (in_dtype == PSB_DT_U8 && amax > 127u));
-  if (!range_checked && !gathers && (ctx->checks & PSB_CHECK_RANGE) && amax < no_limit) {
+  const bool gathers = tensor_ok && wt->packed_k;
+  if (!range_checked && !gathers && ((ctx->checks & PSB_CHECK_RANGE) || (direct && needs_offset)) && amax < no_limit) {
     if (launch_range_check(a.x, (size_t)n * c * h * w, in_dtype == PSB_DT_S8, amax, ctx->err_dev, s) != cudaSuccess)
       return PSB_ERR_CUDA;
     range_checked = true;
@@ -145,31 +190,23 @@ psb_status run_layer(psb_ctx* ctx, const psb_weights* wt, const void* x_dev, uin
   const uint32_t gather_limit = range_checked ? no_limit : amax;
 
   if (tensor_ok) {
-    bool add_corr = false;
     if (wt->packed_k) {
       // gather the activation matrix [M][kpad] once, then run the layer as a plain GEMM
-      st = ensure_scratch(ctx, 1, (size_t)M * wt->kpad);
+      st = ensure_scratch(sc, 1, (size_t)M * wt->kpad);
       if (st != PSB_OK) return st;
       const uint32_t offset = in_dtype == PSB_DT_U8 ? 128u : 0u;
-      if (launch_im2col_s8(a, wt->kpad, wt->run_pitch, offset, (int8_t*)ctx->scratch[1], gather_limit, s) != cudaSuccess)
+      if (launch_im2col_s8(a, wt->kpad, wt->run_pitch, offset, (int8_t*)sc.buf[1], gather_limit, s) != cudaSuccess)
         return PSB_ERR_CUDA;
-      a.x = ctx->scratch[1];
+      a.x = sc.buf[1];
       a.in_dtype = PSB_DT_S8;
       a.C = wt->kpad;
       a.H = oh; a.W = ow;
       a.KH = 1; a.KW = 1; a.stride = 1; a.pad = 0;
-      add_corr = offset != 0;
-      amax = 128;
-    } else if (in_dtype == PSB_DT_U8 && amax > 127u) {
-      const size_t bytes = (size_t)n * c * h * w;   // a multiple of 16: c is
-      st = ensure_scratch(ctx, 1, bytes);
-      if (st != PSB_OK) return st;
-      if (launch_offset128(a.x, ctx->scratch[1], bytes, gather_limit, ctx->err_dev, s) != cudaSuccess) return PSB_ERR_CUDA;
-      a.x = ctx->scratch[1];
-      a.in_dtype = PSB_DT_S8;
-      add_corr = true;
-      amax = 128;
+    } else {
+      a.C = pitch;
     }
+    const bool flip = direct && needs_offset;
+    const bool add_corr = flip || (wt->packed_k && in_dtype == PSB_DT_U8);
     if (add_corr) {
       // 128 * (row sums of the integer filter) for every level this call may use
       for (uint32_t l = 0; l < (uint32_t)kMaxLevels; ++l)
@@ -183,24 +220,24 @@ psb_status run_layer(psb_ctx* ctx, const psb_weights* wt, const void* x_dev, uin
       const uint32_t tiles = sorted_tiles_bound(M);
       const size_t ctl_bytes = (sort_ctl_bytes() + 255u) & ~(size_t)255u;
       const size_t perm_bytes = (size_t)tiles * 128u * sizeof(uint32_t);
-      if (ctx->scratch_bytes[2] < ctl_bytes + perm_bytes + tiles) ctx->sorted_rows = 0;    // the buffer moves
-      st = ensure_scratch(ctx, 2, ctl_bytes + perm_bytes + tiles);
+      if (sc.bytes[2] < ctl_bytes + perm_bytes + tiles) sc.sorted_rows = 0;    // the buffer moves
+      st = ensure_scratch(sc, 2, ctl_bytes + perm_bytes + tiles);
       if (st != PSB_OK) return st;
-      uint8_t* base = (uint8_t*)ctx->scratch[2];
+      uint8_t* base = (uint8_t*)sc.buf[2];
       uint32_t* perm = (uint32_t*)(base + ctl_bytes);
       uint8_t* tile_mask = base + ctl_bytes + perm_bytes;
-      if (ctx->sorted_map != a.kmap || ctx->sorted_rows != (uint32_t)M) {
+      if (sc.sorted_map != a.kmap || sc.sorted_rows != (uint32_t)M) {
         if (launch_level_sort(a.kmap, (uint32_t)M, base, perm, tile_mask, s) != cudaSuccess) return PSB_ERR_CUDA;
-        ctx->sorted_map = a.kmap;
-        ctx->sorted_rows = (uint32_t)M;
+        sc.sorted_map = a.kmap;
+        sc.sorted_rows = (uint32_t)M;
       }
       // the matrix: K index (kh * KW + kw) * cpad + ci, cpad = channel blocks of the filter's plane layout
       const uint32_t cpad = wt->packed_k ? wt->n_cb * wt->bk : ((a.C + wt->bk - 1) / wt->bk) * wt->bk;
       const size_t row_bytes = (size_t)a.KH * a.KW * cpad;
-      st = ensure_scratch(ctx, 3, (size_t)tiles * 128u * row_bytes);
+      st = ensure_scratch(sc, 3, (size_t)tiles * 128u * row_bytes);
       if (st != PSB_OK) return st;
-      if (launch_gather_sorted(a, perm, base, cpad, (uint8_t*)ctx->scratch[3], s) != cudaSuccess) return PSB_ERR_CUDA;
-      a.x = ctx->scratch[3];
+      if (launch_gather_sorted(a, perm, base, cpad, (uint8_t*)sc.buf[3], s) != cudaSuccess) return PSB_ERR_CUDA;
+      a.x = sc.buf[3];
       a.C = (uint32_t)row_bytes;
       a.H = oh; a.W = ow;
       a.KH = 1; a.KW = 1; a.stride = 1; a.pad = 0;
@@ -208,7 +245,7 @@ psb_status run_layer(psb_ctx* ctx, const psb_weights* wt, const void* x_dev, uin
       sorted.tile_mask = tile_mask;
       sorted.tiles = tiles;
     }
-    st = launch_tensor(ctx, wt, a, amax, add_corr, a.kmap ? &sorted : nullptr, s);
+    st = launch_tensor(ctx, wt, a, amax, flip, add_corr, a.kmap ? &sorted : nullptr, s);
     if (st != PSB_OK) return st;
     ctx->last_path = PSB_PATH_TENSOR;
     return PSB_OK;
@@ -217,6 +254,21 @@ psb_status run_layer(psb_ctx* ctx, const psb_weights* wt, const void* x_dev, uin
   for (int l = 0; l < kMaxLevels; ++l) tab.w[l] = wt->level[l].wint;
   if (launch_shift_add(a, tab, wt->rowsum256, amax, s) != cudaSuccess) return PSB_ERR_CUDA;
   ctx->last_path = PSB_PATH_SHIFT_ADD;
+  return PSB_OK;
+}
+
+psb_status set_map(psb_ctx* ctx, const uint8_t* log2k_dev, uint32_t n, uint32_t oh, uint32_t ow,
+                   uint32_t uniform_log2k) {
+  if (log2k_dev) {
+    if (!n || !oh || !ow) return PSB_ERR_INVALID_ARG;
+    ctx->kmap = log2k_dev;
+    ctx->map_n = n; ctx->map_oh = oh; ctx->map_ow = ow;
+  } else {
+    if (!pow2_level_ok(uniform_log2k)) return PSB_ERR_BAD_K;
+    ctx->kmap = nullptr;
+    ctx->map_n = ctx->map_oh = ctx->map_ow = 0;
+    ctx->uniform_log2k = uniform_log2k;
+  }
   return PSB_OK;
 }
 
@@ -267,8 +319,9 @@ psb_status psb_destroy(psb_ctx* ctx) {
   if (!ctx) return PSB_ERR_INVALID_ARG;
   cudaSetDevice(ctx->device);
   cudaDeviceSynchronize();
-  for (int i = 0; i < 4; ++i)
-    if (ctx->scratch[i]) cudaFree(ctx->scratch[i]);
+  for (ScratchSet& sc : ctx->scratch)
+    for (void* b : sc.buf)
+      if (b) cudaFree(b);
   if (ctx->err_dev) cudaFree(ctx->err_dev);
   for (int i = 0; i < psb_ctx::kTimedLaunches; ++i) {
     if (ctx->t_begin[i]) cudaEventDestroy(ctx->t_begin[i]);
@@ -360,7 +413,8 @@ psb_status psb_sample_weights(psb_ctx* ctx, const float* w_dev, const psb_wshape
     w->cfg = cfg;
     w->device = ctx->device;
     w->d = (uint32_t)d64;
-    const bool wide = shape->in_ch_per_group % 16 == 0 && shape->in_ch_per_group >= 32;
+    // fewer than 16 channels: the flat K axis wastes less than a padded channel block per tap
+    const bool wide = shape->in_ch_per_group >= 16;
     w->packed_k = shape->groups == 1 && !wide && d64 >= 16;
     w->has_planes = shape->groups == 1 && (wide || w->packed_k);
     w->cpad = shape->in_ch_per_group;
@@ -425,18 +479,8 @@ psb_status psb_weights_free(psb_ctx* ctx, psb_weights* weights) {
 psb_status psb_set_sample_map(psb_ctx* ctx, const uint8_t* log2k_dev, uint32_t n, uint32_t oh,
                               uint32_t ow, uint32_t uniform_log2k) {
   if (!ctx) return PSB_ERR_INVALID_ARG;
-  ctx->sorted_rows = 0;      // whatever was derived from an earlier map is dropped
-  if (log2k_dev) {
-    if (!n || !oh || !ow) return PSB_ERR_INVALID_ARG;
-    ctx->kmap = log2k_dev;
-    ctx->map_n = n; ctx->map_oh = oh; ctx->map_ow = ow;
-  } else {
-    if (!pow2_level_ok(uniform_log2k)) return PSB_ERR_BAD_K;
-    ctx->kmap = nullptr;
-    ctx->map_n = ctx->map_oh = ctx->map_ow = 0;
-    ctx->uniform_log2k = uniform_log2k;
-  }
-  return PSB_OK;
+  for (ScratchSet& sc : ctx->scratch) sc.sorted_rows = 0;      // whatever was derived from an earlier map is dropped
+  return set_map(ctx, log2k_dev, n, oh, ow, uniform_log2k);
 }
 
 psb_status psb_conv2d(psb_ctx* ctx, const psb_weights* weights, const void* x_dev,
@@ -535,6 +579,7 @@ psb_status psb_sample_batch_free(psb_ctx* ctx, psb_sample_batch* batch) {
 
 psb_status psb_run(psb_ctx* ctx, const psb_op* ops, uint32_t n_ops, void* stream) {
   if (!ctx || (!ops && n_ops)) return PSB_ERR_INVALID_ARG;
+  for (ScratchSet& sc : ctx->scratch) sc.sorted_rows = 0;
   for (uint32_t i = 0; i < n_ops; ++i) {
     const psb_op& op = ops[i];
     psb_status st;
@@ -542,13 +587,9 @@ psb_status psb_run(psb_ctx* ctx, const psb_op* ops, uint32_t n_ops, void* stream
       case PSB_OP_CONV2D:
       case PSB_OP_GEMM: {
         // within one list a map that several operations name is sorted by level once (the maps must not
-        // change while the list runs); psb_set_sample_map drops the sorted order, so it is kept across it
-        const uint8_t* kept_map = ctx->sorted_map;
-        const uint32_t kept_rows = i ? ctx->sorted_rows : 0u;
-        st = psb_set_sample_map(ctx, op.map_dev, op.map_n, op.map_oh, op.map_ow, op.uniform_log2k);
+        // change while the list runs)
+        st = set_map(ctx, op.map_dev, op.map_n, op.map_oh, op.map_ow, op.uniform_log2k);
         if (st != PSB_OK) return st;
-        ctx->sorted_map = kept_map;
-        ctx->sorted_rows = kept_rows;
         st = op.kind == PSB_OP_CONV2D ? psb_conv2d(ctx, op.weights, op.x_dev, &op.conv, stream)
                                       : psb_gemm(ctx, op.weights, op.x_dev, &op.gemm, stream);
         break;

@@ -79,19 +79,30 @@ struct psb_weights {
   int device;
 };
 
+// Work buffers of the calls on one stream: [0] layout conversion, [1] gathered activation matrix, [2] level-sorted
+// order of the current draw-count map (control block, permutation, tile levels), [3] activation rows in that
+// order.  Calls of one stream follow one another, so they share the buffers; calls of different streams may
+// overlap and get their own.
+struct ScratchSet {
+  cudaStream_t stream = nullptr;
+  bool used = false;
+  unsigned long long last_use = 0;
+  void* buf[4] = {nullptr, nullptr, nullptr, nullptr};
+  size_t bytes[4] = {0, 0, 0, 0};
+  // the sorted order in buf[2] belongs to this map (pointer and dimensions); 0 rows = none
+  const uint8_t* sorted_map = nullptr;
+  uint32_t sorted_rows = 0;
+};
+
 struct psb_ctx {
   int device;
   uint32_t* err_dev = nullptr;      // device error word
   const uint8_t* kmap = nullptr;    // borrowed
   uint32_t map_n = 0, map_oh = 0, map_ow = 0;
   uint32_t uniform_log2k = 0;
-  // scratch: [0] layout conversion, [1] gathered / offset activation matrix, [2] level-sorted order of the
-  // current draw-count map (control block, permutation, tile levels), [3] activation rows in that order
-  void* scratch[4] = {nullptr, nullptr, nullptr, nullptr};
-  size_t scratch_bytes[4] = {0, 0, 0, 0};
-  // the sorted order in scratch[2] belongs to this map (pointer and dimensions); 0 rows = none
-  const uint8_t* sorted_map = nullptr;
-  uint32_t sorted_rows = 0;
+  static constexpr int kScratchStreams = 8;   // streams with buffers of their own; the one unused longest gives way
+  ScratchSet scratch[kScratchStreams];
+  unsigned long long scratch_clock = 0;
   int32_t last_path = 0;
   int sm_count = 0;
   unsigned long long wait_limit_cycles = psb::kDefaultWaitLimitCycles;   // bound of every device-side wait
@@ -235,12 +246,13 @@ size_t im2col_s8_smem(const ConvArgs& a, uint32_t run_pitch);   // shared memory
 cudaError_t launch_im2col_s8(const ConvArgs& a, uint32_t kpad, uint32_t run_pitch, uint32_t offset, int8_t* dst,
                              uint32_t limit, cudaStream_t s);
 cudaError_t launch_corr128(const psb_weights* wt, uint32_t level, cudaStream_t s);
-// `limit`: largest byte magnitude allowed (255 for unsigned / 128 for signed data = no check); a byte beyond
-// it raises kDevErrRange in *err
-cudaError_t launch_offset128(const void* src, void* dst, size_t bytes, uint32_t limit, uint32_t* err, cudaStream_t s);
-cudaError_t launch_nchw_to_nhwc(const void* src, void* dst, uint32_t N, uint32_t C, uint32_t HW,
-                                uint32_t elem_bytes, uint32_t is_signed, uint32_t limit, uint32_t* err,
-                                cudaStream_t s);
+// [rows][C] -> [rows][pitch] bytes, zero beyond C.  `limit`: largest byte magnitude allowed (255 for unsigned / 128
+// for signed data = no check); a byte beyond it raises kDevErrRange in *err
+cudaError_t launch_repack_rows(const void* src, void* dst, size_t rows, uint32_t C, uint32_t pitch, uint32_t is_signed,
+                               uint32_t limit, uint32_t* err, cudaStream_t s);
+// planar -> channels-last with `pitch` >= C bytes per location, zero beyond C
+cudaError_t launch_nchw_to_nhwc(const void* src, void* dst, uint32_t N, uint32_t C, uint32_t HW, uint32_t pitch,
+                                uint32_t is_signed, uint32_t limit, uint32_t* err, cudaStream_t s);
 cudaError_t launch_range_check(const void* x, size_t bytes, uint32_t is_signed, uint32_t limit, uint32_t* err,
                                cudaStream_t s);
 // one tiny CTA waits, with the context's bound, on a barrier that nobody arrives at (psb_tensor.cu)
@@ -259,7 +271,8 @@ struct SortedRows {
   const uint8_t* tile_mask;   // [tiles] the level of every tile as a one-bit mask (0 = unused tile)
   uint32_t tiles;             // upper bound of the tiles in use
 };
-psb_status launch_tensor(psb_ctx* ctx, const psb_weights* wt, const ConvArgs& a, uint32_t amax,
+// amax: largest activation magnitude; flip: the bytes are unsigned and reach the MMA as x - 128
+psb_status launch_tensor(psb_ctx* ctx, const psb_weights* wt, const ConvArgs& a, uint32_t amax, bool flip,
                          bool add_corr128, const SortedRows* sorted, cudaStream_t s);
 
 // level-sorted rows for draw-count maps (psb_sort.cu)

@@ -1,0 +1,6 @@
+// The contraction kernel (psb_mma.cuh) for K blocks of 128 bytes.
+#include "psb_mma_launch.cuh"
+
+namespace psb {
+template cudaError_t launch_mma_kernel<128>(const cudaLaunchConfig_t&, const TmapSet&, const TensorParams&, int, bool);
+}  // namespace psb

@@ -1,0 +1,6 @@
+// The contraction kernel (psb_mma.cuh) for K blocks of 32 bytes.
+#include "psb_mma_launch.cuh"
+
+namespace psb {
+template cudaError_t launch_mma_kernel<32>(const cudaLaunchConfig_t&, const TmapSet&, const TensorParams&, int, bool);
+}  // namespace psb

@@ -400,18 +400,47 @@ __global__ void __launch_bounds__(256, 3) dwconv3x3_row32_kernel(const ConvArgs 
     if ((uint32_t)i < n_out) *reinterpret_cast<uint32_t*>((uint8_t*)a.q_out + obase + (size_t)i * C) = qw[i];
 }
 
-// x ^ 0x80 over a whole tensor: unsigned bytes become (x - 128) as signed bytes, 16 per thread.
-__global__ void offset128_kernel(const uint4* src, uint4* dst, size_t n16, uint32_t limit,
-                                 uint32_t* __restrict__ err) {
+// [rows][C] -> [rows][pitch] (pitch a multiple of 16, zero beyond C): the copy engine wants rows that are 16-byte
+// multiples at 16-byte addresses.  Bound by memory; a thread writes one 16-byte piece, put together from the aligned
+// words it overlaps (byte loads at the tensor's two ends only).
+__global__ void __launch_bounds__(256) repack_rows_kernel(const uint8_t* src, uint8_t* __restrict__ dst, size_t rows,
+                                                         uint32_t C, uint32_t pitch, uint32_t is_signed, uint32_t limit,
+                                                         uint32_t* __restrict__ err) {
   pdl_prologue();
+  const uint32_t pieces = pitch / 16u;
+  const size_t total = rows * pieces;
+  const uint8_t* const end = src + rows * C;
   bool bad = false;
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n16; i += (size_t)gridDim.x * blockDim.x) {
-    uint4 v = __ldcg(src + i);
-    if (limit < 255u)
-      bad |= bytes_beyond(v.x, 0u, limit) | bytes_beyond(v.y, 0u, limit) | bytes_beyond(v.z, 0u, limit) |
-             bytes_beyond(v.w, 0u, limit);
-    v.x ^= 0x80808080u; v.y ^= 0x80808080u; v.z ^= 0x80808080u; v.w ^= 0x80808080u;
-    dst[i] = v;
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
+    const size_t row = i / pieces;
+    const uint32_t c0 = (uint32_t)(i - row * pieces) * 16u;
+    const uint32_t count = c0 < C ? min(16u, C - c0) : 0u;
+    const uint8_t* from = src + row * C + c0;
+    const uint32_t mis = (uint32_t)((uintptr_t)from & 3u);
+    const uint8_t* word = from - mis;
+    uint32_t w[5];
+#pragma unroll
+    for (int j = 0; j < 5; ++j) {
+      w[j] = 0u;
+      const uint8_t* q = word + 4 * j;
+      if ((uint32_t)(4 * j) >= mis + count) continue;
+      if (q >= src && q + 4 <= end) {
+        w[j] = __ldca(reinterpret_cast<const uint32_t*>(q));
+      } else {
+#pragma unroll
+        for (int b = 0; b < 4; ++b)
+          if (q + b >= src && q + b < end) w[j] |= (uint32_t)q[b] << (8 * b);
+      }
+    }
+    uint32_t v[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      v[j] = __funnelshift_r(w[j], w[j + 1], 8u * mis);
+      const uint32_t have = count > (uint32_t)(4 * j) ? count - 4 * j : 0u;      // bytes of this word that exist
+      if (have < 4u) v[j] &= (1u << (8u * have)) - 1u;
+      bad |= bytes_beyond(v[j], is_signed, limit);
+    }
+    *reinterpret_cast<uint4*>(dst + row * pitch + c0) = make_uint4(v[0], v[1], v[2], v[3]);
   }
   if (bad) atomicOr(err, kDevErrRange);
 }
@@ -552,28 +581,28 @@ __global__ void __launch_bounds__(256) im2col_s8_kernel(const ConvArgs a, uint32
   }
 }
 
-// [N][C][HW] -> [N][HW][C], elements of 1 byte, through a 32x33 tile.
-__global__ void nchw_to_nhwc_u8_kernel(const uint8_t* src, uint8_t* dst,
-                                       uint32_t C, uint32_t HW, uint32_t is_signed, uint32_t limit,
-                                       uint32_t* __restrict__ err) {
+// [N][C][HW] -> [N][HW][pitch], elements of 1 byte, zero beyond C, through a 32x33 tile.
+__global__ void nchw_to_nhwc_u8_kernel(const uint8_t* src, uint8_t* dst, uint32_t C, uint32_t HW, uint32_t pitch,
+                                       uint32_t is_signed, uint32_t limit, uint32_t* __restrict__ err) {
   pdl_prologue();
   __shared__ uint8_t tile[32][33];
-  const size_t base = (size_t)blockIdx.z * C * HW;
+  const size_t base = (size_t)blockIdx.z * C * HW, dbase = (size_t)blockIdx.z * pitch * HW;
   const uint32_t p0 = blockIdx.x * 32, c0 = blockIdx.y * 32;
   bool bad = false;
   for (uint32_t r = threadIdx.y; r < 32; r += blockDim.y) {
     uint32_t c = c0 + r, p = p0 + threadIdx.x;
+    uint8_t v = 0;
     if (c < C && p < HW) {
-      const uint8_t v = src[base + (size_t)c * HW + p];
+      v = src[base + (size_t)c * HW + p];
       bad |= bytes_beyond((uint32_t)v, is_signed, limit);
-      tile[r][threadIdx.x] = v;
     }
+    tile[r][threadIdx.x] = v;
   }
   if (bad) atomicOr(err, kDevErrRange);
   __syncthreads();
   for (uint32_t r = threadIdx.y; r < 32; r += blockDim.y) {
     uint32_t p = p0 + r, c = c0 + threadIdx.x;
-    if (c < C && p < HW) dst[base + (size_t)p * C + c] = tile[threadIdx.x][r];
+    if (c < pitch && p < HW) dst[dbase + (size_t)p * pitch + c] = tile[threadIdx.x][r];
   }
 }
 
@@ -585,11 +614,11 @@ __global__ void nchw_to_nhwc_u8_kernel(const uint8_t* src, uint8_t* dst,
 // (row pitch 132 words: bank = 4 * quad + location).
 __global__ void __launch_bounds__(256) nchw_to_nhwc_u8x4_kernel(const uint8_t* src,
                                                                uint8_t* __restrict__ dst, uint32_t C,
-                                                               uint32_t HW, uint32_t is_signed, uint32_t limit,
-                                                               uint32_t* __restrict__ err) {
+                                                               uint32_t HW, uint32_t pitch, uint32_t is_signed,
+                                                               uint32_t limit, uint32_t* __restrict__ err) {
   pdl_prologue();
   __shared__ __align__(16) uint32_t tile[8][132];
-  const size_t base = (size_t)blockIdx.z * C * HW;
+  const size_t base = (size_t)blockIdx.z * C * HW, dbase = (size_t)blockIdx.z * pitch * HW;
   const uint32_t p0 = blockIdx.x * 128u, c0 = blockIdx.y * 32u;
   const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u;
   {
@@ -615,7 +644,7 @@ __global__ void __launch_bounds__(256) nchw_to_nhwc_u8x4_kernel(const uint8_t* s
   for (int r = 0; r < 4; ++r) {
     const uint32_t pl = (threadIdx.x >> 3) + 32u * r;
     const uint32_t p = p0 + pl, c = c0 + 4u * q;
-    if (p < HW && c < C) *reinterpret_cast<uint32_t*>(dst + base + (size_t)p * C + c) = tile[q][pl];
+    if (p < HW && c < pitch) *reinterpret_cast<uint32_t*>(dst + dbase + (size_t)p * pitch + c) = tile[q][pl];
   }
 }
 
@@ -733,9 +762,10 @@ uint32_t grid_for(size_t total, uint32_t threads) {
 
 }  // namespace
 
-cudaError_t launch_offset128(const void* src, void* dst, size_t bytes, uint32_t limit, uint32_t* err, cudaStream_t s) {
-  const size_t n16 = bytes / 16;
-  launch_pdl(offset128_kernel, grid_for(n16, 256), 256, 0, s, (const uint4*)src, (uint4*)dst, n16, limit, err);
+cudaError_t launch_repack_rows(const void* src, void* dst, size_t rows, uint32_t C, uint32_t pitch, uint32_t is_signed,
+                               uint32_t limit, uint32_t* err, cudaStream_t s) {
+  launch_pdl(repack_rows_kernel, grid_for(rows * (pitch / 16u), 256), 256, 0, s, (const uint8_t*)src, (uint8_t*)dst, rows, C,
+             pitch, is_signed, limit, err);
   note_launch();
   return cudaGetLastError();
 }
@@ -821,17 +851,15 @@ cudaError_t launch_im2col_s8(const ConvArgs& a, uint32_t kpad, uint32_t run_pitc
   return cudaGetLastError();
 }
 
-cudaError_t launch_nchw_to_nhwc(const void* src, void* dst, uint32_t N, uint32_t C, uint32_t HW,
-                                uint32_t elem_bytes, uint32_t is_signed, uint32_t limit, uint32_t* err,
-                                cudaStream_t s) {
-  if (elem_bytes != 1) return cudaErrorInvalidValue;
-  if (C % 4u == 0 && HW % 4u == 0 && !(((uintptr_t)src | (uintptr_t)dst) & 3u)) {
-    dim3 grid4((HW + 127) / 128, (C + 31) / 32, N);
-    launch_pdl(nchw_to_nhwc_u8x4_kernel, grid4, 256, 0, s, (const uint8_t*)src, (uint8_t*)dst, C, HW, is_signed, limit,
-               err);
+cudaError_t launch_nchw_to_nhwc(const void* src, void* dst, uint32_t N, uint32_t C, uint32_t HW, uint32_t pitch,
+                                uint32_t is_signed, uint32_t limit, uint32_t* err, cudaStream_t s) {
+  if (C % 4u == 0 && pitch % 4u == 0 && HW % 4u == 0 && !(((uintptr_t)src | (uintptr_t)dst) & 3u)) {
+    dim3 grid4((HW + 127) / 128, (pitch + 31) / 32, N);
+    launch_pdl(nchw_to_nhwc_u8x4_kernel, grid4, 256, 0, s, (const uint8_t*)src, (uint8_t*)dst, C, HW, pitch, is_signed,
+               limit, err);
   } else {
-    dim3 grid((HW + 31) / 32, (C + 31) / 32, N), block(32, 8);
-    launch_pdl(nchw_to_nhwc_u8_kernel, grid, block, 0, s, (const uint8_t*)src, (uint8_t*)dst, C, HW, is_signed, limit,
+    dim3 grid((HW + 31) / 32, (pitch + 31) / 32, N), block(32, 8);
+    launch_pdl(nchw_to_nhwc_u8_kernel, grid, block, 0, s, (const uint8_t*)src, (uint8_t*)dst, C, HW, pitch, is_signed, limit,
                err);
   }
   note_launch();

@@ -1,0 +1,72 @@
+"""GPU parity of the tensor path's routes for channel counts that are no multiple of 16, output rows without 16-byte
+alignment, and full-range unsigned bytes with padding (bit-exact against the CPU oracle)."""
+import numpy as np
+import pytest
+
+from psb_testlib import compare, gpu_layer, oracle_layer
+
+pytestmark = pytest.mark.gpu
+
+# (N, C, H, W, O, K, stride, pad, layout, dtype, largest magnitude, shortcut dtype or None, levels or None)
+CASES = [
+    (3, 100, 9, 13, 150, 3, 1, 1, 1, np.uint8, 255, None, None),       # rows of 2-byte units, two channel blocks
+    (2, 17, 11, 9, 33, 3, 1, 1, 1, np.uint8, 255, np.uint8, None),     # single bytes, padded to one K block
+    (4, 31, 13, 12, 20, 5, 2, 2, 0, np.uint8, 255, np.int8, None),     # planar in and out, 4-byte units
+    (5, 36, 8, 7, 100, 1, 1, 0, 1, np.int8, 127, np.uint8, None),      # plain matrix product, rows of 4-byte units
+    (2, 64, 12, 11, 64, 3, 1, 1, 1, np.uint8, 255, None, None),        # no repacking, the flip only
+    (2, 96, 15, 9, 72, 3, 2, 1, 1, np.uint8, 200, np.uint8, None),     # partly filled last channel block, in_max < 255
+    (3, 40, 7, 9, 24, 3, 1, 1, 1, np.uint8, 255, None, (0, 3, 4)),     # draw-count map on flipped, repacked rows
+    (150, 333, 1, 1, 31, 1, 1, 0, 1, np.uint8, 255, None, None),       # fully connected, odd everything
+    (4, 16, 9, 9, 48, 1, 1, 0, 1, np.uint8, 15, None, None),           # rows narrower than a K block
+]
+
+
+@pytest.mark.parametrize("want", [("q",), ("q", "f32", "acc")])
+@pytest.mark.parametrize("case", CASES)
+def test_odd_layers_on_the_tensor_path(case, want, oracle):
+    import paper_1904_02205_b200 as psb
+
+    N, C, H, W, O, K, stride, pad, layout, dtype, top, res_dtype, levels = case
+    ctx = psb.Context(0)
+    rng = np.random.default_rng(C * 7 + O)
+    w = rng.normal(0, np.sqrt(2.0 / (C * K * K)), size=(O, C, K, K)).astype(np.float32)
+    x = rng.integers(0 if dtype == np.uint8 else -top, top + 1, size=(N, C, H, W) if layout == 0 else (N, H, W, C)).astype(dtype)
+    oh, ow = (H + 2 * pad - K) // stride + 1, (W + 2 * pad - K) // stride + 1
+    res = None
+    if res_dtype is not None:
+        lo = 0 if res_dtype == np.uint8 else -128
+        res = rng.integers(lo, lo + 256, size=(N, O, oh, ow) if layout == 0 else (N, oh, ow, O)).astype(res_dtype)
+    kmap = None if levels is None else rng.choice(levels, size=(N, oh, ow)).astype(np.uint8)
+    args = (w, x, layout, 1, stride, pad, 5, 3, list(levels or (3,)), kmap, 3, rng.uniform(0.5, 1.5, O).astype(np.float32),
+            rng.normal(0, 0.5, O).astype(np.float32), True, np.float32(0.02), 0, 255)
+    o = oracle_layer(oracle, *args, residual=res, res_scale=np.float32(0.3))
+    g = gpu_layer(psb, ctx, *args, psb.PSB_DT_U8, residual=res, res_scale=np.float32(0.3), in_max=top, path=psb.PSB_PATH_TENSOR,
+                  want=want)
+    compare(g, o, list(levels or (3,)))
+    assert g["path"] == psb.PSB_PATH_TENSOR
+    ctx.close()
+
+
+def test_rows_that_start_at_odd_addresses(oracle):
+    """An input tensor at an address the copy engine cannot take is repacked first."""
+    import torch
+
+    import paper_1904_02205_b200 as psb
+
+    ctx = psb.Context(0)
+    rng = np.random.default_rng(3)
+    w = rng.normal(0, 0.2, size=(32, 48, 1, 1)).astype(np.float32)
+    x = rng.integers(0, 16, size=(200, 48)).astype(np.uint8)
+    flat = torch.zeros(200 * 48 + 16, dtype=torch.uint8, device=ctx.device)
+    wt = ctx.sample_weights(torch.from_numpy(w).to(ctx.device), seed=1, level_mask=8)
+    ctx.set_sample_map(None, 3)
+    one = torch.ones(32, device=ctx.device)
+    W, eb, _ = oracle.sample_level(w, 1, 0, 3)
+    acc = x.astype(np.int64) @ W.reshape(32, 48).astype(np.int64).T
+    for shift in (1, 4, 7, 8):
+        flat[shift:shift + x.size] = torch.from_numpy(x.ravel()).to(ctx.device)
+        got = ctx.gemm(wt, flat[shift:shift + x.size].view(200, 48), one, one, False, 1.0, 0, 255, in_max=15,
+                       path=psb.PSB_PATH_TENSOR, want=("acc",))["acc"].cpu().numpy()
+        assert ctx.device_status() == 0 and np.array_equal(got, acc)
+    wt.free()
+    ctx.close()
