@@ -14,7 +14,7 @@ CASES = [
     (4, 31, 13, 12, 20, 5, 2, 2, 0, np.uint8, 255, np.int8, None),     # planar in and out, 4-byte units
     (5, 36, 8, 7, 100, 1, 1, 0, 1, np.int8, 127, np.uint8, None),      # plain matrix product, rows of 4-byte units
     (2, 64, 12, 11, 64, 3, 1, 1, 1, np.uint8, 255, None, None),        # no repacking, the flip only
-    (2, 96, 15, 9, 72, 3, 2, 1, 1, np.uint8, 200, np.uint8, None),     # partly filled last channel block, in_max < 255
+    (4, 96, 15, 9, 72, 3, 2, 1, 1, np.uint8, 200, np.uint8, None),     # partly filled last channel block, in_max < 255
     (3, 40, 7, 9, 24, 3, 1, 1, 1, np.uint8, 255, None, (0, 3, 4)),     # draw-count map on flipped, repacked rows
     (150, 333, 1, 1, 31, 1, 1, 0, 1, np.uint8, 255, None, None),       # fully connected, odd everything
     (4, 16, 9, 9, 48, 1, 1, 0, 1, np.uint8, 15, None, None),           # rows narrower than a K block
