@@ -55,21 +55,6 @@ psb_status ensure_scratch(ScratchSet& sc, int slot, size_t bytes) {
   return PSB_OK;
 }
 
-void free_weights_storage(psb_weights* w) {
-  for (int l = 0; l < kMaxLevels; ++l) {
-    if (w->level[l].wint) cudaFree(w->level[l].wint);
-    if (w->level[l].planes) cudaFree(w->level[l].planes);
-    if (w->level[l].corr128) cudaFree(w->level[l].corr128);
-    w->level[l] = LevelStore();
-  }
-  if (w->e_base) cudaFree(w->e_base);
-  if (w->e_max) cudaFree(w->e_max);
-  if (w->rowsum256) cudaFree(w->rowsum256);
-  w->e_base = nullptr;
-  w->e_max = nullptr;
-  w->rowsum256 = nullptr;
-}
-
 psb_status check_epilogue(const psb_epilogue& ep) {
   if (!ep.scale_dev || !ep.bias_dev) return PSB_ERR_INVALID_ARG;
   if (!ep.q_out_dev && !ep.f32_out_dev && !ep.acc_out_dev) return PSB_ERR_INVALID_ARG;
@@ -207,12 +192,6 @@ psb_status run_layer(psb_ctx* ctx, const psb_weights* wt, const void* x_dev, uin
     }
     const bool flip = direct && needs_offset;
     const bool add_corr = flip || (wt->packed_k && in_dtype == PSB_DT_U8);
-    if (add_corr) {
-      // 128 * (row sums of the integer filter) for every level this call may use
-      for (uint32_t l = 0; l < (uint32_t)kMaxLevels; ++l)
-        if (wt->level[l].corr128 && (ctx->kmap || l == ctx->uniform_log2k))
-          if (launch_corr128(wt, l, s) != cudaSuccess) return PSB_ERR_CUDA;
-    }
     SortedRows sorted;
     if (a.kmap) {
       // per-location draw counts: sort the locations by level (once per map), gather the activation rows in
@@ -252,6 +231,27 @@ psb_status run_layer(psb_ctx* ctx, const psb_weights* wt, const void* x_dev, uin
   }
   WintTable tab;
   for (int l = 0; l < kMaxLevels; ++l) tab.w[l] = wt->level[l].wint;
+  if (wt->has_planes) {
+    if (gemv_planes_ok(a, wt)) {
+      if (launch_gemv_planes(a, wt, s) != cudaSuccess) return PSB_ERR_CUDA;
+      ctx->last_path = PSB_PATH_SHIFT_ADD;
+      return PSB_OK;
+    }
+    // the direct kernels read 32-bit weights: put them together from the digit planes
+    const size_t words = (size_t)sh.out_ch * wt->d;
+    uint32_t used = 0, n_used = 0;
+    for (uint32_t l = 0; l < (uint32_t)kMaxLevels; ++l)
+      if (wt->level[l].planes && (a.kmap || l == a.uniform_log2k)) { used |= 1u << l; ++n_used; }
+    st = ensure_scratch(sc, 1, sizeof(int32_t) * words * n_used);
+    if (st != PSB_OK) return st;
+    int32_t* at = (int32_t*)sc.buf[1];
+    for (uint32_t l = 0; l < (uint32_t)kMaxLevels; ++l) {
+      if (!((used >> l) & 1u)) continue;
+      if (launch_expand(wt, l, false, at, s) != cudaSuccess) return PSB_ERR_CUDA;
+      tab.w[l] = at;
+      at += words;
+    }
+  }
   if (launch_shift_add(a, tab, wt->rowsum256, amax, s) != cudaSuccess) return PSB_ERR_CUDA;
   ctx->last_path = PSB_PATH_SHIFT_ADD;
   return PSB_OK;
@@ -425,32 +425,49 @@ psb_status psb_sample_weights(psb_ctx* ctx, const float* w_dev, const psb_wshape
     w->bk = tensor_bk(w->packed_k ? w->kpad : shape->in_ch_per_group);
     w->n_cb = ((w->packed_k ? w->kpad : shape->in_ch_per_group) + w->bk - 1) / w->bk;
     w->n_kb = w->packed_k ? w->n_cb : shape->kh * shape->kw * w->n_cb;
-    bool ok = cudaMalloc(&w->e_base, sizeof(int32_t) * shape->out_ch) == cudaSuccess &&
-              cudaMalloc(&w->e_max, sizeof(uint32_t) * shape->out_ch) == cudaSuccess &&
-              cudaMalloc(&w->rowsum256, sizeof(uint32_t) * kMaxLevels * shape->out_ch) == cudaSuccess &&
-              cudaMemsetAsync(w->e_max, 0, sizeof(uint32_t) * shape->out_ch, s) == cudaSuccess;
-    for (uint32_t l = 0; ok && l < (uint32_t)kMaxLevels; ++l) {
+    // one allocation for the whole handle; the digit planes come last and start as zeros (rows beyond out_ch and
+    // columns beyond the filter are never written)
+    const size_t O = shape->out_ch;
+    size_t bytes = 0;
+    auto place = [&bytes](size_t want) {
+      const size_t at = bytes;
+      bytes = (bytes + want + 1023u) & ~(size_t)1023u;
+      return at;
+    };
+    const size_t at_corr = place(w->has_planes ? sizeof(long long) * kMaxLevels * O : 0), at_base = place(sizeof(int32_t) * O);
+    const size_t at_rows = place(sizeof(uint32_t) * kMaxLevels * O), at_emax = place(sizeof(uint32_t) * O);
+    const size_t levels_from = bytes;
+    size_t at_level[kMaxLevels] = {};
+    for (uint32_t l = 0; l < (uint32_t)kMaxLevels; ++l) {
       if (!((cfg.level_mask >> l) & 1u)) continue;
-      ok = cudaMalloc(&w->level[l].wint, sizeof(int32_t) * d64 * shape->out_ch) == cudaSuccess;
-      if (ok && w->has_planes) {
-        int P = planes_for(cfg.exp_bits, l);
-        size_t bytes = (size_t)w->o_tiles * w->n_kb * P * kTileN * w->bk;
-        w->level[l].planes_count = P;
-        ok = cudaMalloc(&w->level[l].planes, bytes) == cudaSuccess &&
-             cudaMemsetAsync(w->level[l].planes, 0, bytes, s) == cudaSuccess;
-        if (ok)
-          ok = cudaMalloc(&w->level[l].corr128, sizeof(long long) * shape->out_ch) == cudaSuccess;
-      }
+      if (w->has_planes) w->level[l].planes_count = planes_for(cfg.exp_bits, l);
+      at_level[l] = place(w->has_planes ? (size_t)w->o_tiles * w->n_kb * w->level[l].planes_count * kTileN * w->bk
+                                        : sizeof(int32_t) * d64 * O);
     }
-    if (!ok) {
+    if (cudaMalloc(&w->storage, bytes) != cudaSuccess) {
       cudaGetLastError();
-      free_weights_storage(w);
+      delete w;
+      return PSB_ERR_ALLOC;
+    }
+    uint8_t* base = (uint8_t*)w->storage;
+    w->corr128 = w->has_planes ? (long long*)(base + at_corr) : nullptr;
+    w->e_base = (int32_t*)(base + at_base);
+    w->rowsum256 = (uint32_t*)(base + at_rows);
+    w->e_max = (uint32_t*)(base + at_emax);
+    for (uint32_t l = 0; l < (uint32_t)kMaxLevels; ++l) {
+      if (!((cfg.level_mask >> l) & 1u)) continue;
+      if (w->has_planes) w->level[l].planes = (int8_t*)(base + at_level[l]);
+      else w->level[l].wint = (int32_t*)(base + at_level[l]);
+    }
+    if (cudaMemsetAsync(base + at_emax, 0, (w->has_planes ? bytes : levels_from) - at_emax, s) != cudaSuccess) {
+      cudaGetLastError();
+      cudaFree(w->storage);
       delete w;
       return PSB_ERR_ALLOC;
     }
   }
   if (launch_sampler(w_dev, w, ctx->err_dev, s) != cudaSuccess) {
-    if (!*weights) { free_weights_storage(w); delete w; }
+    if (!*weights) { cudaFree(w->storage); delete w; }
     return PSB_ERR_CUDA;
   }
   *weights = w;
@@ -471,7 +488,7 @@ psb_status psb_weights_free(psb_ctx* ctx, psb_weights* weights) {
   if (!ctx || !weights) return PSB_ERR_INVALID_ARG;
   cudaSetDevice(ctx->device);
   cudaDeviceSynchronize();
-  free_weights_storage(weights);
+  cudaFree(weights->storage);
   delete weights;
   return PSB_OK;
 }

@@ -19,55 +19,76 @@ namespace psb {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kStage = 2048;  // weights staged in shared memory per block
+constexpr int kStage = 8192;  // most weights staged in shared memory per block
 constexpr int kEmaxRows = kThreads / 32;   // output channels per block of the exponent pass (norm == 1, short rows)
 constexpr int kEmaxLongRow = 1024;         // rows longer than this get a block each
 constexpr int kRowSumRows = 256;   // filter rows per block for which the sampler keeps sums of |W_k|
+constexpr int kPlaneRows = 64;     // the same for filters with digit planes, which need the signed sums too
 
-// Philox4x32-10 (Salmon et al., SC'11): ten rounds of two 32x32->64 multiplies and
-// xors; the key advances by the two Weyl constants after every round.  The ten round keys
-// depend on the seed only: the host computes them once per launch (PhiloxKeys) and hands them to the kernel as a
-// parameter, so every round reads its key straight from the constant bank and no register holds one.
+// Philox4x32-10 (Salmon et al., SC'11): ten rounds of two 32x32->64 multiplies and xors; the key advances by the
+// two Weyl constants after every round.  What the counters of this library allow to be known beforehand is
+// computed once per launch on the host and read from the constant bank:
+//   - the ten round keys;
+//   - of call q of a weight, counter (q, layer, index, 0) (a filter has at most 2^31 weights, so the high index word
+//     is 0): the products of the first two rounds that see only q.  With M0, M1 the multipliers, Q = M0 q,
+//     U = M1 (hi(Q) ^ k1[0]):  x = hi(U) ^ k0[1],  y = lo(Q) ^ k1[1],  z = lo(U) ^ k0[2].
+// The two products of those rounds that see only the index serve every call of the weight (PhiloxWeight), so a
+// call costs 16 multiplies instead of 20.
+constexpr uint32_t kPhiloxM0 = 0xD2511F53u, kPhiloxM1 = 0xCD9E8D57u;
+constexpr int kPhiloxCalls = 16;      // calls of a weight at k = 64
+
 struct PhiloxKeys {
   uint32_t k0[10], k1[10];
+  uint32_t x[kPhiloxCalls], y[kPhiloxCalls], z[kPhiloxCalls];
   __host__ __device__ __forceinline__ PhiloxKeys(uint32_t seed_lo, uint32_t seed_hi) {
 #pragma unroll
     for (int r = 0; r < 10; ++r) {
       k0[r] = seed_lo + (uint32_t)r * 0x9E3779B9u;
       k1[r] = seed_hi + (uint32_t)r * 0xBB67AE85u;
     }
+#pragma unroll
+    for (int q = 0; q < kPhiloxCalls; ++q) {
+      const unsigned long long Q = (unsigned long long)kPhiloxM0 * (uint32_t)q;
+      const unsigned long long U = (unsigned long long)kPhiloxM1 * ((uint32_t)(Q >> 32) ^ k1[0]);
+      x[q] = (uint32_t)(U >> 32) ^ k0[1];
+      y[q] = (uint32_t)Q ^ k1[1];
+      z[q] = (uint32_t)U ^ k0[2];
+    }
   }
 };
 
-__device__ __forceinline__ void philox4x32_10(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3,
-                                              const PhiloxKeys& key, uint32_t (&out)[4]) {
-  const uint32_t M0 = 0xD2511F53u, M1 = 0xCD9E8D57u;
-#pragma unroll
-  for (int r = 0; r < 10; ++r) {
-    // one widening multiply gives both halves
-    const unsigned long long p0 = (unsigned long long)M0 * c0, p1 = (unsigned long long)M1 * c2;
-    const uint32_t hi0 = (uint32_t)(p0 >> 32), lo0 = (uint32_t)p0;
-    const uint32_t hi1 = (uint32_t)(p1 >> 32), lo1 = (uint32_t)p1;
-    const uint32_t n0 = hi1 ^ c1 ^ key.k0[r];
-    const uint32_t n2 = hi0 ^ c3 ^ key.k1[r];
-    c0 = n0; c1 = lo1; c2 = n2; c3 = lo0;
+// What the calls of one weight share.  layer_key = layer_id ^ k0[0].
+struct PhiloxWeight {
+  uint32_t a_lo, b_lo, b_hi;
+  __device__ __forceinline__ PhiloxWeight(uint32_t index, uint32_t layer_key) {
+    const unsigned long long A = (unsigned long long)kPhiloxM1 * index;
+    const unsigned long long B = (unsigned long long)kPhiloxM0 * ((uint32_t)(A >> 32) ^ layer_key);
+    a_lo = (uint32_t)A;
+    b_lo = (uint32_t)B;
+    b_hi = (uint32_t)(B >> 32);
   }
-  out[0] = c0; out[1] = c1; out[2] = c2; out[3] = c3;
-}
-
-__device__ __forceinline__ void philox4x32_10(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3,
-                                              uint32_t k0, uint32_t k1, uint32_t (&out)[4]) {
-  const PhiloxKeys key(k0, k1);
-  philox4x32_10(c0, c1, c2, c3, key, out);
-}
+  __device__ __forceinline__ void call(uint32_t q, const PhiloxKeys& key, uint32_t (&out)[4]) const {
+    uint32_t c0 = a_lo ^ key.x[q], c2 = b_hi ^ key.y[q], c3 = b_lo, c1 = 0u;
+#pragma unroll
+    for (int r = 2; r < 10; ++r) {
+      // one widening multiply gives both halves
+      const unsigned long long p0 = (unsigned long long)kPhiloxM0 * c0, p1 = (unsigned long long)kPhiloxM1 * c2;
+      c0 = (uint32_t)(p1 >> 32) ^ (r == 2 ? key.z[q] : c1 ^ key.k0[r]);
+      c2 = (uint32_t)(p0 >> 32) ^ c3 ^ key.k1[r];
+      c1 = (uint32_t)p1;
+      c3 = (uint32_t)p0;
+    }
+    out[0] = c0; out[1] = c1; out[2] = c2; out[3] = c3;
+  }
+};
 
 // Counts with a B-bit comparator (Sec. 4.4; supplement, "Stochastic multiplier"): draw j is bit field
 // (j mod n) of word ((j / n) mod 4) of Philox call j / (4 n), n = 32 / B; cnt[l] = ones among the first 2^l
 // draws.  Every index is a compile-time constant here, so the loops unroll into one extract / compare / add
 // per draw.
 template <int B>
-__device__ __forceinline__ void packed_counts(uint32_t thr, uint32_t max_level, uint32_t layer_id, uint32_t i_lo,
-                                              uint32_t i_hi, const PhiloxKeys& keys, uint32_t (&cnt)[kMaxLevels]) {
+__device__ __forceinline__ void packed_counts(uint32_t thr, uint32_t max_level, const PhiloxWeight& pw,
+                                              const PhiloxKeys& keys, uint32_t (&cnt)[kMaxLevels]) {
   constexpr int n = 32 / B, per_call = 4 * n, calls = (64 + per_call - 1) / per_call;
   const uint32_t kmax = 1u << max_level;
   uint32_t c = 0;
@@ -75,7 +96,7 @@ __device__ __forceinline__ void packed_counts(uint32_t thr, uint32_t max_level, 
   for (int q = 0; q < calls; ++q) {
     if ((uint32_t)(q * per_call) < kmax) {
       uint32_t rnd[4];
-      philox4x32_10((uint32_t)q, layer_id, i_lo, i_hi, keys, rnd);
+      pw.call((uint32_t)q, keys, rnd);
 #pragma unroll
       for (int wd = 0; wd < 4; ++wd) {
 #pragma unroll
@@ -96,14 +117,13 @@ __device__ __forceinline__ void packed_counts(uint32_t thr, uint32_t max_level, 
 }
 
 // The same for any width 1..8, indices at run time.
-__device__ __forceinline__ void packed_counts_any(uint32_t pbits, uint32_t thr, uint32_t max_level, uint32_t layer_id,
-                                               uint32_t i_lo, uint32_t i_hi, const PhiloxKeys& keys,
-                                               uint32_t (&cnt)[kMaxLevels]) {
+__device__ __forceinline__ void packed_counts_any(uint32_t pbits, uint32_t thr, uint32_t max_level, const PhiloxWeight& pw,
+                                                  const PhiloxKeys& keys, uint32_t (&cnt)[kMaxLevels]) {
   const uint32_t n = 32u / pbits, per_call = 4u * n, fmask = (1u << pbits) - 1u, kmax = 1u << max_level;
   unsigned long long drawn = 0ull;      // bit j = draw j
   for (uint32_t q = 0; q * per_call < kmax && q * per_call < 64u; ++q) {
     uint32_t rnd[4];
-    philox4x32_10(q, layer_id, i_lo, i_hi, keys, rnd);
+    pw.call(q, keys, rnd);
 #pragma unroll
     for (int wd = 0; wd < 4; ++wd) {
       uint32_t word = rnd[wd];
@@ -126,24 +146,44 @@ __device__ __forceinline__ uint32_t small_div(uint32_t t, uint32_t magic) { retu
 // Largest biased exponent of the finite weights of each exponent group; flags Inf/NaN (which
 // contribute nothing: the finite weights of the group keep the window they would have without it).
 // norm == 1: one warp (short rows) or one block per output channel.  norm == 0: grid-stride over the layer.
-// Biased exponent of a weight after its probability has been rounded to `pbits` bits (Sec. 4.4): a
-// probability that rounds to 1 is the next power of two.  pbits == 0: the exponent as it is.
-__device__ __forceinline__ uint32_t quantised_exponent(uint32_t u, uint32_t pbits) {
-  const uint32_t E = (u >> 23) & 0xFFu;
+// Bound by memory once an element costs an AND and a max: the pass takes the largest magnitude (as an integer) and
+// turns it into an exponent at the end.  After rounding the probability to `pbits` bits (Sec. 4.4) a probability of 1
+// carries into the exponent; that is monotonic in the magnitude, so rounding the largest one is enough.
+__device__ __forceinline__ uint32_t quantised_exponent(uint32_t mag, uint32_t pbits) {
+  const uint32_t E = mag >> 23;
   if (pbits == 0u || E == 0u || E >= 254u) return E;
-  const uint32_t pq = ((u & 0x7FFFFFu) + (1u << (22u - pbits))) >> (23u - pbits);
-  return E + (pq >> pbits);
+  return (mag + (1u << (22u - pbits))) >> 23;
+}
+
+constexpr uint32_t kInfBits = 0x7F800000u;
+
+// Largest magnitude of n words, Inf and NaN flagged and left out.
+template <int kN>
+__device__ __forceinline__ uint32_t max_magnitude(const uint32_t (&u)[kN], uint32_t best, bool& bad) {
+  uint32_t m = 0u;
+#pragma unroll
+  for (int j = 0; j < kN; ++j) m = max(m, u[j] & 0x7FFFFFFFu);
+  if (m >= kInfBits) {
+    bad = true;
+    m = 0u;
+#pragma unroll
+    for (int j = 0; j < kN; ++j) m = max(m, (u[j] & 0x7FFFFFFFu) >= kInfBits ? 0u : u[j] & 0x7FFFFFFFu);
+  }
+  return max(best, m);
 }
 
 __device__ __forceinline__ void emax_block(const float* __restrict__ w, uint32_t O, uint32_t d,
                                            uint32_t norm, uint32_t* __restrict__ e_max,
                                            uint32_t* __restrict__ err, uint32_t block, uint32_t blocks,
-                                           uint32_t tag, uint32_t* __restrict__ rowsum, uint32_t pbits) {
+                                           uint32_t tag, uint32_t* __restrict__ rowsum,
+                                           long long* __restrict__ corr, uint32_t pbits) {
   __shared__ uint32_t red[kThreads / 32];
-  // the sampling pass that follows adds its row sums of |W_k| into these words: start them at zero
+  // the sampling pass that follows adds its row sums into these words: start them at zero
   if (rowsum)
-    for (uint32_t i = block * blockDim.x + threadIdx.x; i < (uint32_t)kMaxLevels * O; i += blocks * blockDim.x)
+    for (uint32_t i = block * blockDim.x + threadIdx.x; i < (uint32_t)kMaxLevels * O; i += blocks * blockDim.x) {
       rowsum[i] = 0u;
+      if (corr) corr[i] = 0;
+    }
   uint32_t best = 0;
   bool bad = false;
   if (norm) {
@@ -159,19 +199,13 @@ __device__ __forceinline__ void emax_block(const float* __restrict__ w, uint32_t
         for (uint32_t i = lane * 4u; i < d; i += lanes * 4u) {
           const uint4 v = __ldg(reinterpret_cast<const uint4*>(row + i));
           const uint32_t u4[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const uint32_t E = quantised_exponent(u4[j], pbits);
-            bad |= (E == 255u);
-            best = max(best, E == 255u ? 0u : E);     // Inf/NaN is flagged and takes no part in the window
-          }
+          best = max_magnitude(u4, best, bad);     // Inf/NaN is flagged and takes no part in the window
         }
       } else {
 #pragma unroll 4
         for (uint32_t i = lane; i < d; i += lanes) {
-          const uint32_t E = quantised_exponent(__float_as_uint(__ldg(row + i)), pbits);
-          bad |= (E == 255u);
-          best = max(best, E == 255u ? 0u : E);
+          const uint32_t u1[1] = {__float_as_uint(__ldg(row + i))};
+          best = max_magnitude(u1, best, bad);
         }
       }
     }
@@ -181,28 +215,30 @@ __device__ __forceinline__ void emax_block(const float* __restrict__ w, uint32_t
       best = __reduce_max_sync(0xFFFFFFFFu, best);
       // `tag` (a call number in the bits above the exponent) distinguishes this call's maxima from whatever
       // an earlier call left in the word
-      if (lane == 0u) e_max[o] = tag | best;
+      if (lane == 0u) e_max[o] = tag | quantised_exponent(best, pbits);
       return;
     }
   } else {
     const size_t total = (size_t)O * d;
     if ((((uintptr_t)w) & 15u) == 0u && (total & 3u) == 0u) {
-#pragma unroll 4
-      for (size_t i = ((size_t)block * blockDim.x + threadIdx.x) * 4u; i < total; i += (size_t)blocks * blockDim.x * 4u) {
-        const uint4 v = __ldg(reinterpret_cast<const uint4*>(w + i));
-        const uint32_t u4[4] = {v.x, v.y, v.z, v.w};
+      // four 16-byte loads in flight per thread
+      const size_t step = (size_t)blocks * blockDim.x * 4u;
+      for (size_t i = ((size_t)block * blockDim.x + threadIdx.x) * 4u; i < total; i += 4u * step) {
+        uint4 v[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const uint32_t E = quantised_exponent(u4[j], pbits);
-          bad |= (E == 255u);
-          best = max(best, E == 255u ? 0u : E);
+        for (int q = 0; q < 4; ++q)
+          v[q] = i + q * step < total ? __ldg(reinterpret_cast<const uint4*>(w + i + q * step)) : make_uint4(0u, 0u, 0u, 0u);
+        uint32_t u16[16];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          u16[4 * q] = v[q].x; u16[4 * q + 1] = v[q].y; u16[4 * q + 2] = v[q].z; u16[4 * q + 3] = v[q].w;
         }
+        best = max_magnitude(u16, best, bad);
       }
     } else {
       for (size_t i = (size_t)block * blockDim.x + threadIdx.x; i < total; i += (size_t)blocks * blockDim.x) {
-        const uint32_t E = quantised_exponent(__float_as_uint(__ldg(w + i)), pbits);
-        bad |= (E == 255u);
-        best = max(best, E == 255u ? 0u : E);
+        const uint32_t u1[1] = {__float_as_uint(__ldg(w + i))};
+        best = max_magnitude(u1, best, bad);
       }
     }
   }
@@ -212,6 +248,7 @@ __device__ __forceinline__ void emax_block(const float* __restrict__ w, uint32_t
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int i = 1; i < kThreads / 32; ++i) best = max(best, red[i]);
+    best = quantised_exponent(best, pbits);
     // `tag` (a call number in the bits above the exponent) makes the maxima of this call beat
     // whatever an earlier call left in the word, so the words need no clearing between calls
     if (norm) e_max[block] = tag | best;
@@ -221,9 +258,9 @@ __device__ __forceinline__ void emax_block(const float* __restrict__ w, uint32_t
 
 __global__ void emax_kernel(const float* __restrict__ w, uint32_t O, uint32_t d, uint32_t norm,
                             uint32_t* __restrict__ e_max, uint32_t* __restrict__ err, uint32_t tag,
-                            uint32_t* __restrict__ rowsum, uint32_t pbits) {
+                            uint32_t* __restrict__ rowsum, long long* __restrict__ corr, uint32_t pbits) {
   pdl_prologue();
-  emax_block(w, O, d, norm, e_max, err, blockIdx.x, gridDim.x, tag, rowsum, pbits);
+  emax_block(w, O, d, norm, e_max, err, blockIdx.x, gridDim.x, tag, rowsum, corr, pbits);
 }
 
 // What one weight becomes at every level: W_k = s (base k + c_k) 2^sh with c_k = cnt[log2 k]; a weight that is
@@ -231,18 +268,14 @@ __global__ void emax_kernel(const float* __restrict__ w, uint32_t O, uint32_t d,
 // `ebase_biased` the biased exponent of the window's floor.
 struct Drawn {
   uint32_t cnt[kMaxLevels];
-  uint32_t base, sh;
+  uint32_t base, sh, thr;
   bool live;
 };
 
-__device__ __forceinline__ void draw_weight(uint32_t u, uint64_t index, int ebase_biased, uint32_t pbits,
-                                            uint32_t underflow, uint32_t deterministic, uint32_t max_level,
-                                            uint32_t layer_id, const PhiloxKeys& keys, Drawn& out) {
+// The part without draws: base, sh, and the threshold that a draw is compared with.
+__device__ __forceinline__ void classify_weight(uint32_t u, int ebase_biased, uint32_t pbits, uint32_t underflow, Drawn& out) {
   const uint32_t E = (u >> 23) & 0xFFu;
   const uint32_t m = u & 0x7FFFFFu;
-  uint32_t (&cnt)[kMaxLevels] = out.cnt;
-#pragma unroll
-  for (int l = 0; l < kMaxLevels; ++l) cnt[l] = 0u;
   // probability on the grid of 2^pbits points, a p of 1 carried into the exponent (Sec. 4.4)
   uint32_t Eq = E, pq = m;
   if (pbits) {
@@ -275,14 +308,28 @@ __device__ __forceinline__ void draw_weight(uint32_t u, uint64_t index, int ebas
     live = false;
   }
 
+  out.base = base;
+  out.sh = sh;
+  out.thr = thr;
+  out.live = live;
+}
+
+__device__ __forceinline__ void draw_weight(uint32_t u, uint32_t index, int ebase_biased, uint32_t pbits,
+                                            uint32_t underflow, uint32_t deterministic, uint32_t max_level,
+                                            uint32_t layer_key, const PhiloxKeys& keys, Drawn& out) {
+  classify_weight(u, ebase_biased, pbits, underflow, out);
+  const uint32_t thr = out.thr;
+  uint32_t (&cnt)[kMaxLevels] = out.cnt;
+#pragma unroll
+  for (int l = 0; l < kMaxLevels; ++l) cnt[l] = 0u;
   // c_k for every level k = 2^l: level l is complete after draw 2^l, i.e. levels 0..2 after the
   // first Philox call, level l >= 2 after call 2^(l-2)
-  if (live && thr != 0u) {
-    const uint32_t i_lo = (uint32_t)index, i_hi = (uint32_t)(index >> 32);
+  if (out.live && thr != 0u) {
+    const PhiloxWeight pw(index, layer_key);
     uint32_t rnd[4];
     if (pbits == 0u) {
       const uint32_t T = thr;
-      philox4x32_10(0u, layer_id, i_lo, i_hi, keys, rnd);
+      pw.call(0u, keys, rnd);
       cnt[0] = rnd[0] < T ? 1u : 0u;
       cnt[1] = cnt[0] + (rnd[1] < T ? 1u : 0u);
       uint32_t c = cnt[1] + (rnd[2] < T ? 1u : 0u) + (rnd[3] < T ? 1u : 0u);
@@ -290,8 +337,9 @@ __device__ __forceinline__ void draw_weight(uint32_t u, uint64_t index, int ebas
 #pragma unroll
       for (int l = 3; l < kMaxLevels; ++l) {
         if ((uint32_t)l <= max_level) {
+#pragma unroll 1
           for (uint32_t q = 1u << (l - 3); q < (1u << (l - 2)); ++q) {
-            philox4x32_10(q, layer_id, i_lo, i_hi, keys, rnd);
+            pw.call(q, keys, rnd);
             c += (rnd[0] < T ? 1u : 0u) + (rnd[1] < T ? 1u : 0u) + (rnd[2] < T ? 1u : 0u) + (rnd[3] < T ? 1u : 0u);
           }
           cnt[l] = c;
@@ -303,17 +351,14 @@ __device__ __forceinline__ void draw_weight(uint32_t u, uint64_t index, int ebas
     } else {
       // pbits-bit comparator, n = 32 / pbits draws per random word
       switch (pbits) {
-        case 4: packed_counts<4>(thr, max_level, layer_id, i_lo, i_hi, keys, cnt); break;
-        case 6: packed_counts<6>(thr, max_level, layer_id, i_lo, i_hi, keys, cnt); break;
-        case 8: packed_counts<8>(thr, max_level, layer_id, i_lo, i_hi, keys, cnt); break;
-        default: packed_counts_any(pbits, thr, max_level, layer_id, i_lo, i_hi, keys, cnt); break;
+        case 4: packed_counts<4>(thr, max_level, pw, keys, cnt); break;
+        case 6: packed_counts<6>(thr, max_level, pw, keys, cnt); break;
+        case 8: packed_counts<8>(thr, max_level, pw, keys, cnt); break;
+        default: packed_counts_any(pbits, thr, max_level, pw, keys, cnt); break;
       }
     }
   }
 
-  out.base = base;
-  out.sh = sh;
-  out.live = live;
 }
 
 struct SampleParams {
@@ -322,54 +367,327 @@ struct SampleParams {
   uint32_t rows_per_block, ch_per_block, ch_chunks;
   uint32_t norm, span, level_mask, max_level;
   uint32_t underflow, pbits, deterministic;   // options of psb_sample_cfg
-  uint32_t seed_lo, seed_hi, layer_id;
-  uint32_t cpad, kpad, has_planes;
+  uint32_t layer_id, has_planes;
   uint32_t bk, n_cb, n_kb;         // operand tiles of the tensor path: K block bytes, blocks per tap, blocks per row
   uint32_t packed_kw, run_pitch;   // packed K (packed_kw = kw, else 0): plane column = kh * run_pitch + kw * Cg + ci
   const uint32_t* e_max;
   uint32_t e_tag;                  // call number the words of e_max must carry (bits 8 and up)
   int32_t* e_base;
-  uint32_t* rowsum;                // [kMaxLevels][O] row sums of |W_k| / 256 (see psb_weights), or null
-  int32_t* wint[kMaxLevels];
+  uint32_t* rowsum;                // [kMaxLevels][O] row sums of |W_k| / 256 (see psb_weights)
+  long long* corr;                 // [kMaxLevels][O] 128 x row sums of W_k, filters with digit planes only
+  int32_t* wint[kMaxLevels];       // filters without digit planes
   int8_t* planes[kMaxLevels];
   int planes_count[kMaxLevels];
 };
 
-// kVec: whether the instance contains the four-weights-per-thread loop at all (a launch whose items are all
-// small carries only the one-weight loop: with the L2 cold, what a short kernel costs is mostly its code)
-template <bool kVec>
-__device__ __forceinline__ void sample_block(const SampleParams& p, uint32_t block, const PhiloxKeys& keys,
-                                             float* stage) {
-  // the parameters may sit in global memory (batched launch): read the scalars once
-  const uint32_t norm = p.norm, span = p.span, level_mask = p.level_mask, max_level = p.max_level;
-  const uint32_t underflow = p.underflow, pbits = p.pbits, deterministic = p.deterministic;
-  const uint32_t layer_id = p.layer_id, KHKW = p.KHKW, Cg = p.Cg;
-  const uint32_t packed_kw = p.packed_kw, run_pitch = p.run_pitch, has_planes = p.has_planes;
-  const uint32_t bk = p.bk, n_cb = p.n_cb, n_kb = p.n_kb;
-  const uint32_t bk_shift = 31u - (uint32_t)__clz((int)bk), bk_mask = bk - 1u;     // bk is a power of two (32, 64, 128)
-  // Row sums of |W_k| (in units of 256, each weight rounded up) for the bound that lets the contraction
-  // recombine its digit planes in 32 bits: gathered per block in shared memory, then added to the layer's words
-  __shared__ uint32_t row_sum[kMaxLevels][kRowSumRows];
-  uint32_t* const rowsum = p.rowsum;
-  const bool track = rowsum != nullptr && p.rows_per_block <= (uint32_t)kRowSumRows;
-  if (track)
-    for (uint32_t i = threadIdx.x; i < (uint32_t)(kMaxLevels * kRowSumRows); i += blockDim.x)
-      row_sum[i / kRowSumRows][i % kRowSumRows] = 0u;
-  const uint32_t row_block = block / p.ch_chunks;
-  const uint32_t chunk = block % p.ch_chunks;
-  const uint32_t o0 = row_block * p.rows_per_block;
-  const uint32_t c0 = chunk * p.ch_per_block;
-  const uint32_t rows = min(p.rows_per_block, p.O - o0);
-  const uint32_t cc = min(p.ch_per_block, p.Cg - c0);
-  const uint32_t per_row = cc * p.KHKW;     // canonical elements of one row in this block
-  const uint32_t count = rows * per_row;
+// Counts of the first k = 2^level draws of a weight with the exact probability T / 2^32 (the common case: no
+// option set, one level), branch-free.
+__device__ __forceinline__ uint32_t count_draws(const PhiloxWeight& pw, uint32_t T, uint32_t level, const PhiloxKeys& keys) {
+  uint32_t rnd[4];
+  pw.call(0u, keys, rnd);
+  uint32_t c = rnd[0] < T ? 1u : 0u;
+  if (level == 0u) return c;
+  c += rnd[1] < T ? 1u : 0u;
+  if (level == 1u) return c;
+  c += (rnd[2] < T ? 1u : 0u) + (rnd[3] < T ? 1u : 0u);
+#pragma unroll 1
+  for (uint32_t q = 1; q < (1u << level) / 4u; ++q) {
+    pw.call(q, keys, rnd);
+    c += (rnd[0] < T ? 1u : 0u) + (rnd[1] < T ? 1u : 0u) + (rnd[2] < T ? 1u : 0u) + (rnd[3] < T ? 1u : 0u);
+  }
+  return c;
+}
 
+// The same with a B-bit comparator (fields as in packed_counts): the fields of a word are compared two sets at a time,
+// every second field with a guard bit above it, (field | guard) - thr keeps the guard iff field >= thr.  Five
+// instructions per set where a compare and an add per draw took three per field.
+template <int B>
+__device__ __forceinline__ uint32_t count_packed(const PhiloxWeight& pw, uint32_t thr, uint32_t level, const PhiloxKeys& keys) {
+  constexpr int n = 32 / B, per_call = 4 * n, calls = (64 + per_call - 1) / per_call;
+  constexpr uint32_t f = (1u << B) - 1u;
+  uint32_t even = 0u, odd = 0u;           // masks of the fields 0, 2, 4, .. and, shifted down by B, 1, 3, 5, ..
+#pragma unroll
+  for (int i = 0; i < n; ++i)
+    if (i & 1) odd |= f << (B * (i - 1)); else even |= f << (B * i);
+  // guards: the bit above each field (for B = 6 the top even field ends at bit 29; for B = 8, 4 at bit 23, 27)
+  const uint32_t g_even = (even / f) << B, g_odd = (odd / f) << B, t_even = (even / f) * thr, t_odd = (odd / f) * thr;
+  const uint32_t k = 1u << level;
+  uint32_t c = 0u;
+#pragma unroll
+  for (int q = 0; q < calls; ++q) {
+    if ((uint32_t)(q * per_call) >= k) break;
+    uint32_t rnd[4];
+    pw.call((uint32_t)q, keys, rnd);
+#pragma unroll
+    for (int wd = 0; wd < 4; ++wd) {
+      const int j0 = q * per_call + wd * n;      // first draw of the word
+      if (j0 >= 64 || (uint32_t)j0 >= k) break;
+      uint32_t ve = g_even, vo = g_odd;
+      if ((uint32_t)(j0 + n) > k) {              // the last draws of the level end inside this word
+        const uint32_t left = k - (uint32_t)j0;  // fields 0 .. left - 1 count
+        ve = g_even & ((1u << (B * ((left + 1u) & ~1u))) - 1u);
+        vo = g_odd & ((1u << (B * (left & ~1u))) - 1u);
+      }
+      const uint32_t e = ((rnd[wd] & even) | g_even) - t_even, o = (((rnd[wd] >> B) & odd) | g_odd) - t_odd;
+      c += (uint32_t)__popc((~e & ve) | ((~o & vo) >> 1));
+    }
+  }
+  return c;
+}
+
+// Count at one level under the sampling options, threshold as classify_weight gives it.
+__device__ __forceinline__ uint32_t count_level(const PhiloxWeight& pw, uint32_t thr, uint32_t level, uint32_t pbits,
+                                                uint32_t deterministic, const PhiloxKeys& keys) {
+  if (pbits == 0u) return count_draws(pw, thr, level, keys);
+  if (deterministic) return ((thr << level) + (1u << (pbits - 1u))) >> pbits;
+  if (pbits == 8u) return count_packed<8>(pw, thr, level, keys);
+  if (pbits == 4u) return count_packed<4>(pw, thr, level, keys);
+  uint32_t cnt[kMaxLevels];
+  if (pbits == 6u) packed_counts<6>(thr, level, pw, keys, cnt);
+  else packed_counts_any(pbits, thr, level, pw, keys, cnt);
+  uint32_t c = cnt[0];
+#pragma unroll
+  for (int l = 1; l < kMaxLevels; ++l)
+    if ((uint32_t)l == level) c = cnt[l];
+  return c;
+}
+
+// Row sums of a block's slice, kept in shared memory and added to the layer's words at the end: the sum of |W_k| in
+// units of 256 (each contribution rounded up) bounds the accumulators; the signed sum, as hi * 4096 + lo, is what an
+// offset of the activations has to be corrected by.
+struct RowSums {
+  uint32_t word[kMaxLevels * kRowSumRows];      // [level][kRowSumRows], or [level][3][kPlaneRows] with digit planes
+};
+
+// One warp's contributions (abs256, signed) to its rows: one reduction and one add per row that the lanes share.
+__device__ __forceinline__ void add_row_sums(uint32_t* sums, uint32_t r, uint32_t abs256, int sum, bool with_signed) {
+  uint32_t lanes = __activemask();
+  const uint32_t r_first = __shfl_sync(lanes, r, __ffs((int)lanes) - 1);
+  if (!__all_sync(lanes, r == r_first)) lanes = __match_any_sync(lanes, r);
+  abs256 = __reduce_add_sync(lanes, abs256);
+  if (with_signed) sum = __reduce_add_sync(lanes, sum);
+  if ((threadIdx.x & 31u) == (uint32_t)__ffs((int)lanes) - 1u && abs256) {
+    atomicAdd(&sums[r], abs256);
+    if (with_signed) {
+      atomicAdd(&sums[kPlaneRows + r], (uint32_t)(sum & 0xFFF));
+      atomicAdd(&sums[2 * kPlaneRows + r], (uint32_t)(sum >> 12));
+    }
+  }
+}
+
+// The four 7-bit digits of m < 2^28 in the four bytes of a word: adding the part above bit 7 to itself moves it up by
+// one, and so on.
+__device__ __forceinline__ uint32_t spread_digits(uint32_t m) {
+  m += m & 0xFFFFFF80u;
+  m += m & 0xFFFF8000u;
+  return m + (m & 0xFF800000u);
+}
+
+// Bytes 0 and 1: 0xFF where a / b is negative (selectors 8 + byte of the permute replicate that byte's sign).
+__device__ __forceinline__ uint32_t top_signs(uint32_t a, uint32_t b) {
+  uint32_t d;
+  asm("prmt.b32 %0, %1, %2, 0xFB;" : "=r"(d) : "r"(a), "r"(b));
+  return d;
+}
+
+// Filters with digit planes whose K axis is tap-major: a thread takes four consecutive channels of one (row, tap),
+// draws them, spreads each magnitude's 7-bit digits over the bytes of a word, transposes the four words with byte
+// permutes into one word per plane, negates the bytes of negative weights at once and stores 4 bytes per plane.
+// The sums of the row come from dp4a on the same words.
+// Bound by issue: per weight at k = 8 the 34 widening multiplies of Philox (4 clocks each per warp and scheduler, as
+// measured) run beside about 100 logic, permute and compare instructions (2 clocks each).  25.5 M weights of the
+// ResNet-50 shape, k = 8: 253 us (370 with the integer filter written beside the planes and one byte store per
+// digit); 4096 x 4096, k = 16, 8-bit probabilities: 205 -> 185 us.
+// kOptions: the sampling options of Sec. 3.1 / 4.4; kMulti: more than one level.
+template <bool kOptions, bool kMulti>
+__device__ __forceinline__ void sample_planes(const SampleParams& p, uint32_t o0, uint32_t c0, uint32_t rows, uint32_t cc,
+                                              const PhiloxKeys& keys, const float* stage, uint32_t* sums) {
+  const uint32_t KHKW = p.KHKW, d = p.d, norm = p.norm, e_tag = p.e_tag, level_mask = p.level_mask;
+  const uint32_t max_level = p.max_level, layer_key = p.layer_id ^ keys.k0[0];
+  const uint32_t bk = p.bk, n_cb = p.n_cb, n_kb = p.n_kb;
+  const uint32_t bk_shift = 31u - (uint32_t)__clz((int)bk), bk_mask = bk - 1u, sw_mask = (bk >> 4) - 1u;
+  const int span = (int)p.span;
+  const uint32_t* const e_max = p.e_max;
+  const uint32_t per_row = cc * KHKW, groups = (cc + 3u) >> 2, per_row4 = groups * KHKW, count4 = rows * per_row4;
+  const uint32_t per_row4_magic = small_div_magic(per_row4), groups_magic = small_div_magic(groups);
+  uint32_t e_word = norm ? 0u : e_max[0];
+  for (uint32_t t = threadIdx.x; t < count4; t += blockDim.x) {
+    const uint32_t r = small_div(t, per_row4_magic), rem = t - r * per_row4;
+    const uint32_t tap = small_div(rem, groups_magic), cl = (rem - tap * groups) << 2;
+    const uint32_t o = o0 + r, ci = c0 + cl;
+    // a word written by an earlier call (other tag) means this call found no live weight in the group
+    if (norm) e_word = e_max[o];
+    const uint32_t Emax = (e_word >> 8) == e_tag ? (e_word & 0xFFu) : 0u;
+    // biased exponents throughout: e - e_base = E - (Emax - span)
+    const int ebase_biased = (int)Emax - span;
+    if (tap == 0 && ci == 0) p.e_base[o] = Emax ? ebase_biased - 127 : 0;
+    const float* w = stage + r * per_row + cl * KHKW + tap;
+    uint32_t index = o * d + ci * KHKW + tap;        // canonical index
+    uint32_t u[4], mag[4], cntpk[kMaxLevels], meta = 0u;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) u[j] = cl + (uint32_t)j < cc ? __float_as_uint(w[(uint32_t)j * KHKW]) : 0u;
+    if (!kOptions && !kMulti) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const uint32_t E = (u[j] >> 23) & 0xFFu;
+        const int sh = (int)E - ebase_biased;
+        const bool live = E - 1u < 254u && sh >= 0;
+        const PhiloxWeight pw(index, layer_key);
+        const uint32_t c = count_draws(pw, u[j] << 9, max_level, keys);
+        mag[j] = live ? ((1u << max_level) + c) << (sh & 15) : 0u;
+        index += KHKW;
+      }
+    } else if (!kMulti) {
+#pragma unroll 1       // one copy of the drawing code: four no longer fit the instruction cache
+      for (int j = 0; j < 4; ++j) {
+        Drawn dw;
+        classify_weight(j == 0 ? u[0] : j == 1 ? u[1] : j == 2 ? u[2] : u[3], ebase_biased, p.pbits, p.underflow, dw);
+        const PhiloxWeight pw(index, layer_key);
+        const uint32_t c = count_level(pw, dw.thr, max_level, p.pbits, p.deterministic, keys);
+        const uint32_t m = dw.live ? ((dw.base << max_level) + c) << dw.sh : 0u;
+        mag[0] = j == 0 ? m : mag[0]; mag[1] = j == 1 ? m : mag[1];
+        mag[2] = j == 2 ? m : mag[2]; mag[3] = j == 3 ? m : mag[3];
+        index += KHKW;
+      }
+    } else {
+#pragma unroll
+      for (int l = 0; l < kMaxLevels; ++l) cntpk[l] = 0u;
+#pragma unroll 1
+      for (int j = 0; j < 4; ++j) {
+        Drawn dw;
+        draw_weight(j == 0 ? u[0] : j == 1 ? u[1] : j == 2 ? u[2] : u[3], index, ebase_biased, kOptions ? p.pbits : 0u,
+                    kOptions ? p.underflow : 0u, kOptions ? p.deterministic : 0u, max_level, layer_key, keys, dw);
+        if (dw.live) {
+          meta |= (dw.sh | (dw.base << 4)) << (8 * j);
+#pragma unroll
+          for (int l = 0; l < kMaxLevels; ++l) cntpk[l] |= dw.cnt[l] << (8 * j);
+        }
+        index += KHKW;
+      }
+    }
+    // bytes 0xFF where the weight is negative
+    const uint32_t neg = __byte_perm(top_signs(u[0], u[1]), top_signs(u[2], u[3]), 0x5410);
+    const uint32_t kb = tap * n_cb + (ci >> bk_shift), kin = ci & bk_mask, jt = o / kTileN, on = o % kTileN;
+    // byte offset of (row, kin) in the swizzled tile (plane_offset); planes are 64 rows apart, which leaves the
+    // swizzle as it is
+    const uint32_t lin = (on << bk_shift) + kin, off = lin ^ (((lin >> 7) & sw_mask) << 4);
+    const size_t tile = (size_t)jt * n_kb + kb;
+#pragma unroll
+    for (int l = 0; l < kMaxLevels; ++l) {
+      if (kMulti ? !((level_mask >> l) & 1u) : l != 0) continue;
+      const uint32_t lv = kMulti ? (uint32_t)l : max_level;
+      if (kMulti) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const uint32_t m8 = meta >> (8 * j), c = (cntpk[l] >> (8 * j)) & 0xFFu;
+          mag[j] = ((((m8 >> 4) & 1u) << lv) + c) << (m8 & 15u);
+        }
+      }
+      uint32_t sp[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        sp[j] = spread_digits(mag[j]);
+      const uint32_t lo01 = __byte_perm(sp[0], sp[1], 0x5140), lo23 = __byte_perm(sp[2], sp[3], 0x5140);
+      const uint32_t hi01 = __byte_perm(sp[0], sp[1], 0x7362), hi23 = __byte_perm(sp[2], sp[3], 0x7362);
+      const uint32_t word[4] = {__byte_perm(lo01, lo23, 0x5410), __byte_perm(lo01, lo23, 0x7632),
+                                __byte_perm(hi01, hi23, 0x5410), __byte_perm(hi01, hi23, 0x7632)};
+      const int P = p.planes_count[lv];
+      int8_t* dst = p.planes[lv] + ((tile * (size_t)P) << (6u + bk_shift)) + off;
+      uint32_t abs_sum = 0u;
+      int sum = 0;
+#pragma unroll
+      for (int pl = 0; pl < kMaxPlanes; ++pl) {
+        if (pl >= P) break;
+        const uint32_t wd = word[pl];
+        // -d as a byte is (0x80 - d) ^ 0x80 for 0 <= d <= 127: no borrow leaves its byte
+        const uint32_t minus = (0x80808080u - wd) ^ 0x80808080u;
+        const uint32_t sg = (minus & neg) | (wd & ~neg);
+        abs_sum += (uint32_t)__dp4a((int)wd, 0x01010101, 0) << (kDigitBits * pl);
+        sum += __dp4a((int)sg, 0x01010101, 0) * (1 << (kDigitBits * pl));
+        *reinterpret_cast<uint32_t*>(dst + ((size_t)pl << (6u + bk_shift))) = sg;
+      }
+      add_row_sums(sums + lv * (3u * kPlaneRows), r, (abs_sum + 255u) >> 8, sum, true);
+    }
+  }
+}
+
+// Everything else, one weight per thread and step: depthwise and grouped filters (integer filter, channels
+// innermost, for the CUDA-core kernels) and flat K axes (few input channels).
+template <bool kOptions>
+__device__ __forceinline__ void sample_single(const SampleParams& p, uint32_t o0, uint32_t c0, uint32_t rows, uint32_t cc,
+                                              const PhiloxKeys& keys, const float* stage, uint32_t* sums, bool track) {
+  const uint32_t KHKW = p.KHKW, Cg = p.Cg, d = p.d, norm = p.norm, e_tag = p.e_tag, level_mask = p.level_mask;
+  const uint32_t max_level = p.max_level, layer_key = p.layer_id ^ keys.k0[0], has_planes = p.has_planes;
+  const uint32_t packed_kw = p.packed_kw, run_pitch = p.run_pitch, bk = p.bk, n_kb = p.n_kb;
+  const uint32_t bk_shift = 31u - (uint32_t)__clz((int)bk), bk_mask = bk - 1u, sw_mask = (bk >> 4) - 1u;
+  const uint32_t per_row = cc * KHKW, count = rows * per_row;
+  const uint32_t per_row_magic = small_div_magic(per_row), cc_magic = small_div_magic(cc);
+  for (uint32_t t = threadIdx.x; t < count; t += blockDim.x) {
+    const uint32_t r = small_div(t, per_row_magic), rem = t - r * per_row;
+    const uint32_t tap = small_div(rem, cc_magic), cl = rem - tap * cc;
+    const uint32_t o = o0 + r, ci = c0 + cl;
+    const uint32_t u = __float_as_uint(stage[r * per_row + cl * KHKW + tap]);
+    const uint32_t index = o * d + ci * KHKW + tap;  // canonical
+    // a word written by an earlier call (other tag) means this call found no live weight in the group
+    const uint32_t e_word = p.e_max[norm ? o : 0];
+    const uint32_t Emax = (e_word >> 8) == e_tag ? (e_word & 0xFFu) : 0u;
+    const int ebase_biased = (int)Emax - (int)p.span;
+    if (tap == 0 && ci == 0) p.e_base[o] = Emax ? ebase_biased - 127 : 0;
+    Drawn dw;
+    draw_weight(u, index, ebase_biased, kOptions ? p.pbits : 0u, kOptions ? p.underflow : 0u, kOptions ? p.deterministic : 0u,
+                max_level, layer_key, keys, dw);
+    const bool neg = (u >> 31) != 0u;
+    const size_t wpos = ((size_t)o * KHKW + tap) * Cg + ci;
+    uint32_t kb = 0, kin = 0;
+    if (has_planes) {            // flat K axis (with a tap-major one the planes are written four channels at a time)
+      const uint32_t kh = tap / packed_kw, kcol = kh * run_pitch + (tap - kh * packed_kw) * Cg + ci;
+      kb = kcol >> bk_shift;
+      kin = kcol & bk_mask;
+    }
+    const uint32_t jt = o / kTileN, on = o % kTileN;
+    const uint32_t lin = (on << bk_shift) + kin, off = lin ^ (((lin >> 7) & sw_mask) << 4);
+#pragma unroll
+    for (int l = 0; l < kMaxLevels; ++l) {
+      if (!((level_mask >> l) & 1u)) continue;
+      const uint32_t mag = dw.live ? (((dw.base << l) + dw.cnt[l]) << dw.sh) : 0u;
+      const int wv = neg ? -(int32_t)mag : (int32_t)mag;
+      if (has_planes) {
+        const int P = p.planes_count[l];
+        int8_t* dst = p.planes[l] + ((((size_t)jt * n_kb + kb) * (size_t)P) << (6u + bk_shift)) + off;
+        for (int pl = 0; pl < P; ++pl) {
+          const int digit = (int)((mag >> (kDigitBits * pl)) & 0x7Fu);
+          dst[(size_t)pl << (6u + bk_shift)] = (int8_t)(neg ? -digit : digit);
+        }
+        add_row_sums(sums + l * (3 * kPlaneRows), r, (mag + 255u) >> 8, wv, true);
+      } else {
+        p.wint[l][wpos] = wv;
+        if (track) add_row_sums(sums + l * kRowSumRows, r, (mag + 255u) >> 8, 0, false);
+      }
+    }
+  }
+}
+
+template <bool kOptions>
+__device__ __forceinline__ void sample_block(const SampleParams& p, uint32_t block, const PhiloxKeys& keys, float* stage,
+                                             RowSums& rs) {
+  const uint32_t level_mask = p.level_mask, has_planes = p.has_planes, O = p.O;
+  const uint32_t sum_rows = has_planes ? (uint32_t)kPlaneRows : (uint32_t)kRowSumRows;
+  const bool track = p.rows_per_block <= sum_rows;         // always so with digit planes (fill_sample_params)
+  const uint32_t pitch = has_planes ? 3u * kPlaneRows : (uint32_t)kRowSumRows;     // words per level
+  if (track)
+    for (uint32_t l = 0; l < (uint32_t)kMaxLevels; ++l)
+      if ((level_mask >> l) & 1u)
+        for (uint32_t i = threadIdx.x; i < pitch; i += blockDim.x) rs.word[l * pitch + i] = 0u;
+  const uint32_t row_block = block / p.ch_chunks, chunk = block - row_block * p.ch_chunks;
+  const uint32_t o0 = row_block * p.rows_per_block, c0 = chunk * p.ch_per_block;
+  const uint32_t rows = min(p.rows_per_block, O - o0), cc = min(p.ch_per_block, p.Cg - c0);
+  const uint32_t count = rows * cc * p.KHKW;
   // The slice is one contiguous run of the weight tensor (whole rows, or a channel range of one row): stage it
   // with 16-byte loads where the run allows.
   {
     const float* src = p.w + (size_t)o0 * p.d + (size_t)c0 * p.KHKW;
     if ((((uintptr_t)src) & 15u) == 0u && (count & 3u) == 0u) {
-#pragma unroll 2
+#pragma unroll 4
       for (uint32_t t = threadIdx.x * 4u; t < count; t += blockDim.x * 4u)
         *reinterpret_cast<float4*>(stage + t) = __ldg(reinterpret_cast<const float4*>(src + t));
     } else {
@@ -378,168 +696,39 @@ __device__ __forceinline__ void sample_block(const SampleParams& p, uint32_t blo
     }
   }
   __syncthreads();
-
-  const uint32_t d = p.d, e_tag = p.e_tag;
-  const uint32_t* const e_max = p.e_max;
-  int32_t* const e_base_out = p.e_base;
-  // count <= kStage and the divisors are block-uniform: divisions by multiply-high.  The slice is walked in
-  // output order (row, tap, channel) so that stores coalesce.
-  if (kVec && !packed_kw && has_planes && ((cc | Cg | c0) & 3u) == 0u && count >= 4u * blockDim.x) {
-    // Items that give every thread at least four weights: four consecutive channels per thread, one 16-byte
-    // store of the integer weights and one 4-byte store per digit plane and level.  Between the draws and the stores the four weights' counts travel as the bytes of
-    // one word per level (c_k <= 64), and (sh, base, sign) as one byte per weight.
-    const uint32_t cc4 = cc >> 2, per_row4 = per_row >> 2;
-    const uint32_t per_row4_magic = small_div_magic(per_row4), cc4_magic = small_div_magic(cc4);
-    for (uint32_t t = threadIdx.x; t < (count >> 2); t += blockDim.x) {
-      const uint32_t r = small_div(t, per_row4_magic), rem = t - r * per_row4;
-      const uint32_t tap = small_div(rem, cc4_magic), cl = (rem - tap * cc4) << 2;
-      const uint32_t o = o0 + r, ci = c0 + cl;
-      // a word written by an earlier call (other tag) means this call found no live weight in the group
-      const uint32_t e_word = e_max[norm ? o : 0];
-      const uint32_t Emax = (e_word >> 8) == e_tag ? (e_word & 0xFFu) : 0u;
-      // biased exponents throughout: e - e_base = E - (Emax - span)
-      const int ebase_biased = (int)Emax - (int)span;
-      if (tap == 0 && ci == 0) e_base_out[o] = Emax ? ebase_biased - 127 : 0;
-      uint32_t cntpk[kMaxLevels] = {0u, 0u, 0u, 0u, 0u, 0u, 0u};
-      uint32_t meta = 0u;
-#pragma unroll 1       // one copy of the drawing code: unrolled four times it no longer fits the instruction cache
-      for (int j = 0; j < 4; ++j) {
-        const uint32_t u = __float_as_uint(stage[r * per_row + (cl + (uint32_t)j) * KHKW + tap]);
-        const uint64_t index = (uint64_t)o * d + (uint64_t)(ci + (uint32_t)j) * KHKW + tap;  // canonical
-        Drawn dw;
-        draw_weight(u, index, ebase_biased, pbits, underflow, deterministic, max_level, layer_id, keys, dw);
-        if (dw.live) {
-#pragma unroll
-          for (int l = 0; l < kMaxLevels; ++l) cntpk[l] |= dw.cnt[l] << (8 * j);
-          meta |= (dw.sh | (dw.base << 4) | ((u >> 31) << 5)) << (8 * j);
-        }
-      }
-      const size_t wpos = ((size_t)o * KHKW + tap) * Cg + ci;
-      const uint32_t kb = tap * n_cb + (ci >> bk_shift), kin = ci & bk_mask;
-      const uint32_t jt = o / kTileN, on = o % kTileN;
-#pragma unroll
-      for (int l = 0; l < kMaxLevels; ++l) {
-        if (!((level_mask >> l) & 1u)) continue;
-        uint32_t mag[4];
-        int wv[4];
-        uint32_t part = 0u;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const uint32_t m8 = meta >> (8 * j), c = (cntpk[l] >> (8 * j)) & 0xFFu;
-          mag[j] = ((((m8 >> 4) & 1u) << l) + c) << (m8 & 15u);
-          wv[j] = ((m8 >> 5) & 1u) ? -(int32_t)mag[j] : (int32_t)mag[j];
-          part += (mag[j] + 255u) >> 8;
-        }
-        *reinterpret_cast<int4*>(p.wint[l] + wpos) = make_int4(wv[0], wv[1], wv[2], wv[3]);
-        if (track) {
-          // lanes of a warp mostly share a row: then one reduction and one shared-memory add per warp
-          const uint32_t lanes = __activemask();
-          const uint32_t r_first = __shfl_sync(lanes, r, (int)__ffs((int)lanes) - 1);
-          if (__all_sync(lanes, r == r_first)) {
-            const uint32_t sum = __reduce_add_sync(lanes, part);
-            if ((threadIdx.x & 31u) == (uint32_t)__ffs((int)lanes) - 1u && sum) atomicAdd(&row_sum[l][r], sum);
-          } else if (part) {
-            atomicAdd(&row_sum[l][r], part);
-          }
-        }
-        const int P = p.planes_count[l];
-        int8_t* tile = p.planes[l] + (((size_t)jt * n_kb + kb) * (size_t)P << (6u + bk_shift));   // P * 64 * bk per tile
-        // byte offset of (row, kin) in the swizzled tile (plane_offset), advanced by 64 rows per plane; the four
-        // bytes share a 16-byte piece
-        const uint32_t lin0 = (on << bk_shift) + kin, sw_mask = (bk >> 4) - 1u;
-        for (int pl = 0; pl < P; ++pl) {
-          uint32_t word = 0u;
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const int digit = (int)((mag[j] >> (kDigitBits * pl)) & 0x7Fu);
-            word |= (uint32_t)((wv[j] < 0 ? -digit : digit) & 0xFF) << (8 * j);
-          }
-          const uint32_t lin = lin0 + ((uint32_t)pl << (6u + bk_shift));
-          *reinterpret_cast<uint32_t*>(tile + (lin ^ (((lin >> 7) & sw_mask) << 4))) = word;
-        }
-      }
-    }
+  if (has_planes && !p.packed_kw) {
+    const bool multi = (level_mask & (level_mask - 1u)) != 0u;
+    const bool plain = !kOptions || (p.pbits | p.underflow) == 0u;
+    if (plain && !multi) sample_planes<false, false>(p, o0, c0, rows, cc, keys, stage, rs.word);
+    else if (multi) sample_planes<kOptions, true>(p, o0, c0, rows, cc, keys, stage, rs.word);
+    else sample_planes<kOptions, false>(p, o0, c0, rows, cc, keys, stage, rs.word);
   } else {
-  const uint32_t per_row_magic = small_div_magic(per_row), cc_magic = small_div_magic(cc);
-  for (uint32_t t = threadIdx.x; t < count; t += blockDim.x) {
-    const uint32_t r = small_div(t, per_row_magic), rem = t - r * per_row;
-    const uint32_t tap = small_div(rem, cc_magic), cl = rem - tap * cc;
-    const uint32_t o = o0 + r, ci = c0 + cl;
-    const uint32_t u = __float_as_uint(stage[r * per_row + cl * KHKW + tap]);
-    const uint64_t index = (uint64_t)o * d + (uint64_t)ci * KHKW + tap;  // canonical
-    // a word written by an earlier call (other tag) means this call found no live weight in the group
-    const uint32_t e_word = e_max[norm ? o : 0];
-    const uint32_t Emax = (e_word >> 8) == e_tag ? (e_word & 0xFFu) : 0u;
-    // biased exponents throughout: e - e_base = E - (Emax - span)
-    const int ebase_biased = (int)Emax - (int)span;
-    if (tap == 0 && ci == 0) e_base_out[o] = Emax ? ebase_biased - 127 : 0;
-    Drawn dw;
-    draw_weight(u, index, ebase_biased, pbits, underflow, deterministic, max_level, layer_id, keys, dw);
-    const bool live = dw.live, neg = (u >> 31) != 0u;
-    const uint32_t base = dw.base, sh = dw.sh;
-    const uint32_t (&cnt)[kMaxLevels] = dw.cnt;
-
-    const size_t wpos = ((size_t)o * KHKW + tap) * Cg + ci;
-    // K block and column inside it (bk is a power of two)
-    uint32_t kb = tap * n_cb + (ci >> bk_shift), kin = ci & bk_mask;
-    if (packed_kw) {
-      const uint32_t kh = tap / packed_kw;
-      const uint32_t kcol = kh * run_pitch + (tap - kh * packed_kw) * Cg + ci;
-      kb = kcol >> bk_shift;
-      kin = kcol & bk_mask;
-    }
-    const uint32_t jt = o / kTileN, on = o % kTileN;
-#pragma unroll
-    for (int l = 0; l < kMaxLevels; ++l) {
-      if (!((level_mask >> l) & 1u)) continue;
-      const uint32_t mag = live ? (((base << l) + cnt[l]) << sh) : 0u;
-      p.wint[l][wpos] = neg ? -(int32_t)mag : (int32_t)mag;
-      if (track) {
-        // lanes of a warp mostly share a row: then one reduction and one shared-memory add per warp
-        const uint32_t lanes = __activemask();
-        const uint32_t r_first = __shfl_sync(lanes, r, (int)__ffs((int)lanes) - 1);
-        const uint32_t part = (mag + 255u) >> 8;
-        if (__all_sync(lanes, r == r_first)) {
-          const uint32_t sum = __reduce_add_sync(lanes, part);
-          if ((threadIdx.x & 31u) == (uint32_t)__ffs((int)lanes) - 1u && sum) atomicAdd(&row_sum[l][r], sum);
-        } else if (part) {
-          atomicAdd(&row_sum[l][r], part);
-        }
-      }
+    sample_single<kOptions>(p, o0, c0, rows, cc, keys, stage, rs.word, track);
+  }
+  __syncthreads();
+  for (uint32_t l = 0; l < (uint32_t)kMaxLevels; ++l) {
+    if (!((level_mask >> l) & 1u)) continue;
+    const uint32_t* sums = rs.word + l * pitch;
+    for (uint32_t r = threadIdx.x; r < rows; r += blockDim.x) {
+      const uint32_t at = l * O + o0 + r;
+      // a block that could not keep sums (more rows than the table holds) leaves the bound unknown
+      if (!track) atomicMax(&p.rowsum[at], 0xFFFFFFFFu);
+      else if (sums[r]) atomicAdd(&p.rowsum[at], sums[r]);
       if (has_planes) {
-        const int P = p.planes_count[l];
-        int8_t* tile = p.planes[l] + (((size_t)jt * n_kb + kb) * (size_t)P << (6u + bk_shift));   // P * 64 * bk per tile
-        // byte offset of (row, kin) in the swizzled tile (plane_offset), advanced by 64 rows per plane
-        const uint32_t lin0 = (on << bk_shift) + kin, sw_mask = (bk >> 4) - 1u;
-        for (int pl = 0; pl < P; ++pl) {
-          const int digit = (int)((mag >> (kDigitBits * pl)) & 0x7Fu);
-          const uint32_t lin = lin0 + ((uint32_t)pl << (6u + bk_shift));
-          tile[lin ^ (((lin >> 7) & sw_mask) << 4)] = (int8_t)(neg ? -digit : digit);
-        }
-      }
-    }
-  }
-  }
-  if (rowsum) {
-    __syncthreads();
-#pragma unroll
-    for (int l = 0; l < kMaxLevels; ++l) {
-      if (!((level_mask >> l) & 1u)) continue;
-      for (uint32_t r = threadIdx.x; r < rows; r += blockDim.x) {
-        // a block that could not keep sums (more rows than the table holds) leaves the bound unknown
-        if (!track) atomicMax(&rowsum[(uint32_t)l * p.O + o0 + r], 0xFFFFFFFFu);
-        else if (row_sum[l][r]) atomicAdd(&rowsum[(uint32_t)l * p.O + o0 + r], row_sum[l][r]);
+        const long long sum = (long long)(int)sums[2 * kPlaneRows + r] * 4096 + (long long)sums[kPlaneRows + r];
+        if (sum) atomicAdd(reinterpret_cast<unsigned long long*>(p.corr + at), (unsigned long long)(sum * 128));
       }
     }
   }
 }
 
-template <bool kVec>
+template <bool kOptions>
 __global__ void __launch_bounds__(kThreads) sample_kernel(const __grid_constant__ SampleParams p,
                                                           const __grid_constant__ PhiloxKeys keys) {
   pdl_prologue();
-  __shared__ float stage[kStage];
-  sample_block<kVec>(p, blockIdx.x, keys, stage);
+  __shared__ __align__(16) float stage[kStage];
+  __shared__ RowSums rs;
+  sample_block<kOptions>(p, blockIdx.x, keys, stage, rs);
 }
 
 // All layers of a network in two launches.  Entry i owns blocks [first, first + count) of each
@@ -561,32 +750,52 @@ __device__ __forceinline__ uint32_t find_entry(const BatchEntry* __restrict__ e,
 }
 
 __global__ void __launch_bounds__(kThreads) emax_batch_kernel(const BatchEntry* __restrict__ entries, uint32_t n,
-                                                              uint32_t* __restrict__ err) {
+                                                              uint32_t* __restrict__ err, uint32_t tag) {
   pdl_prologue();
   const BatchEntry& e = entries[find_entry(entries, n, blockIdx.x, true)];
   emax_block(e.p.w, e.p.O, e.p.d, e.p.norm, const_cast<uint32_t*>(e.p.e_max), err,
-             blockIdx.x - e.emax_first, e.emax_blocks, 0u, e.p.rowsum, e.p.pbits);
+             blockIdx.x - e.emax_first, e.emax_blocks, tag << 8, e.p.rowsum, e.p.corr, e.p.pbits);
 }
 
+template <bool kOptions>
 __global__ void __launch_bounds__(kThreads) sample_batch_kernel(const BatchEntry* __restrict__ entries, uint32_t n,
-                                                                const __grid_constant__ PhiloxKeys keys) {
+                                                                uint32_t tag, const __grid_constant__ PhiloxKeys keys) {
   pdl_prologue();
-  __shared__ float stage[kStage];
+  __shared__ __align__(16) float stage[kStage];
+  __shared__ RowSums rs;
+  __shared__ SampleParams p;
   const BatchEntry& e = entries[find_entry(entries, n, blockIdx.x, false)];
-  sample_block<true>(e.p, blockIdx.x - e.sample_first, keys, stage);
+  // the entry's parameters, once per block
+  for (uint32_t i = threadIdx.x; i < sizeof(SampleParams) / 4u; i += blockDim.x)
+    reinterpret_cast<uint32_t*>(&p)[i] = reinterpret_cast<const uint32_t*>(&e.p)[i];
+  const uint32_t first = e.sample_first;
+  __syncthreads();
+  if (threadIdx.x == 0) p.e_tag = tag;
+  __syncthreads();
+  sample_block<kOptions>(p, blockIdx.x - first, keys, stage, rs);
 }
 
-// 128 * (sum of each filter row): the constant that restores sum x*W from sum (x-128)*W when
-// unsigned activations are fed to the signed MMA with an offset of 128.  One warp per row.
-__global__ void corr128_kernel(const int32_t* wint, uint32_t O, uint32_t d,
-                               long long* __restrict__ corr) {
+// The integer filter of one level put together from its digit planes, in canonical order or channels innermost: the
+// export hook, and the CUDA-core kernels when they are asked to run a filter that has planes.
+__global__ void expand_planes_kernel(const int8_t* planes, int P, uint32_t O, uint32_t Cg, uint32_t KHKW, uint32_t bk,
+                                     uint32_t n_cb, uint32_t n_kb, uint32_t packed_kw, uint32_t run_pitch,
+                                     uint32_t canonical, int32_t* __restrict__ out) {
   pdl_prologue();
-  const uint32_t row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31u;
-  if (row >= O) return;
-  long long sum = 0;
-  for (uint32_t i = lane; i < d; i += 32u) sum += wint[(size_t)row * d + i];
-  for (int off = 16; off; off >>= 1) sum += __shfl_down_sync(0xFFFFFFFFu, sum, off);
-  if (lane == 0) corr[row] = sum * 128;
+  const size_t total = (size_t)O * Cg * KHKW;
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
+    const uint32_t inner = canonical ? KHKW : Cg;
+    const uint32_t a = (uint32_t)(i % inner);
+    const size_t rest = i / inner;
+    const uint32_t outer = canonical ? Cg : KHKW;
+    const uint32_t b = (uint32_t)(rest % outer), o = (uint32_t)(rest / outer);
+    const uint32_t tap = canonical ? a : b, ci = canonical ? b : a;
+    uint32_t kcol = tap * n_cb * bk + ci;
+    if (packed_kw) kcol = (tap / packed_kw) * run_pitch + (tap % packed_kw) * Cg + ci;
+    const int8_t* tile = planes + ((size_t)(o / kTileN) * n_kb + kcol / bk) * (size_t)P * kTileN * bk;
+    int w = 0;
+    for (int pl = 0; pl < P; ++pl) w += (int)tile[plane_offset((uint32_t)pl * kTileN + o % kTileN, kcol % bk, bk)] * (1 << (kDigitBits * pl));
+    out[i] = w;
+  }
 }
 
 // Canonical-order copy of one level for the test hook.
@@ -624,21 +833,21 @@ uint32_t fill_sample_params(const float* w_dev, const psb_weights* wt, uint32_t*
   const uint32_t O = sh.out_ch, Cg = sh.in_ch_per_group, KHKW = sh.kh * sh.kw, d = wt->d;
   p.w = w_dev;
   p.O = O; p.Cg = Cg; p.KHKW = KHKW; p.d = d;
-  // weights per block: the whole staging buffer for large layers; a layer sampled by a launch of its own
-  // gets less if it is small, so that it still spreads over a few hundred blocks (in a batched launch the
-  // other layers' blocks fill the machine)
+  // weights per block: enough that what a block does once (its parameters, sums, barriers) is a small part of it, yet
+  // several blocks per SM: a batched launch is filled by the other layers, a layer of its own is cut finer
   const uint64_t total = (uint64_t)O * d;
-  uint32_t budget = batched ? (uint32_t)kStage
-                            : (uint32_t)std::min<uint64_t>((uint64_t)kStage, std::max<uint64_t>(256u, total / 296u));
-  if (budget < KHKW) budget = KHKW;   // at least one channel (host validation keeps kh*kw <= kStage)
+  uint32_t budget = batched ? 4096u : (uint32_t)std::min<uint64_t>(4096u, std::max<uint64_t>(256u, total / 592u));
+  if (budget < 4u * KHKW) budget = 4u * KHKW;   // at least four channels (host validation keeps kh*kw <= 2048)
+  const uint32_t sum_rows = wt->has_planes ? (uint32_t)kPlaneRows : (uint32_t)kRowSumRows;
   if (d <= budget) {
-    p.rows_per_block = std::min<uint32_t>(budget / d, (uint32_t)kRowSumRows);   // the rows a block keeps sums for
+    p.rows_per_block = std::min<uint32_t>(budget / d, sum_rows);   // the rows a block keeps sums for
     p.ch_per_block = Cg;
     p.ch_chunks = 1;
   } else {
     p.rows_per_block = 1;
     p.ch_per_block = budget / KHKW;
     if (p.ch_per_block > 16u) p.ch_per_block &= ~15u;   // whole 16-byte pieces of the plane rows
+    else p.ch_per_block &= ~3u;
     p.ch_chunks = (Cg + p.ch_per_block - 1) / p.ch_per_block;
   }
   p.norm = wt->cfg.norm;
@@ -650,10 +859,8 @@ uint32_t fill_sample_params(const float* w_dev, const psb_weights* wt, uint32_t*
   p.max_level = 0;
   for (uint32_t l = 0; l < (uint32_t)kMaxLevels; ++l)
     if ((p.level_mask >> l) & 1u) p.max_level = l;
-  p.seed_lo = (uint32_t)wt->cfg.seed;
-  p.seed_hi = (uint32_t)(wt->cfg.seed >> 32);
   p.layer_id = wt->cfg.layer_id;
-  p.cpad = wt->cpad; p.kpad = wt->kpad; p.has_planes = wt->has_planes ? 1u : 0u;
+  p.has_planes = wt->has_planes ? 1u : 0u;
   p.bk = wt->bk; p.n_cb = wt->n_cb; p.n_kb = wt->n_kb;
   p.packed_kw = wt->packed_k ? wt->shape.kw : 0u;
   p.run_pitch = wt->run_pitch;
@@ -661,6 +868,7 @@ uint32_t fill_sample_params(const float* w_dev, const psb_weights* wt, uint32_t*
   p.e_tag = 0;
   p.e_base = wt->e_base;
   p.rowsum = wt->rowsum256;
+  p.corr = wt->corr128;
   for (int l = 0; l < kMaxLevels; ++l) {
     p.wint[l] = wt->level[l].wint;
     p.planes[l] = wt->level[l].planes;
@@ -672,10 +880,14 @@ uint32_t fill_sample_params(const float* w_dev, const psb_weights* wt, uint32_t*
 
 }  // namespace
 
-cudaError_t launch_corr128(const psb_weights* wt, uint32_t level, cudaStream_t s) {
-  const uint32_t O = wt->shape.out_ch;
-  launch_pdl(corr128_kernel, (O * 32 + kThreads - 1) / kThreads, kThreads, 0, s, (const int32_t*)wt->level[level].wint, O,
-             wt->d, wt->level[level].corr128); note_launch();
+cudaError_t launch_expand(const psb_weights* wt, uint32_t level, bool canonical, int32_t* out, cudaStream_t s) {
+  const psb_wshape& sh = wt->shape;
+  const size_t total = (size_t)sh.out_ch * wt->d;
+  const uint32_t blocks = (uint32_t)std::min<size_t>((total + kThreads - 1) / kThreads, 148u * 16u);
+  launch_pdl(expand_planes_kernel, blocks, kThreads, 0, s, (const int8_t*)wt->level[level].planes, wt->level[level].planes_count,
+             sh.out_ch, sh.in_ch_per_group, sh.kh * sh.kw, wt->bk, wt->n_cb, wt->n_kb, wt->packed_k ? sh.kw : 0u, wt->run_pitch,
+             canonical ? 1u : 0u, out);
+  note_launch();
   return cudaGetLastError();
 }
 
@@ -690,16 +902,13 @@ cudaError_t launch_sampler(const float* w_dev, psb_weights* wt, uint32_t* err_de
     wt->e_calls = 1u;
   }
   launch_pdl(emax_kernel, emax_blocks_for(O, wt->d, wt->cfg.norm), kThreads, 0, s, w_dev, O, wt->d, wt->cfg.norm,
-             wt->e_max, err_dev, wt->e_calls << 8, wt->rowsum256, wt->cfg.prob_bits); note_launch();
+             wt->e_max, err_dev, wt->e_calls << 8, wt->rowsum256, wt->corr128, wt->cfg.prob_bits); note_launch();
   SampleParams p;
   const uint32_t blocks = fill_sample_params(w_dev, wt, wt->e_max, p, false);
   p.e_tag = wt->e_calls;
-  // items of fewer than four weights per thread never take the four-weights loop: launch the instance without it
-  const uint64_t item_weights = (uint64_t)p.rows_per_block * std::min<uint64_t>(p.ch_per_block, p.Cg) * p.KHKW;
-  if (item_weights >= 4u * (uint64_t)kThreads)
-    launch_pdl(sample_kernel<true>, blocks, kThreads, 0, s, p, PhiloxKeys(p.seed_lo, p.seed_hi));
-  else
-    launch_pdl(sample_kernel<false>, blocks, kThreads, 0, s, p, PhiloxKeys(p.seed_lo, p.seed_hi));
+  const PhiloxKeys keys((uint32_t)wt->cfg.seed, (uint32_t)(wt->cfg.seed >> 32));
+  if (p.pbits | p.underflow) launch_pdl(sample_kernel<true>, blocks, kThreads, 0, s, p, keys);
+  else launch_pdl(sample_kernel<false>, blocks, kThreads, 0, s, p, keys);
   note_launch();
   return cudaGetLastError();
 }
@@ -710,8 +919,10 @@ cudaError_t launch_sampler(const float* w_dev, psb_weights* wt, uint32_t* err_de
 struct psb_sample_batch {
   uint32_t n = 0;
   psb::BatchEntry* entries_dev = nullptr;
-  uint32_t* e_max_pool = nullptr;     // one word per output channel of every layer
+  uint32_t* e_max_pool = nullptr;     // one word per output channel of every layer: (call number << 8) | exponent
   size_t e_max_words = 0;
+  uint32_t calls = 0;                 // runs made on this batch, modulo 2^24
+  bool options = false;               // some layer uses a sampling option
   uint32_t emax_grid = 0, sample_grid = 0;
   int device = 0;
 };
@@ -726,6 +937,7 @@ psb_status sample_batch_create(psb_ctx* ctx, uint32_t n, const float* const* w_d
   size_t words = 0;
   for (uint32_t i = 0; i < n; ++i) words += weights[i]->shape.out_ch;
   bool ok = cudaMalloc(&b->e_max_pool, sizeof(uint32_t) * words) == cudaSuccess &&
+            cudaMemset(b->e_max_pool, 0, sizeof(uint32_t) * words) == cudaSuccess &&
             cudaMalloc(&b->entries_dev, sizeof(BatchEntry) * n) == cudaSuccess;
   if (ok) {
     size_t off = 0;
@@ -734,6 +946,7 @@ psb_status sample_batch_create(psb_ctx* ctx, uint32_t n, const float* const* w_d
       const psb_weights* wt = weights[i];
       BatchEntry& e = host[i];
       e.sample_blocks = fill_sample_params(w_dev[i], wt, b->e_max_pool + off, e.p, true);
+      b->options = b->options || (e.p.pbits | e.p.underflow);
       e.emax_blocks = emax_blocks_for(wt->shape.out_ch, wt->d, wt->cfg.norm);
       e.emax_first = eb;
       e.sample_first = sb;
@@ -761,12 +974,18 @@ psb_status sample_batch_create(psb_ctx* ctx, uint32_t n, const float* const* w_d
 }
 
 psb_status sample_batch_run(psb_ctx* ctx, psb_sample_batch* b, uint64_t seed, cudaStream_t s) {
-  if (cudaMemsetAsync(b->e_max_pool, 0, sizeof(uint32_t) * b->e_max_words, s) != cudaSuccess)
-    return PSB_ERR_CUDA;
-  launch_pdl(emax_batch_kernel, b->emax_grid, kThreads, 0, s, (const BatchEntry*)b->entries_dev, b->n, ctx->err_dev);
+  b->calls = (b->calls + 1u) & 0xFFFFFFu;
+  if (b->calls == 0u) {       // the words of earlier calls would compare as later ones
+    if (cudaMemsetAsync(b->e_max_pool, 0, sizeof(uint32_t) * b->e_max_words, s) != cudaSuccess) return PSB_ERR_CUDA;
+    b->calls = 1u;
+  }
+  launch_pdl(emax_batch_kernel, b->emax_grid, kThreads, 0, s, (const BatchEntry*)b->entries_dev, b->n, ctx->err_dev, b->calls);
   note_launch();
-  launch_pdl(sample_batch_kernel, b->sample_grid, kThreads, 0, s, (const BatchEntry*)b->entries_dev, b->n,
-             PhiloxKeys((uint32_t)seed, (uint32_t)(seed >> 32)));
+  const PhiloxKeys keys((uint32_t)seed, (uint32_t)(seed >> 32));
+  if (b->options)
+    launch_pdl(sample_batch_kernel<true>, b->sample_grid, kThreads, 0, s, (const BatchEntry*)b->entries_dev, b->n, b->calls, keys);
+  else
+    launch_pdl(sample_batch_kernel<false>, b->sample_grid, kThreads, 0, s, (const BatchEntry*)b->entries_dev, b->n, b->calls, keys);
   note_launch();
   return cudaGetLastError() == cudaSuccess ? PSB_OK : PSB_ERR_CUDA;
 }
@@ -780,7 +999,10 @@ void sample_batch_free(psb_sample_batch* b) {
 cudaError_t launch_export(const psb_weights* wt, uint32_t level, int32_t* wint_out,
                           int32_t* e_base_out, cudaStream_t s) {
   const psb_wshape& sh = wt->shape;
-  if (wint_out) {
+  if (wint_out && wt->has_planes) {
+    const cudaError_t e = launch_expand(wt, level, true, wint_out, s);
+    if (e != cudaSuccess) return e;
+  } else if (wint_out) {
     size_t total = (size_t)sh.out_ch * wt->d;
     uint32_t blocks = (uint32_t)((total + 255) / 256);
     blocks = blocks > 4096 ? 4096 : (blocks < 1 ? 1 : blocks);
@@ -820,9 +1042,9 @@ uint32_t* g_static_scratch_addr[kMaxDevices] = {};   // device address per devic
 // the device address of the static scratch, filled by emax_kernel just before.
 __global__ void __launch_bounds__(kThreads)
 sample_level_canonical_kernel(const float* __restrict__ w, uint32_t O, uint32_t d, uint32_t norm,
-                              uint32_t span, uint32_t log2k, uint32_t seed_lo, uint32_t seed_hi,
-                              uint32_t layer_id, const uint32_t* __restrict__ e_max,
-                              int32_t* __restrict__ wint_out, int32_t* __restrict__ e_base_out) {
+                              uint32_t span, uint32_t log2k, uint32_t layer_id, const uint32_t* __restrict__ e_max,
+                              int32_t* __restrict__ wint_out, int32_t* __restrict__ e_base_out,
+                              const __grid_constant__ PhiloxKeys keys) {
   pdl_prologue();
   const size_t total = (size_t)O * d;
   for (size_t index = (size_t)blockIdx.x * blockDim.x + threadIdx.x; index < total;
@@ -838,9 +1060,10 @@ sample_level_canonical_kernel(const float* __restrict__ w, uint32_t O, uint32_t 
     uint32_t c = 0;
     if (live && m != 0u) {
       const uint32_t T = m << 9, k = 1u << log2k;
+      const PhiloxWeight pw((uint32_t)index, layer_id ^ keys.k0[0]);
       for (uint32_t q = 0; q * 4u < k; ++q) {
         uint32_t rnd[4];
-        philox4x32_10(q, layer_id, (uint32_t)index, (uint32_t)(index >> 32), seed_lo, seed_hi, rnd);
+        pw.call(q, keys, rnd);
 #pragma unroll
         for (int v = 0; v < 4; ++v)
           if (q * 4u + v < k) c += (rnd[v] < T) ? 1u : 0u;
@@ -893,18 +1116,18 @@ extern "C" psb_status psb_sample_level_static(const float* w_dev, const psb_wsha
   // the array keeps the previous call's maxima: the reduction must start from zero
   if (cudaMemsetAsync(e_max, 0, sizeof(uint32_t) * O, s) != cudaSuccess) return PSB_ERR_CUDA;
   if (cfg->norm) {
-    emax_kernel<<<emax_blocks_for(O, d, 1), kThreads, 0, s>>>(w_dev, O, d, 1, e_max, err_sink, 0u, nullptr, 0u); note_launch();
+    emax_kernel<<<emax_blocks_for(O, d, 1), kThreads, 0, s>>>(w_dev, O, d, 1, e_max, err_sink, 0u, nullptr, nullptr, 0u); note_launch();
   } else {
     size_t total = (size_t)O * d;
     uint32_t blocks = (uint32_t)((total + kThreads * 8 - 1) / (kThreads * 8));
     blocks = blocks < 1 ? 1 : (blocks > 1184 ? 1184 : blocks);
-    emax_kernel<<<blocks, kThreads, 0, s>>>(w_dev, O, d, 0, e_max, err_sink, 0u, nullptr, 0u); note_launch();
+    emax_kernel<<<blocks, kThreads, 0, s>>>(w_dev, O, d, 0, e_max, err_sink, 0u, nullptr, nullptr, 0u); note_launch();
   }
   size_t total = (size_t)O * d;
   uint32_t blocks = (uint32_t)((total + kThreads - 1) / kThreads);
   blocks = blocks > 148u * 16u ? 148u * 16u : blocks;
   sample_level_canonical_kernel<<<blocks, kThreads, 0, s>>>(
-      w_dev, O, d, cfg->norm, (1u << exp_bits) - 1u, log2k, (uint32_t)cfg->seed,
-      (uint32_t)(cfg->seed >> 32), cfg->layer_id, e_max, wint_out_dev, e_base_out_dev); note_launch();
+      w_dev, O, d, cfg->norm, (1u << exp_bits) - 1u, log2k, cfg->layer_id, e_max, wint_out_dev, e_base_out_dev,
+      PhiloxKeys((uint32_t)cfg->seed, (uint32_t)(cfg->seed >> 32))); note_launch();
   return cudaGetLastError() == cudaSuccess ? PSB_OK : PSB_ERR_CUDA;
 }

@@ -79,31 +79,105 @@ __global__ void __launch_bounds__(256) conv_direct_kernel(const ConvArgs a, cons
   }
 }
 
-// Fully connected layers at small batch (1x1 filter on a 1x1 image, one group): a warp per output
-// element, the lanes stride over the input features (coalesced runs of the filter row and of the
-// activation row) and the 64-bit partial sums meet in a shuffle tree.  With one thread per output the
-// 256 dependent loads of a 256-feature row made the layer ten times longer than its launch.
-__global__ void __launch_bounds__(256) gemv_warp_kernel(const ConvArgs a, const WintTable wt) {
+// Four byte products of an unsigned / signed activation word with a signed digit word, accumulated.
+template <bool kSignedIn>
+__device__ __forceinline__ int dp4a_act(uint32_t x, uint32_t w, int acc) {
+  int d;
+  if (kSignedIn) asm("dp4a.s32.s32 %0, %1, %2, %3;" : "=r"(d) : "r"(x), "r"(w), "r"(acc));
+  else asm("dp4a.u32.s32 %0, %1, %2, %3;" : "=r"(d) : "r"(x), "r"(w), "r"(acc));
+  return d;
+}
+
+// Matrix products with few rows (fully connected layers at small batch, 1x1 filters on a few locations), straight from
+// the digit planes: a group of lanes per output channel, each lane 16 input features at a time (one 16-byte load per
+// plane, four dp4a per plane and activation row), kNB activation rows per pass over the weights; a plane's sum stays
+// in 32 bits (gemv_planes_ok), the planes meet in 64 bits and the lanes in a shuffle tree.  The activation rows of the
+// block sit in shared memory, kGemvFeatures at a time, padded with zeros to whole K blocks.  Bound by the latency of
+// its few loads; P bytes per weight are read instead of the 4 of an integer filter.
+constexpr int kGemvRows = 4;
+constexpr uint32_t kGemvFeatures = 8192;      // kGemvRows rows of them take 32 KB
+
+struct GemvPlanes {
+  const int8_t* p[kMaxLevels];
+  int count[kMaxLevels];
+  uint32_t bk, n_kb;
+};
+
+template <int kNB, bool kSignedIn>
+__global__ void __launch_bounds__(256) gemv_planes_kernel(const ConvArgs a, const GemvPlanes w, uint32_t M,
+                                                          uint32_t lanes_per_row) {
   pdl_prologue();
-  const size_t total = (size_t)a.N * a.O;
-  const uint32_t lane = threadIdx.x & 31u;
-  for (size_t idx = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; idx < total;
-       idx += ((size_t)gridDim.x * blockDim.x) >> 5) {
-    const uint32_t o = (uint32_t)(idx % a.O);
-    const uint32_t n = (uint32_t)(idx / a.O);
-    const uint32_t level = a.kmap ? a.kmap[n] : a.uniform_log2k;
-    if (level >= (uint32_t)kMaxLevels || !((a.level_mask >> level) & 1u)) {
-      if (lane == 0) atomicOr(a.err, kDevErrBadLevel);
-      continue;
-    }
-    const int32_t* w = wt.w[level] + (size_t)o * a.C;
-    const size_t xoff = (size_t)n * a.C;
-    long long acc = 0;
-    for (uint32_t ci = lane; ci < a.C; ci += 32u)
-      acc += (long long)load_act(a.x, a.in_dtype, xoff + ci) * (long long)__ldca(w + ci);
+  extern __shared__ __align__(16) uint8_t gemv_x[];     // [kNB][min(kp, kGemvFeatures)]
+  const uint32_t bk = w.bk, kp = w.n_kb * bk, C = a.C, seg = min(kp, kGemvFeatures);
+  const uint32_t n0 = blockIdx.y * (uint32_t)kNB, nb = min((uint32_t)kNB, M - n0);
+  const uint8_t* x = (const uint8_t*)a.x + (size_t)n0 * C;
+  const bool vec = C % 16u == 0u && ((uintptr_t)x & 15u) == 0u;
+  const uint32_t sub = threadIdx.x & (lanes_per_row - 1u);
+  const uint32_t o = blockIdx.x * (blockDim.x / lanes_per_row) + threadIdx.x / lanes_per_row;
+  const uint32_t level = a.kmap ? a.kmap[n0] : a.uniform_log2k;      // with a map kNB is 1
+  const bool level_ok = level < (uint32_t)kMaxLevels && ((a.level_mask >> level) & 1u);
+  if (!level_ok && threadIdx.x == 0) atomicOr(a.err, kDevErrBadLevel);
+  int acc[kMaxPlanes][kNB];
 #pragma unroll
-    for (int d = 16; d > 0; d >>= 1) acc += __shfl_down_sync(0xFFFFFFFFu, acc, d);
-    if (lane == 0) store_outputs(a, idx, o, level, acc);
+  for (int pl = 0; pl < kMaxPlanes; ++pl)
+#pragma unroll
+    for (int r = 0; r < kNB; ++r) acc[pl][r] = 0;
+  for (uint32_t k0 = 0; k0 < kp; k0 += seg) {
+    const uint32_t len = min(seg, kp - k0);
+    if (k0) __syncthreads();
+    for (uint32_t r = 0; r < (uint32_t)kNB; ++r)
+      for (uint32_t i = threadIdx.x * 16u; i < len; i += blockDim.x * 16u) {
+        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+        if (r < nb && k0 + i < C) {
+          const uint8_t* src = x + (size_t)r * C + k0 + i;
+          if (vec) {
+            v = __ldcg(reinterpret_cast<const uint4*>(src));
+          } else {
+            uint32_t b[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+            for (int j = 0; j < 16; ++j)
+              if (k0 + i + j < C) b[j >> 2] |= (uint32_t)src[j] << (8 * (j & 3));
+            v = make_uint4(b[0], b[1], b[2], b[3]);
+          }
+        }
+        *reinterpret_cast<uint4*>(gemv_x + r * seg + i) = v;
+      }
+    __syncthreads();
+    if (!level_ok || o >= a.O) continue;
+    const int P = w.count[level];
+    const uint32_t shift = 31u - (uint32_t)__clz((int)bk), on = o % kTileN, chunks = len / 16u;
+    const size_t tile_bytes = (size_t)P * kTileN * bk;
+    const int8_t* base = w.p[level] + (size_t)(o / kTileN) * w.n_kb * tile_bytes;
+#pragma unroll 4
+    for (uint32_t c = sub; c < chunks; c += lanes_per_row) {
+      const uint32_t k = k0 + c * 16u, off = plane_offset(on, k & (bk - 1u), bk);
+      const int8_t* tile = base + (size_t)(k >> shift) * tile_bytes + off;
+      uint4 d[kMaxPlanes];
+#pragma unroll
+      for (int pl = 0; pl < kMaxPlanes; ++pl)
+        if (pl < P) d[pl] = __ldcg(reinterpret_cast<const uint4*>(tile + (size_t)pl * kTileN * bk));
+#pragma unroll
+      for (int r = 0; r < kNB; ++r) {
+        const uint4 v = *reinterpret_cast<const uint4*>(gemv_x + (uint32_t)r * seg + c * 16u);
+#pragma unroll
+        for (int pl = 0; pl < kMaxPlanes; ++pl)
+          if (pl < P) {
+            acc[pl][r] = dp4a_act<kSignedIn>(v.x, d[pl].x, acc[pl][r]);
+            acc[pl][r] = dp4a_act<kSignedIn>(v.y, d[pl].y, acc[pl][r]);
+            acc[pl][r] = dp4a_act<kSignedIn>(v.z, d[pl].z, acc[pl][r]);
+            acc[pl][r] = dp4a_act<kSignedIn>(v.w, d[pl].w, acc[pl][r]);
+          }
+      }
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < kNB; ++r) {
+    long long sum = acc[0][r];
+#pragma unroll
+    for (int pl = 1; pl < kMaxPlanes; ++pl) sum += (long long)acc[pl][r] * (1ll << (kDigitBits * pl));
+    for (uint32_t d = lanes_per_row / 2u; d > 0; d >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, d);
+    if (level_ok && o < a.O && (uint32_t)r < nb && sub == ((uint32_t)r & (lanes_per_row - 1u)))
+      store_outputs(a, (size_t)(n0 + r) * a.O + o, o, level, sum);
   }
 }
 
@@ -825,12 +899,42 @@ cudaError_t launch_shift_add(const ConvArgs& a, const WintTable& wt, const uint3
     launch_pdl(dwconv_nhwc8_kernel, blocks, 256, dw_smem, s, a, wt.w[a.uniform_log2k]); note_launch();
     return cudaGetLastError();
   }
-  if (a.KH == 1 && a.KW == 1 && a.H == 1 && a.W == 1 && a.groups == 1 && a.C >= 64u && !a.out_nchw &&
-      total < (1u << 24)) {
-    launch_pdl(gemv_warp_kernel, grid_for(total * 32u, 256), 256, 0, s, a, wt); note_launch();
-    return cudaGetLastError();
-  }
   launch_pdl(conv_direct_kernel, grid_for(total, 256), 256, 0, s, a, wt); note_launch();
+  return cudaGetLastError();
+}
+
+// Rows of the product: locations of a 1x1 filter with stride 1 on channels-last data.  A plane's sum of one lane: at most
+// 2^20 / lanes * 255 * 127 < 2^31 (filters of 512 features and more have 32 lanes per output).
+bool gemv_planes_ok(const ConvArgs& a, const psb_weights* wt) {
+  const uint64_t M = (uint64_t)a.N * a.OH * a.OW;
+  return a.KH == 1u && a.KW == 1u && a.stride == 1u && a.pad == 0u && !a.out_nchw && !wt->packed_k &&
+         wt->n_kb * wt->bk <= (1u << 20) && M * a.O < (1u << 24) &&
+         (a.kmap ? M : (M + kGemvRows - 1u) / kGemvRows) <= 65535u;
+}
+
+cudaError_t launch_gemv_planes(const ConvArgs& a, const psb_weights* wt, cudaStream_t s) {
+  GemvPlanes w;
+  for (int l = 0; l < kMaxLevels; ++l) {
+    w.p[l] = wt->level[l].planes;
+    w.count[l] = wt->level[l].planes_count;
+  }
+  w.bk = wt->bk;
+  w.n_kb = wt->n_kb;
+  const uint32_t kp = w.n_kb * w.bk, M = a.N * a.OH * a.OW;
+  uint32_t lanes = 1;
+  while (lanes < 32u && lanes * 16u < kp) lanes *= 2u;
+  const bool one = a.kmap || M == 1u;
+  const dim3 grid((a.O + 256u / lanes - 1u) / (256u / lanes), one ? M : (M + kGemvRows - 1u) / kGemvRows);
+  const size_t smem = (size_t)(one ? 1 : kGemvRows) * (kp < kGemvFeatures ? kp : kGemvFeatures);
+  const bool sg = a.in_dtype == PSB_DT_S8;
+  if (one) {
+    if (sg) launch_pdl(gemv_planes_kernel<1, true>, grid, dim3(256), smem, s, a, w, M, lanes);
+    else launch_pdl(gemv_planes_kernel<1, false>, grid, dim3(256), smem, s, a, w, M, lanes);
+  } else {
+    if (sg) launch_pdl(gemv_planes_kernel<kGemvRows, true>, grid, dim3(256), smem, s, a, w, M, lanes);
+    else launch_pdl(gemv_planes_kernel<kGemvRows, false>, grid, dim3(256), smem, s, a, w, M, lanes);
+  }
+  note_launch();
   return cudaGetLastError();
 }
 

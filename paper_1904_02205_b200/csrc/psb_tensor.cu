@@ -167,7 +167,7 @@ psb_status launch_tensor(psb_ctx* ctx, const psb_weights* wt, const ConvArgs& a,
   p.stages = stages;
   const size_t smem_bytes = (p.band ? (size_t)stages * p.band_bytes : (size_t)stages * group * sub_bytes) +
                             p.resident_bytes + ctl_bytes;
-  for (int l = 0; l < kMaxLevels; ++l) p.corr[l] = add_corr128 ? wt->level[l].corr128 : nullptr;
+  for (int l = 0; l < kMaxLevels; ++l) p.corr[l] = add_corr128 && wt->level[l].planes ? wt->corr128 + (size_t)l * a.O : nullptr;
   p.rowsum256 = wt->rowsum256;
   p.amax = amax;
   const CUtensorMapSwizzle swz = swizzle_for(bk);
