@@ -7,6 +7,7 @@ fallback: loading fails loudly if the library has not been built, and
 """
 import ctypes as C
 import os
+import struct
 
 import torch
 
@@ -69,6 +70,21 @@ class psb_op(C.Structure):
 
 PSB_OP_CONV2D, PSB_OP_GEMM, PSB_OP_MAXPOOL, PSB_OP_AVGPOOL = 0, 1, 2, 3
 
+# The argument blocks of the calls that a program makes once per layer, packed in one go: filling the ctypes structures
+# field by field took 3 us of a 10 us call.  Values that do not fit their field go through ctypes, which wraps them.
+_EP_FMT = "3QfIIfiiI4x3Q"
+_CONV_BLOCK, _GEMM_BLOCK = struct.Struct("=10I" + _EP_FMT), struct.Struct("=5I4x" + _EP_FMT)
+_SHAPE_BLOCK, _CFG_BLOCK = struct.Struct("=5I"), struct.Struct("=Q8I")
+assert _CONV_BLOCK.size == C.sizeof(psb_conv_desc) and _GEMM_BLOCK.size == C.sizeof(psb_gemm_desc)
+assert _SHAPE_BLOCK.size == C.sizeof(psb_wshape) and _CFG_BLOCK.size == C.sizeof(psb_sample_cfg)
+
+
+def _block(packer, ctype, head, ep=()):
+    try:
+        return packer.pack(*head, *ep)
+    except struct.error:
+        return bytes(ctype(*head, psb_epilogue(*ep)) if ep else ctype(*head))
+
 _lib = None
 
 
@@ -86,13 +102,12 @@ def load_library():
     lib.psb_status_string.argtypes = [i32]
     lib.psb_status_string.restype = C.c_char_p
     lib.psb_device_status.argtypes = [vp, vp]
-    lib.psb_sample_weights.argtypes = [vp, vp, C.POINTER(psb_wshape), C.POINTER(psb_sample_cfg),
-                                       C.POINTER(vp), vp]
+    lib.psb_sample_weights.argtypes = [vp, vp, vp, vp, C.POINTER(vp), vp]    # argument blocks: bytes or byref()
     lib.psb_weights_export.argtypes = [vp, vp, u32, vp, vp, vp]
     lib.psb_weights_free.argtypes = [vp, vp]
     lib.psb_set_sample_map.argtypes = [vp, vp, u32, u32, u32, u32]
-    lib.psb_conv2d.argtypes = [vp, vp, vp, C.POINTER(psb_conv_desc), vp]
-    lib.psb_gemm.argtypes = [vp, vp, vp, C.POINTER(psb_gemm_desc), vp]
+    lib.psb_conv2d.argtypes = [vp, vp, vp, vp, vp]
+    lib.psb_gemm.argtypes = [vp, vp, vp, vp, vp]
     lib.psb_last_path.argtypes = [vp]
     lib.psb_int8_mma_probe.argtypes = [vp, u32, u32, C.POINTER(C.c_double), C.POINTER(C.c_double), vp]
     lib.psb_contraction_timing.argtypes = [vp, u32]
@@ -136,11 +151,14 @@ def _ptr(t):
 
 
 def _stream(stream):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return C.c_void_p(s.cuda_stream)
+    # the raw handle of the current stream: torch.cuda.current_stream() builds a Stream object around it (3 us)
+    if stream is None:
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return stream.cuda_stream
 
 
 _TORCH_DT = {PSB_DT_U8: torch.uint8, PSB_DT_S8: torch.int8}
+_OUT_DT = {"f32": torch.float32, "acc": torch.int64}
 
 
 def _dt_of(t):
@@ -259,14 +277,16 @@ class Context:
         assert w.is_cuda and w.dtype == torch.float32 and w.is_contiguous()
         if w.dim() == 2:
             w = w.view(w.shape[0], w.shape[1], 1, 1)
-        shape = psb_wshape(w.shape[0], w.shape[1], w.shape[2], w.shape[3], groups)
-        cfg = psb_sample_cfg(seed, layer_id, level_mask, exp_bits, norm, underflow, prob_bits, deterministic, 0)
+        dims = tuple(w.shape)
+        shape = _block(_SHAPE_BLOCK, psb_wshape, (*dims, groups))
+        cfg = _block(_CFG_BLOCK, psb_sample_cfg,
+                     (seed, layer_id, level_mask, exp_bits, norm, underflow, prob_bits, deterministic, 0))
         h = C.c_void_p(into.handle.value if into is not None else None)
-        _check(self.lib.psb_sample_weights(self.handle, _ptr(w), C.byref(shape), C.byref(cfg),
-                                           C.byref(h), _stream(stream)), "psb_sample_weights")
+        _check(self.lib.psb_sample_weights(self.handle, w.data_ptr(), shape, cfg, C.byref(h), _stream(stream)),
+               "psb_sample_weights")
         if into is not None:
             return into
-        return Weights(self, h, tuple(w.shape) + (groups,), level_mask)
+        return Weights(self, h, dims + (groups,), level_mask)
 
     def weights_export(self, weights, log2k, stream=None):
         O, Cg, KH, KW, _ = weights.shape
@@ -293,22 +313,16 @@ class Context:
     # -- psb_conv2d / psb_gemm ----------------------------------------------
     def _epilogue(self, out_shape, scale, bias, relu, inv_step, qmin, qmax, out_dtype, residual,
                   residual_scale, want, out):
-        out = dict(out or {})
-        if "q" in want and "q" not in out:
-            out["q"] = torch.empty(out_shape, dtype=_TORCH_DT[out_dtype], device=self.device)
-        if "f32" in want and "f32" not in out:
-            out["f32"] = torch.empty(out_shape, dtype=torch.float32, device=self.device)
-        if "acc" in want and "acc" not in out:
-            out["acc"] = torch.empty(out_shape, dtype=torch.int64, device=self.device)
-        ep = psb_epilogue()
-        ep.scale_dev, ep.bias_dev = scale.data_ptr(), bias.data_ptr()
-        ep.residual_dev = None if residual is None else residual.data_ptr()
-        ep.residual_scale = float(residual_scale)
-        ep.residual_dtype = PSB_DT_U8 if residual is None else _dt_of(residual)
-        ep.relu, ep.inv_step, ep.qmin, ep.qmax, ep.out_dtype = int(relu), float(inv_step), qmin, qmax, out_dtype
-        ep.q_out_dev = out["q"].data_ptr() if "q" in out else None
-        ep.f32_out_dev = out["f32"].data_ptr() if "f32" in out else None
-        ep.acc_out_dev = out["acc"].data_ptr() if "acc" in out else None
+        out = dict(out) if out else {}
+        for kind in want:
+            if kind not in out:
+                dt = _TORCH_DT[out_dtype] if kind == "q" else _OUT_DT.get(kind)
+                if dt is not None:
+                    out[kind] = torch.empty(out_shape, dtype=dt, device=self.device)
+        q, f32, acc = out.get("q"), out.get("f32"), out.get("acc")
+        ep = (scale.data_ptr(), bias.data_ptr(), 0 if residual is None else residual.data_ptr(), float(residual_scale),
+              PSB_DT_U8 if residual is None else _dt_of(residual), int(relu), float(inv_step), qmin, qmax, out_dtype,
+              0 if q is None else q.data_ptr(), 0 if f32 is None else f32.data_ptr(), 0 if acc is None else acc.data_ptr())
         return ep, out
 
     def conv2d(self, weights, x, layout, stride, pad, scale, bias, relu, inv_step, qmin, qmax,
@@ -326,9 +340,8 @@ class Context:
         oshape = (n, O, oh, ow) if layout == PSB_LAYOUT_NCHW else (n, oh, ow, O)
         ep, out = self._epilogue(oshape, scale, bias, relu, inv_step, qmin, qmax, out_dtype, residual,
                                  residual_scale, want, out)
-        d = psb_conv_desc(layout, _dt_of(x), in_max, n, c, h, w, stride, pad, path, ep)
-        _check(self.lib.psb_conv2d(self.handle, weights.handle, _ptr(x), C.byref(d), _stream(stream)),
-               "psb_conv2d")
+        d = _block(_CONV_BLOCK, psb_conv_desc, (layout, _dt_of(x), in_max, n, c, h, w, stride, pad, path), ep)
+        _check(self.lib.psb_conv2d(self.handle, weights.handle, x.data_ptr(), d, _stream(stream)), "psb_conv2d")
         return out
 
     def gemm(self, weights, x, scale, bias, relu, inv_step, qmin, qmax, out_dtype=PSB_DT_U8,
@@ -339,9 +352,8 @@ class Context:
         batch, fin = x.shape
         ep, out = self._epilogue((batch, weights.shape[0]), scale, bias, relu, inv_step, qmin, qmax,
                                  out_dtype, residual, residual_scale, want, out)
-        d = psb_gemm_desc(_dt_of(x), in_max, batch, fin, path, ep)
-        _check(self.lib.psb_gemm(self.handle, weights.handle, _ptr(x), C.byref(d), _stream(stream)),
-               "psb_gemm")
+        d = _block(_GEMM_BLOCK, psb_gemm_desc, (_dt_of(x), in_max, batch, fin, path), ep)
+        _check(self.lib.psb_gemm(self.handle, weights.handle, x.data_ptr(), d, _stream(stream)), "psb_gemm")
         return out
 
     # -- attention proposal (Sec. 4.5) -----------------------------------------
