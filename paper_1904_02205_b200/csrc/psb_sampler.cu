@@ -490,6 +490,10 @@ __device__ __forceinline__ uint32_t top_signs(uint32_t a, uint32_t b) {
   return d;
 }
 
+// Biased exponent of a window from its word.  A word written by an earlier call (other tag) means this call found no
+// live weight in the group.
+__device__ __forceinline__ uint32_t window_exponent(uint32_t word, uint32_t tag) { return (word >> 8) == tag ? (word & 0xFFu) : 0u; }
+
 // Filters with digit planes whose K axis is tap-major: a thread takes four consecutive channels of one (row, tap),
 // draws them, spreads each magnitude's 7-bit digits over the bytes of a word, transposes the four words with byte
 // permutes into one word per plane, negates the bytes of negative weights at once and stores 4 bytes per plane.
@@ -500,24 +504,22 @@ __device__ __forceinline__ uint32_t top_signs(uint32_t a, uint32_t b) {
 // digit); 4096 x 4096, k = 16, 8-bit probabilities: 205 -> 185 us.
 // kOptions: the sampling options of Sec. 3.1 / 4.4; kMulti: more than one level.
 template <bool kOptions, bool kMulti>
-__device__ __forceinline__ void sample_planes(const SampleParams& p, uint32_t o0, uint32_t c0, uint32_t rows, uint32_t cc,
+__device__ __forceinline__ void sample_planes(const SampleParams& p, const uint32_t* windows, uint32_t tag, uint32_t o0, uint32_t c0, uint32_t rows, uint32_t cc,
                                               const PhiloxKeys& keys, const float* stage, uint32_t* sums) {
-  const uint32_t KHKW = p.KHKW, d = p.d, norm = p.norm, e_tag = p.e_tag, level_mask = p.level_mask;
+  const uint32_t KHKW = p.KHKW, d = p.d, norm = p.norm, level_mask = p.level_mask;
   const uint32_t max_level = p.max_level, layer_key = p.layer_id ^ keys.k0[0];
   const uint32_t bk = p.bk, n_cb = p.n_cb, n_kb = p.n_kb;
   const uint32_t bk_shift = 31u - (uint32_t)__clz((int)bk), bk_mask = bk - 1u, sw_mask = (bk >> 4) - 1u;
   const int span = (int)p.span;
-  const uint32_t* const e_max = p.e_max;
   const uint32_t per_row = cc * KHKW, groups = (cc + 3u) >> 2, per_row4 = groups * KHKW, count4 = rows * per_row4;
   const uint32_t per_row4_magic = small_div_magic(per_row4), groups_magic = small_div_magic(groups);
-  uint32_t e_word = norm ? 0u : e_max[0];
+  uint32_t e_word = norm ? 0u : windows[0];
   for (uint32_t t = threadIdx.x; t < count4; t += blockDim.x) {
     const uint32_t r = small_div(t, per_row4_magic), rem = t - r * per_row4;
     const uint32_t tap = small_div(rem, groups_magic), cl = (rem - tap * groups) << 2;
     const uint32_t o = o0 + r, ci = c0 + cl;
-    // a word written by an earlier call (other tag) means this call found no live weight in the group
-    if (norm) e_word = e_max[o];
-    const uint32_t Emax = (e_word >> 8) == e_tag ? (e_word & 0xFFu) : 0u;
+    if (norm) e_word = windows[r];
+    const uint32_t Emax = window_exponent(e_word, tag);
     // biased exponents throughout: e - e_base = E - (Emax - span)
     const int ebase_biased = (int)Emax - span;
     if (tap == 0 && ci == 0) p.e_base[o] = Emax ? ebase_biased - 127 : 0;
@@ -614,9 +616,10 @@ __device__ __forceinline__ void sample_planes(const SampleParams& p, uint32_t o0
 // Everything else, one weight per thread and step: depthwise and grouped filters (integer filter, channels
 // innermost, for the CUDA-core kernels) and flat K axes (few input channels).
 template <bool kOptions>
-__device__ __forceinline__ void sample_single(const SampleParams& p, uint32_t o0, uint32_t c0, uint32_t rows, uint32_t cc,
-                                              const PhiloxKeys& keys, const float* stage, uint32_t* sums, bool track) {
-  const uint32_t KHKW = p.KHKW, Cg = p.Cg, d = p.d, norm = p.norm, e_tag = p.e_tag, level_mask = p.level_mask;
+__device__ __forceinline__ void sample_single(const SampleParams& p, const uint32_t* windows, uint32_t tag, uint32_t o0,
+                                              uint32_t c0, uint32_t rows, uint32_t cc, const PhiloxKeys& keys, const float* stage,
+                                              uint32_t* sums) {
+  const uint32_t KHKW = p.KHKW, Cg = p.Cg, d = p.d, level_mask = p.level_mask;
   const uint32_t max_level = p.max_level, layer_key = p.layer_id ^ keys.k0[0], has_planes = p.has_planes;
   const uint32_t packed_kw = p.packed_kw, run_pitch = p.run_pitch, bk = p.bk, n_kb = p.n_kb;
   const uint32_t bk_shift = 31u - (uint32_t)__clz((int)bk), bk_mask = bk - 1u, sw_mask = (bk >> 4) - 1u;
@@ -628,9 +631,7 @@ __device__ __forceinline__ void sample_single(const SampleParams& p, uint32_t o0
     const uint32_t o = o0 + r, ci = c0 + cl;
     const uint32_t u = __float_as_uint(stage[r * per_row + cl * KHKW + tap]);
     const uint32_t index = o * d + ci * KHKW + tap;  // canonical
-    // a word written by an earlier call (other tag) means this call found no live weight in the group
-    const uint32_t e_word = p.e_max[norm ? o : 0];
-    const uint32_t Emax = (e_word >> 8) == e_tag ? (e_word & 0xFFu) : 0u;
+    const uint32_t Emax = window_exponent(windows[p.norm ? r : 0u], tag);
     const int ebase_biased = (int)Emax - (int)p.span;
     if (tap == 0 && ci == 0) p.e_base[o] = Emax ? ebase_biased - 127 : 0;
     Drawn dw;
@@ -661,23 +662,22 @@ __device__ __forceinline__ void sample_single(const SampleParams& p, uint32_t o0
         add_row_sums(sums + l * (3 * kPlaneRows), r, (mag + 255u) >> 8, wv, true);
       } else {
         p.wint[l][wpos] = wv;
-        if (track) add_row_sums(sums + l * kRowSumRows, r, (mag + 255u) >> 8, 0, false);
+        add_row_sums(sums + l * kRowSumRows, r, (mag + 255u) >> 8, 0, false);
       }
     }
   }
 }
 
-template <bool kOptions>
+// kFused: the block finds its windows itself instead of reading the words of an exponent pass, and owns whole rows, so
+// it stores their sums where the others add to words that the exponent pass has cleared.
+template <bool kOptions, bool kFused>
 __device__ __forceinline__ void sample_block(const SampleParams& p, uint32_t block, const PhiloxKeys& keys, float* stage,
-                                             RowSums& rs) {
+                                             RowSums& rs, uint32_t* err) {
   const uint32_t level_mask = p.level_mask, has_planes = p.has_planes, O = p.O;
-  const uint32_t sum_rows = has_planes ? (uint32_t)kPlaneRows : (uint32_t)kRowSumRows;
-  const bool track = p.rows_per_block <= sum_rows;         // always so with digit planes (fill_sample_params)
   const uint32_t pitch = has_planes ? 3u * kPlaneRows : (uint32_t)kRowSumRows;     // words per level
-  if (track)
-    for (uint32_t l = 0; l < (uint32_t)kMaxLevels; ++l)
-      if ((level_mask >> l) & 1u)
-        for (uint32_t i = threadIdx.x; i < pitch; i += blockDim.x) rs.word[l * pitch + i] = 0u;
+  for (uint32_t l = 0; l < (uint32_t)kMaxLevels; ++l)
+    if ((level_mask >> l) & 1u)
+      for (uint32_t i = threadIdx.x; i < pitch; i += blockDim.x) rs.word[l * pitch + i] = 0u;
   const uint32_t row_block = block / p.ch_chunks, chunk = block - row_block * p.ch_chunks;
   const uint32_t o0 = row_block * p.rows_per_block, c0 = chunk * p.ch_per_block;
   const uint32_t rows = min(p.rows_per_block, O - o0), cc = min(p.ch_per_block, p.Cg - c0);
@@ -695,15 +695,59 @@ __device__ __forceinline__ void sample_block(const SampleParams& p, uint32_t blo
       for (uint32_t t = threadIdx.x; t < count; t += blockDim.x) stage[t] = __ldg(src + t);
     }
   }
+  const uint32_t* windows = p.e_max + (p.norm ? o0 : 0u);      // of the rows of this block, or the layer's
+  uint32_t tag = p.e_tag;
+  if (kFused) {
+    __shared__ uint32_t window[kRowSumRows];
+    const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u, d = p.d;
+    bool bad = false;
+    if (p.norm) {
+      __syncthreads();
+      for (uint32_t r = warp; r < rows; r += kThreads / 32) {
+        uint32_t best = 0u;
+        for (uint32_t i = lane; i < d; i += 32u) {
+          const uint32_t u1[1] = {__float_as_uint(stage[r * d + i])};
+          best = max_magnitude(u1, best, bad);
+        }
+        best = __reduce_max_sync(0xFFFFFFFFu, best);
+        if (lane == 0u) window[r] = quantised_exponent(best, p.pbits);
+      }
+    } else {
+      // one window for a small layer: every block looks at all of it
+      const uint32_t total = O * d, head = (((uintptr_t)p.w) & 15u) == 0u ? total & ~3u : 0u;
+      uint32_t best = 0u;
+      const uint4* w4 = reinterpret_cast<const uint4*>(p.w);
+#pragma unroll 8
+      for (uint32_t i = threadIdx.x; i < head / 4u; i += kThreads) {
+        const uint4 v = __ldg(w4 + i);
+        const uint32_t u4[4] = {v.x, v.y, v.z, v.w};
+        best = max_magnitude(u4, best, bad);
+      }
+      for (uint32_t i = head + threadIdx.x; i < total; i += kThreads) {
+        const uint32_t u1[1] = {__float_as_uint(__ldg(p.w + i))};
+        best = max_magnitude(u1, best, bad);
+      }
+      best = __reduce_max_sync(0xFFFFFFFFu, best);
+      if (lane == 0u) window[1u + warp] = best;
+      __syncthreads();
+      if (threadIdx.x == 0u) {
+        for (uint32_t i = 2u; i <= kThreads / 32; ++i) best = max(best, window[i]);
+        window[0] = quantised_exponent(best, p.pbits);
+      }
+    }
+    if (__any_sync(0xFFFFFFFFu, bad) && lane == 0u) atomicOr(err, kDevErrNonFinite);
+    windows = window;
+    tag = 0u;
+  }
   __syncthreads();
   if (has_planes && !p.packed_kw) {
     const bool multi = (level_mask & (level_mask - 1u)) != 0u;
     const bool plain = !kOptions || (p.pbits | p.underflow) == 0u;
-    if (plain && !multi) sample_planes<false, false>(p, o0, c0, rows, cc, keys, stage, rs.word);
-    else if (multi) sample_planes<kOptions, true>(p, o0, c0, rows, cc, keys, stage, rs.word);
-    else sample_planes<kOptions, false>(p, o0, c0, rows, cc, keys, stage, rs.word);
+    if (plain && !multi) sample_planes<false, false>(p, windows, tag, o0, c0, rows, cc, keys, stage, rs.word);
+    else if (multi) sample_planes<kOptions, true>(p, windows, tag, o0, c0, rows, cc, keys, stage, rs.word);
+    else sample_planes<kOptions, false>(p, windows, tag, o0, c0, rows, cc, keys, stage, rs.word);
   } else {
-    sample_single<kOptions>(p, o0, c0, rows, cc, keys, stage, rs.word, track);
+    sample_single<kOptions>(p, windows, tag, o0, c0, rows, cc, keys, stage, rs.word);
   }
   __syncthreads();
   for (uint32_t l = 0; l < (uint32_t)kMaxLevels; ++l) {
@@ -711,24 +755,25 @@ __device__ __forceinline__ void sample_block(const SampleParams& p, uint32_t blo
     const uint32_t* sums = rs.word + l * pitch;
     for (uint32_t r = threadIdx.x; r < rows; r += blockDim.x) {
       const uint32_t at = l * O + o0 + r;
-      // a block that could not keep sums (more rows than the table holds) leaves the bound unknown
-      if (!track) atomicMax(&p.rowsum[at], 0xFFFFFFFFu);
-      else if (sums[r]) atomicAdd(&p.rowsum[at], sums[r]);
-      if (has_planes) {
-        const long long sum = (long long)(int)sums[2 * kPlaneRows + r] * 4096 + (long long)sums[kPlaneRows + r];
-        if (sum) atomicAdd(reinterpret_cast<unsigned long long*>(p.corr + at), (unsigned long long)(sum * 128));
+      const long long sum = has_planes ? 128 * ((long long)(int)sums[2 * kPlaneRows + r] * 4096 + (long long)sums[kPlaneRows + r]) : 0;
+      if (kFused) {
+        p.rowsum[at] = sums[r];
+        if (has_planes) p.corr[at] = sum;
+      } else {
+        if (sums[r]) atomicAdd(&p.rowsum[at], sums[r]);
+        if (sum) atomicAdd(reinterpret_cast<unsigned long long*>(p.corr + at), (unsigned long long)sum);
       }
     }
   }
 }
 
-template <bool kOptions>
-__global__ void __launch_bounds__(kThreads) sample_kernel(const __grid_constant__ SampleParams p,
-                                                          const __grid_constant__ PhiloxKeys keys) {
+template <bool kOptions, bool kFused>
+__global__ void __launch_bounds__(kThreads, 4) sample_kernel(const __grid_constant__ SampleParams p,
+                                                          const __grid_constant__ PhiloxKeys keys, uint32_t* err) {
   pdl_prologue();
   __shared__ __align__(16) float stage[kStage];
   __shared__ RowSums rs;
-  sample_block<kOptions>(p, blockIdx.x, keys, stage, rs);
+  sample_block<kOptions, kFused>(p, blockIdx.x, keys, stage, rs, err);
 }
 
 // All layers of a network in two launches.  Entry i owns blocks [first, first + count) of each
@@ -772,7 +817,7 @@ __global__ void __launch_bounds__(kThreads) sample_batch_kernel(const BatchEntry
   __syncthreads();
   if (threadIdx.x == 0) p.e_tag = tag;
   __syncthreads();
-  sample_block<kOptions>(p, blockIdx.x - first, keys, stage, rs);
+  sample_block<kOptions, false>(p, blockIdx.x - first, keys, stage, rs, nullptr);
 }
 
 // The integer filter of one level put together from its digit planes, in canonical order or channels innermost: the
@@ -826,9 +871,20 @@ uint32_t emax_blocks_for(uint32_t O, uint32_t d, uint32_t norm) {
   return blocks < 1 ? 1 : (blocks > 1184 ? 1184 : blocks);
 }
 
+// A layer sampled by a launch of its own needs no exponent pass before it (a launch of about 3 us on the host and on
+// the device) where a block holds whole rows and their windows are its own (norm == 1), or where the layer is so small
+// that every block can look at all of it.  4096 x 4096 with a window per row and its contraction 224 -> 216 us;
+// 256 -> 128 features (32768 weights in blocks of 256) 18.2 -> 16.2 us in a stream of calls; 3x3 64 -> 64 channels
+// (36864 weights, 576 a row) 27.1 -> 33.2: too few blocks, each reading too much.
+bool fused_sampling(const psb_weights* wt) {
+  return wt->cfg.norm ? wt->d <= 4096u : wt->d <= 256u && (uint64_t)wt->shape.out_ch * wt->d <= 32768u;
+}
+
+enum class SampleLaunch { kBatch, kTwoPass, kFused };
+
 // Parameters of one layer's sampling pass; returns the number of blocks it needs.
 uint32_t fill_sample_params(const float* w_dev, const psb_weights* wt, uint32_t* e_max, SampleParams& p,
-                            bool batched) {
+                            SampleLaunch how) {
   const psb_wshape& sh = wt->shape;
   const uint32_t O = sh.out_ch, Cg = sh.in_ch_per_group, KHKW = sh.kh * sh.kw, d = wt->d;
   p.w = w_dev;
@@ -836,7 +892,8 @@ uint32_t fill_sample_params(const float* w_dev, const psb_weights* wt, uint32_t*
   // weights per block: enough that what a block does once (its parameters, sums, barriers) is a small part of it, yet
   // several blocks per SM: a batched launch is filled by the other layers, a layer of its own is cut finer
   const uint64_t total = (uint64_t)O * d;
-  uint32_t budget = batched ? 4096u : (uint32_t)std::min<uint64_t>(4096u, std::max<uint64_t>(256u, total / 592u));
+  uint32_t budget = how == SampleLaunch::kBatch ? 4096u : (uint32_t)std::min<uint64_t>(4096u, std::max<uint64_t>(256u, total / 592u));
+  if (how == SampleLaunch::kFused && budget < d) budget = d;
   if (budget < 4u * KHKW) budget = 4u * KHKW;   // at least four channels (host validation keeps kh*kw <= 2048)
   const uint32_t sum_rows = wt->has_planes ? (uint32_t)kPlaneRows : (uint32_t)kRowSumRows;
   if (d <= budget) {
@@ -892,6 +949,15 @@ cudaError_t launch_expand(const psb_weights* wt, uint32_t level, bool canonical,
 }
 
 cudaError_t launch_sampler(const float* w_dev, psb_weights* wt, uint32_t* err_dev, cudaStream_t s) {
+  const PhiloxKeys keys((uint32_t)wt->cfg.seed, (uint32_t)(wt->cfg.seed >> 32));
+  SampleParams p;
+  if (fused_sampling(wt)) {
+    const uint32_t blocks = fill_sample_params(w_dev, wt, wt->e_max, p, SampleLaunch::kFused);
+    if (p.pbits | p.underflow) launch_pdl(sample_kernel<true, true>, blocks, kThreads, 0, s, p, keys, err_dev);
+    else launch_pdl(sample_kernel<false, true>, blocks, kThreads, 0, s, p, keys, err_dev);
+    note_launch();
+    return cudaGetLastError();
+  }
   const uint32_t O = wt->shape.out_ch;
   // the exponent maxima carry the number of the call that wrote them; the words were cleared when
   // the handle was made and are cleared again only when the 24-bit call number wraps
@@ -903,12 +969,10 @@ cudaError_t launch_sampler(const float* w_dev, psb_weights* wt, uint32_t* err_de
   }
   launch_pdl(emax_kernel, emax_blocks_for(O, wt->d, wt->cfg.norm), kThreads, 0, s, w_dev, O, wt->d, wt->cfg.norm,
              wt->e_max, err_dev, wt->e_calls << 8, wt->rowsum256, wt->corr128, wt->cfg.prob_bits); note_launch();
-  SampleParams p;
-  const uint32_t blocks = fill_sample_params(w_dev, wt, wt->e_max, p, false);
+  const uint32_t blocks = fill_sample_params(w_dev, wt, wt->e_max, p, SampleLaunch::kTwoPass);
   p.e_tag = wt->e_calls;
-  const PhiloxKeys keys((uint32_t)wt->cfg.seed, (uint32_t)(wt->cfg.seed >> 32));
-  if (p.pbits | p.underflow) launch_pdl(sample_kernel<true>, blocks, kThreads, 0, s, p, keys);
-  else launch_pdl(sample_kernel<false>, blocks, kThreads, 0, s, p, keys);
+  if (p.pbits | p.underflow) launch_pdl(sample_kernel<true, false>, blocks, kThreads, 0, s, p, keys, err_dev);
+  else launch_pdl(sample_kernel<false, false>, blocks, kThreads, 0, s, p, keys, err_dev);
   note_launch();
   return cudaGetLastError();
 }
@@ -945,7 +1009,7 @@ psb_status sample_batch_create(psb_ctx* ctx, uint32_t n, const float* const* w_d
     for (uint32_t i = 0; i < n; ++i) {
       const psb_weights* wt = weights[i];
       BatchEntry& e = host[i];
-      e.sample_blocks = fill_sample_params(w_dev[i], wt, b->e_max_pool + off, e.p, true);
+      e.sample_blocks = fill_sample_params(w_dev[i], wt, b->e_max_pool + off, e.p, SampleLaunch::kBatch);
       b->options = b->options || (e.p.pbits | e.p.underflow);
       e.emax_blocks = emax_blocks_for(wt->shape.out_ch, wt->d, wt->cfg.norm);
       e.emax_first = eb;
