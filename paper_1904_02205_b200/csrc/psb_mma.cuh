@@ -13,11 +13,8 @@
 //   warps 0-1 producers (one thread each, taking the stages in turns): TMA loads of the activation tile (im2col mode for
 //            filters with taps, stride or padding; plain 2-D tiles otherwise) and
 //            of the digit-plane tile into a ring of shared-memory stages
-//   warps 2-3 MMA issuers (one thread each; warp 3 also allocates TMEM): the pipeline stages
-//            alternate between them.  The tensor pipe takes only a few MMAs ahead of the one it
-//            executes, so whatever else an issuing thread does (barrier waits, commits, tile
-//            bookkeeping: a few hundred clocks per stage) would leave the pipe idle; with two
-//            issuers one thread's bookkeeping runs under the other's MMAs
+//   warp 2 issues the MMAs
+//   warp 3 allocates TMEM; issues half of the MMAs in band mode; flips the top bit of unsigned activations
 //   warps 4-19 epilogue: TMEM -> registers, recombine planes, dequantise, bias,
 //            shortcut, ReLU, re-quantise, vectorised stores; overlaps the next
 //            tile's MMAs through two TMEM accumulator buffers
@@ -40,8 +37,9 @@ namespace {
 
 constexpr int kTileM = 128;
 constexpr int kProducerWarps = 2;    // one issuing thread each: their barrier waits overlap
-constexpr int kMmaWarp0 = kProducerWarps;          // issues the even passes
-constexpr int kMmaWarp1 = kMmaWarp0 + 1;           // issues the odd passes; owns the TMEM allocation
+constexpr int kMmaWarp0 = kProducerWarps;          // issues the MMAs
+constexpr int kMmaWarp1 = kMmaWarp0 + 1;           // band mode: issues half of them; flips unsigned activations; owns the
+                                                   // TMEM allocation
 constexpr int kFirstEpilogueWarp = kMmaWarp1 + 1;  // a multiple of 4: warp & 3 = TMEM lane quarter
 constexpr int kPlaneBars = 4;        // resident digit planes arrive in this many parts, each with its barrier
 constexpr int kEpilogueWarps = 16;
@@ -51,8 +49,6 @@ constexpr uint32_t kTmemBufStride = 256;
 constexpr int kMaxStages = 12;
 constexpr uint32_t kResidentMaxBytes = 112 * 1024;          // digit planes kept in shared memory
 constexpr size_t kSmemBudget = 227 * 1024;
-constexpr int kTapBatch = 6;                                // descriptor offsets fetched ahead of their MMAs
-constexpr int kMaxBandMmas = 128;                           // MMAs per tile (taps x K steps) that band mode handles
 
 }  // namespace
 
@@ -215,27 +211,25 @@ __device__ __forceinline__ void tc_commit(uint32_t bar) {
                : "memory");
 }
 
-// The same instruction for the issue loops: accumulate always, descriptors given as (low word, high word),
-// no memory clobber (the loop's own loads of descriptor offsets may then be scheduled ahead of it; the
-// operands are written by the copy engine and ordered by the barrier waits, which keep their clobbers).
-template <bool ACC>
-__device__ __forceinline__ void tc_mma_i8_lohi(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t desc_hi,
-                                               uint32_t idesc) {
+// One lane of the (converged) warp.  The MMA role runs with all 32 lanes and lets one of them issue: its addresses are
+// then warp-uniform values, which is where the instruction wants its descriptors.  In code that only one lane enters,
+// every descriptor word is moved from a vector register first, about 100 clocks per MMA.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t e;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(e));
+  return e != 0u;
+}
+
+// Descriptors given as (low word, high word); `acc` 0 overwrites the accumulator.
+__device__ __forceinline__ void tc_mma_i8(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t desc_hi, uint32_t idesc,
+                                          uint32_t acc) {
   asm volatile(
       "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
       "setp.ne.b32 p, %5, 0;\n\t"
       "mov.b64 da, {%1, %3};\n\t"
       "mov.b64 db, {%2, %3};\n\t"
       "tcgen05.mma.cta_group::1.kind::i8 [%0], da, db, %4, p;\n\t}"
-      ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(ACC ? 1u : 0u));
-}
-__device__ __forceinline__ void tc_mma_i8_acc(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t desc_hi,
-                                              uint32_t idesc) {
-  tc_mma_i8_lohi<true>(d_tmem, a_lo, b_lo, desc_hi, idesc);
-}
-__device__ __forceinline__ void tc_mma_i8_zero(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t desc_hi,
-                                               uint32_t idesc) {
-  tc_mma_i8_lohi<false>(d_tmem, a_lo, b_lo, desc_hi, idesc);
+      ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(acc));
 }
 
 __device__ __forceinline__ void tc_ld16(uint32_t taddr, uint32_t (&v)[16]) {
@@ -302,11 +296,10 @@ struct SharedCtl {
   unsigned long long acc_full[2];
   unsigned long long acc_empty[2];
   unsigned long long planes_full[kPlaneBars];
-  unsigned long long started[2];        // per accumulator buffer: the zeroing MMA of the pass has been issued
-  unsigned long long pass_issued;       // all but the last K block of a pass have been issued (phase = pass number)
-  uint2 tap_tab[2][kMaxBandMmas];       // band mode, per issuing thread: (activation, plane) descriptor offsets of the
-                                        // tile's MMAs, in units of 16 bytes
+  unsigned long long started[2];        // band mode, per accumulator buffer: the overwriting MMA of the tile has been issued
+  unsigned long long flipped[kMaxStages];   // full, and the top bits flipped (unsigned activations)
   uint32_t tmem_base;
+  uint32_t rowmax[kMaxLevels];          // largest row sum of |W_k| per level (units of 256), see find_row_maxima
   WaitCtl wait;
   alignas(16) int32_t corr32[kEpilogueWarps][16];   // low words of the integer addends
   alignas(16) float2 scb[kEpilogueWarps][16];   // per epilogue warp: (scale * 2^(e_base - log2 k), bias), read two
@@ -640,17 +633,28 @@ struct RowMapBand {
   }
 };
 
-// Whether the accumulators of level l stay below 2^31 in magnitude: (largest row sum of |W_k|, kept by the
-// sampler in units of 256, each weight rounded up) x (largest activation magnitude; with an integer addend the
-// magnitude before the offset, since the sum that counts is the one after the addend).  Warp-collective: the
-// lanes share the scan over the rows.
-__device__ __forceinline__ bool fits_32_bits(const TensorParams& p, uint32_t l) {
-  if (!p.rowsum256) return false;
-  const uint32_t* sums = p.rowsum256 + (size_t)l * p.a.O;
-  uint32_t best = 0;
-  for (uint32_t o = threadIdx.x & 31u; o < p.a.O; o += 32u) best = max(best, sums[o]);
-  best = __reduce_max_sync(0xFFFFFFFFu, best);
-  // (a sum that wrapped or was marked unknown reads as huge either way)
+// Largest row sum of |W_k| (kept by the sampler in units of 256, each contribution rounded up) of every sampled level the
+// call may use, by all epilogue warps together: one warp alone scans 2048 rows in 16 rounds of L2 latency, once per
+// level.  (Draw-count maps with five levels, ResNet-50 shape, batch 128: 5541 -> 5512 us.)
+__device__ __forceinline__ void find_row_maxima(const TensorParams& p, SharedCtl* ctl, uint32_t levels) {
+  const uint32_t et = threadIdx.x - 32u * (uint32_t)kFirstEpilogueWarp;
+  for (uint32_t l = 0; l < (uint32_t)kMaxLevels; ++l) {
+    if (!((levels >> l) & 1u)) continue;
+    const uint32_t* sums = p.rowsum256 + (size_t)l * p.a.O;
+    uint32_t best = 0;
+#pragma unroll 4
+    for (uint32_t o = et; o < p.a.O; o += 32u * (uint32_t)kEpilogueWarps) best = max(best, sums[o]);
+    best = __reduce_max_sync(0xFFFFFFFFu, best);
+    if ((threadIdx.x & 31u) == 0u && best) atomicMax(&ctl->rowmax[l], best);
+  }
+  asm volatile("bar.sync 1, %0;" ::"n"(32 * kEpilogueWarps) : "memory");
+}
+
+// Whether the accumulators of level l stay below 2^31 in magnitude: row sum x largest activation magnitude (with an
+// integer addend the magnitude before the offset, since the sum that counts is the one after the addend).
+__device__ __forceinline__ bool fits_32_bits(const TensorParams& p, const SharedCtl* ctl, uint32_t l) {
+  const uint32_t best = ctl->rowmax[l];
+  // (a sum that wrapped reads as huge)
   return (unsigned long long)best * 256ull * (unsigned long long)p.amax < (1ull << 31) && best < (1u << 24);
 }
 
@@ -849,195 +853,107 @@ __device__ __forceinline__ bool uniform_dispatch(const TensorParams& p, SharedCt
   return uniform_dispatch_tail<P, false, 2>(p, ctl, tmem_base, ew, lane, c, fast_u8);
 }
 
-// The MMA issuing role, one thread of warp kMmaWarp0 (mine = 0) and one of kMmaWarp1 (mine = 1).
-// Both walk the same sequence of passes and ring stages; stage uses are numbered through the
-// whole kernel and the number's parity selects the thread.  The thread that owns the first
-// stage of a pass waits for the accumulator buffer and issues the zeroing MMA; the other one
-// joins the pass after that (`started`).  Integer accumulation is exact, so the order in
-// which the two threads' MMAs reach the accumulator is immaterial.  A parity wait on a stage
-// barrier is meaningful while the waiter is less than two uses of that stage ahead of it; the
-// ring has an even number of stages, so a thread always meets the same slots and its wait for
-// a slot follows its own previous use of that slot.  Kept out of line and fed from local copies of
-// the parameters so that its loop state lives in registers: the pipe idles for every clock this
-// thread spends between two MMAs beyond what the other thread covers.  Returns true on a timeout.
-//
-// Passes of a single stage are issued in their order: the first MMA of a pass follows the last but one K block
-// of the pass before it (`pass_issued`; the waits for the stage and the accumulator buffer are done by then).  Without
-// the rule both threads issue at once whenever both have a stage ready, the MMAs of two tiles interleave in
-// the pipe, both tiles complete late and together, and the pipe then idles until the output stage has
-// emptied an accumulator buffer.
-// Unsigned activations (p.flip): the 32 lanes of the issuing warp flip the top bit of every byte of the stage's
-// activation tiles in shared memory, between the copy's arrival and the MMAs (16 bytes per lane and step: a 16 KB
-// tile is 32 steps, which run under the other issuing thread's MMAs), and make the writes visible to the tensor
-// core's proxy.  A separate pass over the tensor in global memory, as there was before, cost a launch and a read and a
-// write of all activations, and could not serve padded filters.
-__device__ __forceinline__ void flip_tile(uint32_t addr, uint32_t bytes, uint32_t lane) {
-#pragma unroll 8
-  for (uint32_t b = lane * 16u; b < bytes; b += 512u) {
-    uint32_t x, y, z, w;
-    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(x), "=r"(y), "=r"(z), "=r"(w) : "r"(addr + b));
-    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(addr + b), "r"(x ^ 0x80808080u), "r"(y ^ 0x80808080u),
-                 "r"(z ^ 0x80808080u), "r"(w ^ 0x80808080u) : "memory");
-  }
+// All lanes of the warp wait together; false when a wait ran out.
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, WaitCtl* wc) {
+  return __all_sync(0xFFFFFFFFu, mbar_wait(bar, parity, wc, kNoSleep)) != 0;
 }
 
-// kWarp: the instance for layers with unsigned activations or a partly filled last channel block, run by the whole
-// warp; the other one, run by one thread, carries none of that code (it cost the plain layers 1 %).
-template <int BK, bool kWarp>
-__device__ __noinline__ bool mma_role(const TensorParams& p, SharedCtl* ctl, uint32_t tmem_base, uint32_t ring_addr,
-                                      uint32_t planes_addr, uint32_t stage_bytes, uint32_t sub_bytes,
-                                      uint32_t k_iters, uint32_t mine) {
-  WaitCtl* abort = &ctl->wait;
-  // kWarp: the lanes leave the waits together
-  const uint32_t lane = threadIdx.x & 31u;
-  const bool leader = !kWarp || lane == 0u, flip = kWarp && p.flip != 0u;
-  auto wait = [&](uint32_t bar, uint32_t parity, uint32_t backoff = 0u) {
-    const bool ok = mbar_wait(bar, parity, abort, backoff);
-    return kWarp ? __all_sync(0xFFFFFFFFu, ok) != 0 : ok;
-  };
-  const uint32_t group = p.group, stages = p.stages, resident = p.resident, stage_bytes_a = p.stage_bytes_a;
-  const uint32_t level_mask = p.a.level_mask;
-  const uint32_t n_groups = (k_iters + group - 1) / group;
-  const uint32_t n_cb = p.n_cb, tail_ksteps = p.tail_ksteps;
-  const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
+// The MMA issuing role: one warp, inlined into the kernel so that its parameters come from the constant bank and its
+// addresses stay uniform.  Two single threads taking turns, out of line, as there were before, needed 100 to 250 clocks
+// per MMA and hand-overs between them (K block of 4 MMAs, streamed planes, 3x3 256 -> 256 channels: 753 -> 640 clocks;
+// the copies of a K block, 40 KB at the 68 bytes per clock and SM that L2 delivers to all SMs at once, take 600).
+// Returns true on a timeout.
+template <int BK>
+__device__ __forceinline__ bool mma_role(const TensorParams& p, SharedCtl* ctl, uint32_t tmem_base, uint32_t ring_addr,
+                                         uint32_t planes_addr, uint32_t stage_bytes, uint32_t sub_bytes, uint32_t k_iters) {
+  WaitCtl* wc = &ctl->wait;
+  const bool leader = elect_one();
+  const uint32_t full0 = smem_u32(p.flip ? &ctl->flipped[0] : &ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
   const uint32_t acc_full0 = smem_u32(&ctl->acc_full[0]), acc_empty0 = smem_u32(&ctl->acc_empty[0]);
-  const uint32_t started0 = smem_u32(&ctl->started[0]);
-  const uint32_t pass_issued = smem_u32(&ctl->pass_issued);
-  // (passes of several stages already have both threads at work on the same pass in turns; there the rule
-  // only took the overlap at the pass boundaries away and cost a few per cent)
-  const bool ordered = n_groups == 1u;
   const uint32_t desc_hi = smem_desc_hi(BK);
+  const bool whole = p.tail_ksteps == (uint32_t)(BK / 32);     // every K block is full of channels
   // resident digit planes: K blocks below planes_upto are known to have landed
   const uint32_t plane_part = (k_iters + kPlaneBars - 1) / kPlaneBars;
-  uint32_t planes_ready = 0, planes_upto = resident ? 0u : 0xFFFFFFFFu;
-  uint32_t s = 0, ph = 0, pass = 0, use = 0;
+  uint32_t planes_ready = 0, planes_upto = p.resident ? 0u : 0xFFFFFFFFu;
+  uint32_t s = 0, ph = 0, pass = 0;
   TileIter ti;
   for (ti.init(p); ti.valid(); ti.next()) {
-    const uint32_t levels = tile_levels(p, ti.m_tile) & level_mask;
-    for (uint32_t todo = levels & 0x7Fu; todo; todo &= todo - 1u) {
-      const uint32_t l = (uint32_t)__ffs((int)todo) - 1u;
-      const uint32_t P = p.planes[l];
-      const uint32_t buf = pass & 1u, aph = (pass >> 1) & 1u;
-      // instruction descriptor: s32 accumulators, s8 x s8, both K-major, M = 128, N = P * 64
-      const uint32_t idesc = (2u << 4) | (1u << 7) | (1u << 10) | (((P * kTileN) >> 3) << 17) |
-                             ((kTileM >> 4) << 24);
-      const uint32_t d_tmem = tmem_base + buf * kTmemBufStride;
-      const uint32_t blk = P * kTileN * BK;
-      bool joined = (use & 1u) == mine;
-      if (joined) {
-        if (!wait(acc_empty0 + 8u * buf, aph ^ 1u)) return true;
-        tc_fence_after();
+    const uint32_t levels = tile_levels(p, ti.m_tile) & p.a.level_mask & 0x7Fu;
+    if (!levels) continue;      // no sampled level: no pass from any role
+    const uint32_t P = p.planes[(uint32_t)__ffs((int)levels) - 1u];
+    const uint32_t buf = pass & 1u, aph = (pass >> 1) & 1u;
+    ++pass;
+    // instruction descriptor: s32 accumulators, s8 x s8, both K-major, M = 128, N = P * 64
+    const uint32_t idesc = (2u << 4) | (1u << 7) | (1u << 10) | (((P * kTileN) >> 3) << 17) | ((kTileM >> 4) << 24);
+    const uint32_t d_tmem = tmem_base + buf * kTmemBufStride;
+    const uint32_t blk = P * kTileN * BK;
+    if (!warp_wait(acc_empty0 + 8u * buf, aph ^ 1u, wc)) return true;
+    tc_fence_after();
+    uint32_t b_res = planes_addr, acc = 0u, cb = 0u;
+    for (uint32_t it = 0; it < k_iters;) {
+      const uint32_t cnt = min(p.group, k_iters - it);
+      if (!warp_wait(full0 + 8u * s, ph, wc)) return true;
+      while (it + cnt > planes_upto) {
+        if (!warp_wait(smem_u32(&ctl->planes_full[planes_ready]), 0u, wc)) return true;
+        ++planes_ready;
+        planes_upto = planes_ready == (uint32_t)kPlaneBars ? 0xFFFFFFFFu : planes_upto + plane_part;
       }
-      uint32_t b_res = planes_addr, g = 0;
-      for (uint32_t it = 0; it < k_iters; ++g, ++use) {
-        const uint32_t cnt = min(group, k_iters - it);
-        if ((use & 1u) == mine) {
-          if (!joined) {
-            if (!wait(started0 + 8u * buf, aph)) return true;
-            joined = true;
-          }
-          if (!wait(full0 + 8u * s, ph)) return true;
-          while (it + cnt > planes_upto) {
-            if (!wait(smem_u32(&ctl->planes_full[planes_ready]), 0u)) return true;
-            ++planes_ready;
-            planes_upto = planes_ready == (uint32_t)kPlaneBars ? 0xFFFFFFFFu : planes_upto + plane_part;
-          }
-          if (flip) {
-            for (uint32_t j = 0; j < cnt; ++j) flip_tile(ring_addr + s * stage_bytes + j * sub_bytes, stage_bytes_a, lane);
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            __syncwarp();
-          }
-          if (ordered && pass != 0u) {
-            if (!wait(pass_issued, (pass - 1u) & 1u, kNoSleep)) return true;
-          }
-          tc_fence_after();
-          // K blocks of the stage: activation tiles sub_bytes apart, planes beside them or resident; only the
-          // low words of the descriptors move (by bytes / 16)
-          uint32_t a_lo = smem_desc_lo(ring_addr + s * stage_bytes);
-          uint32_t b_lo = resident ? smem_desc_lo(b_res) : a_lo + (stage_bytes_a >> 4);
-          const uint32_t a_step = sub_bytes >> 4, b_step = resident ? blk >> 4 : sub_bytes >> 4;
+      tc_fence_after();
+      // K blocks of the stage: activation tiles sub_bytes apart, planes beside them or resident; only the
+      // low words of the descriptors move (by bytes / 16)
+      uint32_t a_lo = smem_desc_lo(ring_addr + s * stage_bytes);
+      uint32_t b_lo = p.resident ? smem_desc_lo(b_res) : a_lo + (p.stage_bytes_a >> 4);
+      const uint32_t a_step = sub_bytes >> 4, b_step = p.resident ? blk >> 4 : sub_bytes >> 4;
+      for (uint32_t j = 0; j < cnt; ++j, a_lo += a_step, b_lo += b_step) {
+        // a tap's last channel block: only the K steps that hold channels
+        const bool tail = ++cb == p.n_cb;
+        if (tail) cb = 0u;
+        if (whole || !tail) {
           if (leader) {
-            if (!kWarp) {
-              for (uint32_t j = 0; j < cnt; ++j, a_lo += a_step, b_lo += b_step) {
-                // the pass after this one may start under this pass's last K block
-                if (ordered && j + 1u == cnt) mbar_arrive(pass_issued);
-                if (it == 0 && j == 0) {
-                  tc_mma_i8_zero(d_tmem, a_lo, b_lo, desc_hi, idesc);
+            tc_mma_i8(d_tmem, a_lo, b_lo, desc_hi, idesc, acc);
 #pragma unroll
-                  for (int ks = 1; ks < BK / 32; ++ks) tc_mma_i8_acc(d_tmem, a_lo + 2 * ks, b_lo + 2 * ks, desc_hi, idesc);
-                } else {
-#pragma unroll
-                  for (int ks = 0; ks < BK / 32; ++ks) tc_mma_i8_acc(d_tmem, a_lo + 2 * ks, b_lo + 2 * ks, desc_hi, idesc);
-                }
-              }
-            } else {
-              uint32_t cb = it % n_cb;
-              for (uint32_t j = 0; j < cnt; ++j, a_lo += a_step, b_lo += b_step) {
-                if (ordered && j + 1u == cnt) mbar_arrive(pass_issued);
-                const bool tail = ++cb == n_cb;      // the tap's last channel block: only the K steps that hold channels
-                if (tail) cb = 0u;
-                if (it == 0 && j == 0) tc_mma_i8_zero(d_tmem, a_lo, b_lo, desc_hi, idesc);
-                else tc_mma_i8_acc(d_tmem, a_lo, b_lo, desc_hi, idesc);
-#pragma unroll
-                for (int ks = 1; ks < BK / 32; ++ks)
-                  if (!tail || (uint32_t)ks < tail_ksteps) tc_mma_i8_acc(d_tmem, a_lo + 2 * ks, b_lo + 2 * ks, desc_hi, idesc);
-              }
-            }
-            if (it == 0 && n_groups > 1u) {
-              tc_fence_before();
-              mbar_arrive(started0 + 8u * buf);
-            }
-            tc_commit(empty0 + 8u * s);
-            // this thread's last stage of the pass: the last or the last but one
-            if (g + 2u >= n_groups) tc_commit(acc_full0 + 8u * buf);
+            for (int ks = 1; ks < BK / 32; ++ks) tc_mma_i8(d_tmem, a_lo + 2 * ks, b_lo + 2 * ks, desc_hi, idesc, 1u);
           }
-          if (kWarp) __syncwarp();
+        } else {
+          for (uint32_t ks = 0; ks < p.tail_ksteps; ++ks)
+            if (leader) tc_mma_i8(d_tmem, a_lo + 2 * ks, b_lo + 2 * ks, desc_hi, idesc, ks ? 1u : acc);
         }
-        b_res += cnt * blk;
-        it += cnt;
-        if (++s == stages) { s = 0; ph ^= 1u; }
+        acc = 1u;
       }
-      ++pass;
+      if (leader) tc_commit(empty0 + 8u * s);
+      b_res += cnt * blk;
+      it += cnt;
+      if (++s == p.stages) { s = 0; ph ^= 1u; }
     }
+    if (leader) tc_commit(acc_full0 + 8u * buf);
+    __syncwarp();
   }
   return false;
 }
 
-// The same role in band mode, where a ring stage holds the band of a whole tile: both threads work on every
-// tile, thread 0 on the first half of its MMAs (taps x K steps), thread 1 on the second half, both into the
-// one accumulator (the order of integer additions is immaterial).  One thread alone needs about 115 clocks
-// per MMA where the pipe needs 96, and a hand-over between tiles costs a few hundred more; two threads on
-// the same tile keep the pipe fed and the tiles in order.  Thread 0 issues the zeroing MMA first (`started`);
-// both commit to the stage's and the accumulator's barriers (count 2 in this mode).  The descriptor offsets of
-// a thread's MMAs are computed once (a table in shared memory, read a few entries ahead of the MMAs); the
-// issue loop then spends two additions per MMA.
+// The same role in band mode, where a ring stage holds the band of a whole tile: two warps work on every tile, the first
+// on the first half of its taps, the second (mine = 1) on the rest, both into the one accumulator (the order of integer
+// additions is immaterial), so that one's bookkeeping between tiles runs under the other's MMAs (3x3 64 -> 64 channels,
+// 56x56, batch 64: 23.4 us with one warp).  The first one issues the overwriting MMA (`started`); both commit to the
+// stage's and the accumulator's barriers (count 2 in this mode).
 template <int BK>
-__device__ __noinline__ bool mma_role_band(const TensorParams& p, SharedCtl* ctl, uint32_t tmem_base,
-                                           uint32_t ring_addr, uint32_t planes_addr, uint32_t stage_bytes,
-                                           uint32_t mine) {
-  WaitCtl* abort = &ctl->wait;
-  const uint32_t stages = p.stages, row_bytes = p.Wp * p.a.C, KH = p.a.KH, KW = p.a.KW;
+__device__ __forceinline__ bool mma_role_band(const TensorParams& p, SharedCtl* ctl, uint32_t tmem_base,
+                                              uint32_t ring_addr, uint32_t planes_addr, uint32_t stage_bytes, uint32_t mine) {
+  WaitCtl* wc = &ctl->wait;
+  const bool leader = elect_one();
   const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
   const uint32_t acc_full0 = smem_u32(&ctl->acc_full[0]), acc_empty0 = smem_u32(&ctl->acc_empty[0]);
   const uint32_t started0 = smem_u32(&ctl->started[0]);
   const uint32_t desc_hi = smem_desc_hi(BK);
   const uint32_t P = p.planes[p.a.uniform_log2k];
   const uint32_t idesc = (2u << 4) | (1u << 7) | (1u << 10) | (((P * kTileN) >> 3) << 17) | ((kTileM >> 4) << 24);
-  const uint32_t blk = P * kTileN * BK;
-  constexpr uint32_t kSteps = BK / 32;
-  const uint32_t n_mmas = KH * KW * kSteps, half = (n_mmas + 1u) / 2u;
-  const uint32_t j_begin = mine ? half : 0u, cnt = mine ? n_mmas - half : half;
-  uint2* const tab = ctl->tap_tab[mine];
-  for (uint32_t i = 0; i < (cnt + kTapBatch - 1) / kTapBatch * kTapBatch; ++i) {
-    const uint32_t j = j_begin + i, tap = j / kSteps, ks = j - tap * kSteps, kh = tap / KW, kw = tap - kh * KW;
-    tab[i] = i < cnt ? make_uint2((kh * row_bytes + kw * (uint32_t)BK + ks * 32u) >> 4, (tap * blk + ks * 32u) >> 4)
-                     : make_uint2(0u, 0u);
-  }
-  // resident digit planes arrive in kPlaneBars parts of `plane_part` K blocks (= taps): this thread needs the
-  // parts up to the one that holds its last tap
-  const uint32_t k_iters = KH * KW, plane_part = (k_iters + kPlaneBars - 1) / kPlaneBars;
-  const uint32_t parts_needed = min((uint32_t)kPlaneBars, (j_begin + cnt - 1u) / kSteps / plane_part + 1u);
-  const uint32_t planes_lo = smem_desc_lo(planes_addr);
+  const uint32_t b_step = P * kTileN * BK / 16u, row_step = p.Wp * p.a.C / 16u;
+  const uint32_t taps = p.a.KH * p.a.KW, half = (taps + 1u) / 2u;
+  const uint32_t tap0 = mine ? half : 0u, tap1 = mine ? taps : half;
+  const uint32_t kh0 = tap0 / p.a.KW, kw0 = tap0 - kh0 * p.a.KW;
+  // resident digit planes arrive in kPlaneBars parts of `plane_part` K blocks (= taps)
+  const uint32_t plane_part = (taps + kPlaneBars - 1) / kPlaneBars;
+  const uint32_t parts_needed = tap1 > tap0 ? min((uint32_t)kPlaneBars, (tap1 - 1u) / plane_part + 1u) : 0u;
   uint32_t s = 0, ph = 0, pass = 0;
   TileIter ti;
   for (ti.init(p); ti.valid(); ti.next(), ++pass) {
@@ -1046,33 +962,69 @@ __device__ __noinline__ bool mma_role_band(const TensorParams& p, SharedCtl* ctl
     // byte offset of the tile's first position in its band
     const uint32_t t0 = (ti.m_tile - __umulhi(ti.m_tile, p.tpi_magic) * p.tpi) * kTileM;
     const uint32_t band_off = (t0 - __umulhi(t0, p.Wp_magic) * p.Wp) * (uint32_t)BK;
-    if (!mbar_wait(acc_empty0 + 8u * buf, aph ^ 1u, abort)) return true;
-    if (mine && !mbar_wait(started0 + 8u * buf, aph, abort, kNoSleep)) return true;
-    if (!mbar_wait(full0 + 8u * s, ph, abort)) return true;
+    if (!warp_wait(acc_empty0 + 8u * buf, aph ^ 1u, wc)) return true;
+    if (!warp_wait(full0 + 8u * s, ph, wc)) return true;
     if (pass == 0u)
       for (uint32_t b = 0; b < parts_needed; ++b)
-        if (!mbar_wait(smem_u32(&ctl->planes_full[b]), 0u, abort)) return true;
+        if (!warp_wait(smem_u32(&ctl->planes_full[b]), 0u, wc)) return true;
+    if (mine && !warp_wait(started0 + 8u * buf, aph, wc)) return true;
     tc_fence_after();
-    const uint32_t a0 = smem_desc_lo(ring_addr + s * stage_bytes + band_off);
-    for (uint32_t i0 = 0; i0 < cnt; i0 += kTapBatch) {
-      uint2 t[kTapBatch];
-#pragma unroll
-      for (int j = 0; j < kTapBatch; ++j) t[j] = tab[i0 + j];
-#pragma unroll
-      for (int j = 0; j < kTapBatch; ++j) {
-        if (i0 + (uint32_t)j >= cnt) break;
-        if (j == 0 && i0 == 0u && !mine) {
-          tc_mma_i8_zero(d_tmem, a0 + t[0].x, planes_lo + t[0].y, desc_hi, idesc);
+    uint32_t a_row = smem_desc_lo(ring_addr + s * stage_bytes + band_off) + kh0 * row_step, kw = kw0;
+    uint32_t b_lo = smem_desc_lo(planes_addr) + tap0 * b_step;
+    for (uint32_t tap = tap0; tap < tap1; ++tap, b_lo += b_step) {
+      const uint32_t a_lo = a_row + kw * (BK / 16u);
+      if (leader) {
+        tc_mma_i8(d_tmem, a_lo, b_lo, desc_hi, idesc, tap ? 1u : 0u);
+        if (tap == 0u) {
           tc_fence_before();
           mbar_arrive(started0 + 8u * buf);
-        } else {
-          tc_mma_i8_acc(d_tmem, a0 + t[j].x, planes_lo + t[j].y, desc_hi, idesc);
+        }
+#pragma unroll
+        for (int ks = 1; ks < BK / 32; ++ks) tc_mma_i8(d_tmem, a_lo + 2 * ks, b_lo + 2 * ks, desc_hi, idesc, 1u);
+      }
+      if (++kw == p.a.KW) { kw = 0; a_row += row_step; }
+    }
+    if (leader) {
+      tc_commit(empty0 + 8u * s);
+      tc_commit(acc_full0 + 8u * buf);
+    }
+    __syncwarp();
+    if (++s == p.stages) { s = 0; ph ^= 1u; }
+  }
+  return false;
+}
+
+// Unsigned activations (p.flip): a warp of its own flips the top bit of every byte of the stages' activation tiles in
+// shared memory, between the copy's arrival and the MMAs, makes the writes visible to the tensor core's proxy and
+// hands the stage on (`flipped`).  A 16 KB tile is 32 steps of 16 bytes per lane, about the time of the four MMAs of its K
+// block, under which it runs.  (A pass over the tensor in global memory cost a launch and a read and a write of all
+// activations, and could not serve padded filters.)
+__device__ __forceinline__ bool flip_role(const TensorParams& p, SharedCtl* ctl, uint32_t ring_addr, uint32_t stage_bytes,
+                                          uint32_t sub_bytes, uint32_t k_iters) {
+  const uint32_t lane = threadIdx.x & 31u;
+  uint32_t s = 0, ph = 0;
+  TileIter ti;
+  for (ti.init(p); ti.valid(); ti.next()) {
+    if (!(tile_levels(p, ti.m_tile) & p.a.level_mask & 0x7Fu)) continue;
+    for (uint32_t it = 0; it < k_iters;) {
+      const uint32_t cnt = min(p.group, k_iters - it);
+      if (!warp_wait(smem_u32(&ctl->full[s]), ph, &ctl->wait)) return true;
+      for (uint32_t j = 0; j < cnt; ++j) {
+        const uint32_t addr = ring_addr + s * stage_bytes + j * sub_bytes;
+#pragma unroll 8
+        for (uint32_t b = lane * 16u; b < p.stage_bytes_a; b += 512u) {
+          uint32_t x, y, z, w;
+          asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(x), "=r"(y), "=r"(z), "=r"(w) : "r"(addr + b));
+          asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(addr + b), "r"(x ^ 0x80808080u), "r"(y ^ 0x80808080u),
+                       "r"(z ^ 0x80808080u), "r"(w ^ 0x80808080u) : "memory");
         }
       }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&ctl->flipped[s]));
+      it += cnt;
+      if (++s == p.stages) { s = 0; ph ^= 1u; }
     }
-    tc_commit(empty0 + 8u * s);
-    tc_commit(acc_full0 + 8u * buf);
-    if (++s == stages) { s = 0; ph ^= 1u; }
   }
   return false;
 }
@@ -1099,11 +1051,11 @@ psb_mma_kernel(const __grid_constant__ TmapSet maps, const __grid_constant__ Ten
   if (threadIdx.x == 0) {
     for (uint32_t s = 0; s < p.stages; ++s) {
       mbar_init(smem_u32(&ctl->full[s]), 1);
-      mbar_init(smem_u32(&ctl->empty[s]), p.band ? 2u : 1u);     // band mode: both issuing threads use every stage
+      mbar_init(smem_u32(&ctl->empty[s]), p.band ? 2u : 1u);     // band mode: two warps use every stage
+      mbar_init(smem_u32(&ctl->flipped[s]), 1);
     }
     for (int b = 0; b < 2; ++b) {
-      // both issuing threads commit to it when a pass has more than one stage, and in band mode
-      mbar_init(smem_u32(&ctl->acc_full[b]), (p.band || (k_iters + p.group - 1) / p.group > 1u) ? 2u : 1u);
+      mbar_init(smem_u32(&ctl->acc_full[b]), p.band ? 2u : 1u);
       mbar_init(smem_u32(&ctl->acc_empty[b]), kEpilogueWarps);
     }
     {  // part b of the resident planes holds K blocks [b * part, (b + 1) * part): one arrival per block
@@ -1114,7 +1066,7 @@ psb_mma_kernel(const __grid_constant__ TmapSet maps, const __grid_constant__ Ten
       }
     }
     for (int b = 0; b < 2; ++b) mbar_init(smem_u32(&ctl->started[b]), 1);
-    mbar_init(smem_u32(&ctl->pass_issued), 1);
+    for (int l = 0; l < kMaxLevels; ++l) ctl->rowmax[l] = 0u;
     ctl->wait.abort = 0;
     ctl->wait.limit = p.wait_limit;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -1219,15 +1171,12 @@ psb_mma_kernel(const __grid_constant__ TmapSet maps, const __grid_constant__ Ten
     }
   } else if (warp == (uint32_t)kMmaWarp0 || warp == (uint32_t)kMmaWarp1) {
     // ---------------------------------------------------------------- MMA
-    if (p.flip || p.tail_ksteps != (uint32_t)(BK / 32))
-      failed = mma_role<BK, true>(p, ctl, tmem_base, smem_u32(ring), smem_u32(smem), stage_bytes, sub_bytes, k_iters,
-                                  warp - (uint32_t)kMmaWarp0);
-    else if (lane == 0)
-      failed = p.band ? mma_role_band<BK>(p, ctl, tmem_base, smem_u32(ring), smem_u32(smem), stage_bytes,
-                                          warp - (uint32_t)kMmaWarp0)
-                      : mma_role<BK, false>(p, ctl, tmem_base, smem_u32(ring), smem_u32(smem), stage_bytes, sub_bytes,
-                                            k_iters, warp - (uint32_t)kMmaWarp0);
-    failed = __shfl_sync(0xFFFFFFFFu, failed ? 1 : 0, 0) != 0;
+    if (p.band)
+      failed = mma_role_band<BK>(p, ctl, tmem_base, smem_u32(ring), smem_u32(smem), stage_bytes, warp - (uint32_t)kMmaWarp0);
+    else if (warp == (uint32_t)kMmaWarp0)
+      failed = mma_role<BK>(p, ctl, tmem_base, smem_u32(ring), smem_u32(smem), stage_bytes, sub_bytes, k_iters);
+    else if (p.flip)
+      failed = flip_role(p, ctl, smem_u32(ring), stage_bytes, sub_bytes, k_iters);
   } else {
     // ----------------------------------------------------------- epilogue
     // 16 warps: warp & 3 selects the TMEM lane quarter (32 rows), ew >> 2 the 16 of the tile's 64
@@ -1264,14 +1213,15 @@ psb_mma_kernel(const __grid_constant__ TmapSet maps, const __grid_constant__ Ten
                   bar);
       }
     }
+    find_row_maxima(p, ctl, a.kmap ? a.level_mask : 1u << a.uniform_log2k);
     if (!kGeneral) {
       // (an integer addend takes the 64-bit loop here: a branch for it in the 32-bit one cost every layer 1 %)
       bool w32 = p.corr[(uint32_t)__ffs((int)(a.level_mask & 0x7Fu)) - 1u] == nullptr;
       if (a.kmap) {          // every level a tile may have must fit
         for (uint32_t lv = 0; lv < (uint32_t)kMaxLevels; ++lv)
-          if ((a.level_mask >> lv) & 1u) w32 = fits_32_bits(p, lv) && w32;
+          if ((a.level_mask >> lv) & 1u) w32 = fits_32_bits(p, ctl, lv) && w32;
       } else {
-        w32 = fits_32_bits(p, a.uniform_log2k) && w32;
+        w32 = fits_32_bits(p, ctl, a.uniform_log2k) && w32;
       }
       if (P0 == 4u) failed = uniform_dispatch<4>(p, ctl, tmem_base, ew, lane, ec, fast_u8, w32, res_kind);
       else if (P0 == 3u) failed = uniform_dispatch<3>(p, ctl, tmem_base, ew, lane, ec, fast_u8, w32, res_kind);
@@ -1284,7 +1234,7 @@ psb_mma_kernel(const __grid_constant__ TmapSet maps, const __grid_constant__ Ten
       uint32_t w32_levels = 0;      // levels whose accumulators are known to fit 32 bits
       if (q_only)
         for (uint32_t l = 0; l < (uint32_t)kMaxLevels; ++l)
-          if (((a.level_mask >> l) & 1u) && fits_32_bits(p, l)) w32_levels |= 1u << l;
+          if (((a.level_mask >> l) & 1u) && fits_32_bits(p, ctl, l)) w32_levels |= 1u << l;
       TileIter ti;
       for (ti.init(p); !failed && ti.valid(); ti.next()) {
         const uint32_t m0 = ti.m_tile * kTileM, o_tile = ti.o_tile;

@@ -128,7 +128,7 @@ psb_status launch_tensor(psb_ctx* ctx, const psb_weights* wt, const ConvArgs& a,
       const bool quotients_ok = Wp >= 2u && tpi >= 2u && tpi * kTileM * Wp < (1ull << 32) &&
                                 (uint64_t)a.N * tpi * tpi < (1ull << 32);
       if (codes_only && !flip && p.im2col && a.stride == 1 && a.KH * a.KW > 1u && a.C == bk && (bk == 64u || bk == 128u) &&
-          Wp <= 256u && rows <= 256u && a.KH * a.KW * (bk / 32u) <= (uint32_t)(kMaxBandMmas - kTapBatch) && (kSmemBudget - ctl_bytes - need) / bytes >= 2u && quotients_ok) {
+          Wp <= 256u && rows <= 256u && (kSmemBudget - ctl_bytes - need) / bytes >= 2u && quotients_ok) {
         p.band = 1;
         p.Wp = Wp;
         p.tpi = (uint32_t)tpi;
