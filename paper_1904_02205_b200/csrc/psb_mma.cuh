@@ -14,7 +14,8 @@
 //            filters with taps, stride or padding; plain 2-D tiles otherwise) and
 //            of the digit-plane tile into a ring of shared-memory stages
 //   warp 2 issues the MMAs
-//   warp 3 allocates TMEM; issues half of the MMAs in band mode; flips the top bit of unsigned activations
+//   warp 3 allocates TMEM; issues half of the MMAs in band mode; flips the top bit of unsigned activations;
+//            staged outputs: moves shortcut tiles into and output tiles out of shared memory
 //   warps 4-19 epilogue: TMEM -> registers, recombine planes, dequantise, bias,
 //            shortcut, ReLU, re-quantise, vectorised stores; overlaps the next
 //            tile's MMAs through two TMEM accumulator buffers
@@ -43,7 +44,9 @@ constexpr int kMmaWarp1 = kMmaWarp0 + 1;           // band mode: issues half of 
 constexpr int kFirstEpilogueWarp = kMmaWarp1 + 1;  // a multiple of 4: warp & 3 = TMEM lane quarter
 constexpr int kPlaneBars = 4;        // resident digit planes arrive in this many parts, each with its barrier
 constexpr int kEpilogueWarps = 16;
-constexpr int kThreadsTensor = 32 * (kFirstEpilogueWarp + kEpilogueWarps);
+constexpr int kThreadsTensor = 32 * (kFirstEpilogueWarp + kEpilogueWarps);   // five warps of 96 registers per scheduler: no room for another
+constexpr int kIoSlots = 4;                          // staged outputs: a tile being loaded, two worked on, one stored
+constexpr uint32_t kIoTileBytes = kTileM * kTileN;   // a tile of codes: 128 rows x 64 bytes
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kTmemBufStride = 256;
 constexpr int kMaxStages = 12;
@@ -54,6 +57,7 @@ constexpr size_t kSmemBudget = 227 * 1024;
 
 struct TmapSet {
   CUtensorMap a;     // activations; the digit planes need none: their tiles are contiguous
+  CUtensorMap out, res;   // staged outputs: codes and shortcut as [M][O] bytes, boxes of a tile
 };
 
 struct TensorParams {
@@ -69,6 +73,7 @@ struct TensorParams {
   const uint8_t* tile_mask;   // per row tile: levels present (bit l = level l), or null without a map
   uint32_t unit;        // widest store (bytes: 16, 8, 4, 2, 1) that every channels-last output row allows
   uint32_t tail_ksteps; // MMA K steps of a tap's last channel block (the rest of the block lies beyond the channels)
+  uint32_t staged;      // 1: output tiles leave (and shortcut tiles arrive) through shared memory and the copy engine
   uint32_t flip;        // 1: the activations are unsigned bytes; their top bit is flipped in shared memory (x - 128)
                         // and `corr` restores the sum.  Positions the copy engine fills with zeros become -128, i.e.
                         // x = 0, so padding needs no case of its own
@@ -170,6 +175,11 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
       " [%0], [%1, {%3, %4}], [%2];"
       ::"r"(dst), "l"(map), "r"(bar), "r"(x), "r"(y)
       : "memory");
+}
+
+__device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, uint32_t src, int x, int y) {
+  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%2, %3}], [%1];"
+               ::"l"(map), "r"(src), "r"(x), "r"(y) : "memory");
 }
 
 // Plain bulk copy of a contiguous, 16-byte aligned run of global memory.
@@ -296,15 +306,17 @@ struct SharedCtl {
   unsigned long long acc_full[2];
   unsigned long long acc_empty[2];
   unsigned long long planes_full[kPlaneBars];
+  unsigned long long slot_ready[kIoSlots];  // staged outputs: the shortcut tile has landed
+  unsigned long long slot_done[kIoSlots];   // the codes of the tile are in the slot
   unsigned long long started[2];        // band mode, per accumulator buffer: the overwriting MMA of the tile has been issued
   unsigned long long flipped[kMaxStages];   // full, and the top bits flipped (unsigned activations)
   uint32_t tmem_base;
   uint32_t rowmax[kMaxLevels];          // largest row sum of |W_k| per level (units of 256), see find_row_maxima
   WaitCtl wait;
   alignas(16) int32_t corr32[kEpilogueWarps][16];   // low words of the integer addends
-  alignas(16) float2 scb[kEpilogueWarps][16];   // per epilogue warp: (scale * 2^(e_base - log2 k), bias), read two
+  alignas(16) float2 scb[kEpilogueWarps][32];   // per epilogue warp: (scale * 2^(e_base - log2 k), bias), read two
                                                 // channels (16 bytes) at a time
-  long long corr[kEpilogueWarps][16];   // per epilogue warp: integer addend per channel
+  long long corr[kEpilogueWarps][32];   // per epilogue warp: integer addend per channel
 };
 
 // Output arithmetic of one 16-channel chunk held in registers (v[plane][channel]), common case:
@@ -826,10 +838,160 @@ __device__ __noinline__ bool epilogue_uniform(const TensorParams& p, SharedCtl* 
   return false;
 }
 
+// 16 channels with the planes recombined in 32 bits.
+template <int P>
+__device__ __forceinline__ void load_folded(uint32_t taddr, uint32_t (&a)[1][16]) {
+  uint32_t v[P][16];
+#pragma unroll
+  for (int pl = 0; pl < P; ++pl) tc_ld16(taddr + pl * kTileN, v[pl]);
+  tc_wait_ld();
+#pragma unroll
+  for (int j = 0; j < 16; ++j) {
+    int acc = (int)v[0][j];
+#pragma unroll
+    for (int pl = 1; pl < P; ++pl) acc += (int)v[pl][j] << (kDigitBits * pl);
+    a[0][j] = (uint32_t)acc;
+  }
+}
+
+// The loop for layers with a shortcut and several tiles per CTA, channels-last rows of whole 16-byte pieces in tile order (p.staged).
+// Two things differ.  Codes and shortcut bytes pass through slots of shared memory, moved as one box per tile by the
+// copy engine (io_role): direct accesses, 16 bytes of a different row per lane, cost 32 cache-line look-ups and half-used
+// sectors per instruction.  And the sixteen warps form two groups that take alternate tiles, each with the accumulator
+// buffer of its parity, a warp taking 32 rows x 32 channels, so that the bookkeeping of a tile is spent on twice as many
+// outputs.  1x1 64 -> 256 channels @56 with a shortcut, batch 64: 55.4 -> 40.3 us (staged without the groups 48.4; 17.7 us
+// at memory rate).
+template <int P, bool W32, int RES, bool FAST_U8>
+__device__ __noinline__ bool epilogue_staged(const TensorParams& p, SharedCtl* ctl, uint32_t tmem_base, uint32_t slots_addr,
+                                             uint32_t ew, uint32_t lane, EpiConst c) {
+  const ConvArgs& a = p.a;
+  const uint32_t quarter = ew & 3u, half = (ew >> 2) & 1u, group = ew >> 3, row = quarter * 32u + lane;
+  const uint32_t l = a.uniform_log2k, O = a.O;
+  const bool use_corr = p.corr[l] != nullptr;
+  WaitCtl* abort = &ctl->wait;
+  const float2* scb = ctl->scb[ew];
+  const long long* corr = ctl->corr[ew];
+  // this lane's two 16-byte pieces of a slot: rows of 64 bytes, pieces permuted by the copy engine's 64-byte swizzle
+  const uint32_t sw = (row >> 1) & 3u, row_addr = slots_addr + group * kIoTileBytes + row * (uint32_t)kTileN;
+  const uint32_t piece[2] = {((2u * half) ^ sw) << 4, ((2u * half + 1u) ^ sw) << 4};
+  const uint32_t ready0 = smem_u32(&ctl->slot_ready[group]), done0 = smem_u32(&ctl->slot_done[group]);
+  const uint32_t acc_full = smem_u32(&ctl->acc_full[group]), acc_empty = smem_u32(&ctl->acc_empty[group]);
+  const uint32_t taddr = tmem_base + group * kTmemBufStride + ((quarter * 32u) << 16) + half * 32u;
+  TileIter ti;
+  ti.init(p);
+  if (group) ti.next();
+  uint32_t n = 0, cur_o_tile = 0xFFFFFFFFu;      // n: tiles of this group so far; their slots alternate
+  while (ti.valid()) {
+    const uint32_t o_tile = ti.o_tile, o_base = o_tile * kTileN + half * 32u;
+    const bool active = o_base < O;             // warp-uniform
+    ti.next();
+    ti.next();
+    if (o_tile != cur_o_tile) {
+      // per-channel constants of this channel tile: the warp keeps its own copy of its 32 channels
+      __syncwarp();
+      const uint32_t o = o_base + lane;
+      float2 sb = make_float2(0.f, 0.f);
+      long long cr = 0;
+      if (o < O) {
+        sb.x = ldexpf(a.scale[o], a.e_base[o] - (int)l);
+        sb.y = a.bias[o];
+        if (use_corr) cr = p.corr[l][o];
+      }
+      ctl->scb[ew][lane] = sb;
+      if (!W32) ctl->corr[ew][lane] = cr;
+      cur_o_tile = o_tile;
+      __syncwarp();
+    }
+    bool ok = mbar_wait(acc_full, n & 1u, abort, 32);
+    if (__any_sync(0xFFFFFFFFu, !ok)) return true;
+    tc_fence_after();
+    const uint32_t slot = (n & 1u) * 2u, addr = row_addr + slot * kIoTileBytes;
+    auto release = [&]() {
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(acc_empty);
+    };
+    auto shortcut = [&](uint32_t at) {
+      uint4 r;
+      asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "r"(at));
+      return r;
+    };
+    auto store = [&](uint32_t at, uint4 q) {
+      asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(q.x), "r"(q.y), "r"(q.z), "r"(q.w) : "memory");
+    };
+    if (W32) {
+      uint32_t a0[1][16], a1[1][16];
+      if (active) {
+        load_folded<P>(taddr, a0);
+        load_folded<P>(taddr + 16u, a1);
+      }
+      release();
+      ok = mbar_wait(ready0 + 8u * slot, (n >> 1) & 1u, abort, 32);
+      if (__any_sync(0xFFFFFFFFu, !ok)) return true;
+      if (active) {
+        store(addr + piece[0], chunk_math<1, true, RES, FAST_U8>(a0, shortcut(addr + piece[0]), scb, corr, c));
+        store(addr + piece[1], chunk_math<1, true, RES, FAST_U8>(a1, shortcut(addr + piece[1]), scb + 16, corr + 16, c));
+      }
+    } else {
+      ok = mbar_wait(ready0 + 8u * slot, (n >> 1) & 1u, abort, 32);
+      if (__any_sync(0xFFFFFFFFu, !ok)) return true;
+      uint32_t v[P][16];
+      if (active) {
+        load_chunk<P, false>(taddr, v);
+        store(addr + piece[0], chunk_math<P, false, RES, FAST_U8>(v, shortcut(addr + piece[0]), scb, corr, c));
+        load_chunk<P, false>(taddr + 16u, v);
+      }
+      release();
+      if (active) store(addr + piece[1], chunk_math<P, false, RES, FAST_U8>(v, shortcut(addr + piece[1]), scb + 16, corr + 16, c));
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncwarp();
+    if (lane == 0) mbar_arrive(done0 + 8u * slot);
+    ++n;
+  }
+  return false;
+}
+
+// One thread moves the tiles of epilogue_staged: the shortcuts of up to three tiles ahead in, the codes out.  Rows and channels
+// beyond the tensor read as zeros and are not written.
+__device__ __noinline__ bool io_role(const TensorParams& p, const TmapSet& maps, SharedCtl* ctl, uint32_t slots_addr) {
+  TileIter out, in;
+  out.init(p);
+  in.init(p);
+  auto prepare = [&](uint32_t slot) {
+    if (!in.valid()) return;
+    const uint32_t bar = smem_u32(&ctl->slot_ready[slot]);
+    mbar_expect_tx(bar, kIoTileBytes);
+    tma_load_2d(slots_addr + slot * kIoTileBytes, &maps.res, bar, (int)(in.o_tile * kTileN), (int)(in.m_tile * kTileM));
+    in.next();
+  };
+  prepare(0u);
+  prepare(1u);
+  prepare(2u);
+  bool ok = true;
+  uint32_t slot = 0, phase = 0;
+  for (; out.valid(); out.next()) {
+    ok = mbar_wait(smem_u32(&ctl->slot_done[slot]), phase, &ctl->wait);
+    if (!ok) break;
+    tma_store_2d(&maps.out, slots_addr + slot * kIoTileBytes, (int)(out.o_tile * kTileN), (int)(out.m_tile * kTileM));
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+    // all but this store have read their slots: the one of the tile before is free
+    asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+    prepare((slot + (uint32_t)kIoSlots - 1u) % (uint32_t)kIoSlots);
+    if (++slot == (uint32_t)kIoSlots) { slot = 0; phase ^= 1u; }
+  }
+  asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+  return !ok;
+}
+
 // Run-time options of the uniform output stage -> template instance.
 template <int P, bool W32, int RES>
 __device__ __forceinline__ bool uniform_dispatch_tail(const TensorParams& p, SharedCtl* ctl, uint32_t tmem_base,
-                                                      uint32_t ew, uint32_t lane, const EpiConst& c, bool fast_u8) {
+                                                      uint32_t slots_addr, uint32_t ew, uint32_t lane, const EpiConst& c,
+                                                      bool fast_u8) {
+  if (RES && p.staged)
+    return fast_u8 ? epilogue_staged<P, W32, RES ? RES : 1, true>(p, ctl, tmem_base, slots_addr, ew, lane, c)
+                   : epilogue_staged<P, W32, RES ? RES : 1, false>(p, ctl, tmem_base, slots_addr, ew, lane, c);
   if (p.band)
     return fast_u8 ? epilogue_uniform<P, W32, RES, true, RowMapBand>(p, ctl, tmem_base, ew, lane, c)
                    : epilogue_uniform<P, W32, RES, false, RowMapBand>(p, ctl, tmem_base, ew, lane, c);
@@ -840,17 +1002,17 @@ __device__ __forceinline__ bool uniform_dispatch_tail(const TensorParams& p, Sha
                  : epilogue_uniform<P, W32, RES, false, RowMap>(p, ctl, tmem_base, ew, lane, c);
 }
 template <int P>
-__device__ __forceinline__ bool uniform_dispatch(const TensorParams& p, SharedCtl* ctl, uint32_t tmem_base,
+__device__ __forceinline__ bool uniform_dispatch(const TensorParams& p, SharedCtl* ctl, uint32_t tmem_base, uint32_t slots_addr,
                                                  uint32_t ew, uint32_t lane, const EpiConst& c, bool fast_u8,
                                                  bool w32, uint32_t res) {
   if (w32) {
-    if (res == 0u) return uniform_dispatch_tail<P, true, 0>(p, ctl, tmem_base, ew, lane, c, fast_u8);
-    if (res == 1u) return uniform_dispatch_tail<P, true, 1>(p, ctl, tmem_base, ew, lane, c, fast_u8);
-    return uniform_dispatch_tail<P, true, 2>(p, ctl, tmem_base, ew, lane, c, fast_u8);
+    if (res == 0u) return uniform_dispatch_tail<P, true, 0>(p, ctl, tmem_base, slots_addr, ew, lane, c, fast_u8);
+    if (res == 1u) return uniform_dispatch_tail<P, true, 1>(p, ctl, tmem_base, slots_addr, ew, lane, c, fast_u8);
+    return uniform_dispatch_tail<P, true, 2>(p, ctl, tmem_base, slots_addr, ew, lane, c, fast_u8);
   }
-  if (res == 0u) return uniform_dispatch_tail<P, false, 0>(p, ctl, tmem_base, ew, lane, c, fast_u8);
-  if (res == 1u) return uniform_dispatch_tail<P, false, 1>(p, ctl, tmem_base, ew, lane, c, fast_u8);
-  return uniform_dispatch_tail<P, false, 2>(p, ctl, tmem_base, ew, lane, c, fast_u8);
+  if (res == 0u) return uniform_dispatch_tail<P, false, 0>(p, ctl, tmem_base, slots_addr, ew, lane, c, fast_u8);
+  if (res == 1u) return uniform_dispatch_tail<P, false, 1>(p, ctl, tmem_base, slots_addr, ew, lane, c, fast_u8);
+  return uniform_dispatch_tail<P, false, 2>(p, ctl, tmem_base, slots_addr, ew, lane, c, fast_u8);
 }
 
 // All lanes of the warp wait together; false when a wait ran out.
@@ -1043,7 +1205,9 @@ psb_mma_kernel(const __grid_constant__ TmapSet maps, const __grid_constant__ Ten
   // a stage holds `group` K blocks, each an activation tile followed (streaming mode) by planes
   const uint32_t sub_bytes = p.stage_bytes_a + (p.resident ? 0u : p.stage_bytes_b_max);
   const uint32_t stage_bytes = p.band ? p.band_bytes : sub_bytes * p.group;
-  SharedCtl* ctl = reinterpret_cast<SharedCtl*>(ring + (size_t)p.stages * stage_bytes);
+  // staged outputs: kIoSlots tiles between the ring and the control block
+  const uint32_t slots_addr = smem_u32(ring) + p.stages * stage_bytes;
+  SharedCtl* ctl = reinterpret_cast<SharedCtl*>(ring + (size_t)p.stages * stage_bytes + (p.staged ? kIoSlots * kIoTileBytes : 0u));
 
   const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u;
   const uint32_t k_iters = p.a.KH * p.a.KW * p.n_cb;
@@ -1056,7 +1220,7 @@ psb_mma_kernel(const __grid_constant__ TmapSet maps, const __grid_constant__ Ten
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(smem_u32(&ctl->acc_full[b]), p.band ? 2u : 1u);
-      mbar_init(smem_u32(&ctl->acc_empty[b]), kEpilogueWarps);
+      mbar_init(smem_u32(&ctl->acc_empty[b]), p.staged ? kEpilogueWarps / 2 : kEpilogueWarps);   // staged: a group of warps per tile
     }
     {  // part b of the resident planes holds K blocks [b * part, (b + 1) * part): one arrival per block
       const uint32_t part = (k_iters + kPlaneBars - 1) / kPlaneBars;
@@ -1067,6 +1231,10 @@ psb_mma_kernel(const __grid_constant__ TmapSet maps, const __grid_constant__ Ten
     }
     for (int b = 0; b < 2; ++b) mbar_init(smem_u32(&ctl->started[b]), 1);
     for (int l = 0; l < kMaxLevels; ++l) ctl->rowmax[l] = 0u;
+    for (int b = 0; b < kIoSlots; ++b) {
+      mbar_init(smem_u32(&ctl->slot_ready[b]), 1);
+      mbar_init(smem_u32(&ctl->slot_done[b]), kEpilogueWarps / 2);
+    }
     ctl->wait.abort = 0;
     ctl->wait.limit = p.wait_limit;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -1175,7 +1343,10 @@ psb_mma_kernel(const __grid_constant__ TmapSet maps, const __grid_constant__ Ten
       failed = mma_role_band<BK>(p, ctl, tmem_base, smem_u32(ring), smem_u32(smem), stage_bytes, warp - (uint32_t)kMmaWarp0);
     else if (warp == (uint32_t)kMmaWarp0)
       failed = mma_role<BK>(p, ctl, tmem_base, smem_u32(ring), smem_u32(smem), stage_bytes, sub_bytes, k_iters);
-    else if (p.flip)
+    else if (p.staged) {
+      if (lane == 0) failed = io_role(p, maps, ctl, slots_addr);
+      failed = __shfl_sync(0xFFFFFFFFu, failed ? 1 : 0, 0) != 0;
+    } else if (p.flip)
       failed = flip_role(p, ctl, smem_u32(ring), stage_bytes, sub_bytes, k_iters);
   } else {
     // ----------------------------------------------------------- epilogue
@@ -1223,9 +1394,9 @@ psb_mma_kernel(const __grid_constant__ TmapSet maps, const __grid_constant__ Ten
       } else {
         w32 = fits_32_bits(p, ctl, a.uniform_log2k) && w32;
       }
-      if (P0 == 4u) failed = uniform_dispatch<4>(p, ctl, tmem_base, ew, lane, ec, fast_u8, w32, res_kind);
-      else if (P0 == 3u) failed = uniform_dispatch<3>(p, ctl, tmem_base, ew, lane, ec, fast_u8, w32, res_kind);
-      else failed = uniform_dispatch<2>(p, ctl, tmem_base, ew, lane, ec, fast_u8, w32, res_kind);
+      if (P0 == 4u) failed = uniform_dispatch<4>(p, ctl, tmem_base, slots_addr, ew, lane, ec, fast_u8, w32, res_kind);
+      else if (P0 == 3u) failed = uniform_dispatch<3>(p, ctl, tmem_base, slots_addr, ew, lane, ec, fast_u8, w32, res_kind);
+      else failed = uniform_dispatch<2>(p, ctl, tmem_base, slots_addr, ew, lane, ec, fast_u8, w32, res_kind);
     } else {
       // general loop: per-location draw counts, any outputs and layouts, ragged channel counts
       const float2* scb = ctl->scb[ew];

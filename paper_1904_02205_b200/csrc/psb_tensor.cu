@@ -6,6 +6,12 @@ namespace psb {
 
 namespace {
 
+// Layers with a shortcut use the staged output stage from this many tiles per SM.  Below, the time to the first and the
+// last tile counts, and half of the warps per tile lose it: 1x1 256 -> 1024 @14, batch 1 (32 tiles) 5.7 us directly, 6.5
+// staged; batch 64 (1568 tiles) 18.4 and 15.7.  Without a shortcut both take the same, or the direct one less: 1x1
+// 64 -> 256 @56 35.4 and 34.7, 256 -> 64 13.7 and 14.8, 3x3 128 -> 128 @28 24.3 and 25.3, 96 -> 16 @112 34.4 and 36.8.
+constexpr uint64_t kStagedMinTiles = 3;
+
 // One warp waits, with the given bound, on a barrier that has no other party: the wait runs out,
 // the kernel raises the error word and returns.  Exercises mbar_wait's give-up path as the contraction
 // kernel would take it, with nothing in flight.
@@ -141,10 +147,14 @@ psb_status launch_tensor(psb_ctx* ctx, const psb_weights* wt, const ConvArgs& a,
       p.ctas_per_otile = cpo < p.m_tiles ? cpo : p.m_tiles;
     }
   }
+  // Staged outputs (epilogue_staged): channels-last codes in rows of whole 16-byte pieces, rows in tile order
+  p.staged = (uniform_epilogue(p) && !a.kmap && !p.band && !a.out_nchw && p.unit == 16u && !flip && a.residual &&
+              (uint64_t)p.m_tiles * p.o_tiles >= kStagedMinTiles * (uint64_t)ctx->sm_count) ? 1u : 0u;
+  const size_t io_bytes = p.staged ? (size_t)kIoSlots * kIoTileBytes : 0u;
   // K blocks are handed over in groups: every barrier round trip costs the issuing thread a
   // few hundred cycles, so a stage should carry about eight MMAs (M=128, N=P*64, K=32 each)
   const uint32_t sub_bytes = p.stage_bytes_a + (p.resident ? 0u : p.stage_bytes_b_max);
-  const size_t avail = kSmemBudget - ctl_bytes - p.resident_bytes;
+  const size_t avail = kSmemBudget - ctl_bytes - p.resident_bytes - io_bytes;
   uint32_t group = 8u / (bk / 32u);
   if (group < 1) group = 1;
   if (group > k_iters) group = k_iters;
@@ -166,7 +176,7 @@ psb_status launch_tensor(psb_ctx* ctx, const psb_weights* wt, const ConvArgs& a,
   if (stages < 2) return PSB_ERR_UNSUPPORTED;
   p.stages = stages;
   const size_t smem_bytes = (p.band ? (size_t)stages * p.band_bytes : (size_t)stages * group * sub_bytes) +
-                            p.resident_bytes + ctl_bytes;
+                            p.resident_bytes + io_bytes + ctl_bytes;
   for (int l = 0; l < kMaxLevels; ++l) p.corr[l] = add_corr128 && wt->level[l].planes ? wt->corr128 + (size_t)l * a.O : nullptr;
   p.rowsum256 = wt->rowsum256;
   p.amax = amax;
@@ -201,6 +211,17 @@ psb_status launch_tensor(psb_ctx* ctx, const psb_weights* wt, const ConvArgs& a,
                   estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swz, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
       return PSB_ERR_CUDA;
+  }
+  if (p.staged) {
+    cuuint64_t dims[2] = {a.O, p.M};
+    cuuint64_t strides[1] = {(cuuint64_t)a.O};
+    cuuint32_t box[2] = {(cuuint32_t)kTileN, kTileM};
+    cuuint32_t estr[2] = {1, 1};
+    for (int i = 0; i < 2; ++i)
+      if (enc_tiled(i ? &maps.res : &maps.out, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, i ? const_cast<void*>(a.residual) : a.q_out, dims,
+                    strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
+                    CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return PSB_ERR_CUDA;
   }
   for (int l = 0; l < kMaxLevels; ++l) p.planes_ptr[l] = wt->level[l].planes;
 

@@ -70,3 +70,43 @@ def test_rows_that_start_at_odd_addresses(oracle):
         assert ctx.device_status() == 0 and np.array_equal(got, acc)
     wt.free()
     ctx.close()
+
+
+@pytest.mark.parametrize("case", [
+    # (N, H, W, C, O, shortcut dtype, exp_bits, log2k, in_max): several tiles per SM, ragged last rows and channel tiles
+    (19, 56, 55, 64, 64, np.uint8, 4, 3, 15), (30, 49, 41, 32, 80, np.int8, 4, 3, 15), (19, 56, 55, 64, 64, np.int8, 3, 0, 15),
+    (8, 57, 61, 128, 144, np.uint8, 4, 6, 15), (19, 56, 57, 256, 64, np.int8, 4, 6, 127),
+])
+@pytest.mark.parametrize("signed_out", [False, True])
+def test_shortcut_tiles_through_shared_memory(case, signed_out, oracle):
+    """Layers with a shortcut and enough tiles for the staged output stage: two to four planes, 32- and 64-bit
+    recombination, a second channel tile that is partly or wholly beyond the channels."""
+    import torch
+
+    import paper_1904_02205_b200 as psb
+
+    N, H, W, C, O, res_dtype, exp_bits, log2k, top = case
+    assert -(-N * H * W // 128) * -(-O // 64) >= 3 * 148
+    ctx = psb.Context(0)
+    rng = np.random.default_rng(O + H)
+    w = rng.normal(0, np.sqrt(2.0 / C), size=(O, C, 1, 1)).astype(np.float32)
+    x = rng.integers(0, top + 1, size=(N, H, W, C)).astype(np.uint8)
+    lo = 0 if res_dtype == np.uint8 else -128
+    res = rng.integers(lo, lo + 256, size=(N, H, W, O)).astype(res_dtype)
+    scale, bias = rng.uniform(0.5, 1.5, O).astype(np.float32), rng.normal(0, 0.5, O).astype(np.float32)
+    dev = lambda t: torch.from_numpy(t).to(ctx.device)
+    wt = ctx.sample_weights(dev(w), seed=5, layer_id=3, level_mask=1 << log2k, exp_bits=exp_bits)
+    ctx.set_sample_map(None, log2k)
+    qmin, qmax = (-100, 101) if signed_out else (0, 15)
+    inv_step = np.float32(0.5)
+    q = ctx.conv2d(wt, dev(x), psb.PSB_LAYOUT_NHWC, 1, 0, dev(scale), dev(bias), not signed_out, inv_step, qmin, qmax,
+                   out_dtype=psb.PSB_DT_S8 if signed_out else psb.PSB_DT_U8, residual=dev(res), residual_scale=0.3, in_max=top,
+                   path=psb.PSB_PATH_TENSOR)["q"].cpu().numpy()
+    assert ctx.device_status() == 0
+    # first and last image against the oracle
+    for n in (0, N - 1):
+        o = oracle_layer(oracle, w, x[n:n + 1], 1, 1, 1, 0, 5, 3, [log2k], None, log2k, scale, bias, not signed_out, inv_step, qmin,
+                         qmax, residual=res[n:n + 1], res_scale=np.float32(0.3), exp_bits=exp_bits)
+        assert np.array_equal(q[n:n + 1].astype(np.int32), o["q"])
+    wt.free()
+    ctx.close()
