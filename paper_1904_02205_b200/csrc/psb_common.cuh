@@ -181,18 +181,6 @@ __device__ __forceinline__ float acc_to_float(long long acc) {
   return __fmaf_rn((float)hi, 16777216.0f, (float)lo);
 }
 
-// The same for |acc| < 2^45, without the conversion unit: the parts get their float form by
-// exponent arithmetic,
-//   float(n) = as_float(0x4B400000 + n) - 1.5 * 2^23   for |n| < 2^22,
-//   float(n) = as_float(0x4B000000 | n) - 2^23         for 0 <= n < 2^23.
-__device__ __forceinline__ float acc_to_float_small(long long acc) {
-  const int hi = (int)(acc >> 23);
-  const unsigned int lo = (unsigned int)acc & 0x7FFFFFu;
-  const float hi_f = __int_as_float(0x4B400000 + hi) - 12582912.0f;
-  const float lo_f = __uint_as_float(0x4B000000u | lo) - 8388608.0f;
-  return __fmaf_rn(hi_f, 8388608.0f, lo_f);
-}
-
 // Programmatic dependent launch: a kernel launched through launch_pdl may be scheduled while the
 // kernel before it in the stream is still running; it must call pdl_prologue() before it touches
 // global memory, which waits for the earlier grids to complete (and lets the kernel after it be

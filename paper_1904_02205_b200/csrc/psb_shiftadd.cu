@@ -9,6 +9,8 @@
 // activations, and it honours per-location draw counts directly.
 #include "psb_common.cuh"
 
+#include <algorithm>
+
 namespace psb {
 
 namespace {
@@ -244,234 +246,209 @@ __global__ void __launch_bounds__(256) dwconv_nhwc8_kernel(const ConvArgs a, con
   }
 }
 
-// Depthwise 3x3, channels-last, one draw count, only codes wanted.  A thread owns 4 channels
-// and kDwSeg consecutive output columns of one output row: its 36 filter values and 8 output
-// constants stay in registers, every input column of the 3-row band is loaded once (one 32-bit
-// load per row) and serves up to three outputs.  All loads of the band are issued before the
-// arithmetic; positions outside the image read as zero through a predicate.  The output stage
-// is dequant()/requant() written without the conversion unit (exponent arithmetic, see
-// acc_to_float_small).  Adjacent threads take adjacent channel quads, so a warp's loads and
-// stores are contiguous runs of the channels-last rows.
+// Depthwise 3x3, channels-last, one draw count, only codes wanted: a thread owns 4 channels x kDwCols output columns and
+// walks down the rows of an image with its 36 filter values in registers.  Every input row is read once per thread, its
+// bytes are extracted once and serve up to three output rows, whose sums are open at the same time (unrolled by three
+// so that no sum moves).  The integer sum x * W_k over the nine taps (Eq. 9 summed over the draws) fits 32 bits whenever
+// (largest activation) x (sum of |W_k| of the channel) stays below 2^31; the sampler keeps those sums, and a thread with
+// a channel where it does not computes its outputs one by one in 64 bits.  The output stage is dequant()/requant() with
+// the relu folded into the lower clamp (inv_step > 0), rounded by adding 1.5 * 2^23.
+// Bound by the nine 32-bit multiply-adds per output (2 clocks each): 15 us for 144 channels @56, batch 64.  That layer
+// with its sampling: 78.6 -> 65.8 us (a thread with 8 outputs of one row spent 48 logic clocks per output and spilled).
+constexpr int kDwCols = 2;
+
+struct DwConst {
+  float res_scale, inv_step, lo_f, hi_f;
+};
+
 template <int S>
-struct DwSeg { static constexpr int kOut = S == 1 ? 8 : 4; static constexpr int kCols = (kOut - 1) * S + 3; };
+struct DwIn { static constexpr int kCols = (kDwCols - 1) * S + 3; };
 
-template <int S, bool kSignedIn>
-__global__ void __launch_bounds__(256, 2) dwconv3x3_row_kernel(const ConvArgs a, const int32_t* wint) {
-  pdl_prologue();
-  constexpr int L = DwSeg<S>::kOut, NC = DwSeg<S>::kCols;
-  const uint32_t C = a.C, G = C / 4u;
-  const uint32_t segs = (a.OW + L - 1) / L;
-  const uint32_t total = a.N * a.OH * segs * G;   // the launcher keeps this below 2^32
-  const uint32_t idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= total) return;
-  uint32_t t = idx / G;
-  const uint32_t c0 = (idx - t * G) * 4u;
-  const uint32_t seg = t % segs; t /= segs;
-  const uint32_t oy = t % a.OH, n = t / a.OH;
-  const uint32_t ox0 = seg * L;
-
-  // band of input: rows iy0..iy0+2, columns ix0..ix0+NC-1
-  const int iy0 = (int)(oy * S) - (int)a.pad, ix0 = (int)(ox0 * S) - (int)a.pad;
-  const uint32_t last_ox = min(ox0 + (uint32_t)L, a.OW) - 1u;
-  const int ix_end = (int)(last_ox * S) - (int)a.pad + 2;     // last column any output of the segment reads
-  uint32_t raw[3][NC];
-#pragma unroll
-  for (int r = 0; r < 3; ++r) {
-    const int iy = iy0 + r;
-    const bool row_in = (unsigned)iy < a.H;
-    const uint8_t* rp = (const uint8_t*)a.x + ((size_t)(n * a.H + (row_in ? iy : 0)) * a.W) * C + c0;
-#pragma unroll
-    for (int cidx = 0; cidx < NC; ++cidx) {
-      const int ix = ix0 + cidx;
-      raw[r][cidx] = 0u;
-      if (row_in && (unsigned)ix < a.W && ix <= ix_end)
-        raw[r][cidx] = __ldcg(reinterpret_cast<const uint32_t*>(rp + (size_t)ix * C));
+// One output in 64 bits, straight from global memory (channels whose sums may not fit 32).
+template <bool kSignedIn>
+__device__ __noinline__ void dw_output64(const ConvArgs& a, const int32_t* wch, uint32_t n, uint32_t oy, uint32_t ox, uint32_t o) {
+  long long acc = 0;
+  for (uint32_t kh = 0; kh < 3u; ++kh) {
+    const int iy = (int)(oy * a.stride + kh) - (int)a.pad;
+    if ((unsigned)iy >= a.H) continue;
+    for (uint32_t kw = 0; kw < 3u; ++kw) {
+      const int ix = (int)(ox * a.stride + kw) - (int)a.pad;
+      if ((unsigned)ix >= a.W) continue;
+      acc += (long long)load_act(a.x, kSignedIn ? PSB_DT_S8 : PSB_DT_U8, (((size_t)n * a.H + iy) * a.W + ix) * a.C + o) *
+             (long long)__ldca(wch + kh * 3u + kw);
     }
   }
-  // filter [channel][tap] and output constants of the 4 channels
-  int w[36];
-  {
+  store_outputs(a, (((size_t)n * a.OH + oy) * a.OW + ox) * a.C + o, o, a.uniform_log2k, acc);
+}
+
+// kVec: channel counts that are multiples of 4 at 4-byte aligned addresses; otherwise words are put together from bytes.
+template <int S, bool kSignedIn, bool kVec>
+__global__ void __launch_bounds__(256, 2) dwconv3x3_kernel(const ConvArgs a, const int32_t* wint, const uint32_t* rowsum256,
+                                                           uint32_t amax, uint32_t rows_per_thread) {
+  pdl_prologue();
+  constexpr int NC = DwIn<S>::kCols;
+  const uint32_t C = a.C, G = (C + 3u) / 4u;
+  const uint32_t segs = (a.OW + kDwCols - 1) / kDwCols, strips = (a.OH + rows_per_thread - 1u) / rows_per_thread;
+  const uint32_t idx = blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= a.N * strips * segs * G) return;      // the launcher keeps this below 2^32
+  uint32_t t = idx / G;
+  const uint32_t c0 = (idx - t * G) * 4u, left = kVec ? 4u : min(4u, C - c0);
+  const uint32_t seg = t % segs; t /= segs;
+  const uint32_t strip = t % strips, n = t / strips;
+  const uint32_t ox0 = seg * kDwCols, oy0 = strip * rows_per_thread, oy1 = min(oy0 + rows_per_thread, a.OH);
+  const uint32_t level = a.uniform_log2k;
+  // (a sum marked unknown, 0xFFFFFFFF, fails the test like a large one)
+  bool fits = true;
+  for (uint32_t j = 0; j < left; ++j)
+    fits = fits && (unsigned long long)__ldca(rowsum256 + (size_t)level * a.O + c0 + j) * 256ull * amax < (1ull << 31);
+  if (!fits) {
+    for (uint32_t oy = oy0; oy < oy1; ++oy)
+      for (uint32_t ox = ox0; ox < min(ox0 + (uint32_t)kDwCols, a.OW); ++ox)
+        for (uint32_t j = 0; j < left; ++j) dw_output64<kSignedIn>(a, wint + (size_t)(c0 + j) * 9u, n, oy, ox, c0 + j);
+    return;
+  }
+  int w[4][9];
+  if (kVec) {
     const int4* wp = reinterpret_cast<const int4*>(wint + (size_t)c0 * 9u);
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
       const int4 v = __ldca(wp + i);
-      w[4 * i] = v.x; w[4 * i + 1] = v.y; w[4 * i + 2] = v.z; w[4 * i + 3] = v.w;
+      const int e[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int q = 0; q < 4; ++q) w[(4 * i + q) / 9][(4 * i + q) % 9] = e[q];
     }
+  } else {
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int q = 0; q < 9; ++q) w[j][q] = (uint32_t)j < left ? __ldca(wint + (size_t)(c0 + j) * 9u + q) : 0;
   }
   float sc[4], bi[4];
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
-    sc[j] = ldexpf(a.scale[c0 + j], a.e_base[c0 + j] - (int)a.uniform_log2k);
-    bi[j] = a.bias[c0 + j];
+    const uint32_t o = (uint32_t)j < left ? c0 + j : c0;
+    sc[j] = ldexpf(a.scale[o], a.e_base[o] - (int)level);
+    bi[j] = a.bias[o];
   }
-  const bool has_res = a.residual != nullptr;
-  const uint32_t res_sign = a.residual_dtype == PSB_DT_S8 ? 0x80u : 0u;
-  const float res_bias = 8388608.0f + (float)res_sign;
-  const float relu_floor = (a.relu && a.qmin < 0) ? 0.0f : __int_as_float(0xFF800000);
-  const float qmin_f = (float)a.qmin, qmax_f = (float)a.qmax;
-  const size_t obase = ((size_t)(n * a.OH + oy) * a.OW + ox0) * C + c0;
+  const float lo_f = a.relu && a.qmin < 0 ? 0.0f : (float)a.qmin, hi_f = (float)a.qmax;
+  const bool has_res = a.residual != nullptr, res_signed = a.residual_dtype == PSB_DT_S8;
+  const int ix0 = (int)(ox0 * S) - (int)a.pad;
+  bool col_in[NC];
+#pragma unroll
+  for (int q = 0; q < NC; ++q) col_in[q] = (unsigned)(ix0 + q) < a.W;
+  const uint8_t* const xcol = (const uint8_t*)a.x + ((ptrdiff_t)n * a.H * a.W + ix0) * (ptrdiff_t)C + c0;
+  const size_t row_bytes = (size_t)a.W * C;
 
+  auto load_word = [&](const uint8_t* at) -> uint32_t {
+    if (kVec) return __ldcg(reinterpret_cast<const uint32_t*>(at));
+    uint32_t v = 0u;
 #pragma unroll
-  for (int i = 0; i < L; ++i) {
-    if (ox0 + i > last_ox) break;
-    const size_t oidx = obase + (size_t)i * C;
-    uint32_t rv = 0u;
-    if (has_res) rv = __ldcg(reinterpret_cast<const uint32_t*>((const uint8_t*)a.residual + oidx));
-    long long acc[4] = {0, 0, 0, 0};
+    for (int j = 0; j < 4; ++j)
+      if ((uint32_t)j < left) v |= (uint32_t)at[j] << (8 * j);
+    return v;
+  };
+  auto load_row = [&](int iy, uint32_t (&raw)[NC]) {
+    const bool in = (unsigned)iy < a.H;
+    const uint8_t* rp = xcol + (ptrdiff_t)iy * (ptrdiff_t)row_bytes;
 #pragma unroll
-    for (int r = 0; r < 3; ++r) {
-#pragma unroll
-      for (int kw = 0; kw < 3; ++kw) {
-        const uint32_t v = raw[r][i * S + kw];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const uint32_t b = (v >> (8 * j)) & 0xFFu;
-          const int xi = kSignedIn ? (int)(int8_t)b : (int)b;
-          acc[j] += (long long)xi * (long long)w[j * 9 + r * 3 + kw];
-        }
-      }
+    for (int q = 0; q < NC; ++q) {
+      raw[q] = 0u;
+      if (in && col_in[q]) raw[q] = load_word(rp + (size_t)q * C);
     }
-    uint32_t q[4];
+  };
+  int acc[3][kDwCols][4];
+  // adds row `kh` of the filter on one input row to a set of sums (kh == 0 starts them)
+  auto add_row = [&](const uint32_t (&raw)[NC], int (&sum)[kDwCols][4], const int kh) {
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      float y = __fmaf_rn(acc_to_float_small(acc[j]), sc[j], bi[j]);
-      if (has_res) {
-        const uint32_t rb = ((rv >> (8 * j)) & 0xFFu) ^ res_sign;   // byte + 128 if signed
-        y = __fmaf_rn(__uint_as_float(0x4B000000u | rb) - res_bias, a.residual_scale, y);
+      int x[NC];
+#pragma unroll
+      for (int q = 0; q < NC; ++q) {
+        const uint32_t b = (raw[q] >> (8 * j)) & 0xFFu;
+        x[q] = kSignedIn ? (int)(signed char)b : (int)b;
       }
-      y = fmaxf(y, relu_floor);
-      // clamp, then round half to even by adding 1.5 * 2^23: the low byte of the sum is the code
-      const float tq = fminf(fmaxf(__fmul_rn(y, a.inv_step), qmin_f), qmax_f);
-      q[j] = __float_as_uint(tq + 12582912.0f);
+#pragma unroll
+      for (int i = 0; i < kDwCols; ++i) {
+        int v = kh == 0 ? 0 : sum[i][j];
+        v += x[i * S] * w[j][kh * 3];
+        v += x[i * S + 1] * w[j][kh * 3 + 1];
+        v += x[i * S + 2] * w[j][kh * 3 + 2];
+        sum[i][j] = v;
+      }
     }
-    *reinterpret_cast<uint32_t*>((uint8_t*)a.q_out + oidx) =
-        __byte_perm(__byte_perm(q[0], q[1], 0x0040), __byte_perm(q[2], q[3], 0x0040), 0x5410);
-  }
-}
-
-// The same layer class with the arithmetic cut down to what the bytes need.  The integer sum x * W_k over the
-// nine taps (Eq. 9 summed over the draws) fits 32 bits whenever (largest activation) x (sum of |W_k| of the
-// channel) stays below 2^31; the sampler keeps those sums, so a thread knows per channel whether 32-bit
-// multiply-adds are exact and falls back to 64-bit ones where they are not.  A thread owns 4 channels and kOut
-// consecutive outputs of one row and works channel by channel: the bytes of the 3 x kCols input words are
-// extracted once per row and channel and serve up to three outputs each, one multiply-add per tap; the output
-// stage is dequant()/requant() with conversion-unit instructions (one int -> float, one float -> int, both
-// round to nearest even as the definitions ask).  About 25 instructions per output where the 64-bit kernel
-// above needs about 70.
-template <typename Acc>
-__device__ __forceinline__ float dw_acc_to_float(Acc acc);
-template <>
-__device__ __forceinline__ float dw_acc_to_float<int>(int acc) { return __int2float_rn(acc); }
-template <>
-__device__ __forceinline__ float dw_acc_to_float<long long>(long long acc) { return acc_to_float(acc); }
-
-template <int S, bool kSignedIn, typename Acc>
-__device__ __forceinline__ void dw_channel(const uint32_t (&raw)[3][DwSeg<S>::kCols], int j, const int32_t* wch,
-                                           float sc, float bi, bool has_res, const uint32_t (&rv)[DwSeg<S>::kOut],
-                                           bool res_signed, float res_scale, float relu_floor, float inv_step,
-                                           float lo_f, float hi_f, uint32_t n_out, uint32_t (&qw)[DwSeg<S>::kOut]) {
-  constexpr int L = DwSeg<S>::kOut, NC = DwSeg<S>::kCols;
-  Acc acc[L];
+  };
+  auto emit = [&](uint32_t oy, const int (&sum)[kDwCols][4]) {
 #pragma unroll
-  for (int i = 0; i < L; ++i) acc[i] = 0;
+    for (int i = 0; i < kDwCols; ++i) {
+      if (ox0 + (uint32_t)i >= a.OW) break;
+      const size_t at = (((size_t)n * a.OH + oy) * a.OW + ox0 + i) * C + c0;
+      uint32_t rw = 0u;
+      if (has_res) {
+        const uint8_t* rp = (const uint8_t*)a.residual + at;
+        rw = load_word(rp);
+      }
+      uint32_t q[4];
 #pragma unroll
-  for (int r = 0; r < 3; ++r) {
-    const int w0 = __ldca(wch + r * 3), w1 = __ldca(wch + r * 3 + 1), w2 = __ldca(wch + r * 3 + 2);
-    int xb[NC];
+      for (int j = 0; j < 4; ++j) {
+        float y = __fmaf_rn(__int2float_rn(sum[i][j]), sc[j], bi[j]);
+        if (has_res) {
+          const uint32_t rb = (rw >> (8 * j)) & 0xFFu;
+          y = __fmaf_rn(res_signed ? (float)(int)(signed char)rb : (float)rb, a.residual_scale, y);
+        }
+        q[j] = __float_as_uint(__fadd_rn(fminf(fmaxf(__fmul_rn(y, a.inv_step), lo_f), hi_f), 12582912.0f));
+      }
+      const uint32_t word = __byte_perm(__byte_perm(q[0], q[1], 0x0040), __byte_perm(q[2], q[3], 0x0040), 0x5410);
+      if (kVec) {
+        *reinterpret_cast<uint32_t*>((uint8_t*)a.q_out + at) = word;
+      } else {
 #pragma unroll
-    for (int cidx = 0; cidx < NC; ++cidx) {
-      const uint32_t b = (raw[r][cidx] >> (8 * j)) & 0xFFu;
-      xb[cidx] = kSignedIn ? (int)(signed char)b : (int)b;
+        for (int j = 0; j < 4; ++j)
+          if ((uint32_t)j < left) ((uint8_t*)a.q_out)[at + j] = (uint8_t)(word >> (8 * j));
+      }
     }
+  };
+  const int iy0 = (int)(oy0 * S) - (int)a.pad;
+  const uint32_t rows = oy1 - oy0;
+  uint32_t cur[NC], nxt[NC];
+  load_row(iy0, cur);
+  load_row(iy0 + 1, nxt);
+  if (S == 1) {
+    // input row r opens output r, adds to output r - 1 and closes output r - 2
+    auto step = [&](uint32_t r, int (&open)[kDwCols][4], int (&mid)[kDwCols][4], int (&close)[kDwCols][4]) {
+      uint32_t raw[NC];
 #pragma unroll
-    for (int i = 0; i < L; ++i) {
-      acc[i] += (Acc)xb[i * S] * (Acc)w0;
-      acc[i] += (Acc)xb[i * S + 1] * (Acc)w1;
-      acc[i] += (Acc)xb[i * S + 2] * (Acc)w2;
+      for (int q = 0; q < NC; ++q) { raw[q] = cur[q]; cur[q] = nxt[q]; }
+      if (r + 2u < rows + 2u) load_row(iy0 + (int)r + 2, nxt);
+      add_row(raw, open, 0);
+      add_row(raw, mid, 1);
+      add_row(raw, close, 2);
+      if (r >= 2u && r - 2u < rows) emit(oy0 + r - 2u, close);
+    };
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+#pragma unroll
+      for (int i = 0; i < kDwCols; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[k][i][j] = 0;
+    for (uint32_t r = 0; r < rows + 2u; r += 3u) {
+      step(r, acc[0], acc[2], acc[1]);
+      step(r + 1u, acc[1], acc[0], acc[2]);
+      step(r + 2u, acc[2], acc[1], acc[0]);
     }
-  }
+  } else {
+    add_row(cur, acc[0], 0);
+    for (uint32_t r = 0; r < rows; ++r) {
+      uint32_t mid[NC];
 #pragma unroll
-  for (int i = 0; i < L; ++i) {
-    if ((uint32_t)i >= n_out) break;
-    float y = __fmaf_rn(dw_acc_to_float<Acc>(acc[i]), sc, bi);
-    if (has_res) {
-      const uint32_t rb = (rv[i] >> (8 * j)) & 0xFFu;
-      y = __fmaf_rn(res_signed ? (float)(int)(signed char)rb : (float)rb, res_scale, y);
-    }
-    y = fmaxf(y, relu_floor);
-    const float t = fminf(fmaxf(__fmul_rn(y, inv_step), lo_f), hi_f);
-    const uint32_t q = (uint32_t)__float2int_rn(t) & 0xFFu;
-    qw[i] |= q << (8 * j);
-  }
-}
-
-template <int S, bool kSignedIn>
-__global__ void __launch_bounds__(256, 3) dwconv3x3_row32_kernel(const ConvArgs a, const int32_t* wint,
-                                                                 const uint32_t* rowsum256,
-                                                                 uint32_t amax) {
-  pdl_prologue();
-  constexpr int L = DwSeg<S>::kOut, NC = DwSeg<S>::kCols;
-  const uint32_t C = a.C, G = C / 4u;
-  const uint32_t segs = (a.OW + L - 1) / L;
-  const uint32_t total = a.N * a.OH * segs * G;   // the launcher keeps this below 2^32
-  const uint32_t idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= total) return;
-  uint32_t t = idx / G;
-  const uint32_t c0 = (idx - t * G) * 4u;
-  const uint32_t seg = t % segs; t /= segs;
-  const uint32_t oy = t % a.OH, n = t / a.OH;
-  const uint32_t ox0 = seg * L;
-
-  // band of input: rows iy0..iy0+2, columns ix0..ix0+NC-1, every word = 4 channels of one position
-  const int iy0 = (int)(oy * S) - (int)a.pad, ix0 = (int)(ox0 * S) - (int)a.pad;
-  const uint32_t last_ox = min(ox0 + (uint32_t)L, a.OW) - 1u;
-  const int ix_end = (int)(last_ox * S) - (int)a.pad + 2;     // last column any output of the segment reads
-  uint32_t raw[3][NC];
-#pragma unroll
-  for (int r = 0; r < 3; ++r) {
-    const int iy = iy0 + r;
-    const bool row_in = (unsigned)iy < a.H;
-    const uint8_t* rp = (const uint8_t*)a.x + ((size_t)(n * a.H + (row_in ? iy : 0)) * a.W) * C + c0;
-#pragma unroll
-    for (int cidx = 0; cidx < NC; ++cidx) {
-      const int ix = ix0 + cidx;
-      raw[r][cidx] = 0u;
-      if (row_in && (unsigned)ix < a.W && ix <= ix_end)
-        raw[r][cidx] = __ldcg(reinterpret_cast<const uint32_t*>(rp + (size_t)ix * C));
+      for (int q = 0; q < NC; ++q) mid[q] = nxt[q];
+      load_row(iy0 + 2 * (int)r + 2, cur);
+      if (r + 1u < rows) load_row(iy0 + 2 * (int)r + 3, nxt);
+      add_row(mid, acc[0], 1);
+      add_row(cur, acc[0], 2);
+      emit(oy0 + r, acc[0]);
+      add_row(cur, acc[0], 0);
     }
   }
-  const bool has_res = a.residual != nullptr;
-  const size_t obase = ((size_t)(n * a.OH + oy) * a.OW + ox0) * C + c0;
-  const uint32_t n_out = last_ox - ox0 + 1u;
-  uint32_t rv[L], qw[L];
-#pragma unroll
-  for (int i = 0; i < L; ++i) {
-    qw[i] = 0u;
-    rv[i] = 0u;
-    if (has_res && (uint32_t)i < n_out)
-      rv[i] = __ldcg(reinterpret_cast<const uint32_t*>((const uint8_t*)a.residual + obase + (size_t)i * C));
-  }
-  const float relu_floor = a.relu ? 0.0f : __int_as_float(0xFF800000);
-  const float lo_f = (float)a.qmin, hi_f = (float)a.qmax;
-  const bool res_signed = a.residual_dtype == PSB_DT_S8;
-  const uint32_t level = a.uniform_log2k;
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const uint32_t o = c0 + j;
-    const float sc = ldexpf(a.scale[o], a.e_base[o] - (int)level), bi = a.bias[o];
-    const int32_t* wch = wint + (size_t)o * 9u;
-    // (a sum marked unknown, 0xFFFFFFFF, fails the test like a large one)
-    const unsigned long long bound = (unsigned long long)__ldca(rowsum256 + (size_t)level * a.O + o) * 256ull * amax;
-    if (bound < (1ull << 31))
-      dw_channel<S, kSignedIn, int>(raw, j, wch, sc, bi, has_res, rv, res_signed, a.residual_scale, relu_floor,
-                                    a.inv_step, lo_f, hi_f, n_out, qw);
-    else
-      dw_channel<S, kSignedIn, long long>(raw, j, wch, sc, bi, has_res, rv, res_signed, a.residual_scale, relu_floor,
-                                          a.inv_step, lo_f, hi_f, n_out, qw);
-  }
-#pragma unroll
-  for (int i = 0; i < L; ++i)
-    if ((uint32_t)i < n_out) *reinterpret_cast<uint32_t*>((uint8_t*)a.q_out + obase + (size_t)i * C) = qw[i];
 }
 
 // [rows][C] -> [rows][pitch] (pitch a multiple of 16, zero beyond C): the copy engine wants rows that are 16-byte
@@ -856,7 +833,30 @@ cudaError_t launch_range_check(const void* x, size_t bytes, uint32_t is_signed, 
 cudaError_t launch_shift_add(const ConvArgs& a, const WintTable& wt, const uint32_t* rowsum256, uint32_t amax,
                              cudaStream_t s) {
   size_t total = (size_t)a.N * a.OH * a.OW * a.O;
-  // depthwise, channels-last, one draw count, only codes wanted: the vectorised kernel
+  // depthwise 3x3, channels-last, one draw count, only codes wanted
+  if (a.groups == a.C && a.O == a.C && a.KH == 3 && a.KW == 3 && a.stride <= 2u && !a.kmap && a.q_out && !a.f32_out && !a.acc_out &&
+      !a.out_nchw && a.inv_step > 0.0f) {
+    // rows per thread: as many as leave two waves of threads (148 SMs x 512), for each strip reads two rows more
+    const uint64_t columns = (uint64_t)a.N * ((a.OW + kDwCols - 1) / kDwCols) * ((a.C + 3u) / 4u);
+    const uint64_t strips = std::min<uint64_t>(std::max<uint64_t>((2ull * 148 * 512 + columns - 1) / columns, (a.OH + 27u) / 28u), (a.OH + 1u) / 2u);
+    const uint32_t rows = (uint32_t)((a.OH + strips - 1) / strips);
+    const uint64_t threads = columns * ((a.OH + rows - 1) / rows);
+    if (threads < (1ull << 32) - 256u) {
+      const uint32_t blocks = (uint32_t)((threads + 255u) / 256u);
+      const int32_t* wl = wt.w[a.uniform_log2k];
+      const bool vec = a.C % 4u == 0 && !(((uintptr_t)a.x | (uintptr_t)a.q_out | (uintptr_t)a.residual) & 3u);
+#define PSB_DW(SV, SG, VC) launch_pdl(dwconv3x3_kernel<SV, SG, VC>, blocks, 256, 0, s, a, wl, rowsum256, amax, rows)
+#define PSB_DW_V(SV, SG) do { if (vec) PSB_DW(SV, SG, true); else PSB_DW(SV, SG, false); } while (0)
+      const bool sg = a.in_dtype == PSB_DT_S8;
+      if (a.stride == 1) { if (sg) PSB_DW_V(1, true); else PSB_DW_V(1, false); }
+      else { if (sg) PSB_DW_V(2, true); else PSB_DW_V(2, false); }
+#undef PSB_DW_V
+#undef PSB_DW
+      note_launch();
+      return cudaGetLastError();
+    }
+  }
+  // other depthwise filters, channel counts that are multiples of 8: eight channels per thread
   const size_t dw_smem = (size_t)a.KH * a.KW * a.C * sizeof(int32_t);
   if (a.groups == a.C && a.O == a.C && a.C % 8u == 0 && !a.kmap && a.q_out && !a.f32_out && !a.acc_out &&
       !a.out_nchw && dw_smem <= 64 * 1024 &&
@@ -867,32 +867,6 @@ cudaError_t launch_shift_add(const ConvArgs& a, const WintTable& wt, const uint3
     if (dev >= 0 && dev < 64 && !attr_set[dev]) {
       cudaFuncSetAttribute(dwconv_nhwc8_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
       attr_set[dev] = true;
-    }
-    if (a.KH == 3 && a.KW == 3 && (a.stride == 1 || a.stride == 2)) {
-      const uint32_t seg_out = a.stride == 1 ? DwSeg<1>::kOut : DwSeg<2>::kOut;
-      const uint64_t threads = (uint64_t)a.N * a.OH * ((a.OW + seg_out - 1) / seg_out) * (a.C / 4u);
-      if (threads < (1ull << 32) - 256u) {
-        const uint32_t blocks = (uint32_t)((threads + 255u) / 256u);
-        const int32_t* wl = wt.w[a.uniform_log2k];
-        const bool sg = a.in_dtype == PSB_DT_S8;
-        if (rowsum256) {
-          if (a.stride == 1) {
-            if (sg) launch_pdl(dwconv3x3_row32_kernel<1, true>, blocks, 256, 0, s, a, wl, rowsum256, amax);
-            else launch_pdl(dwconv3x3_row32_kernel<1, false>, blocks, 256, 0, s, a, wl, rowsum256, amax);
-          } else {
-            if (sg) launch_pdl(dwconv3x3_row32_kernel<2, true>, blocks, 256, 0, s, a, wl, rowsum256, amax);
-            else launch_pdl(dwconv3x3_row32_kernel<2, false>, blocks, 256, 0, s, a, wl, rowsum256, amax);
-          }
-        } else if (a.stride == 1) {
-          if (sg) launch_pdl(dwconv3x3_row_kernel<1, true>, blocks, 256, 0, s, a, wl);
-          else launch_pdl(dwconv3x3_row_kernel<1, false>, blocks, 256, 0, s, a, wl);
-        } else {
-          if (sg) launch_pdl(dwconv3x3_row_kernel<2, true>, blocks, 256, 0, s, a, wl);
-          else launch_pdl(dwconv3x3_row_kernel<2, false>, blocks, 256, 0, s, a, wl);
-        }
-        note_launch();
-        return cudaGetLastError();
-      }
     }
     uint32_t blocks = grid_for(total / 8, 256);
     if (blocks > 148u * 4u) blocks = 148u * 4u;

@@ -110,3 +110,35 @@ def test_shortcut_tiles_through_shared_memory(case, signed_out, oracle):
         assert np.array_equal(q[n:n + 1].astype(np.int32), o["q"])
     wt.free()
     ctx.close()
+
+
+@pytest.mark.parametrize("case", [
+    # (N, C, H, W, stride, dtype, shortcut dtype or None): odd channel counts, one row or column, long strips, wide sums
+    (2, 37, 9, 11, 1, np.uint8, None), (1, 5, 7, 1, 2, np.int8, None), (3, 64, 1, 13, 1, np.uint8, np.int8),
+    (1, 8, 61, 9, 1, np.int8, np.uint8), (2, 12, 64, 33, 2, np.uint8, None), (130, 48, 14, 15, 1, np.uint8, None),
+    (2, 39, 30, 17, 2, np.uint8, np.uint8),
+])
+@pytest.mark.parametrize("log2k,flat", [(4, False), (6, True)])
+def test_depthwise_strips(case, log2k, flat, oracle):
+    """flat: all weights near the window's top, so that the sums do not fit 32 bits."""
+    import paper_1904_02205_b200 as psb
+
+    N, C, H, W, stride, dtype, res_dtype = case
+    ctx = psb.Context(0)
+    rng = np.random.default_rng(C * 3 + H)
+    w = rng.normal(0, 0.3, size=(C, 1, 3, 3)).astype(np.float32)
+    if flat:
+        w = (np.sign(w) * rng.uniform(1.5, 1.99, size=w.shape)).astype(np.float32)
+    lo, hi = (0, 256) if dtype == np.uint8 else (-128, 128)
+    x = rng.integers(lo, hi, size=(N, H, W, C)).astype(dtype)
+    oh, ow = (H - 1) // stride + 1, (W - 1) // stride + 1
+    res = None
+    if res_dtype is not None:
+        lo = 0 if res_dtype == np.uint8 else -128
+        res = rng.integers(lo, lo + 256, size=(N, oh, ow, C)).astype(res_dtype)
+    args = (w, x, 1, C, stride, 1, 5, 3, [log2k], None, log2k, rng.uniform(0.5, 1.5, C).astype(np.float32),
+            rng.normal(0, 0.5, C).astype(np.float32), False, np.float32(0.05 if not flat else 0.01), -100, 101)
+    o = oracle_layer(oracle, *args, residual=res, res_scale=np.float32(0.3))
+    g = gpu_layer(psb, ctx, *args, psb.PSB_DT_S8, residual=res, res_scale=np.float32(0.3), want=("q",))
+    compare(g, o, [log2k])
+    ctx.close()
