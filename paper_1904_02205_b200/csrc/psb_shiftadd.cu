@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(256) dwconv_nhwc8_kernel(const ConvArgs a, con
 // a channel where it does not computes its outputs one by one in 64 bits.  The output stage is dequant()/requant() with
 // the relu folded into the lower clamp (inv_step > 0), rounded by adding 1.5 * 2^23.
 // Bound by the nine 32-bit multiply-adds per output (2 clocks each): 15 us for 144 channels @56, batch 64.  That layer
-// with its sampling: 78.6 -> 65.8 us (a thread with 8 outputs of one row spent 48 logic clocks per output and spilled).
+// with its sampling: 78.6 -> 58.4 us (a thread with 8 outputs of one row spent 48 logic clocks per output and spilled).
 constexpr int kDwCols = 2;
 
 struct DwConst {
@@ -336,8 +336,14 @@ __global__ void __launch_bounds__(256, 2) dwconv3x3_kernel(const ConvArgs a, con
   bool col_in[NC];
 #pragma unroll
   for (int q = 0; q < NC; ++q) col_in[q] = (unsigned)(ix0 + q) < a.W;
-  const uint8_t* const xcol = (const uint8_t*)a.x + ((ptrdiff_t)n * a.H * a.W + ix0) * (ptrdiff_t)C + c0;
-  const size_t row_bytes = (size_t)a.W * C;
+  const size_t row_bytes = (size_t)a.W * C, out_row_bytes = (size_t)a.OW * C;
+  const int iy0 = (int)(oy0 * S) - (int)a.pad;
+  // the next input row to load (its number and address) and the next output row to write, both moved on row by row
+  int iy = iy0;
+  const uint8_t* in_row = (const uint8_t*)a.x + (((ptrdiff_t)n * a.H + iy0) * (ptrdiff_t)a.W + ix0) * (ptrdiff_t)C + c0;
+  size_t out_at = (((size_t)n * a.OH + oy0) * a.OW + ox0) * C + c0;
+  const bool second = ox0 + 1u < a.OW;
+  static_assert(kDwCols == 2, "the last segment of a row has one or two columns");
 
   auto load_word = [&](const uint8_t* at) -> uint32_t {
     if (kVec) return __ldcg(reinterpret_cast<const uint32_t*>(at));
@@ -347,41 +353,40 @@ __global__ void __launch_bounds__(256, 2) dwconv3x3_kernel(const ConvArgs a, con
       if ((uint32_t)j < left) v |= (uint32_t)at[j] << (8 * j);
     return v;
   };
-  auto load_row = [&](int iy, uint32_t (&raw)[NC]) {
+  auto load_row = [&](uint32_t (&raw)[NC]) {
     const bool in = (unsigned)iy < a.H;
-    const uint8_t* rp = xcol + (ptrdiff_t)iy * (ptrdiff_t)row_bytes;
 #pragma unroll
     for (int q = 0; q < NC; ++q) {
       raw[q] = 0u;
-      if (in && col_in[q]) raw[q] = load_word(rp + (size_t)q * C);
+      if (in && col_in[q]) raw[q] = load_word(in_row + (uint32_t)q * C);
+    }
+    ++iy;
+    in_row += row_bytes;
+  };
+  auto extract = [&](const uint32_t (&raw)[NC], const int j, int (&x)[NC]) {
+#pragma unroll
+    for (int q = 0; q < NC; ++q) {
+      const uint32_t b = (raw[q] >> (8 * j)) & 0xFFu;
+      x[q] = kSignedIn ? (int)(signed char)b : (int)b;
+    }
+  };
+  // adds row `kh` of the filter on one input row to the sums of channel j (kh == 0 starts them)
+  auto add_row = [&](const int (&x)[NC], int (&sum)[kDwCols][4], const int j, const int kh) {
+#pragma unroll
+    for (int i = 0; i < kDwCols; ++i) {
+      int v = kh == 0 ? 0 : sum[i][j];
+      v += x[i * S] * w[j][kh * 3];
+      v += x[i * S + 1] * w[j][kh * 3 + 1];
+      v += x[i * S + 2] * w[j][kh * 3 + 2];
+      sum[i][j] = v;
     }
   };
   int acc[3][kDwCols][4];
-  // adds row `kh` of the filter on one input row to a set of sums (kh == 0 starts them)
-  auto add_row = [&](const uint32_t (&raw)[NC], int (&sum)[kDwCols][4], const int kh) {
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      int x[NC];
-#pragma unroll
-      for (int q = 0; q < NC; ++q) {
-        const uint32_t b = (raw[q] >> (8 * j)) & 0xFFu;
-        x[q] = kSignedIn ? (int)(signed char)b : (int)b;
-      }
-#pragma unroll
-      for (int i = 0; i < kDwCols; ++i) {
-        int v = kh == 0 ? 0 : sum[i][j];
-        v += x[i * S] * w[j][kh * 3];
-        v += x[i * S + 1] * w[j][kh * 3 + 1];
-        v += x[i * S + 2] * w[j][kh * 3 + 2];
-        sum[i][j] = v;
-      }
-    }
-  };
-  auto emit = [&](uint32_t oy, const int (&sum)[kDwCols][4]) {
+  auto emit = [&](const int (&sum)[kDwCols][4]) {
 #pragma unroll
     for (int i = 0; i < kDwCols; ++i) {
-      if (ox0 + (uint32_t)i >= a.OW) break;
-      const size_t at = (((size_t)n * a.OH + oy) * a.OW + ox0 + i) * C + c0;
+      if (i && !second) break;
+      const size_t at = out_at + (uint32_t)i * C;
       uint32_t rw = 0u;
       if (has_res) {
         const uint8_t* rp = (const uint8_t*)a.residual + at;
@@ -406,23 +411,28 @@ __global__ void __launch_bounds__(256, 2) dwconv3x3_kernel(const ConvArgs a, con
           if ((uint32_t)j < left) ((uint8_t*)a.q_out)[at + j] = (uint8_t)(word >> (8 * j));
       }
     }
+    out_at += out_row_bytes;
   };
-  const int iy0 = (int)(oy0 * S) - (int)a.pad;
   const uint32_t rows = oy1 - oy0;
   uint32_t cur[NC], nxt[NC];
-  load_row(iy0, cur);
-  load_row(iy0 + 1, nxt);
+  load_row(cur);
+  load_row(nxt);
   if (S == 1) {
     // input row r opens output r, adds to output r - 1 and closes output r - 2
     auto step = [&](uint32_t r, int (&open)[kDwCols][4], int (&mid)[kDwCols][4], int (&close)[kDwCols][4]) {
       uint32_t raw[NC];
 #pragma unroll
       for (int q = 0; q < NC; ++q) { raw[q] = cur[q]; cur[q] = nxt[q]; }
-      if (r + 2u < rows + 2u) load_row(iy0 + (int)r + 2, nxt);
-      add_row(raw, open, 0);
-      add_row(raw, mid, 1);
-      add_row(raw, close, 2);
-      if (r >= 2u && r - 2u < rows) emit(oy0 + r - 2u, close);
+      if (r < rows) load_row(nxt);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        int x[NC];
+        extract(raw, j, x);
+        add_row(x, open, j, 0);
+        add_row(x, mid, j, 1);
+        add_row(x, close, j, 2);
+      }
+      if (r >= 2u && r - 2u < rows) emit(close);
     };
 #pragma unroll
     for (int k = 0; k < 3; ++k)
@@ -436,17 +446,33 @@ __global__ void __launch_bounds__(256, 2) dwconv3x3_kernel(const ConvArgs a, con
       step(r + 2u, acc[2], acc[1], acc[0]);
     }
   } else {
-    add_row(cur, acc[0], 0);
-    for (uint32_t r = 0; r < rows; ++r) {
-      uint32_t mid[NC];
+    // two input rows per output row; the second one closes it and opens the next
 #pragma unroll
-      for (int q = 0; q < NC; ++q) mid[q] = nxt[q];
-      load_row(iy0 + 2 * (int)r + 2, cur);
-      if (r + 1u < rows) load_row(iy0 + 2 * (int)r + 3, nxt);
-      add_row(mid, acc[0], 1);
-      add_row(cur, acc[0], 2);
-      emit(oy0 + r, acc[0]);
-      add_row(cur, acc[0], 0);
+    for (int j = 0; j < 4; ++j) {
+      int x[NC];
+      extract(cur, j, x);
+      add_row(x, acc[0], j, 0);
+    }
+    load_row(cur);
+    for (uint32_t r = 0; r < rows; ++r) {
+      uint32_t mid[NC], end[NC];
+#pragma unroll
+      for (int q = 0; q < NC; ++q) { mid[q] = nxt[q]; end[q] = cur[q]; }
+      if (r + 1u < rows) { load_row(nxt); load_row(cur); }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        int x[NC];
+        extract(mid, j, x);
+        add_row(x, acc[0], j, 1);
+        extract(end, j, x);
+        add_row(x, acc[0], j, 2);
+        add_row(x, acc[1], j, 0);
+      }
+      emit(acc[0]);
+#pragma unroll
+      for (int i = 0; i < kDwCols; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[0][i][j] = acc[1][i][j];
     }
   }
 }
@@ -836,10 +862,17 @@ cudaError_t launch_shift_add(const ConvArgs& a, const WintTable& wt, const uint3
   // depthwise 3x3, channels-last, one draw count, only codes wanted
   if (a.groups == a.C && a.O == a.C && a.KH == 3 && a.KW == 3 && a.stride <= 2u && !a.kmap && a.q_out && !a.f32_out && !a.acc_out &&
       !a.out_nchw && a.inv_step > 0.0f) {
-    // rows per thread: as many as leave two waves of threads (148 SMs x 512), for each strip reads two rows more
+    // Rows per thread: the machine holds two blocks of 256 threads per SM; among the strip lengths the one with the
+    // least (waves of blocks) x (rows + what a thread spends before its first row, about four rows' worth)
     const uint64_t columns = (uint64_t)a.N * ((a.OW + kDwCols - 1) / kDwCols) * ((a.C + 3u) / 4u);
-    const uint64_t strips = std::min<uint64_t>(std::max<uint64_t>((2ull * 148 * 512 + columns - 1) / columns, (a.OH + 27u) / 28u), (a.OH + 1u) / 2u);
-    const uint32_t rows = (uint32_t)((a.OH + strips - 1) / strips);
+    uint32_t rows = a.OH;
+    uint64_t best = ~0ull;
+    for (uint32_t strips = 1; strips <= 32u && strips <= a.OH; ++strips) {
+      const uint32_t r = (a.OH + strips - 1) / strips;
+      const uint64_t waves = (columns * ((a.OH + r - 1) / r) + 2ull * 148 * 256 - 1) / (2ull * 148 * 256);
+      const uint64_t cost = waves * (r + 4u);
+      if (cost < best) { best = cost; rows = r; }
+    }
     const uint64_t threads = columns * ((a.OH + rows - 1) / rows);
     if (threads < (1ull << 32) - 256u) {
       const uint32_t blocks = (uint32_t)((threads + 255u) / 256u);
