@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(256) dwconv_nhwc8_kernel(const ConvArgs a, con
 // a channel where it does not computes its outputs one by one in 64 bits.  The output stage is dequant()/requant() with
 // the relu folded into the lower clamp (inv_step > 0), rounded by adding 1.5 * 2^23.
 // Bound by the nine 32-bit multiply-adds per output (2 clocks each): 15 us for 144 channels @56, batch 64.  That layer
-// with its sampling: 78.6 -> 58.4 us (a thread with 8 outputs of one row spent 48 logic clocks per output and spilled).
+// with its sampling: 78.6 -> 51.4 us (a thread with 8 outputs of one row spent 48 logic clocks per output and spilled).
 constexpr int kDwCols = 2;
 
 struct DwConst {
@@ -283,7 +283,7 @@ __device__ __noinline__ void dw_output64(const ConvArgs& a, const int32_t* wch, 
 
 // kVec: channel counts that are multiples of 4 at 4-byte aligned addresses; otherwise words are put together from bytes.
 template <int S, bool kSignedIn, bool kVec>
-__global__ void __launch_bounds__(256, 2) dwconv3x3_kernel(const ConvArgs a, const int32_t* wint, const uint32_t* rowsum256,
+__global__ void __launch_bounds__(128, 5) dwconv3x3_kernel(const ConvArgs a, const int32_t* wint, const uint32_t* rowsum256,
                                                            uint32_t amax, uint32_t rows_per_thread) {
   pdl_prologue();
   constexpr int NC = DwIn<S>::kCols;
@@ -862,23 +862,23 @@ cudaError_t launch_shift_add(const ConvArgs& a, const WintTable& wt, const uint3
   // depthwise 3x3, channels-last, one draw count, only codes wanted
   if (a.groups == a.C && a.O == a.C && a.KH == 3 && a.KW == 3 && a.stride <= 2u && !a.kmap && a.q_out && !a.f32_out && !a.acc_out &&
       !a.out_nchw && a.inv_step > 0.0f) {
-    // Rows per thread: the machine holds two blocks of 256 threads per SM; among the strip lengths the one with the
+    // Rows per thread: the machine holds five blocks of 128 threads per SM; among the strip lengths the one with the
     // least (waves of blocks) x (rows + what a thread spends before its first row, about four rows' worth)
     const uint64_t columns = (uint64_t)a.N * ((a.OW + kDwCols - 1) / kDwCols) * ((a.C + 3u) / 4u);
     uint32_t rows = a.OH;
     uint64_t best = ~0ull;
     for (uint32_t strips = 1; strips <= 32u && strips <= a.OH; ++strips) {
       const uint32_t r = (a.OH + strips - 1) / strips;
-      const uint64_t waves = (columns * ((a.OH + r - 1) / r) + 2ull * 148 * 256 - 1) / (2ull * 148 * 256);
+      const uint64_t waves = (columns * ((a.OH + r - 1) / r) + 5ull * 148 * 128 - 1) / (5ull * 148 * 128);
       const uint64_t cost = waves * (r + 4u);
       if (cost < best) { best = cost; rows = r; }
     }
     const uint64_t threads = columns * ((a.OH + rows - 1) / rows);
     if (threads < (1ull << 32) - 256u) {
-      const uint32_t blocks = (uint32_t)((threads + 255u) / 256u);
+      const uint32_t blocks = (uint32_t)((threads + 127u) / 128u);
       const int32_t* wl = wt.w[a.uniform_log2k];
       const bool vec = a.C % 4u == 0 && !(((uintptr_t)a.x | (uintptr_t)a.q_out | (uintptr_t)a.residual) & 3u);
-#define PSB_DW(SV, SG, VC) launch_pdl(dwconv3x3_kernel<SV, SG, VC>, blocks, 256, 0, s, a, wl, rowsum256, amax, rows)
+#define PSB_DW(SV, SG, VC) launch_pdl(dwconv3x3_kernel<SV, SG, VC>, blocks, 128, 0, s, a, wl, rowsum256, amax, rows)
 #define PSB_DW_V(SV, SG) do { if (vec) PSB_DW(SV, SG, true); else PSB_DW(SV, SG, false); } while (0)
       const bool sg = a.in_dtype == PSB_DT_S8;
       if (a.stride == 1) { if (sg) PSB_DW_V(1, true); else PSB_DW_V(1, false); }
