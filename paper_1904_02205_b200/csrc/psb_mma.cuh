@@ -14,8 +14,8 @@
 //            filters with taps, stride or padding; plain 2-D tiles otherwise) and
 //            of the digit-plane tile into a ring of shared-memory stages
 //   warp 2 issues the MMAs
-//   warp 3 allocates TMEM; issues half of the MMAs in band mode; flips the top bit of unsigned activations;
-//            staged outputs: moves shortcut tiles into and output tiles out of shared memory
+//   warp 3 allocates TMEM; issues half of the MMAs in band mode and where a tile is one stage; flips the top bit of
+//            unsigned activations; staged outputs: moves shortcut tiles in and output tiles out of shared memory
 //   warps 4-19 epilogue: TMEM -> registers, recombine planes, dequantise, bias,
 //            shortcut, ReLU, re-quantise, vectorised stores; overlaps the next
 //            tile's MMAs through two TMEM accumulator buffers
@@ -79,6 +79,7 @@ struct TensorParams {
                         // x = 0, so padding needs no case of its own
   uint32_t resident;    // 1: the CTA keeps the digit planes of its channel tile in shared memory
   uint32_t ctas_per_otile;
+  uint32_t alternate;   // 1: one pipeline stage per tile, and two warps issue the MMAs of alternate tiles
   uint32_t resident_bytes;
   const uint32_t* rowsum256;   // [level][O] row sums of |W_k| in units of 256 (rounded up), or null
   uint32_t amax;        // largest activation magnitude the caller vouches for
@@ -1024,10 +1025,15 @@ __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, WaitCtl
 // addresses stay uniform.  Two single threads taking turns, out of line, as there were before, needed 100 to 250 clocks
 // per MMA and hand-overs between them (K block of 4 MMAs, streamed planes, 3x3 256 -> 256 channels: 753 -> 640 clocks;
 // the copies of a K block, 40 KB at the 68 bytes per clock and SM that L2 delivers to all SMs at once, take 600).
+// Tiles of a single stage alternate between two warps (p.alternate): what a warp does per tile beside its MMAs (waits,
+// descriptors, commits) takes about 1300 clocks, more than the tile's copies: 1x1 96 -> 16 channels
+// @112, batch 64: 34.6 -> 27.7 us, 256 -> 64 @56 13.7 -> 12.4.  (Not with staged outputs, where that warp moves the tiles:
+// one producer warp for both was slower, 40.2 -> 45.1 us on 64 -> 256 @56 with a shortcut.)
 // Returns true on a timeout.
 template <int BK>
 __device__ __forceinline__ bool mma_role(const TensorParams& p, SharedCtl* ctl, uint32_t tmem_base, uint32_t ring_addr,
-                                         uint32_t planes_addr, uint32_t stage_bytes, uint32_t sub_bytes, uint32_t k_iters) {
+                                         uint32_t planes_addr, uint32_t stage_bytes, uint32_t sub_bytes, uint32_t k_iters,
+                                         uint32_t mine) {
   WaitCtl* wc = &ctl->wait;
   const bool leader = elect_one();
   const uint32_t full0 = smem_u32(p.flip ? &ctl->flipped[0] : &ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
@@ -1042,6 +1048,11 @@ __device__ __forceinline__ bool mma_role(const TensorParams& p, SharedCtl* ctl, 
   for (ti.init(p); ti.valid(); ti.next()) {
     const uint32_t levels = tile_levels(p, ti.m_tile) & p.a.level_mask & 0x7Fu;
     if (!levels) continue;      // no sampled level: no pass from any role
+    if (p.alternate && (pass & 1u) != mine) {      // the other warp's tile and stage
+      ++pass;
+      if (++s == p.stages) { s = 0; ph ^= 1u; }
+      continue;
+    }
     const uint32_t P = p.planes[(uint32_t)__ffs((int)levels) - 1u];
     const uint32_t buf = pass & 1u, aph = (pass >> 1) & 1u;
     ++pass;
@@ -1341,8 +1352,9 @@ psb_mma_kernel(const __grid_constant__ TmapSet maps, const __grid_constant__ Ten
     // ---------------------------------------------------------------- MMA
     if (p.band)
       failed = mma_role_band<BK>(p, ctl, tmem_base, smem_u32(ring), smem_u32(smem), stage_bytes, warp - (uint32_t)kMmaWarp0);
-    else if (warp == (uint32_t)kMmaWarp0)
-      failed = mma_role<BK>(p, ctl, tmem_base, smem_u32(ring), smem_u32(smem), stage_bytes, sub_bytes, k_iters);
+    else if (warp == (uint32_t)kMmaWarp0 || p.alternate)
+      failed = mma_role<BK>(p, ctl, tmem_base, smem_u32(ring), smem_u32(smem), stage_bytes, sub_bytes, k_iters,
+                            warp - (uint32_t)kMmaWarp0);
     else if (p.staged) {
       if (lane == 0) failed = io_role(p, maps, ctl, slots_addr);
       failed = __shfl_sync(0xFFFFFFFFu, failed ? 1 : 0, 0) != 0;

@@ -165,6 +165,7 @@ psb_status launch_tensor(psb_ctx* ctx, const psb_weights* wt, const ConvArgs& a,
   }
   if (p.band) group = k_iters;   // one stage = one band = every tap of a tile
   p.group = group;
+  p.alternate = (!p.band && !p.staged && !flip && group >= k_iters) ? 1u : 0u;
   uint32_t stages = (uint32_t)(p.band ? avail / p.band_bytes : avail / ((size_t)group * sub_bytes));
   if (stages > (uint32_t)kMaxStages) stages = kMaxStages;
   // An even number of stages: the two producer warps and the two MMA issuing threads each take
