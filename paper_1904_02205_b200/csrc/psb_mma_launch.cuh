@@ -6,20 +6,19 @@
 namespace psb {
 
 template <int BK>
-cudaError_t launch_mma_kernel(const cudaLaunchConfig_t& cfg, const TmapSet& maps, const TensorParams& p, int device, bool general) {
+cudaError_t launch_mma_kernel(const cudaLaunchConfig_t& cfg, const TmapSet& maps, const TensorParams& p, int device, int kind) {
+  const auto kernel = kind == kGeneralOutputs ? psb_mma_kernel<BK, kGeneralOutputs>
+                      : kind == kSortedRows   ? psb_mma_kernel<BK, kSortedRows> : psb_mma_kernel<BK, kOneLevel>;
   // the shared-memory limit of an instance is raised once per device, to the most a launch can ask for
   constexpr int kMaxDevicesForAttr = 64;
-  static bool raised[kMaxDevicesForAttr][2];
+  static bool raised[kMaxDevicesForAttr][3];
   const bool known = device >= 0 && device < kMaxDevicesForAttr;
-  if (!known || !raised[device][general]) {
-    const cudaError_t e = general
-        ? cudaFuncSetAttribute(psb_mma_kernel<BK, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget)
-        : cudaFuncSetAttribute(psb_mma_kernel<BK, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget);
+  if (!known || !raised[device][kind]) {
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget);
     if (e != cudaSuccess) return e;
-    if (known) raised[device][general] = true;
+    if (known) raised[device][kind] = true;
   }
-  return general ? cudaLaunchKernelEx(&cfg, psb_mma_kernel<BK, true>, maps, p)
-                 : cudaLaunchKernelEx(&cfg, psb_mma_kernel<BK, false>, maps, p);
+  return cudaLaunchKernelEx(&cfg, kernel, maps, p);
 }
 
 }  // namespace psb

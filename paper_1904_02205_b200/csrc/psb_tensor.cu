@@ -147,8 +147,10 @@ psb_status launch_tensor(psb_ctx* ctx, const psb_weights* wt, const ConvArgs& a,
       p.ctas_per_otile = cpo < p.m_tiles ? cpo : p.m_tiles;
     }
   }
-  // Staged outputs (epilogue_staged): channels-last codes in rows of whole 16-byte pieces, rows in tile order
-  p.staged = (uniform_epilogue(p) && !a.kmap && !p.band && !a.out_nchw && p.unit == 16u && !flip && a.residual &&
+  // Staged outputs: channels-last codes in rows of whole 16-byte pieces.  Rows in tile order (epilogue_staged) only with a
+  // shortcut: a whole row of 16 bytes per lane is written as fast directly.  Rows sorted by level (epilogue_sorted) always:
+  // they lie anywhere, and no role but the output stage takes part, so flipped activations are served too.
+  p.staged = (uniform_epilogue(p) && !p.band && !a.out_nchw && p.unit == 16u && (a.kmap || (a.residual && !flip)) &&
               (uint64_t)p.m_tiles * p.o_tiles >= kStagedMinTiles * (uint64_t)ctx->sm_count) ? 1u : 0u;
   const size_t io_bytes = p.staged ? (size_t)kIoSlots * kIoTileBytes : 0u;
   // K blocks are handed over in groups: every barrier round trip costs the issuing thread a
@@ -165,7 +167,7 @@ psb_status launch_tensor(psb_ctx* ctx, const psb_weights* wt, const ConvArgs& a,
   }
   if (p.band) group = k_iters;   // one stage = one band = every tap of a tile
   p.group = group;
-  p.alternate = (!p.band && !p.staged && !flip && group >= k_iters) ? 1u : 0u;
+  p.alternate = (!p.band && !(p.staged && !a.kmap) && !flip && group >= k_iters) ? 1u : 0u;
   uint32_t stages = (uint32_t)(p.band ? avail / p.band_bytes : avail / ((size_t)group * sub_bytes));
   if (stages > (uint32_t)kMaxStages) stages = kMaxStages;
   // An even number of stages: the two producer warps and the two MMA issuing threads each take
@@ -213,7 +215,7 @@ psb_status launch_tensor(psb_ctx* ctx, const psb_weights* wt, const ConvArgs& a,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
       return PSB_ERR_CUDA;
   }
-  if (p.staged) {
+  if (p.staged && !a.kmap) {
     cuuint64_t dims[2] = {a.O, p.M};
     cuuint64_t strides[1] = {(cuuint64_t)a.O};
     cuuint32_t box[2] = {(cuuint32_t)kTileN, kTileM};
@@ -241,12 +243,12 @@ psb_status launch_tensor(psb_ctx* ctx, const psb_weights* wt, const ConvArgs& a,
   cfg.stream = s;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  const bool general = !uniform_epilogue(p);
+  const int kind = !uniform_epilogue(p) ? kGeneralOutputs : a.kmap ? kSortedRows : kOneLevel;
   const bool timed = ctx->time_contraction && ctx->t_begin[0] && ctx->timed_launches < psb_ctx::kTimedLaunches;
   if (timed) cudaEventRecord(ctx->t_begin[ctx->timed_launches], s);
-  e = bk == 128 ? launch_mma_kernel<128>(cfg, maps, p, ctx->device, general)
-      : bk == 64 ? launch_mma_kernel<64>(cfg, maps, p, ctx->device, general)
-                 : launch_mma_kernel<32>(cfg, maps, p, ctx->device, general);
+  e = bk == 128 ? launch_mma_kernel<128>(cfg, maps, p, ctx->device, kind)
+      : bk == 64 ? launch_mma_kernel<64>(cfg, maps, p, ctx->device, kind)
+                 : launch_mma_kernel<32>(cfg, maps, p, ctx->device, kind);
   note_launch();
   if (timed) {
     cudaEventRecord(ctx->t_end[ctx->timed_launches], s);

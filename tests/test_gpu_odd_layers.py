@@ -142,3 +142,49 @@ def test_depthwise_strips(case, log2k, flat, oracle):
     g = gpu_layer(psb, ctx, *args, psb.PSB_DT_S8, residual=res, res_scale=np.float32(0.3), want=("q",))
     compare(g, o, [log2k])
     ctx.close()
+
+
+@pytest.mark.parametrize("case", [
+    # (N, H, W, C, O, K, shortcut dtype or None, in_max): several tiles per SM on rows sorted by level
+    (19, 56, 57, 64, 64, 1, np.uint8, 15), (30, 49, 41, 32, 80, 1, np.int8, 15), (19, 56, 57, 64, 48, 3, None, 15),
+    (8, 57, 61, 128, 144, 1, np.uint8, 127),
+])
+@pytest.mark.parametrize("levels", [(0, 2, 4), (5, 6)])
+def test_sorted_rows_through_shared_memory(case, levels, oracle):
+    import torch
+
+    import paper_1904_02205_b200 as psb
+
+    N, H, W, C, O, K, res_dtype, top = case
+    assert -(-N * H * W // 128) * -(-O // 64) >= 3 * 148
+    ctx = psb.Context(0)
+    rng = np.random.default_rng(O + H + levels[0])
+    w = rng.normal(0, np.sqrt(2.0 / (C * K * K)), size=(O, C, K, K)).astype(np.float32)
+    x = rng.integers(0, top + 1, size=(N, H, W, C)).astype(np.uint8)
+    scale, bias = rng.uniform(0.5, 1.5, O).astype(np.float32), rng.normal(0, 0.5, O).astype(np.float32)
+    res = None
+    if res_dtype is not None:
+        lo = 0 if res_dtype == np.uint8 else -128
+        res = rng.integers(lo, lo + 256, size=(N, H, W, O)).astype(res_dtype)
+    kmap = rng.choice(levels, size=(N, H, W)).astype(np.uint8)
+    dev = lambda t: torch.from_numpy(t).to(ctx.device)
+    wt = ctx.sample_weights(dev(w), seed=5, layer_id=3, level_mask=sum(1 << l for l in levels))
+    run = lambda: ctx.conv2d(wt, dev(x), psb.PSB_LAYOUT_NHWC, 1, K // 2, dev(scale), dev(bias), True, np.float32(0.2), 0, 15,
+                             residual=None if res is None else dev(res), residual_scale=0.3, in_max=top, path=psb.PSB_PATH_TENSOR)
+    ctx.set_sample_map(dev(kmap))
+    q = run()["q"].cpu().numpy()
+    assert ctx.device_status() == 0
+    for n in (0, N - 1):
+        o = oracle_layer(oracle, w, x[n:n + 1], 1, 1, 1, K // 2, 5, 3, list(levels), kmap[n:n + 1], levels[0], scale, bias, True,
+                         np.float32(0.2), 0, 15, residual=None if res is None else res[n:n + 1], res_scale=np.float32(0.3))
+        assert np.array_equal(q[n:n + 1].astype(np.int32), o["q"])
+    # a level that was not sampled is reported; the other locations keep their results
+    bad = kmap.copy()
+    bad[1, 3, :200] = 1
+    ctx.set_sample_map(dev(bad))
+    again = run()["q"].cpu().numpy()
+    assert ctx.device_status() == psb.PSB_ERR_BAD_K
+    assert np.array_equal(again[2:], q[2:])
+    ctx.set_sample_map(None, 0)
+    wt.free()
+    ctx.close()
