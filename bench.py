@@ -268,10 +268,10 @@ class FcWorkload:
         self.q_host.copy_(self.out["q"], non_blocking=True)
 
     def roofline(self, kernel_ms, peaks):
-        # one launch of 2048 threads: neither bytes (35 KB) nor arithmetic matter, the launch does
+        # one launch, a warp per output: neither bytes (35 KB) nor arithmetic matter, the launch does
         nbytes = self.images * 256 + 128 * 256 * 4 + self.images * 128
         achieved = nbytes / (kernel_ms * 1e-3) / 1e9
-        return dict(bound="hbm", kernel="conv_direct_kernel (latency-bound: one launch of 2048 threads)",
+        return dict(bound="hbm", kernel="gemv_planes_kernel (latency-bound: one warp per output)",
                     achieved=achieved, peak=peaks["hbm_gbs"], unit="GB/s", frac=achieved / peaks["hbm_gbs"],
                     traffic=None, peak_source=peaks["source"], kernel_ms=kernel_ms)
 

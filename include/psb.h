@@ -21,10 +21,11 @@
  *   - `stream` is a cudaStream_t passed as void*.  All compute calls are
  *     asynchronous on that stream and do not synchronise the device, with one
  *     exception: a call that needs a larger internal scratch buffer than any
- *     call before it on this context (layout conversion, gathered matrices,
+ *     call before it on this stream (layout conversion, gathered matrices,
  *     the sorted order of a draw-count map) frees and allocates device
  *     memory, which waits for the device; after one pass over a network's
- *     shapes no call grows anything.  Otherwise only psb_create, psb_destroy,
+ *     shapes no call grows anything.  (A context keeps buffers for eight
+ *     streams; a ninth takes over those unused longest and waits likewise.)  Otherwise only psb_create, psb_destroy,
  *     the first psb_sample_weights for a handle, psb_weights_free and
  *     psb_device_status may block.
  *   - Every function returns a psb_status: 0 on success, negative on error.
