@@ -186,8 +186,8 @@ __device__ __forceinline__ float acc_to_float(long long acc) {
 // global memory, which waits for the earlier grids to complete (and lets the kernel after it be
 // scheduled in turn).  What is saved is the launch latency between the many short kernels of a step.
 //
-// Rule for such kernels: whatever an earlier kernel of the stream may have written (activations, integer
-// filters and their row sums, the sorted order of a draw-count map, scratch matrices) is read with ordinary
+// Rule for such kernels: whatever an earlier kernel of the stream may have written (activations, fp32 filters,
+// integer filters and their row sums, the sorted order of a draw-count map, scratch matrices) is read with ordinary
 // loads (plain, __ldca, __ldcg), never through the read-only path (__ldg, or a const __restrict__ kernel
 // parameter, which the compiler turns into the same instruction).  That path promises data that does not
 // change during the kernel's lifetime, which here begins before the earlier kernel has finished: the compiler

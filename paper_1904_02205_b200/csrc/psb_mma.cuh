@@ -400,16 +400,17 @@ __device__ __forceinline__ uint4 chunk_math(const uint32_t (&v)[P][16], const ui
 // 16 bytes of a channels-last row.  Rows that are only 8-byte aligned (channel counts that are odd
 // multiples of 8) move as two halves; `both` is false for the last 8 channels of such a row.
 // The loads are volatile asm so that they stay where they are written (a tile ahead of their use, before
-// the wait for the accumulator) instead of being sunk to the first use of the value.
+// the wait for the accumulator) instead of being sunk to the first use of the value.  Shortcut bytes are the output of an
+// earlier kernel: ordinary loads (the rule at pdl_prologue).
 __device__ __forceinline__ uint4 load_row16(const uint8_t* src, bool vec16, bool both) {
   uint4 r = make_uint4(0u, 0u, 0u, 0u);
   if (vec16) {
-    asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];"
+    asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];"
                  : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(src));
     return r;
   }
-  asm volatile("ld.global.nc.v2.u32 {%0, %1}, [%2];" : "=r"(r.x), "=r"(r.y) : "l"(src));
-  if (both) asm volatile("ld.global.nc.v2.u32 {%0, %1}, [%2];" : "=r"(r.z), "=r"(r.w) : "l"(src + 8));
+  asm volatile("ld.global.v2.u32 {%0, %1}, [%2];" : "=r"(r.x), "=r"(r.y) : "l"(src));
+  if (both) asm volatile("ld.global.v2.u32 {%0, %1}, [%2];" : "=r"(r.z), "=r"(r.w) : "l"(src + 8));
   return r;
 }
 __device__ __forceinline__ void store_row16(uint8_t* dst, uint4 v, bool vec16, bool both) {

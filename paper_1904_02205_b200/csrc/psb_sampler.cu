@@ -172,7 +172,7 @@ __device__ __forceinline__ uint32_t max_magnitude(const uint32_t (&u)[kN], uint3
   return max(best, m);
 }
 
-__device__ __forceinline__ void emax_block(const float* __restrict__ w, uint32_t O, uint32_t d,
+__device__ __forceinline__ void emax_block(const float* w, uint32_t O, uint32_t d,
                                            uint32_t norm, uint32_t* __restrict__ e_max,
                                            uint32_t* __restrict__ err, uint32_t block, uint32_t blocks,
                                            uint32_t tag, uint32_t* __restrict__ rowsum,
@@ -197,14 +197,14 @@ __device__ __forceinline__ void emax_block(const float* __restrict__ w, uint32_t
       if ((((uintptr_t)row) & 15u) == 0u && (d & 3u) == 0u) {
 #pragma unroll 4
         for (uint32_t i = lane * 4u; i < d; i += lanes * 4u) {
-          const uint4 v = __ldg(reinterpret_cast<const uint4*>(row + i));
+          const uint4 v = __ldcg(reinterpret_cast<const uint4*>(row + i));
           const uint32_t u4[4] = {v.x, v.y, v.z, v.w};
           best = max_magnitude(u4, best, bad);     // Inf/NaN is flagged and takes no part in the window
         }
       } else {
 #pragma unroll 4
         for (uint32_t i = lane; i < d; i += lanes) {
-          const uint32_t u1[1] = {__float_as_uint(__ldg(row + i))};
+          const uint32_t u1[1] = {__float_as_uint(__ldcg(row + i))};
           best = max_magnitude(u1, best, bad);
         }
       }
@@ -227,7 +227,7 @@ __device__ __forceinline__ void emax_block(const float* __restrict__ w, uint32_t
         uint4 v[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q)
-          v[q] = i + q * step < total ? __ldg(reinterpret_cast<const uint4*>(w + i + q * step)) : make_uint4(0u, 0u, 0u, 0u);
+          v[q] = i + q * step < total ? __ldcg(reinterpret_cast<const uint4*>(w + i + q * step)) : make_uint4(0u, 0u, 0u, 0u);
         uint32_t u16[16];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -237,7 +237,7 @@ __device__ __forceinline__ void emax_block(const float* __restrict__ w, uint32_t
       }
     } else {
       for (size_t i = (size_t)block * blockDim.x + threadIdx.x; i < total; i += (size_t)blocks * blockDim.x) {
-        const uint32_t u1[1] = {__float_as_uint(__ldg(w + i))};
+        const uint32_t u1[1] = {__float_as_uint(__ldcg(w + i))};
         best = max_magnitude(u1, best, bad);
       }
     }
@@ -256,7 +256,7 @@ __device__ __forceinline__ void emax_block(const float* __restrict__ w, uint32_t
   }
 }
 
-__global__ void emax_kernel(const float* __restrict__ w, uint32_t O, uint32_t d, uint32_t norm,
+__global__ void emax_kernel(const float* w, uint32_t O, uint32_t d, uint32_t norm,
                             uint32_t* __restrict__ e_max, uint32_t* __restrict__ err, uint32_t tag,
                             uint32_t* __restrict__ rowsum, long long* __restrict__ corr, uint32_t pbits) {
   pdl_prologue();
@@ -689,10 +689,10 @@ __device__ __forceinline__ void sample_block(const SampleParams& p, uint32_t blo
     if ((((uintptr_t)src) & 15u) == 0u && (count & 3u) == 0u) {
 #pragma unroll 4
       for (uint32_t t = threadIdx.x * 4u; t < count; t += blockDim.x * 4u)
-        *reinterpret_cast<float4*>(stage + t) = __ldg(reinterpret_cast<const float4*>(src + t));
+        *reinterpret_cast<float4*>(stage + t) = __ldcg(reinterpret_cast<const float4*>(src + t));
     } else {
 #pragma unroll 4
-      for (uint32_t t = threadIdx.x; t < count; t += blockDim.x) stage[t] = __ldg(src + t);
+      for (uint32_t t = threadIdx.x; t < count; t += blockDim.x) stage[t] = __ldcg(src + t);
     }
   }
   const uint32_t* windows = p.e_max + (p.norm ? o0 : 0u);      // of the rows of this block, or the layer's
@@ -719,12 +719,12 @@ __device__ __forceinline__ void sample_block(const SampleParams& p, uint32_t blo
       const uint4* w4 = reinterpret_cast<const uint4*>(p.w);
 #pragma unroll 8
       for (uint32_t i = threadIdx.x; i < head / 4u; i += kThreads) {
-        const uint4 v = __ldg(w4 + i);
+        const uint4 v = __ldca(w4 + i);
         const uint32_t u4[4] = {v.x, v.y, v.z, v.w};
         best = max_magnitude(u4, best, bad);
       }
       for (uint32_t i = head + threadIdx.x; i < total; i += kThreads) {
-        const uint32_t u1[1] = {__float_as_uint(__ldg(p.w + i))};
+        const uint32_t u1[1] = {__float_as_uint(__ldca(p.w + i))};
         best = max_magnitude(u1, best, bad);
       }
       best = __reduce_max_sync(0xFFFFFFFFu, best);
@@ -783,7 +783,7 @@ struct BatchEntry {
   uint32_t emax_first, emax_blocks, sample_first, sample_blocks;
 };
 
-__device__ __forceinline__ uint32_t find_entry(const BatchEntry* __restrict__ e, uint32_t n, uint32_t block,
+__device__ __forceinline__ uint32_t find_entry(const BatchEntry* e, uint32_t n, uint32_t block,
                                                bool emax) {
   uint32_t lo = 0, hi = n - 1;
   while (lo < hi) {
@@ -794,7 +794,7 @@ __device__ __forceinline__ uint32_t find_entry(const BatchEntry* __restrict__ e,
   return lo;
 }
 
-__global__ void __launch_bounds__(kThreads) emax_batch_kernel(const BatchEntry* __restrict__ entries, uint32_t n,
+__global__ void __launch_bounds__(kThreads) emax_batch_kernel(const BatchEntry* entries, uint32_t n,
                                                               uint32_t* __restrict__ err, uint32_t tag) {
   pdl_prologue();
   const BatchEntry& e = entries[find_entry(entries, n, blockIdx.x, true)];
@@ -803,7 +803,7 @@ __global__ void __launch_bounds__(kThreads) emax_batch_kernel(const BatchEntry* 
 }
 
 template <bool kOptions>
-__global__ void __launch_bounds__(kThreads) sample_batch_kernel(const BatchEntry* __restrict__ entries, uint32_t n,
+__global__ void __launch_bounds__(kThreads) sample_batch_kernel(const BatchEntry* entries, uint32_t n,
                                                                 uint32_t tag, const __grid_constant__ PhiloxKeys keys) {
   pdl_prologue();
   __shared__ __align__(16) float stage[kStage];
@@ -844,7 +844,7 @@ __global__ void expand_planes_kernel(const int8_t* planes, int P, uint32_t O, ui
 }
 
 // Canonical-order copy of one level for the test hook.
-__global__ void export_kernel(const int32_t* __restrict__ wint, int32_t* __restrict__ out, uint32_t O,
+__global__ void export_kernel(const int32_t* wint, int32_t* __restrict__ out, uint32_t O,
                               uint32_t Cg, uint32_t KHKW) {
   pdl_prologue();
   size_t total = (size_t)O * Cg * KHKW;
@@ -1105,8 +1105,8 @@ uint32_t* g_static_scratch_addr[kMaxDevices] = {};   // device address per devic
 // One thread per weight, canonical order in and out (both coalesce).  e_max is
 // the device address of the static scratch, filled by emax_kernel just before.
 __global__ void __launch_bounds__(kThreads)
-sample_level_canonical_kernel(const float* __restrict__ w, uint32_t O, uint32_t d, uint32_t norm,
-                              uint32_t span, uint32_t log2k, uint32_t layer_id, const uint32_t* __restrict__ e_max,
+sample_level_canonical_kernel(const float* w, uint32_t O, uint32_t d, uint32_t norm,
+                              uint32_t span, uint32_t log2k, uint32_t layer_id, const uint32_t* e_max,
                               int32_t* __restrict__ wint_out, int32_t* __restrict__ e_base_out,
                               const __grid_constant__ PhiloxKeys keys) {
   pdl_prologue();
