@@ -1066,9 +1066,11 @@ __device__ __noinline__ bool epilogue_sorted(const TensorParams& p, SharedCtl* c
     auto put = [&](uint32_t at, uint4 q) {
       asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(q.x), "r"(q.y), "r"(q.z), "r"(q.w) : "memory");
     };
-    // the other slot's codes have been stored (a __syncwarp lies between): the next tile's shortcut may come in
+    // Every lane has read the other slot's codes (the barrier orders those reads before the copies): the next tile's
+    // shortcut may come in.
     auto arrive_shortcut = [&]() {
       if (!RES) return;
+      __syncwarp();
       fetch_shortcut((n & 1u) ^ 1u);
       asm volatile("cp.async.wait_group 1;" ::: "memory");       // this tile's
       __syncwarp();
