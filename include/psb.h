@@ -25,9 +25,13 @@
  *     the sorted order of a draw-count map) frees and allocates device
  *     memory, which waits for the device; after one pass over a network's
  *     shapes no call grows anything.  (A context keeps buffers for eight
- *     streams; a ninth takes over those unused longest and waits likewise.)  Otherwise only psb_create, psb_destroy,
- *     the first psb_sample_weights for a handle, psb_weights_free and
- *     psb_device_status may block.
+ *     streams; a ninth takes over those unused longest and waits likewise.)
+ *     Calls on a stream that is being captured have buffers apart from those
+ *     of eager calls: they are allocated beside the capture, wait for nothing
+ *     and stay until psb_destroy, for replays of the graph.  Replays of graphs
+ *     that were captured on one stream must not overlap.
+ *     Otherwise only psb_create, psb_destroy, the first psb_sample_weights for
+ *     a handle, psb_weights_free and psb_device_status may block.
  *   - Every function returns a psb_status: 0 on success, negative on error.
  *     Arguments are validated on the host before anything is launched; a call
  *     that returns an error has launched nothing.  There is no CPU fallback: if

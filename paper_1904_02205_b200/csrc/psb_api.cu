@@ -23,36 +23,87 @@ constexpr uint64_t kRepackMinMacs = 1u << 20;
 
 bool pow2_level_ok(uint32_t log2k) { return log2k < (uint32_t)kMaxLevels; }
 
-// The work buffers of a stream.  A stream not met before takes a free set, or the one unused longest once the device
-// has finished with it.
-ScratchSet& scratch_for(psb_ctx* ctx, cudaStream_t s) {
-  ScratchSet* pick = nullptr;
-  for (ScratchSet& c : ctx->scratch) {
-    if (c.used && c.stream == s) { pick = &c; break; }
-    if (!pick || (pick->used && (!c.used || c.last_use < pick->last_use))) pick = &c;
+// The work buffers of the calls on a stream.  A stream not met before gets a set of its own; the ninth takes over the set
+// unused longest, once the device has finished with it.  Captured calls have sets apart from eager ones, since their graph
+// may run at any time later, and these are never taken over.  (A stream's id cannot be asked for while it is being
+// captured: these sets go by the handle.)
+psb_status scratch_for(psb_ctx* ctx, cudaStream_t s, ScratchSet** out) {
+  unsigned long long key = 0, capture = 0;
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  cudaError_t e = cudaStreamGetCaptureInfo(s, &status, &capture);
+  if (e == cudaSuccess && status == cudaStreamCaptureStatusNone) {
+    capture = 0;
+    e = cudaStreamGetId(s, &key);
+  } else {
+    key = (unsigned long long)(uintptr_t)s;
   }
-  if (!pick->used || pick->stream != s) {
-    if (pick->used) cudaDeviceSynchronize();
-    pick->used = true;
-    pick->stream = s;
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return PSB_ERR_CUDA;
+  }
+  const bool in_graph = status != cudaStreamCaptureStatusNone;
+  ScratchSet *pick = nullptr, *oldest = nullptr;
+  int eager = 0;
+  for (ScratchSet* c = ctx->scratch; c && !pick; c = c->next) {
+    if (c->in_graph == in_graph && c->key == key) pick = c;
+    else if (!c->in_graph) {
+      ++eager;
+      if (!oldest || c->last_use < oldest->last_use) oldest = c;
+    }
+  }
+  if (!pick && !in_graph && eager >= psb_ctx::kScratchStreams) {
+    if (cudaDeviceSynchronize() != cudaSuccess) {
+      cudaGetLastError();
+      return PSB_ERR_CUDA;
+    }
+    pick = oldest;
     pick->sorted_rows = 0;
   }
+  if (!pick) {
+    pick = new (std::nothrow) ScratchSet();
+    if (!pick) return PSB_ERR_ALLOC;
+    pick->in_graph = in_graph;
+    pick->next = ctx->scratch;
+    ctx->scratch = pick;
+  }
+  pick->key = key;
+  if (pick->capture != capture) pick->sorted_rows = 0;      // another capture's order is made by another graph
+  pick->capture = capture;
   pick->last_use = ++ctx->scratch_clock;
-  return *pick;
+  *out = pick;
+  return PSB_OK;
 }
 
-psb_status ensure_scratch(ScratchSet& sc, int slot, size_t bytes) {
+psb_status ensure_scratch(psb_ctx* ctx, ScratchSet& sc, int slot, size_t bytes) {
   if (sc.bytes[slot] >= bytes) return PSB_OK;
-  if (sc.buf[slot]) cudaFree(sc.buf[slot]);
+  if (sc.buf[slot] && sc.in_graph) {
+    KeptBuffer* kept = new (std::nothrow) KeptBuffer{ctx->kept, sc.buf[slot]};
+    if (!kept) return PSB_ERR_ALLOC;
+    ctx->kept = kept;
+  } else if (sc.buf[slot]) {
+    cudaFree(sc.buf[slot]);
+  }
   sc.buf[slot] = nullptr;
   sc.bytes[slot] = 0;
+  if (slot == 2) sc.sorted_rows = 0;     // the order is gone with its buffer
   size_t want = bytes + bytes / 4;
-  if (cudaMalloc(&sc.buf[slot], want) != cudaSuccess) {
+  // an allocation is no operation of the stream: it is made now, beside the capture
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  if (sc.in_graph) cudaThreadExchangeStreamCaptureMode(&mode);
+  const cudaError_t e = cudaMalloc(&sc.buf[slot], want);
+  if (sc.in_graph) cudaThreadExchangeStreamCaptureMode(&mode);
+  if (e != cudaSuccess) {
     cudaGetLastError();
+    sc.buf[slot] = nullptr;
     return PSB_ERR_ALLOC;
   }
   sc.bytes[slot] = want;
   return PSB_OK;
+}
+
+// Whatever was derived from an earlier map is dropped.
+void drop_sorted_orders(psb_ctx* ctx) {
+  for (ScratchSet* sc = ctx->scratch; sc; sc = sc->next) sc->sorted_rows = 0;
 }
 
 psb_status check_epilogue(const psb_epilogue& ep) {
@@ -142,23 +193,30 @@ psb_status run_layer(psb_ctx* ctx, const psb_weights* wt, const void* x_dev, uin
   uint32_t pitch = c;
   if (direct) pitch = sh.kh * sh.kw > 1u || stride > 1u ? round_up(c < wt->bk ? wt->bk : c, 16u) : round_up(c, 16u);
 
-  ScratchSet& sc = scratch_for(ctx, s);
+  ScratchSet* sc = nullptr;      // looked up by the first step that needs a buffer
+  auto scratch = [&](int slot, size_t bytes) -> psb_status {
+    if (!sc) {
+      const psb_status found = scratch_for(ctx, s, &sc);
+      if (found != PSB_OK) return found;
+    }
+    return ensure_scratch(ctx, *sc, slot, bytes);
+  };
   bool range_checked = false;
   if (in_conv) {
-    st = ensure_scratch(sc, 0, (size_t)n * h * w * pitch);
+    st = scratch(0, (size_t)n * h * w * pitch);
     if (st != PSB_OK) return st;
-    if (launch_nchw_to_nhwc(x_dev, sc.buf[0], n, c, h * w, pitch, in_dtype == PSB_DT_S8, amax, ctx->err_dev, s) !=
+    if (launch_nchw_to_nhwc(x_dev, sc->buf[0], n, c, h * w, pitch, in_dtype == PSB_DT_S8, amax, ctx->err_dev, s) !=
         cudaSuccess)
       return PSB_ERR_CUDA;
-    a.x = sc.buf[0];
+    a.x = sc->buf[0];
     range_checked = true;     // the conversion pass has looked at every byte
   } else if (direct && (pitch != c || ((uintptr_t)x_dev & 15u))) {
-    st = ensure_scratch(sc, 0, (size_t)n * h * w * pitch);
+    st = scratch(0, (size_t)n * h * w * pitch);
     if (st != PSB_OK) return st;
-    if (launch_repack_rows(x_dev, sc.buf[0], (size_t)n * h * w, c, pitch, in_dtype == PSB_DT_S8, amax, ctx->err_dev, s) !=
+    if (launch_repack_rows(x_dev, sc->buf[0], (size_t)n * h * w, c, pitch, in_dtype == PSB_DT_S8, amax, ctx->err_dev, s) !=
         cudaSuccess)
       return PSB_ERR_CUDA;
-    a.x = sc.buf[0];
+    a.x = sc->buf[0];
     range_checked = true;
   }
   // in_max is a promise the kernels rely on (bytes above 127 would read as negative on the tensor path):
@@ -177,12 +235,12 @@ psb_status run_layer(psb_ctx* ctx, const psb_weights* wt, const void* x_dev, uin
   if (tensor_ok) {
     if (wt->packed_k) {
       // gather the activation matrix [M][kpad] once, then run the layer as a plain GEMM
-      st = ensure_scratch(sc, 1, (size_t)M * wt->kpad);
+      st = scratch(1, (size_t)M * wt->kpad);
       if (st != PSB_OK) return st;
       const uint32_t offset = in_dtype == PSB_DT_U8 ? 128u : 0u;
-      if (launch_im2col_s8(a, wt->kpad, wt->run_pitch, offset, (int8_t*)sc.buf[1], gather_limit, s) != cudaSuccess)
+      if (launch_im2col_s8(a, wt->kpad, wt->run_pitch, offset, (int8_t*)sc->buf[1], gather_limit, s) != cudaSuccess)
         return PSB_ERR_CUDA;
-      a.x = sc.buf[1];
+      a.x = sc->buf[1];
       a.in_dtype = PSB_DT_S8;
       a.C = wt->kpad;
       a.H = oh; a.W = ow;
@@ -199,24 +257,23 @@ psb_status run_layer(psb_ctx* ctx, const psb_weights* wt, const void* x_dev, uin
       const uint32_t tiles = sorted_tiles_bound(M);
       const size_t ctl_bytes = (sort_ctl_bytes() + 255u) & ~(size_t)255u;
       const size_t perm_bytes = (size_t)tiles * 128u * sizeof(uint32_t);
-      if (sc.bytes[2] < ctl_bytes + perm_bytes + tiles) sc.sorted_rows = 0;    // the buffer moves
-      st = ensure_scratch(sc, 2, ctl_bytes + perm_bytes + tiles);
+      st = scratch(2, ctl_bytes + perm_bytes + tiles);
       if (st != PSB_OK) return st;
-      uint8_t* base = (uint8_t*)sc.buf[2];
+      uint8_t* base = (uint8_t*)sc->buf[2];
       uint32_t* perm = (uint32_t*)(base + ctl_bytes);
       uint8_t* tile_mask = base + ctl_bytes + perm_bytes;
-      if (sc.sorted_map != a.kmap || sc.sorted_rows != (uint32_t)M) {
+      if (sc->sorted_map != a.kmap || sc->sorted_rows != (uint32_t)M) {
         if (launch_level_sort(a.kmap, (uint32_t)M, base, perm, tile_mask, s) != cudaSuccess) return PSB_ERR_CUDA;
-        sc.sorted_map = a.kmap;
-        sc.sorted_rows = (uint32_t)M;
+        sc->sorted_map = a.kmap;
+        sc->sorted_rows = (uint32_t)M;
       }
       // the matrix: K index (kh * KW + kw) * cpad + ci, cpad = channel blocks of the filter's plane layout
       const uint32_t cpad = wt->packed_k ? wt->n_cb * wt->bk : ((a.C + wt->bk - 1) / wt->bk) * wt->bk;
       const size_t row_bytes = (size_t)a.KH * a.KW * cpad;
-      st = ensure_scratch(sc, 3, (size_t)tiles * 128u * row_bytes);
+      st = scratch(3, (size_t)tiles * 128u * row_bytes);
       if (st != PSB_OK) return st;
-      if (launch_gather_sorted(a, perm, base, cpad, (uint8_t*)sc.buf[3], s) != cudaSuccess) return PSB_ERR_CUDA;
-      a.x = sc.buf[3];
+      if (launch_gather_sorted(a, perm, base, cpad, (uint8_t*)sc->buf[3], s) != cudaSuccess) return PSB_ERR_CUDA;
+      a.x = sc->buf[3];
       a.C = (uint32_t)row_bytes;
       a.H = oh; a.W = ow;
       a.KH = 1; a.KW = 1; a.stride = 1; a.pad = 0;
@@ -242,9 +299,9 @@ psb_status run_layer(psb_ctx* ctx, const psb_weights* wt, const void* x_dev, uin
     uint32_t used = 0, n_used = 0;
     for (uint32_t l = 0; l < (uint32_t)kMaxLevels; ++l)
       if (wt->level[l].planes && (a.kmap || l == a.uniform_log2k)) { used |= 1u << l; ++n_used; }
-    st = ensure_scratch(sc, 1, sizeof(int32_t) * words * n_used);
+    st = scratch(1, sizeof(int32_t) * words * n_used);
     if (st != PSB_OK) return st;
-    int32_t* at = (int32_t*)sc.buf[1];
+    int32_t* at = (int32_t*)sc->buf[1];
     for (uint32_t l = 0; l < (uint32_t)kMaxLevels; ++l) {
       if (!((used >> l) & 1u)) continue;
       if (launch_expand(wt, l, false, at, s) != cudaSuccess) return PSB_ERR_CUDA;
@@ -319,9 +376,17 @@ psb_status psb_destroy(psb_ctx* ctx) {
   if (!ctx) return PSB_ERR_INVALID_ARG;
   cudaSetDevice(ctx->device);
   cudaDeviceSynchronize();
-  for (ScratchSet& sc : ctx->scratch)
-    for (void* b : sc.buf)
+  while (ScratchSet* sc = ctx->scratch) {
+    for (void* b : sc->buf)
       if (b) cudaFree(b);
+    ctx->scratch = sc->next;
+    delete sc;
+  }
+  while (KeptBuffer* kept = ctx->kept) {
+    cudaFree(kept->buf);
+    ctx->kept = kept->next;
+    delete kept;
+  }
   if (ctx->err_dev) cudaFree(ctx->err_dev);
   for (int i = 0; i < psb_ctx::kTimedLaunches; ++i) {
     if (ctx->t_begin[i]) cudaEventDestroy(ctx->t_begin[i]);
@@ -496,7 +561,7 @@ psb_status psb_weights_free(psb_ctx* ctx, psb_weights* weights) {
 psb_status psb_set_sample_map(psb_ctx* ctx, const uint8_t* log2k_dev, uint32_t n, uint32_t oh,
                               uint32_t ow, uint32_t uniform_log2k) {
   if (!ctx) return PSB_ERR_INVALID_ARG;
-  for (ScratchSet& sc : ctx->scratch) sc.sorted_rows = 0;      // whatever was derived from an earlier map is dropped
+  drop_sorted_orders(ctx);
   return set_map(ctx, log2k_dev, n, oh, ow, uniform_log2k);
 }
 
@@ -596,7 +661,7 @@ psb_status psb_sample_batch_free(psb_ctx* ctx, psb_sample_batch* batch) {
 
 psb_status psb_run(psb_ctx* ctx, const psb_op* ops, uint32_t n_ops, void* stream) {
   if (!ctx || (!ops && n_ops)) return PSB_ERR_INVALID_ARG;
-  for (ScratchSet& sc : ctx->scratch) sc.sorted_rows = 0;
+  drop_sorted_orders(ctx);
   for (uint32_t i = 0; i < n_ops; ++i) {
     const psb_op& op = ops[i];
     psb_status st;

@@ -83,16 +83,25 @@ struct psb_weights {
 // Work buffers of the calls on one stream: [0] layout conversion, [1] gathered activation matrix, [2] level-sorted
 // order of the current draw-count map (control block, permutation, tile levels), [3] activation rows in that
 // order.  Calls of one stream follow one another, so they share the buffers; calls of different streams may
-// overlap and get their own.
+// overlap and get their own.  Streams are told apart by their unique id: a handle is used again after a stream is
+// destroyed, and cudaStreamPerThread is one handle for a stream per thread.
 struct ScratchSet {
-  cudaStream_t stream = nullptr;
-  bool used = false;
+  ScratchSet* next = nullptr;
+  unsigned long long key = 0;          // of the stream: its id, or of a captured call its handle
   unsigned long long last_use = 0;
+  unsigned long long capture = 0;      // the capture that last used the set, 0 for eager calls
+  bool in_graph = false;               // serves captured calls: the buffers stay until psb_destroy
   void* buf[4] = {nullptr, nullptr, nullptr, nullptr};
   size_t bytes[4] = {0, 0, 0, 0};
   // the sorted order in buf[2] belongs to this map (pointer and dimensions); 0 rows = none
   const uint8_t* sorted_map = nullptr;
   uint32_t sorted_rows = 0;
+};
+
+// A buffer that a captured graph may still name after its set has got a larger one.
+struct KeptBuffer {
+  KeptBuffer* next;
+  void* buf;
 };
 
 struct psb_ctx {
@@ -101,8 +110,9 @@ struct psb_ctx {
   const uint8_t* kmap = nullptr;    // borrowed
   uint32_t map_n = 0, map_oh = 0, map_ow = 0;
   uint32_t uniform_log2k = 0;
-  static constexpr int kScratchStreams = 8;   // streams with buffers of their own; the one unused longest gives way
-  ScratchSet scratch[kScratchStreams];
+  static constexpr int kScratchStreams = 8;   // eager streams with buffers of their own; the one unused longest gives way
+  ScratchSet* scratch = nullptr;
+  KeptBuffer* kept = nullptr;
   unsigned long long scratch_clock = 0;
   int32_t last_path = 0;
   int sm_count = 0;
