@@ -71,7 +71,8 @@ class psb_op(C.Structure):
 PSB_OP_CONV2D, PSB_OP_GEMM, PSB_OP_MAXPOOL, PSB_OP_AVGPOOL = 0, 1, 2, 3
 
 # The argument blocks of the calls that a program makes once per layer, packed in one go: filling the ctypes structures
-# field by field took 3 us of a 10 us call.  Values that do not fit their field go through ctypes, which wraps them.
+# field by field took 3 us of a 10 us call.  Values that do not fit their field go through ctypes, which wraps whole numbers and
+# makes infinities of floats.
 _EP_FMT = "3QfIIfiiI4x3Q"
 _CONV_BLOCK, _GEMM_BLOCK = struct.Struct("=10I" + _EP_FMT), struct.Struct("=5I4x" + _EP_FMT)
 _SHAPE_BLOCK, _CFG_BLOCK = struct.Struct("=5I"), struct.Struct("=Q8I")
@@ -82,7 +83,7 @@ assert _SHAPE_BLOCK.size == C.sizeof(psb_wshape) and _CFG_BLOCK.size == C.sizeof
 def _block(packer, ctype, head, ep=()):
     try:
         return packer.pack(*head, *ep)
-    except struct.error:
+    except (struct.error, OverflowError):
         return bytes(ctype(*head, psb_epilogue(*ep)) if ep else ctype(*head))
 
 _lib = None
