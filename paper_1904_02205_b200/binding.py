@@ -280,7 +280,7 @@ class Context:
         if w.dim() == 2:
             w = w.view(w.shape[0], w.shape[1], 1, 1)
         dims = tuple(w.shape)
-        shape = _block(_SHAPE_BLOCK, psb_wshape, (*dims, groups))
+        shape = _block(_SHAPE_BLOCK, psb_wshape, (dims[0], dims[1], dims[2], dims[3], groups))
         cfg = _block(_CFG_BLOCK, psb_sample_cfg,
                      (seed, layer_id, level_mask, exp_bits, norm, underflow, prob_bits, deterministic, 0))
         h = C.c_void_p(into.handle.value if into is not None else None)

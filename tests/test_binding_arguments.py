@@ -24,3 +24,36 @@ def test_floats_beyond_fp32_become_infinities(inv_step, residual_scale):
     ep, _ = _epilogue(("q",), inv_step, residual_scale)
     head = (B.PSB_DT_U8, 15, 2, 4, 0)
     assert B._block(B._GEMM_BLOCK, B.psb_gemm_desc, head, ep) == bytes(B.psb_gemm_desc(*head, B.psb_epilogue(*ep)))
+
+
+class _Filter:
+    """A stand-in for a CUDA tensor."""
+    is_cuda, dtype = True, torch.float32
+
+    def __init__(self, *shape):
+        self.shape = torch.Size(shape)
+
+    def is_contiguous(self):
+        return True
+
+    def dim(self):
+        return len(self.shape)
+
+    def data_ptr(self):
+        return 256
+
+
+def test_filters_of_more_than_four_dimensions_pass_their_first_four(monkeypatch):
+    seen = []
+
+    def sample(ctx, w, shape, *rest):
+        seen.append(shape)
+        return 0
+
+    monkeypatch.setattr(B, "_stream", lambda s: 0)
+    ctx = SimpleNamespace(handle=None, lib=SimpleNamespace(psb_sample_weights=sample))
+    wt = B.Context.sample_weights(ctx, _Filter(6, 5, 1, 1, 1))
+    assert seen == [bytes(B.psb_wshape(6, 5, 1, 1, 1))] and wt.shape == (6, 5, 1, 1, 1, 1)
+    wt.handle = None
+    with pytest.raises(IndexError):
+        B.Context.sample_weights(ctx, _Filter(6, 5, 3))
