@@ -103,12 +103,18 @@ def load_library():
     lib.psb_status_string.argtypes = [i32]
     lib.psb_status_string.restype = C.c_char_p
     lib.psb_device_status.argtypes = [vp, vp]
-    lib.psb_sample_weights.argtypes = [vp, vp, vp, vp, C.POINTER(vp), vp]    # argument blocks: bytes or byref()
+    lib.psb_sample_weights.argtypes = [vp, vp, C.POINTER(psb_wshape), C.POINTER(psb_sample_cfg), C.POINTER(vp), vp]
     lib.psb_weights_export.argtypes = [vp, vp, u32, vp, vp, vp]
     lib.psb_weights_free.argtypes = [vp, vp]
     lib.psb_set_sample_map.argtypes = [vp, vp, u32, u32, u32, u32]
-    lib.psb_conv2d.argtypes = [vp, vp, vp, vp, vp]
-    lib.psb_gemm.argtypes = [vp, vp, vp, vp, vp]
+    lib.psb_conv2d.argtypes = [vp, vp, vp, C.POINTER(psb_conv_desc), vp]
+    lib.psb_gemm.argtypes = [vp, vp, vp, C.POINTER(psb_gemm_desc), vp]
+    # the same functions for packed argument blocks (bytes)
+    lib.packed_sample_weights, lib.packed_conv2d, lib.packed_gemm = lib["psb_sample_weights"], lib["psb_conv2d"], lib["psb_gemm"]
+    lib.packed_sample_weights.argtypes = [vp, vp, vp, vp, C.POINTER(vp), vp]
+    lib.packed_conv2d.argtypes = lib.packed_gemm.argtypes = [vp, vp, vp, vp, vp]
+    for f in (lib.packed_sample_weights, lib.packed_conv2d, lib.packed_gemm):
+        f.restype = i32
     lib.psb_last_path.argtypes = [vp]
     lib.psb_int8_mma_probe.argtypes = [vp, u32, u32, C.POINTER(C.c_double), C.POINTER(C.c_double), vp]
     lib.psb_contraction_timing.argtypes = [vp, u32]
@@ -284,7 +290,7 @@ class Context:
         cfg = _block(_CFG_BLOCK, psb_sample_cfg,
                      (seed, layer_id, level_mask, exp_bits, norm, underflow, prob_bits, deterministic, 0))
         h = C.c_void_p(into.handle.value if into is not None else None)
-        _check(self.lib.psb_sample_weights(self.handle, w.data_ptr(), shape, cfg, C.byref(h), _stream(stream)),
+        _check(self.lib.packed_sample_weights(self.handle, w.data_ptr(), shape, cfg, C.byref(h), _stream(stream)),
                "psb_sample_weights")
         if into is not None:
             return into
@@ -341,7 +347,7 @@ class Context:
         ep, out = self._epilogue(oshape, scale, bias, relu, inv_step, qmin, qmax, out_dtype, residual,
                                  residual_scale, want, out)
         d = _block(_CONV_BLOCK, psb_conv_desc, (layout, _dt_of(x), in_max, n, c, h, w, stride, pad, path), ep)
-        _check(self.lib.psb_conv2d(self.handle, weights.handle, x.data_ptr(), d, _stream(stream)), "psb_conv2d")
+        _check(self.lib.packed_conv2d(self.handle, weights.handle, x.data_ptr(), d, _stream(stream)), "psb_conv2d")
         return out
 
     def gemm(self, weights, x, scale, bias, relu, inv_step, qmin, qmax, out_dtype=PSB_DT_U8,
@@ -353,7 +359,7 @@ class Context:
         ep, out = self._epilogue((batch, weights.shape[0]), scale, bias, relu, inv_step, qmin, qmax,
                                  out_dtype, residual, residual_scale, want, out)
         d = _block(_GEMM_BLOCK, psb_gemm_desc, (_dt_of(x), in_max, batch, fin, path), ep)
-        _check(self.lib.psb_gemm(self.handle, weights.handle, x.data_ptr(), d, _stream(stream)), "psb_gemm")
+        _check(self.lib.packed_gemm(self.handle, weights.handle, x.data_ptr(), d, _stream(stream)), "psb_gemm")
         return out
 
     # -- attention proposal (Sec. 4.5) -----------------------------------------

@@ -51,9 +51,19 @@ def test_filters_of_more_than_four_dimensions_pass_their_first_four(monkeypatch)
         return 0
 
     monkeypatch.setattr(B, "_stream", lambda s: 0)
-    ctx = SimpleNamespace(handle=None, lib=SimpleNamespace(psb_sample_weights=sample))
+    ctx = SimpleNamespace(handle=None, lib=SimpleNamespace(psb_sample_weights=sample, packed_sample_weights=sample))
     wt = B.Context.sample_weights(ctx, _Filter(6, 5, 1, 1, 1))
     assert seen == [bytes(B.psb_wshape(6, 5, 1, 1, 1))] and wt.shape == (6, 5, 1, 1, 1, 1)
     wt.handle = None
     with pytest.raises(IndexError):
         B.Context.sample_weights(ctx, _Filter(6, 5, 3))
+
+
+def test_the_library_functions_take_argument_structures():
+    """load_library() is public: its functions take the structures of psb.h, by value or by reference."""
+    lib = B.load_library()
+    conv, gemm, shape, cfg = B.psb_conv_desc(), B.psb_gemm_desc(), B.psb_wshape(), B.psb_sample_cfg()
+    for call in (lambda p: lib.psb_conv2d(None, None, None, p(conv), None),
+                 lambda p: lib.psb_gemm(None, None, None, p(gemm), None),
+                 lambda p: lib.psb_sample_weights(None, None, p(shape), p(cfg), None, None)):
+        assert call(lambda s: s) == B.PSB_ERR_INVALID_ARG and call(B.C.byref) == B.PSB_ERR_INVALID_ARG
