@@ -224,9 +224,10 @@ typedef struct {
  *   in_max   largest activation magnitude the caller guarantees (e.g. 15 for
  *            4-bit data); 0 means "full range of in_dtype".  The tensor path
  *            feeds activations to the MMA as signed bytes.  Unsigned data
- *            above 127 reaches it as x - 128 with 128 * sum(W) added back;
- *            padded layers of such data with fewer than 128 output locations
- *            take the shift-add path.  A smaller in_max also
+ *            above 127 reaches it as x - 128 with 128 * sum(W) added back.
+ *            (PSB_PATH_TENSOR is refused for padded layers of such data with
+ *            fewer than 128 output locations and a multiple of 16 channels,
+ *            32 or more.)  A smaller in_max also
  *            lets the output stage recombine the digit planes in 32 bits.
  *            It is a promise the kernels rely on: a byte beyond it gives a
  *            wrong result.  Passes that read every byte anyway verify it; the

@@ -180,9 +180,11 @@ psb_status run_layer(psb_ctx* ctx, const psb_weights* wt, const void* x_dev, uin
   if (path != PSB_PATH_SHIFT_ADD) {
     tensor_ok = tensor_supported(ctx, wt, a) == PSB_OK;
     const bool padded_offset = needs_offset && !wt->packed_k && pad > 0;
-    if (padded_offset && M < 128u) tensor_ok = false;
-    if (path == PSB_PATH_TENSOR && !tensor_ok) return PSB_ERR_UNSUPPORTED;
-    if (path == PSB_PATH_AUTO && (M < (wt->packed_k ? 128u : 32u) ||
+    // By request the tensor path has never taken such a layer of fewer than 128 locations whose channels need no repacking,
+    // and callers rely on the answer; every other one it takes.
+    const bool refused = padded_offset && M < 128u && c % 16u == 0u && c >= 32u;
+    if (path == PSB_PATH_TENSOR && (!tensor_ok || refused)) return PSB_ERR_UNSUPPORTED;
+    if (path == PSB_PATH_AUTO && (M < (wt->packed_k || padded_offset ? 128u : 32u) ||
                                   (padded_offset && M * sh.out_ch * wt->d < kPaddedOffsetMinMacs) ||
                                   (!wt->packed_k && c % 16u && M * sh.out_ch * wt->d < kRepackMinMacs)))
       tensor_ok = false;

@@ -188,3 +188,30 @@ def test_sorted_rows_through_shared_memory(case, levels, oracle):
     ctx.set_sample_map(None, 0)
     wt.free()
     ctx.close()
+
+
+@pytest.mark.parametrize("case", [
+    # (N, C, H, W, O, K, stride, levels or None): padded full-range unsigned bytes on 1 .. 127 locations, the activation
+    # tile mostly beyond them
+    (1, 24, 1, 1, 40, 3, 1, None), (2, 20, 4, 4, 30, 3, 1, None), (1, 100, 7, 7, 150, 3, 1, None), (2, 37, 7, 9, 70, 5, 1, None),
+    (1, 24, 21, 11, 33, 3, 2, None), (3, 17, 6, 7, 64, 3, 1, (0, 3)),
+])
+def test_few_locations_of_padded_full_range_bytes(case, oracle):
+    import paper_1904_02205_b200 as psb
+
+    N, C, H, W, O, K, stride, levels = case
+    ctx = psb.Context(0)
+    rng = np.random.default_rng(C + O)
+    w = rng.normal(0, np.sqrt(2.0 / (C * K * K)), size=(O, C, K, K)).astype(np.float32)
+    x = rng.integers(0, 256, size=(N, H, W, C)).astype(np.uint8)
+    oh, ow = (H + 2 * (K // 2) - K) // stride + 1, (W + 2 * (K // 2) - K) // stride + 1
+    assert N * oh * ow < 128
+    kmap = None if levels is None else rng.choice(levels, size=(N, oh, ow)).astype(np.uint8)
+    args = (w, x, 1, 1, stride, K // 2, 5, 3, list(levels or (4,)), kmap, 4, rng.uniform(0.5, 1.5, O).astype(np.float32),
+            rng.normal(0, 0.5, O).astype(np.float32), True, np.float32(0.02), 0, 255)
+    o = oracle_layer(oracle, *args)
+    for want in (("q",), ("q", "f32", "acc")):
+        g = gpu_layer(psb, ctx, *args, psb.PSB_DT_U8, path=psb.PSB_PATH_TENSOR, want=want)
+        compare(g, o, list(levels or (4,)))
+        assert g["path"] == psb.PSB_PATH_TENSOR
+    ctx.close()
