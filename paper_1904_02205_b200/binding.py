@@ -165,8 +165,7 @@ def _stream(stream):
 
 
 _TORCH_DT = {PSB_DT_U8: torch.uint8, PSB_DT_S8: torch.int8}
-_OUT_DT = {"f32": torch.float32, "acc": torch.int64}     # the codes ("q") have the type the caller asks for
-_OUT_KINDS = ("q", "f32", "acc")
+_OUT_DT = {"f32": torch.float32, "acc": torch.int64}
 
 
 def _dt_of(t):
@@ -322,9 +321,12 @@ class Context:
     def _epilogue(self, out_shape, scale, bias, relu, inv_step, qmin, qmax, out_dtype, residual,
                   residual_scale, want, out):
         out = dict(out) if out else {}
-        for kind in _OUT_KINDS:
-            if kind in want and kind not in out:      # `want` may also be one text, such as "f32" or "q+f32"
-                out[kind] = torch.empty(out_shape, dtype=_OUT_DT.get(kind) or _TORCH_DT[out_dtype], device=self.device)
+        # `want` may also be one text, such as "f32" or "q+f32"
+        for kind in want if type(want) is not str else [k for k in ("q", "f32", "acc") if k in want]:
+            if kind not in out:
+                dt = _TORCH_DT[out_dtype] if kind == "q" else _OUT_DT.get(kind)
+                if dt is not None:
+                    out[kind] = torch.empty(out_shape, dtype=dt, device=self.device)
         q, f32, acc = out.get("q"), out.get("f32"), out.get("acc")
         ep = (scale.data_ptr(), bias.data_ptr(), 0 if residual is None else residual.data_ptr(), float(residual_scale),
               PSB_DT_U8 if residual is None else _dt_of(residual), int(relu), float(inv_step), qmin, qmax, out_dtype,
