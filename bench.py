@@ -268,10 +268,10 @@ class FcWorkload:
         self.q_host.copy_(self.out["q"], non_blocking=True)
 
     def roofline(self, kernel_ms, peaks):
-        # one launch, a warp per output: neither bytes (35 KB) nor arithmetic matter, the launch does
+        # one launch, 16 lanes per output channel and four rows: neither bytes (35 KB) nor arithmetic matter, the launch does
         nbytes = self.images * 256 + 128 * 256 * 4 + self.images * 128
         achieved = nbytes / (kernel_ms * 1e-3) / 1e9
-        return dict(bound="hbm", kernel="gemv_planes_kernel (latency-bound: one warp per output)",
+        return dict(bound="hbm", kernel="dense_planes_kernel (latency-bound: 16 lanes per output channel)",
                     achieved=achieved, peak=peaks["hbm_gbs"], unit="GB/s", frac=achieved / peaks["hbm_gbs"],
                     traffic=None, peak_source=peaks["source"], kernel_ms=kernel_ms)
 

@@ -288,29 +288,13 @@ psb_status run_layer(psb_ctx* ctx, const psb_weights* wt, const void* x_dev, uin
     ctx->last_path = PSB_PATH_TENSOR;
     return PSB_OK;
   }
+  if (wt->has_planes) {
+    if (launch_dense_planes(a, wt, s) != cudaSuccess) return PSB_ERR_CUDA;
+    ctx->last_path = PSB_PATH_SHIFT_ADD;
+    return PSB_OK;
+  }
   WintTable tab;
   for (int l = 0; l < kMaxLevels; ++l) tab.w[l] = wt->level[l].wint;
-  if (wt->has_planes) {
-    if (gemv_planes_ok(a, wt)) {
-      if (launch_gemv_planes(a, wt, s) != cudaSuccess) return PSB_ERR_CUDA;
-      ctx->last_path = PSB_PATH_SHIFT_ADD;
-      return PSB_OK;
-    }
-    // the direct kernels read 32-bit weights: put them together from the digit planes
-    const size_t words = (size_t)sh.out_ch * wt->d;
-    uint32_t used = 0, n_used = 0;
-    for (uint32_t l = 0; l < (uint32_t)kMaxLevels; ++l)
-      if (wt->level[l].planes && (a.kmap || l == a.uniform_log2k)) { used |= 1u << l; ++n_used; }
-    st = scratch(1, sizeof(int32_t) * words * n_used);
-    if (st != PSB_OK) return st;
-    int32_t* at = (int32_t*)sc->buf[1];
-    for (uint32_t l = 0; l < (uint32_t)kMaxLevels; ++l) {
-      if (!((used >> l) & 1u)) continue;
-      if (launch_expand(wt, l, false, at, s) != cudaSuccess) return PSB_ERR_CUDA;
-      tab.w[l] = at;
-      at += words;
-    }
-  }
   if (launch_shift_add(a, tab, wt->rowsum256, amax, s) != cudaSuccess) return PSB_ERR_CUDA;
   ctx->last_path = PSB_PATH_SHIFT_ADD;
   return PSB_OK;

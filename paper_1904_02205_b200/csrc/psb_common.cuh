@@ -239,16 +239,13 @@ cudaError_t launch_export(const psb_weights* wt, uint32_t level, int32_t* wint_o
 // rowsum256: [level][O] row sums of |W_k| / 256 kept by the sampler; amax: largest activation magnitude
 cudaError_t launch_shift_add(const ConvArgs& a, const WintTable& wt, const uint32_t* rowsum256, uint32_t amax,
                              cudaStream_t s);
-// matrix products with few rows (rows of activations contiguous: FC layers, 1x1 filters) from the digit planes
-bool gemv_planes_ok(const ConvArgs& a, const psb_weights* wt);
-cudaError_t launch_gemv_planes(const ConvArgs& a, const psb_weights* wt, cudaStream_t s);
+// dense layers on CUDA cores from the digit planes
+cudaError_t launch_dense_planes(const ConvArgs& a, const psb_weights* wt, cudaStream_t s);
 // gathers [M][kpad] signed bytes (x - offset; zero padding becomes -offset, K padding 0); row kh of the
 // filter window occupies bytes [kh * run_pitch, kh * run_pitch + kw * c) of a matrix row
 size_t im2col_s8_smem(const ConvArgs& a, uint32_t run_pitch);   // shared memory the gather kernel needs
 cudaError_t launch_im2col_s8(const ConvArgs& a, uint32_t kpad, uint32_t run_pitch, uint32_t offset, int8_t* dst,
                              uint32_t limit, cudaStream_t s);
-// the integer filter of one level from its digit planes, canonical order or channels innermost
-cudaError_t launch_expand(const psb_weights* wt, uint32_t level, bool canonical, int32_t* out, cudaStream_t s);
 // [rows][C] -> [rows][pitch] bytes, zero beyond C.  `limit`: largest byte magnitude allowed (255 for unsigned / 128
 // for signed data = no check); a byte beyond it raises kDevErrRange in *err
 cudaError_t launch_repack_rows(const void* src, void* dst, size_t rows, uint32_t C, uint32_t pitch, uint32_t is_signed,

@@ -820,20 +820,16 @@ __global__ void __launch_bounds__(kThreads) sample_batch_kernel(const BatchEntry
   sample_block<kOptions, false>(p, blockIdx.x - first, keys, stage, rs, nullptr);
 }
 
-// The integer filter of one level put together from its digit planes, in canonical order or channels innermost: the
-// export hook, and the CUDA-core kernels when they are asked to run a filter that has planes.
+// The integer filter of one level put together from its digit planes, in canonical order, for the test hook.
 __global__ void expand_planes_kernel(const int8_t* planes, int P, uint32_t O, uint32_t Cg, uint32_t KHKW, uint32_t bk,
                                      uint32_t n_cb, uint32_t n_kb, uint32_t packed_kw, uint32_t run_pitch,
-                                     uint32_t canonical, int32_t* __restrict__ out) {
+                                     int32_t* __restrict__ out) {
   pdl_prologue();
   const size_t total = (size_t)O * Cg * KHKW;
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-    const uint32_t inner = canonical ? KHKW : Cg;
-    const uint32_t a = (uint32_t)(i % inner);
-    const size_t rest = i / inner;
-    const uint32_t outer = canonical ? Cg : KHKW;
-    const uint32_t b = (uint32_t)(rest % outer), o = (uint32_t)(rest / outer);
-    const uint32_t tap = canonical ? a : b, ci = canonical ? b : a;
+    const uint32_t tap = (uint32_t)(i % KHKW);
+    const size_t rest = i / KHKW;
+    const uint32_t ci = (uint32_t)(rest % Cg), o = (uint32_t)(rest / Cg);
     uint32_t kcol = tap * n_cb * bk + ci;
     if (packed_kw) kcol = (tap / packed_kw) * run_pitch + (tap % packed_kw) * Cg + ci;
     const int8_t* tile = planes + ((size_t)(o / kTileN) * n_kb + kcol / bk) * (size_t)P * kTileN * bk;
@@ -936,17 +932,6 @@ uint32_t fill_sample_params(const float* w_dev, const psb_weights* wt, uint32_t*
 }
 
 }  // namespace
-
-cudaError_t launch_expand(const psb_weights* wt, uint32_t level, bool canonical, int32_t* out, cudaStream_t s) {
-  const psb_wshape& sh = wt->shape;
-  const size_t total = (size_t)sh.out_ch * wt->d;
-  const uint32_t blocks = (uint32_t)std::min<size_t>((total + kThreads - 1) / kThreads, 148u * 16u);
-  launch_pdl(expand_planes_kernel, blocks, kThreads, 0, s, (const int8_t*)wt->level[level].planes, wt->level[level].planes_count,
-             sh.out_ch, sh.in_ch_per_group, sh.kh * sh.kw, wt->bk, wt->n_cb, wt->n_kb, wt->packed_k ? sh.kw : 0u, wt->run_pitch,
-             canonical ? 1u : 0u, out);
-  note_launch();
-  return cudaGetLastError();
-}
 
 cudaError_t launch_sampler(const float* w_dev, psb_weights* wt, uint32_t* err_dev, cudaStream_t s) {
   const PhiloxKeys keys((uint32_t)wt->cfg.seed, (uint32_t)(wt->cfg.seed >> 32));
@@ -1064,8 +1049,12 @@ cudaError_t launch_export(const psb_weights* wt, uint32_t level, int32_t* wint_o
                           int32_t* e_base_out, cudaStream_t s) {
   const psb_wshape& sh = wt->shape;
   if (wint_out && wt->has_planes) {
-    const cudaError_t e = launch_expand(wt, level, true, wint_out, s);
-    if (e != cudaSuccess) return e;
+    const size_t total = (size_t)sh.out_ch * wt->d;
+    const uint32_t blocks = (uint32_t)std::min<size_t>((total + kThreads - 1) / kThreads, 148u * 16u);
+    launch_pdl(expand_planes_kernel, blocks, kThreads, 0, s, (const int8_t*)wt->level[level].planes, wt->level[level].planes_count,
+               sh.out_ch, sh.in_ch_per_group, sh.kh * sh.kw, wt->bk, wt->n_cb, wt->n_kb, wt->packed_k ? sh.kw : 0u, wt->run_pitch,
+               wint_out);
+    note_launch();
   } else if (wint_out) {
     size_t total = (size_t)sh.out_ch * wt->d;
     uint32_t blocks = (uint32_t)((total + 255) / 256);

@@ -2,11 +2,12 @@
 //
 // The paper's capacitor unit adds x << (e + B) over the draws (Eq. 9); summed over
 // the k draws that is x * (k + c_k) << (e - e_base), an integer product with the
-// sampled integer weight.  On the GPU one 64-bit integer multiply-add per
-// (activation, weight) pair realises exactly that sum.  This path serves layers
-// that are not dense matrix products for the tensor cores: depthwise filters,
-// fully connected layers at small batch, very few input channels, 8-bit unsigned
-// activations, and it honours per-location draw counts directly.
+// sampled integer weight.  Depthwise and grouped filters hold that weight; dense
+// ones hold its signed digit planes, whose byte products are summed plane by
+// plane.  This path serves layers that are not dense matrix products for the
+// tensor cores (depthwise filters) or too small for them (fully connected layers
+// at small batch, filters on a few locations), and it honours per-location draw
+// counts directly.
 #include "psb_common.cuh"
 
 #include <algorithm>
@@ -90,96 +91,163 @@ __device__ __forceinline__ int dp4a_act(uint32_t x, uint32_t w, int acc) {
   return d;
 }
 
-// Matrix products with few rows (fully connected layers at small batch, 1x1 filters on a few locations), straight from
-// the digit planes: a group of lanes per output channel, each lane 16 input features at a time (one 16-byte load per
-// plane, four dp4a per plane and activation row), kNB activation rows per pass over the weights; a plane's sum stays
-// in 32 bits (gemv_planes_ok), the planes meet in 64 bits and the lanes in a shuffle tree.  The activation rows of the
-// block sit in shared memory, kGemvFeatures at a time, padded with zeros to whole K blocks.  Bound by the latency of
-// its few loads; P bytes per weight are read instead of the 4 of an integer filter.
-constexpr int kGemvRows = 4;
-constexpr uint32_t kGemvFeatures = 8192;      // kGemvRows rows of them take 32 KB
+// Dense layers on CUDA cores (fully connected layers at small batch, filters with and without taps on a few locations),
+// straight from the digit planes: a group of lanes per output channel, each lane 16 bytes of the K axis at a time (one
+// 16-byte load per plane, four dp4a per plane and location), kNB output locations per pass over the weights; a plane's sum
+// stays in 32 bits over one segment of the axis, the planes and segments meet in 64 bits and the lanes in a shuffle tree.
+// The patches of the block's locations sit in shared memory in the order of the planes' K axis, kPlaneSegment bytes at a
+// time, zero outside the image and beyond the channels.  Bound by the latency of its few loads; P bytes per weight are
+// read instead of the 4 of an integer filter.  (One thread per output on an integer filter, which has to be put together
+// from the planes first, took 698 us for 3x3 512 -> 512 on 9 locations, 44 us for 32 -> 32 on 49; this kernel 11.0 and 8.7,
+// the latter in a stream of calls that the host bounds.)
+constexpr int kPlaneLocations = 4;
+constexpr uint32_t kPlaneSegment = 8192;      // kPlaneLocations patches of them take 32 KB
+// Blocks per SM.  More registers than three or two of them leave (loads of four pieces in flight) help a single wave: 3x3 512 -> 512 on 9 locations 11.0 us, with three blocks 15.2.
+constexpr int kPlainBlocks = 3, kTapBlocks = 2;
 
-struct GemvPlanes {
+// (Kept small: with 304 bytes of parameters instead of 280 a launch took 0.35 us longer on the host.)
+struct DensePlanes {
   const int8_t* p[kMaxLevels];
-  int count[kMaxLevels];
+  uint8_t count[kMaxLevels + 1];
   uint32_t bk, n_kb;
+  uint32_t tap_pieces;     // 16-byte pieces of the K axis per tap (channels rounded up to whole K blocks); flat K axis: 0
+  uint32_t run_pitch;      // flat K axis: bytes per filter row
+  float per_tap, per_kw;   // 1 / tap_pieces, 1 / KW
 };
 
-template <int kNB, bool kSignedIn>
-__global__ void __launch_bounds__(256) gemv_planes_kernel(const ConvArgs a, const GemvPlanes w, uint32_t M,
-                                                          uint32_t lanes_per_row) {
-  pdl_prologue();
-  extern __shared__ __align__(16) uint8_t gemv_x[];     // [kNB][min(kp, kGemvFeatures)]
-  const uint32_t bk = w.bk, kp = w.n_kb * bk, C = a.C, seg = min(kp, kGemvFeatures);
-  const uint32_t n0 = blockIdx.y * (uint32_t)kNB, nb = min((uint32_t)kNB, M - n0);
-  const uint8_t* x = (const uint8_t*)a.x + (size_t)n0 * C;
-  const bool vec = C % 16u == 0u && ((uintptr_t)x & 15u) == 0u;
-  const uint32_t sub = threadIdx.x & (lanes_per_row - 1u);
-  const uint32_t o = blockIdx.x * (blockDim.x / lanes_per_row) + threadIdx.x / lanes_per_row;
-  const uint32_t level = a.kmap ? a.kmap[n0] : a.uniform_log2k;      // with a map kNB is 1
-  const bool level_ok = level < (uint32_t)kMaxLevels && ((a.level_mask >> level) & 1u);
-  if (!level_ok && threadIdx.x == 0) atomicOr(a.err, kDevErrBadLevel);
-  int acc[kMaxPlanes][kNB];
+// 16 bytes of the patch of one output location from K-axis byte k on; iy0, ix0: its first tap in image `img`.  kPlain:
+// a filter of one tap without stride and padding, `img` is the location itself.
+template <bool kPlain>
+__device__ __forceinline__ uint4 patch_piece(const ConvArgs& a, const DensePlanes& w, const uint8_t* img, int iy0, int ix0,
+                                             uint32_t k, uint32_t unit) {
+  uint32_t b[4] = {0u, 0u, 0u, 0u};
+  if (kPlain || w.tap_pieces) {
+    uint32_t ci = k;
+    const uint8_t* src = img + k;
+    if (!kPlain) {
+      // quotients of numbers below 2^22 (pieces) and 2^11 (taps) in fp32, the first one put right where it is one off
+      const uint32_t piece = k / 16u;
+      uint32_t tap = __float2uint_rz((float)piece * w.per_tap);
+      if (tap * w.tap_pieces > piece) --tap;
+      else if ((tap + 1u) * w.tap_pieces <= piece) ++tap;
+      const uint32_t kh = __float2uint_rz(((float)tap + 0.5f) * w.per_kw);
+      const int iy = iy0 + (int)kh, ix = ix0 + (int)(tap - kh * a.KW);
+      if ((unsigned)iy >= a.H || (unsigned)ix >= a.W) return make_uint4(0u, 0u, 0u, 0u);
+      ci = (piece - tap * w.tap_pieces) * 16u;
+      src = img + ((size_t)iy * a.W + (uint32_t)ix) * a.C + ci;
+    }
+    if (ci >= a.C) return make_uint4(0u, 0u, 0u, 0u);
+    if (unit == 16u) return __ldcg(reinterpret_cast<const uint4*>(src));
+    if (unit == 4u) {
 #pragma unroll
-  for (int pl = 0; pl < kMaxPlanes; ++pl)
+      for (int j = 0; j < 4; ++j)
+        if (ci + 4u * j < a.C) b[j] = __ldcg(reinterpret_cast<const uint32_t*>(src + 4 * j));
+    } else {
 #pragma unroll
-    for (int r = 0; r < kNB; ++r) acc[pl][r] = 0;
-  for (uint32_t k0 = 0; k0 < kp; k0 += seg) {
-    const uint32_t len = min(seg, kp - k0);
-    if (k0) __syncthreads();
-    for (uint32_t r = 0; r < (uint32_t)kNB; ++r)
-      for (uint32_t i = threadIdx.x * 16u; i < len; i += blockDim.x * 16u) {
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        if (r < nb && k0 + i < C) {
-          const uint8_t* src = x + (size_t)r * C + k0 + i;
-          if (vec) {
-            v = __ldcg(reinterpret_cast<const uint4*>(src));
-          } else {
-            uint32_t b[4] = {0u, 0u, 0u, 0u};
+      for (int j = 0; j < 16; ++j)
+        if (ci + j < a.C) b[j >> 2] |= (uint32_t)src[j] << (8 * (j & 3));
+    }
+  } else {
+    uint32_t kh = k / w.run_pitch, at = k - kh * w.run_pitch, kw = at / a.C, ci = at - kw * a.C;
 #pragma unroll
-            for (int j = 0; j < 16; ++j)
-              if (k0 + i + j < C) b[j >> 2] |= (uint32_t)src[j] << (8 * (j & 3));
-            v = make_uint4(b[0], b[1], b[2], b[3]);
-          }
-        }
-        *reinterpret_cast<uint4*>(gemv_x + r * seg + i) = v;
-      }
-    __syncthreads();
-    if (!level_ok || o >= a.O) continue;
-    const int P = w.count[level];
-    const uint32_t shift = 31u - (uint32_t)__clz((int)bk), on = o % kTileN, chunks = len / 16u;
-    const size_t tile_bytes = (size_t)P * kTileN * bk;
-    const int8_t* base = w.p[level] + (size_t)(o / kTileN) * w.n_kb * tile_bytes;
-#pragma unroll 4
-    for (uint32_t c = sub; c < chunks; c += lanes_per_row) {
-      const uint32_t k = k0 + c * 16u, off = plane_offset(on, k & (bk - 1u), bk);
-      const int8_t* tile = base + (size_t)(k >> shift) * tile_bytes + off;
-      uint4 d[kMaxPlanes];
-#pragma unroll
-      for (int pl = 0; pl < kMaxPlanes; ++pl)
-        if (pl < P) d[pl] = __ldcg(reinterpret_cast<const uint4*>(tile + (size_t)pl * kTileN * bk));
-#pragma unroll
-      for (int r = 0; r < kNB; ++r) {
-        const uint4 v = *reinterpret_cast<const uint4*>(gemv_x + (uint32_t)r * seg + c * 16u);
-#pragma unroll
-        for (int pl = 0; pl < kMaxPlanes; ++pl)
-          if (pl < P) {
-            acc[pl][r] = dp4a_act<kSignedIn>(v.x, d[pl].x, acc[pl][r]);
-            acc[pl][r] = dp4a_act<kSignedIn>(v.y, d[pl].y, acc[pl][r]);
-            acc[pl][r] = dp4a_act<kSignedIn>(v.z, d[pl].z, acc[pl][r]);
-            acc[pl][r] = dp4a_act<kSignedIn>(v.w, d[pl].w, acc[pl][r]);
-          }
-      }
+    for (int j = 0; j < 16; ++j) {
+      const int iy = iy0 + (int)kh, ix = ix0 + (int)kw;
+      if (kh < a.KH && kw < a.KW && (unsigned)iy < a.H && (unsigned)ix < a.W)
+        b[j >> 2] |= (uint32_t)img[((size_t)iy * a.W + (uint32_t)ix) * a.C + ci] << (8 * (j & 3));
+      if (++ci == a.C) { ci = 0u; ++kw; }
+      if (++at == w.run_pitch) { at = kw = ci = 0u; ++kh; }
     }
   }
+  return make_uint4(b[0], b[1], b[2], b[3]);
+}
+
+template <int kNB, bool kSignedIn, bool kPlain>
+__global__ void __launch_bounds__(256, kPlain ? kPlainBlocks : kTapBlocks) dense_planes_kernel(const __grid_constant__ ConvArgs a,
+                                                           const __grid_constant__ DensePlanes w, uint32_t M,
+                                                           uint32_t lanes_per_row) {
+  pdl_prologue();
+  extern __shared__ __align__(16) uint8_t patches[];     // [kNB][min(kp, kPlaneSegment)]
+  const uint32_t bk = w.bk, kp = w.n_kb * bk, seg = min(kp, kPlaneSegment), ohow = a.OH * a.OW;
+  const uint32_t align = a.C | (uint32_t)(uintptr_t)a.x;
+  const uint32_t unit = (align & 15u) == 0u ? 16u : (align & 3u) == 0u ? 4u : 1u;
+  const uint32_t sub = threadIdx.x & (lanes_per_row - 1u);
+  const uint32_t o = blockIdx.x * (blockDim.x / lanes_per_row) + threadIdx.x / lanes_per_row;
+  for (uint32_t n0 = blockIdx.y * (uint32_t)kNB; n0 < M; n0 += gridDim.y * (uint32_t)kNB) {
+    const uint32_t nb = min((uint32_t)kNB, M - n0);
+    const uint8_t* img[kNB];
+    int iy0[kNB], ix0[kNB];
 #pragma unroll
-  for (int r = 0; r < kNB; ++r) {
-    long long sum = acc[0][r];
+    for (int r = 0; r < kNB; ++r) {
+      const uint32_t m = n0 + min((uint32_t)r, nb - 1u);
+      iy0[r] = ix0[r] = 0;
+      if (kPlain) {
+        img[r] = (const uint8_t*)a.x + (size_t)m * a.C;
+        continue;
+      }
+      const uint32_t n = m / ohow, pix = m - n * ohow, oy = pix / a.OW;
+      img[r] = (const uint8_t*)a.x + (size_t)n * a.H * a.W * a.C;
+      iy0[r] = (int)(oy * a.stride) - (int)a.pad;
+      ix0[r] = (int)((pix - oy * a.OW) * a.stride) - (int)a.pad;
+    }
+    const uint32_t level = a.kmap ? a.kmap[n0] : a.uniform_log2k;      // with a map kNB is 1
+    const bool level_ok = level < (uint32_t)kMaxLevels && ((a.level_mask >> level) & 1u);
+    if (!level_ok && threadIdx.x == 0) atomicOr(a.err, kDevErrBadLevel);
+    long long sum[kNB];
 #pragma unroll
-    for (int pl = 1; pl < kMaxPlanes; ++pl) sum += (long long)acc[pl][r] * (1ll << (kDigitBits * pl));
-    for (uint32_t d = lanes_per_row / 2u; d > 0; d >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, d);
-    if (level_ok && o < a.O && (uint32_t)r < nb && sub == ((uint32_t)r & (lanes_per_row - 1u)))
-      store_outputs(a, (size_t)(n0 + r) * a.O + o, o, level, sum);
+    for (int r = 0; r < kNB; ++r) sum[r] = 0;
+    for (uint32_t k0 = 0; k0 < kp; k0 += seg) {
+      const uint32_t len = min(seg, kp - k0), chunks = len / 16u;
+      __syncthreads();                                     // the patches of the step before have been read
+#pragma unroll
+      for (int r = 0; r < kNB; ++r)
+        for (uint32_t i = threadIdx.x * 16u; i < len; i += blockDim.x * 16u)
+          *reinterpret_cast<uint4*>(patches + r * seg + i) = patch_piece<kPlain>(a, w, img[r], iy0[r], ix0[r], k0 + i, unit);
+      __syncthreads();
+      if (!level_ok || o >= a.O) continue;
+      const int P = w.count[level];
+      const uint32_t shift = 31u - (uint32_t)__clz((int)bk), on = o % kTileN;
+      const size_t tile_bytes = (size_t)P * kTileN * bk;
+      const int8_t* base = w.p[level] + (size_t)(o / kTileN) * w.n_kb * tile_bytes;
+      int acc[kMaxPlanes][kNB];
+#pragma unroll
+      for (int pl = 0; pl < kMaxPlanes; ++pl)
+#pragma unroll
+        for (int r = 0; r < kNB; ++r) acc[pl][r] = 0;
+#pragma unroll 4
+      for (uint32_t c = sub; c < chunks; c += lanes_per_row) {
+        const uint32_t k = k0 + c * 16u, off = plane_offset(on, k & (bk - 1u), bk);
+        const int8_t* tile = base + (size_t)(k >> shift) * tile_bytes + off;
+        uint4 d[kMaxPlanes];
+#pragma unroll
+        for (int pl = 0; pl < kMaxPlanes; ++pl)
+          if (pl < P) d[pl] = __ldcg(reinterpret_cast<const uint4*>(tile + (size_t)pl * kTileN * bk));
+#pragma unroll
+        for (int r = 0; r < kNB; ++r) {
+          const uint4 v = *reinterpret_cast<const uint4*>(patches + (uint32_t)r * seg + c * 16u);
+#pragma unroll
+          for (int pl = 0; pl < kMaxPlanes; ++pl)
+            if (pl < P) {
+              acc[pl][r] = dp4a_act<kSignedIn>(v.x, d[pl].x, acc[pl][r]);
+              acc[pl][r] = dp4a_act<kSignedIn>(v.y, d[pl].y, acc[pl][r]);
+              acc[pl][r] = dp4a_act<kSignedIn>(v.z, d[pl].z, acc[pl][r]);
+              acc[pl][r] = dp4a_act<kSignedIn>(v.w, d[pl].w, acc[pl][r]);
+            }
+        }
+      }
+      // a lane's sum over a segment is at most 8192 * 255 * 127 < 2^28
+#pragma unroll
+      for (int r = 0; r < kNB; ++r)
+#pragma unroll
+        for (int pl = 0; pl < kMaxPlanes; ++pl) sum[r] += (long long)acc[pl][r] * (1ll << (kDigitBits * pl));
+    }
+#pragma unroll
+    for (int r = 0; r < kNB; ++r) {
+      for (uint32_t d = lanes_per_row / 2u; d > 0; d >>= 1) sum[r] += __shfl_xor_sync(0xFFFFFFFFu, sum[r], d);
+      if (!level_ok || o >= a.O || (uint32_t)r >= nb || sub != ((uint32_t)r & (lanes_per_row - 1u))) continue;
+      const uint32_t m = n0 + (uint32_t)r, n = m / ohow;
+      const size_t at = a.out_nchw ? ((size_t)n * a.O + o) * ohow + (m - n * ohow) : (size_t)m * a.O + o;
+      store_outputs(a, at, o, level, sum[r]);
+    }
   }
 }
 
@@ -910,37 +978,51 @@ cudaError_t launch_shift_add(const ConvArgs& a, const WintTable& wt, const uint3
   return cudaGetLastError();
 }
 
-// Rows of the product: locations of a 1x1 filter with stride 1 on channels-last data.  A plane's sum of one lane: at most
-// 2^20 / lanes * 255 * 127 < 2^31 (filters of 512 features and more have 32 lanes per output).
-bool gemv_planes_ok(const ConvArgs& a, const psb_weights* wt) {
-  const uint64_t M = (uint64_t)a.N * a.OH * a.OW;
-  return a.KH == 1u && a.KW == 1u && a.stride == 1u && a.pad == 0u && !a.out_nchw && !wt->packed_k &&
-         wt->n_kb * wt->bk <= (1u << 20) && M * a.O < (1u << 24) &&
-         (a.kmap ? M : (M + kGemvRows - 1u) / kGemvRows) <= 65535u;
+namespace {
+struct DenseGrid {
+  uint32_t lanes;      // per output channel
+  bool one;            // one location per block row, not kPlaneLocations
+  bool plain;          // one tap, no stride, no padding
+  uint32_t x, y;
+};
+DenseGrid dense_grid(const ConvArgs& a, const psb_weights* wt) {
+  DenseGrid g;
+  const uint32_t kp = wt->n_kb * wt->bk, M = a.N * a.OH * a.OW;
+  g.lanes = 1;
+  while (g.lanes < 32u && g.lanes * 16u < kp) g.lanes *= 2u;
+  g.one = a.kmap || M == 1u;
+  g.plain = !wt->packed_k && a.KH * a.KW == 1u && a.stride == 1u && a.pad == 0u;
+  g.x = (a.O + 256u / g.lanes - 1u) / (256u / g.lanes);
+  g.y = g.one ? M : (M + kPlaneLocations - 1u) / kPlaneLocations;
+  return g;
 }
+}  // namespace
 
-cudaError_t launch_gemv_planes(const ConvArgs& a, const psb_weights* wt, cudaStream_t s) {
-  GemvPlanes w;
+cudaError_t launch_dense_planes(const ConvArgs& a, const psb_weights* wt, cudaStream_t s) {
+  DensePlanes w;
   for (int l = 0; l < kMaxLevels; ++l) {
     w.p[l] = wt->level[l].planes;
-    w.count[l] = wt->level[l].planes_count;
+    w.count[l] = (uint8_t)wt->level[l].planes_count;
   }
   w.bk = wt->bk;
   w.n_kb = wt->n_kb;
+  w.tap_pieces = wt->packed_k ? 0u : wt->n_cb * wt->bk / 16u;
+  w.run_pitch = wt->run_pitch;
+  w.per_tap = w.tap_pieces ? 1.0f / (float)w.tap_pieces : 0.0f;
+  w.per_kw = 1.0f / (float)a.KW;
+  const DenseGrid g = dense_grid(a, wt);
   const uint32_t kp = w.n_kb * w.bk, M = a.N * a.OH * a.OW;
-  uint32_t lanes = 1;
-  while (lanes < 32u && lanes * 16u < kp) lanes *= 2u;
-  const bool one = a.kmap || M == 1u;
-  const dim3 grid((a.O + 256u / lanes - 1u) / (256u / lanes), one ? M : (M + kGemvRows - 1u) / kGemvRows);
-  const size_t smem = (size_t)(one ? 1 : kGemvRows) * (kp < kGemvFeatures ? kp : kGemvFeatures);
+  const dim3 grid(g.x, g.y < 65535u ? g.y : 65535u);
+  const size_t smem = (size_t)(g.one ? 1 : kPlaneLocations) * (kp < kPlaneSegment ? kp : kPlaneSegment);
   const bool sg = a.in_dtype == PSB_DT_S8;
-  if (one) {
-    if (sg) launch_pdl(gemv_planes_kernel<1, true>, grid, dim3(256), smem, s, a, w, M, lanes);
-    else launch_pdl(gemv_planes_kernel<1, false>, grid, dim3(256), smem, s, a, w, M, lanes);
-  } else {
-    if (sg) launch_pdl(gemv_planes_kernel<kGemvRows, true>, grid, dim3(256), smem, s, a, w, M, lanes);
-    else launch_pdl(gemv_planes_kernel<kGemvRows, false>, grid, dim3(256), smem, s, a, w, M, lanes);
-  }
+#define PSB_DP(NB, SG, PL) launch_pdl(dense_planes_kernel<NB, SG, PL>, grid, dim3(256), smem, s, a, w, M, g.lanes)
+#define PSB_DP_SG(NB, PL) do { if (sg) PSB_DP(NB, true, PL); else PSB_DP(NB, false, PL); } while (0)
+  if (g.one && g.plain) PSB_DP_SG(1, true);
+  else if (g.one) PSB_DP_SG(1, false);
+  else if (g.plain) PSB_DP_SG(kPlaneLocations, true);
+  else PSB_DP_SG(kPlaneLocations, false);
+#undef PSB_DP_SG
+#undef PSB_DP
   note_launch();
   return cudaGetLastError();
 }

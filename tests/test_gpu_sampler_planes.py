@@ -60,3 +60,59 @@ def test_one_level_under_options_alone_and_in_a_batch(opts, log2k, oracle):
     for h in handles:
         h.free()
     ctx.close()
+
+
+@pytest.mark.parametrize("case", [
+    # (N, C, H, W, O, K, stride, layout, levels, signed input): flat and tap-major K axes, patches in pieces of 1, 4 and 16
+    # bytes, one segment of the axis and two, locations that are no multiple of the block's four
+    (1, 3, 9, 7, 17, 5, 2, 0, (3,), False), (2, 7, 4, 5, 40, 3, 1, 1, (0,), True), (1, 17, 5, 5, 70, 3, 1, 1, (6,), False),
+    (3, 36, 3, 4, 33, 3, 2, 0, (4,), True), (1, 64, 7, 7, 130, 5, 1, 1, (2,), False), (1, 1000, 2, 3, 9, 3, 1, 1, (3,), False),
+    (2, 24, 6, 5, 20, 3, 1, 0, (0, 2, 4), False), (1, 4, 8, 8, 12, 7, 3, 1, (1, 5), True), (1, 48, 1, 1, 64, 1, 1, 1, (3,), False),
+    (1, 16, 30, 31, 8, 3, 1, 1, (3,), False),
+])
+def test_filters_with_taps_from_the_digit_planes(case, oracle):
+    import paper_1904_02205_b200 as psb
+
+    N, C, H, W, O, K, stride, layout, levels, signed = case
+    ctx = psb.Context(0)
+    rng = np.random.default_rng(C * 5 + O)
+    w = rng.normal(0, np.sqrt(2.0 / (C * K * K)), size=(O, C, K, K)).astype(np.float32)
+    lo, hi, dt = (-128, 128, np.int8) if signed else (0, 256, np.uint8)
+    x = rng.integers(lo, hi, size=(N, C, H, W) if layout == 0 else (N, H, W, C)).astype(dt)
+    oh, ow = (H + 2 * (K // 2) - K) // stride + 1, (W + 2 * (K // 2) - K) // stride + 1
+    res = rng.integers(0, 256, size=(N, O, oh, ow) if layout == 0 else (N, oh, ow, O)).astype(np.uint8)
+    kmap = rng.choice(levels, size=(N, oh, ow)).astype(np.uint8) if len(levels) > 1 else None
+    args = (w, x, layout, 1, stride, K // 2, 5, 3, list(levels), kmap, levels[0], rng.uniform(0.5, 1.5, O).astype(np.float32),
+            rng.normal(0, 0.5, O).astype(np.float32), True, np.float32(0.02), 0, 255)
+    o = oracle_layer(oracle, *args, residual=res, res_scale=np.float32(0.3))
+    before = ctx.launch_count()
+    g = gpu_layer(psb, ctx, *args, psb.PSB_DT_U8, residual=res, res_scale=np.float32(0.3), path=psb.PSB_PATH_SHIFT_ADD)
+    compare(g, o, list(levels))
+    # sampling, one export per level, one launch for the layer and one for a planar input: nothing is put together first
+    planar = 1 if layout == 0 and C > 1 and H * W > 1 else 0
+    assert ctx.launch_count() - before <= 2 + len(levels) + 1 + planar
+    ctx.close()
+
+
+def test_few_locations_at_odd_addresses(oracle):
+    import torch
+
+    import paper_1904_02205_b200 as psb
+
+    ctx = psb.Context(0)
+    rng = np.random.default_rng(3)
+    w = rng.normal(0, 0.1, size=(32, 48, 3, 3)).astype(np.float32)
+    x = rng.integers(0, 256, size=(1, 4, 5, 48)).astype(np.uint8)
+    wt = ctx.sample_weights(torch.from_numpy(w).to(ctx.device), seed=1, level_mask=8)
+    ctx.set_sample_map(None, 3)
+    one = torch.ones(32, device=ctx.device)
+    W = {3: oracle.sample_level(w, 1, 0, 3)[0]}
+    acc = oracle.conv_acc(x, oracle.geom(x.shape, oracle.NHWC, oracle.U8, w.shape, 1, 1, 1), W, uniform_log2k=3)
+    flat = torch.zeros(x.size + 16, dtype=torch.uint8, device=ctx.device)
+    for shift in (0, 1, 4, 6):
+        flat[shift:shift + x.size] = torch.from_numpy(x.ravel()).to(ctx.device)
+        got = ctx.conv2d(wt, flat[shift:shift + x.size].view(x.shape), 1, 1, 1, one, one, False, 1.0, 0, 255,
+                         path=psb.PSB_PATH_SHIFT_ADD, want=("acc",))["acc"].cpu().numpy()
+        assert ctx.device_status() == 0 and np.array_equal(got, acc)
+    wt.free()
+    ctx.close()
