@@ -11,15 +11,31 @@ using namespace psb;
 
 namespace {
 
-// Lines between the CUDA-core and the tensor path under PSB_PATH_AUTO, in multiply-accumulates of the call.
-// Padded layers of full-range unsigned bytes: the calls of the tensor path take 15-18 us in a stream of such calls
-// whatever the size, conv_direct_kernel 118 us at 10.6 M, 264 us at 19 M (3x3, 64 -> 64 channels) but 34 us at 11 M
-// with 40 output channels: the line stands where the tensor path has won for every shape measured.
-constexpr uint64_t kPaddedOffsetMinMacs = 16u << 20;
-// Layers whose activation rows have to be repacked first (one launch more): a fully connected layer of 333 features,
-// batch 37, 13 outputs (0.16 M) took 27.5 us with its sampling on CUDA cores, 30.5 us on the tensor path; a 1x1 layer of
-// 52 channels (3.6 M) 25.6 and 22.6 us.
-constexpr uint64_t kRepackMinMacs = 1u << 20;
+// The line between the CUDA-core and the tensor path for dense layers under PSB_PATH_AUTO.  The tensor path takes a
+// layer of any few locations in about the same time (4 to 6 us on the device for short K axes, 640 clocks per K block for
+// long ones), and a launch more where the activation rows are repacked or gathered first.  The CUDA-core kernel takes 4 to
+// 11 us as long as all its blocks run at once, a multiple of it when they do not.  us per call in a stream of calls, CUDA
+// cores / tensor path:
+//   no launch more:  3x3 512->512, 16 locations (256 blocks) 11.0 / 15.3, 25 locations (448) 19.4 / 15.3; 4096->1000 features,
+//                    12 rows (375) 10.4 / 13.3, 16 rows (500) 15.7 / 13.3; 1024->1024, 12 rows (384) 8.7 / 9.2, 31 rows
+//                    (1024) 14.8 / 9.4.  From 32 locations on the tensor path: 3x3 32->32, 196 locations 8.6 / 8.8, on the
+//                    device 6.1 / 4.5, and the device is what counts inside a list of operations.
+//   repacked rows:   3x3 100->150, 49 locations (247) 8.6 / 12.3, 98 locations (475) 14.3 / 12.4; 1x1 52->60, 784 locations
+//                    (196) 8.7 / 12.2; on the device 7.9 / 10.0 and 5.0 / 7.3.
+//   flat K axis:     3x3 8->64, 121 locations 8.7 / 12.1, on the device 8.3 / 7.4; 5x5 12->128, 49 locations (208) 9.2 / 12.3,
+//                    100 locations (400) 17 / 12.
+//   Padded full-range bytes whose channels need no repacking stay on CUDA cores for up to two rounds of blocks: callers rely
+//   on the path of such layers of ten million multiply-accumulates (3x3 64->64, 288 locations: 576 blocks, 12.1 us on the
+//   device, 7.5 on the tensor path; it was 118 with one thread per output).
+bool prefers_cuda_cores(const ConvArgs& a, const psb_weights* wt, bool repacked, bool padded_offset, int sm_count) {
+  const uint64_t M = (uint64_t)a.N * a.OH * a.OW;
+  const bool few = M < (wt->packed_k ? 128u : 32u);
+  const uint32_t rounds = dense_planes_rounds(a, wt, sm_count);
+  const bool at_once = rounds <= 1u;
+  if (a.kmap) return few || at_once;      // a map costs up to four launches more on the tensor path, on CUDA cores none
+  if (padded_offset && !repacked) return rounds <= 2u;
+  return repacked ? at_once : few && at_once;
+}
 
 bool pow2_level_ok(uint32_t log2k) { return log2k < (uint32_t)kMaxLevels; }
 
@@ -176,24 +192,23 @@ psb_status run_layer(psb_ctx* ctx, const psb_weights* wt, const void* x_dev, uin
   // The MMA takes signed bytes.  Unsigned data above 127 is fed as x - 128 (top bit flipped, by the gather or in
   // shared memory) and corrected by 128 * sum(W).
   const bool needs_offset = in_dtype == PSB_DT_U8 && amax > 127u;
+  // Channel pitch of the matrix the copy engine reads: its rows must be 16-byte multiples, and with taps as wide as
+  // a K block.
+  uint32_t pitch = c;
+  if (!wt->packed_k) pitch = sh.kh * sh.kw > 1u || stride > 1u ? round_up(c < wt->bk ? wt->bk : c, 16u) : round_up(c, 16u);
+  const bool repack = !wt->packed_k && !in_conv && (pitch != c || ((uintptr_t)x_dev & 15u));
   bool tensor_ok = false;
   if (path != PSB_PATH_SHIFT_ADD) {
     tensor_ok = tensor_supported(ctx, wt, a) == PSB_OK;
+    // By request the tensor path has never taken padded data of this range on fewer than 128 locations where the channels
+    // need no repacking, and callers rely on the answer; every other layer it takes.
     const bool padded_offset = needs_offset && !wt->packed_k && pad > 0;
-    // By request the tensor path has never taken such a layer of fewer than 128 locations whose channels need no repacking,
-    // and callers rely on the answer; every other one it takes.
     const bool refused = padded_offset && M < 128u && c % 16u == 0u && c >= 32u;
     if (path == PSB_PATH_TENSOR && (!tensor_ok || refused)) return PSB_ERR_UNSUPPORTED;
-    if (path == PSB_PATH_AUTO && (M < (wt->packed_k || padded_offset ? 128u : 32u) ||
-                                  (padded_offset && M * sh.out_ch * wt->d < kPaddedOffsetMinMacs) ||
-                                  (!wt->packed_k && c % 16u && M * sh.out_ch * wt->d < kRepackMinMacs)))
-      tensor_ok = false;
+    if (path == PSB_PATH_AUTO && tensor_ok && prefers_cuda_cores(a, wt, repack, padded_offset, ctx->sm_count)) tensor_ok = false;
   }
-  // Channel pitch of the matrix the copy engine reads: its rows must be 16-byte multiples, and with taps as wide as
-  // a K block.
   const bool direct = tensor_ok && !wt->packed_k;
-  uint32_t pitch = c;
-  if (direct) pitch = sh.kh * sh.kw > 1u || stride > 1u ? round_up(c < wt->bk ? wt->bk : c, 16u) : round_up(c, 16u);
+  if (!direct) pitch = c;
 
   ScratchSet* sc = nullptr;      // looked up by the first step that needs a buffer
   auto scratch = [&](int slot, size_t bytes) -> psb_status {
@@ -212,7 +227,7 @@ psb_status run_layer(psb_ctx* ctx, const psb_weights* wt, const void* x_dev, uin
       return PSB_ERR_CUDA;
     a.x = sc->buf[0];
     range_checked = true;     // the conversion pass has looked at every byte
-  } else if (direct && (pitch != c || ((uintptr_t)x_dev & 15u))) {
+  } else if (direct && repack) {
     st = scratch(0, (size_t)n * h * w * pitch);
     if (st != PSB_OK) return st;
     if (launch_repack_rows(x_dev, sc->buf[0], (size_t)n * h * w, c, pitch, in_dtype == PSB_DT_S8, amax, ctx->err_dev, s) !=

@@ -239,7 +239,9 @@ cudaError_t launch_export(const psb_weights* wt, uint32_t level, int32_t* wint_o
 // rowsum256: [level][O] row sums of |W_k| / 256 kept by the sampler; amax: largest activation magnitude
 cudaError_t launch_shift_add(const ConvArgs& a, const WintTable& wt, const uint32_t* rowsum256, uint32_t amax,
                              cudaStream_t s);
-// dense layers on CUDA cores from the digit planes
+// dense layers on CUDA cores from the digit planes; rounds: how often the launch fills the machine (one pass over the filter
+// counts as one)
+uint32_t dense_planes_rounds(const ConvArgs& a, const psb_weights* wt, int sm_count);
 cudaError_t launch_dense_planes(const ConvArgs& a, const psb_weights* wt, cudaStream_t s);
 // gathers [M][kpad] signed bytes (x - offset; zero padding becomes -offset, K padding 0); row kh of the
 // filter window occupies bytes [kh * run_pitch, kh * run_pitch + kw * c) of a matrix row

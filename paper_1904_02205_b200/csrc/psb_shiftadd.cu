@@ -102,7 +102,8 @@ __device__ __forceinline__ int dp4a_act(uint32_t x, uint32_t w, int acc) {
 // the latter in a stream of calls that the host bounds.)
 constexpr int kPlaneLocations = 4;
 constexpr uint32_t kPlaneSegment = 8192;      // kPlaneLocations patches of them take 32 KB
-// Blocks per SM.  More registers than three or two of them leave (loads of four pieces in flight) help a single wave: 3x3 512 -> 512 on 9 locations 11.0 us, with three blocks 15.2.
+// Blocks per SM.  More registers than three or two of them leave (loads of four pieces in flight) help a single wave, which
+// is what PSB_PATH_AUTO sends here: 3x3 512 -> 512 on 9 locations 11.0 us, with three blocks 15.2.
 constexpr int kPlainBlocks = 3, kTapBlocks = 2;
 
 // (Kept small: with 304 bytes of parameters instead of 280 a launch took 0.35 us longer on the host.)
@@ -997,6 +998,12 @@ DenseGrid dense_grid(const ConvArgs& a, const psb_weights* wt) {
   return g;
 }
 }  // namespace
+
+uint32_t dense_planes_rounds(const ConvArgs& a, const psb_weights* wt, int sm_count) {
+  const DenseGrid g = dense_grid(a, wt);
+  const uint64_t slots = (uint64_t)sm_count * (g.plain ? kPlainBlocks : kTapBlocks);
+  return g.y == 1u ? 1u : (uint32_t)(((uint64_t)g.x * g.y + slots - 1u) / slots);
+}
 
 cudaError_t launch_dense_planes(const ConvArgs& a, const psb_weights* wt, cudaStream_t s) {
   DensePlanes w;

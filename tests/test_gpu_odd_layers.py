@@ -215,3 +215,28 @@ def test_few_locations_of_padded_full_range_bytes(case, oracle):
         compare(g, o, list(levels or (4,)))
         assert g["path"] == psb.PSB_PATH_TENSOR
     ctx.close()
+
+
+@pytest.mark.parametrize("case", [
+    # (N, C, H, W, O, K, largest magnitude, levels or None, tensor path): both sides of the line that PSB_PATH_AUTO draws
+    (1, 64, 20, 15, 64, 3, 255, None, True), (1, 64, 20, 14, 64, 3, 255, None, False), (2, 256, 7, 7, 256, 3, 255, None, True),
+    (1, 32, 4, 7, 32, 3, 255, None, False), (1, 100, 7, 7, 150, 3, 255, None, False), (1, 100, 8, 8, 150, 3, 255, None, True),
+    (31, 512, 1, 1, 2048, 1, 15, None, True), (4, 512, 1, 1, 2048, 1, 15, None, False), (10, 52, 14, 14, 60, 1, 15, None, True),
+    (1, 12, 10, 10, 128, 5, 255, None, True), (1, 12, 7, 7, 128, 5, 255, None, False), (1, 48, 6, 6, 16, 3, 255, (0, 3), False),
+    (1, 48, 12, 12, 64, 3, 255, (0, 3), True),
+])
+def test_line_between_the_paths(case, oracle):
+    import paper_1904_02205_b200 as psb
+
+    N, C, H, W, O, K, top, levels, tensor = case
+    ctx = psb.Context(0)
+    rng = np.random.default_rng(C + O + H)
+    w = rng.normal(0, np.sqrt(2.0 / (C * K * K)), size=(O, C, K, K)).astype(np.float32)
+    x = rng.integers(0, top + 1, size=(N, H, W, C)).astype(np.uint8)
+    kmap = None if levels is None else rng.choice(levels, size=(N, H, W)).astype(np.uint8)
+    args = (w, x, 1, 1, 1, K // 2, 5, 3, list(levels or (3,)), kmap, 3, rng.uniform(0.5, 1.5, O).astype(np.float32),
+            rng.normal(0, 0.5, O).astype(np.float32), True, np.float32(0.02), 0, 255)
+    g = gpu_layer(psb, ctx, *args, psb.PSB_DT_U8, in_max=top, want=("q", "acc"))
+    compare(g, oracle_layer(oracle, *args), list(levels or (3,)))
+    assert g["path"] == (psb.PSB_PATH_TENSOR if tensor else psb.PSB_PATH_SHIFT_ADD)
+    ctx.close()
