@@ -177,18 +177,14 @@ __global__ void __launch_bounds__(256, kPlain ? kPlainBlocks : kTapBlocks) dense
     const uint32_t nb = min((uint32_t)kNB, M - n0);
     const uint8_t* img[kNB];
     int iy0[kNB], ix0[kNB];
+    if (!kPlain) {
 #pragma unroll
-    for (int r = 0; r < kNB; ++r) {
-      const uint32_t m = n0 + min((uint32_t)r, nb - 1u);
-      iy0[r] = ix0[r] = 0;
-      if (kPlain) {
-        img[r] = (const uint8_t*)a.x + (size_t)m * a.C;
-        continue;
+      for (int r = 0; r < kNB; ++r) {
+        const uint32_t m = n0 + min((uint32_t)r, nb - 1u), n = m / ohow, pix = m - n * ohow, oy = pix / a.OW;
+        img[r] = (const uint8_t*)a.x + (size_t)n * a.H * a.W * a.C;
+        iy0[r] = (int)(oy * a.stride) - (int)a.pad;
+        ix0[r] = (int)((pix - oy * a.OW) * a.stride) - (int)a.pad;
       }
-      const uint32_t n = m / ohow, pix = m - n * ohow, oy = pix / a.OW;
-      img[r] = (const uint8_t*)a.x + (size_t)n * a.H * a.W * a.C;
-      iy0[r] = (int)(oy * a.stride) - (int)a.pad;
-      ix0[r] = (int)((pix - oy * a.OW) * a.stride) - (int)a.pad;
     }
     const uint32_t level = a.kmap ? a.kmap[n0] : a.uniform_log2k;      // with a map kNB is 1
     const bool level_ok = level < (uint32_t)kMaxLevels && ((a.level_mask >> level) & 1u);
@@ -198,11 +194,26 @@ __global__ void __launch_bounds__(256, kPlain ? kPlainBlocks : kTapBlocks) dense
     for (int r = 0; r < kNB; ++r) sum[r] = 0;
     for (uint32_t k0 = 0; k0 < kp; k0 += seg) {
       const uint32_t len = min(seg, kp - k0), chunks = len / 16u;
-      __syncthreads();                                     // the patches of the step before have been read
+      if (k0 || n0 != blockIdx.y * (uint32_t)kNB) __syncthreads();      // the patches of the step before have been read
+      if (kPlain && kNB > 1) {
+        // the pieces of all rows dealt out to the threads: one load per thread for up to 1024 features, and one copy of the
+        // code (row by row: 64 -> 10 features, 17 rows 3.9 us on the device, 3.4 so; 1024 -> 1024, 12 rows 6.2 and 5.6)
+        for (uint32_t i = threadIdx.x; i < nb * chunks; i += blockDim.x) {
+          uint32_t r = 0;
 #pragma unroll
-      for (int r = 0; r < kNB; ++r)
-        for (uint32_t i = threadIdx.x * 16u; i < len; i += blockDim.x * 16u)
-          *reinterpret_cast<uint4*>(patches + r * seg + i) = patch_piece<kPlain>(a, w, img[r], iy0[r], ix0[r], k0 + i, unit);
+          for (int q = 1; q < kNB; ++q) r += i >= (uint32_t)q * chunks ? 1u : 0u;
+          const uint32_t k = (i - r * chunks) * 16u;
+          *reinterpret_cast<uint4*>(patches + r * seg + k) =
+              patch_piece<true>(a, w, (const uint8_t*)a.x + (size_t)(n0 + r) * a.C, 0, 0, k0 + k, unit);
+        }
+      } else {
+#pragma unroll
+        for (int r = 0; r < kNB; ++r) {
+          const uint8_t* from = kPlain ? (const uint8_t*)a.x + (size_t)n0 * a.C : img[r];
+          for (uint32_t i = threadIdx.x * 16u; i < len; i += blockDim.x * 16u)
+            *reinterpret_cast<uint4*>(patches + r * seg + i) = patch_piece<kPlain>(a, w, from, iy0[r], ix0[r], k0 + i, unit);
+        }
+      }
       __syncthreads();
       if (!level_ok || o >= a.O) continue;
       const int P = w.count[level];
