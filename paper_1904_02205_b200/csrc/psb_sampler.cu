@@ -931,6 +931,14 @@ uint32_t fill_sample_params(const float* w_dev, const psb_weights* wt, uint32_t*
   return row_blocks * p.ch_chunks;
 }
 
+// A captured call carries one number through all its replays, which the words of later calls would beat: its graph clears
+// them each time.
+bool is_captured(cudaStream_t s) {
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &status) != cudaSuccess) cudaGetLastError();
+  return status == cudaStreamCaptureStatusActive;
+}
+
 }  // namespace
 
 cudaError_t launch_sampler(const float* w_dev, psb_weights* wt, uint32_t* err_dev, cudaStream_t s) {
@@ -947,10 +955,10 @@ cudaError_t launch_sampler(const float* w_dev, psb_weights* wt, uint32_t* err_de
   // the exponent maxima carry the number of the call that wrote them; the words were cleared when
   // the handle was made and are cleared again only when the 24-bit call number wraps
   wt->e_calls = (wt->e_calls + 1u) & 0xFFFFFFu;
-  if (wt->e_calls == 0u) {
+  if (wt->e_calls == 0u || is_captured(s)) {
     cudaError_t e = cudaMemsetAsync(wt->e_max, 0, sizeof(uint32_t) * O, s);
     if (e != cudaSuccess) return e;
-    wt->e_calls = 1u;
+    if (wt->e_calls == 0u) wt->e_calls = 1u;
   }
   launch_pdl(emax_kernel, emax_blocks_for(O, wt->d, wt->cfg.norm), kThreads, 0, s, w_dev, O, wt->d, wt->cfg.norm,
              wt->e_max, err_dev, wt->e_calls << 8, wt->rowsum256, wt->corr128, wt->cfg.prob_bits); note_launch();
@@ -1024,9 +1032,9 @@ psb_status sample_batch_create(psb_ctx* ctx, uint32_t n, const float* const* w_d
 
 psb_status sample_batch_run(psb_ctx* ctx, psb_sample_batch* b, uint64_t seed, cudaStream_t s) {
   b->calls = (b->calls + 1u) & 0xFFFFFFu;
-  if (b->calls == 0u) {       // the words of earlier calls would compare as later ones
+  if (b->calls == 0u || is_captured(s)) {       // the words of earlier calls would compare as later ones
     if (cudaMemsetAsync(b->e_max_pool, 0, sizeof(uint32_t) * b->e_max_words, s) != cudaSuccess) return PSB_ERR_CUDA;
-    b->calls = 1u;
+    if (b->calls == 0u) b->calls = 1u;
   }
   launch_pdl(emax_batch_kernel, b->emax_grid, kThreads, 0, s, (const BatchEntry*)b->entries_dev, b->n, ctx->err_dev, b->calls);
   note_launch();

@@ -135,3 +135,47 @@ def test_capture_on_a_stream_not_met_before():
     a.free()
     big.free()
     ctx.close()
+
+
+def test_captured_sampling_replayed_after_later_calls():
+    """One window per layer, in a graph that samples a handle and a batch twice each: replays, with eager calls between them,
+    give the filters of the seeds that were captured."""
+    import torch
+
+    import paper_1904_02205_b200 as psb
+
+    ctx = psb.Context(0)
+    rng = np.random.default_rng(5)
+    w = [torch.from_numpy(rng.normal(0, 0.1, size=s).astype(np.float32)).to(ctx.device)
+         for s in ((64, 64, 3, 3), (72, 40, 3, 3), (33, 300, 1, 1))]
+    alone = ctx.sample_weights(w[0], seed=1, level_mask=8)
+    kept = [ctx.sample_weights(a, seed=1, layer_id=i, level_mask=8) for i, a in enumerate(w)]
+    batch = ctx.sample_batch_create(w, kept)
+
+    def calls(seeds):
+        for seed in seeds:
+            ctx.sample_weights(w[0], seed=seed, level_mask=8, into=alone)
+            ctx.sample_batch_run(batch, seed)
+
+    def filters():
+        torch.cuda.synchronize()
+        return [ctx.weights_export(h, 3)[0].cpu().numpy() for h in [alone] + kept]
+
+    calls([3])
+    ref = filters()
+    assert all(r.any() for r in ref)
+    g = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(g, stream=torch.cuda.Stream()):
+        calls([2, 3])
+    for eager in ([], [], [4, 5]):
+        calls(eager)
+        torch.cuda.synchronize()
+        g.replay()
+        assert _same(filters(), ref)
+    assert ctx.device_status() == 0
+    del g
+    ctx.sample_batch_free(batch)
+    for h in [alone] + kept:
+        h.free()
+    ctx.close()
