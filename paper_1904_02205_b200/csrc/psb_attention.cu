@@ -93,7 +93,7 @@ __global__ void __launch_bounds__(256) attention_maps_kernel(const float* entrop
 cudaError_t launch_entropy(const void* act, uint32_t is_signed, uint32_t locations, uint32_t C, float step,
                            float* entropy, cudaStream_t s) {
   uint32_t blocks = (locations + 7u) / 8u;
-  if (blocks > 148u * 8u) blocks = 148u * 8u;
+  if (blocks > kSms * 8u) blocks = kSms * 8u;
   if (blocks < 1u) blocks = 1u;
   launch_pdl(entropy_kernel, blocks, 256, 0, s, (const uint8_t*)act, is_signed, locations, C, step, entropy);
   note_launch();

@@ -12,6 +12,7 @@ constexpr int kMaxLevels = 7;        // k = 1, 2, 4, ..., 64
 constexpr int kDigitBits = 7;        // magnitude bits per signed digit plane
 constexpr int kTileN = 64;           // output channels per tensor-path tile
 constexpr int kMaxPlanes = 4;
+constexpr uint32_t kSms = 148;       // of a B200: grids of the streaming kernels are sized by it
 
 // Bits of the device error word.
 constexpr uint32_t kDevErrNonFinite = 1u;

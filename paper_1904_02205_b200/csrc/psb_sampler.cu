@@ -5,8 +5,8 @@
 //   draw k Bernoulli(p) bits from Philox4x32-10         the comparator of the
 //                                                       stochastic multiplier
 //   count the upper draws among the first k, every k    Eq. 8 (binomial count)
-//   emit W_k = s (k + c_k) 2^(e - e_base) as int32 and as signed 7-bit digit
-//   planes in the layout the tensor path loads with TMA.
+//   emit W_k = s (k + c_k) 2^(e - e_base) as signed 7-bit digit planes in the
+//   layout the contraction kernels read (dense filters), or as int32 (others).
 // The random bits never leave registers.
 #include <new>
 
@@ -1058,7 +1058,7 @@ cudaError_t launch_export(const psb_weights* wt, uint32_t level, int32_t* wint_o
   const psb_wshape& sh = wt->shape;
   if (wint_out && wt->has_planes) {
     const size_t total = (size_t)sh.out_ch * wt->d;
-    const uint32_t blocks = (uint32_t)std::min<size_t>((total + kThreads - 1) / kThreads, 148u * 16u);
+    const uint32_t blocks = (uint32_t)std::min<size_t>((total + kThreads - 1) / kThreads, kSms * 16u);
     launch_pdl(expand_planes_kernel, blocks, kThreads, 0, s, (const int8_t*)wt->level[level].planes, wt->level[level].planes_count,
                sh.out_ch, sh.in_ch_per_group, sh.kh * sh.kw, wt->bk, wt->n_cb, wt->n_kb, wt->packed_k ? sh.kw : 0u, wt->run_pitch,
                wint_out);
@@ -1186,7 +1186,7 @@ extern "C" psb_status psb_sample_level_static(const float* w_dev, const psb_wsha
   }
   size_t total = (size_t)O * d;
   uint32_t blocks = (uint32_t)((total + kThreads - 1) / kThreads);
-  blocks = blocks > 148u * 16u ? 148u * 16u : blocks;
+  blocks = blocks > kSms * 16u ? kSms * 16u : blocks;
   sample_level_canonical_kernel<<<blocks, kThreads, 0, s>>>(
       w_dev, O, d, cfg->norm, (1u << exp_bits) - 1u, log2k, cfg->layer_id, e_max, wint_out_dev, e_base_out_dev,
       PhiloxKeys((uint32_t)cfg->seed, (uint32_t)(cfg->seed >> 32))); note_launch();

@@ -377,7 +377,6 @@ __global__ void __launch_bounds__(128, 5) dwconv3x3_kernel(const ConvArgs a, con
   const uint32_t strip = t % strips, n = t / strips;
   const uint32_t ox0 = seg * kDwCols, oy0 = strip * rows_per_thread, oy1 = min(oy0 + rows_per_thread, a.OH);
   const uint32_t level = a.uniform_log2k;
-  // (a sum marked unknown, 0xFFFFFFFF, fails the test like a large one)
   bool fits = true;
   for (uint32_t j = 0; j < left; ++j)
     fits = fits && (unsigned long long)__ldca(rowsum256 + (size_t)level * a.O + c0 + j) * 256ull * amax < (1ull << 31);
@@ -913,7 +912,7 @@ __global__ void avgpool_kernel(const uint8_t* x, uint32_t nchw, uint32_t N, uint
 uint32_t grid_for(size_t total, uint32_t threads) {
   size_t b = (total + threads - 1) / threads;
   if (b < 1) b = 1;
-  if (b > 148u * 32u) b = 148u * 32u;
+  if (b > kSms * 32u) b = kSms * 32u;
   return (uint32_t)b;
 }
 
@@ -930,7 +929,7 @@ cudaError_t launch_repack_rows(const void* src, void* dst, size_t rows, uint32_t
 cudaError_t launch_range_check(const void* x, size_t bytes, uint32_t is_signed, uint32_t limit, uint32_t* err,
                                cudaStream_t s) {
   uint32_t blocks = grid_for(bytes / 16 + 1, 256);
-  if (blocks > 148u * 8u) blocks = 148u * 8u;
+  if (blocks > kSms * 8u) blocks = kSms * 8u;
   launch_pdl(range_check_kernel, blocks, 256, 0, s, (const uint8_t*)x, bytes, is_signed, limit, err);
   note_launch();
   return cudaGetLastError();
@@ -949,7 +948,7 @@ cudaError_t launch_shift_add(const ConvArgs& a, const WintTable& wt, const uint3
     uint64_t best = ~0ull;
     for (uint32_t strips = 1; strips <= 32u && strips <= a.OH; ++strips) {
       const uint32_t r = (a.OH + strips - 1) / strips;
-      const uint64_t waves = (columns * ((a.OH + r - 1) / r) + 5ull * 148 * 128 - 1) / (5ull * 148 * 128);
+      const uint64_t waves = (columns * ((a.OH + r - 1) / r) + 5ull * kSms * 128 - 1) / (5ull * kSms * 128);
       const uint64_t cost = waves * (r + 4u);
       if (cost < best) { best = cost; rows = r; }
     }
@@ -982,7 +981,7 @@ cudaError_t launch_shift_add(const ConvArgs& a, const WintTable& wt, const uint3
       attr_set[dev] = true;
     }
     uint32_t blocks = grid_for(total / 8, 256);
-    if (blocks > 148u * 4u) blocks = 148u * 4u;
+    if (blocks > kSms * 4u) blocks = kSms * 4u;
     launch_pdl(dwconv_nhwc8_kernel, blocks, 256, dw_smem, s, a, wt.w[a.uniform_log2k]); note_launch();
     return cudaGetLastError();
   }

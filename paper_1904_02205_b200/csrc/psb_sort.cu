@@ -158,7 +158,7 @@ cudaError_t launch_level_sort(const uint8_t* kmap, uint32_t M, void* ctl, uint32
   cudaError_t e = cudaMemsetAsync(ctl, 0, sizeof(SortCtl), s);
   if (e != cudaSuccess) return e;
   uint32_t blocks = (M + 255u) / 256u;
-  if (blocks > 148u * 8u) blocks = 148u * 8u;
+  if (blocks > kSms * 8u) blocks = kSms * 8u;
   if (blocks < 1u) blocks = 1u;
   launch_pdl(level_count_kernel, blocks, 256, 0, s, kmap, M, (SortCtl*)ctl, perm, max_tiles * kTileRows);
   note_launch();
@@ -174,7 +174,7 @@ cudaError_t launch_gather_sorted(const ConvArgs& a, const uint32_t* perm, const 
   const uint64_t rows = (uint64_t)sorted_tiles_bound((uint64_t)a.N * a.OH * a.OW) * kTileRows;
   const uint32_t rows_per_block = (256u / lanes) * (uint32_t)kGatherRows;
   uint64_t blocks = (rows + rows_per_block - 1) / rows_per_block;
-  if (blocks > 148u * 16u) blocks = 148u * 16u;
+  if (blocks > kSms * 16u) blocks = kSms * 16u;
   if (blocks < 1u) blocks = 1u;
   launch_pdl(gather_sorted_kernel, (uint32_t)blocks, 256, 0, s, a, perm, (const SortCtl*)ctl, cpad, lanes, dst);
   note_launch();
