@@ -867,13 +867,23 @@ uint32_t emax_blocks_for(uint32_t O, uint32_t d, uint32_t norm) {
   return blocks < 1 ? 1 : (blocks > 1184 ? 1184 : blocks);
 }
 
-// A layer sampled by a launch of its own needs no exponent pass before it (a launch of about 3 us on the host and on
-// the device) where a block holds whole rows and their windows are its own (norm == 1), or where the layer is so small
-// that every block can look at all of it.  4096 x 4096 with a window per row and its contraction 224 -> 216 us;
-// 256 -> 128 features (32768 weights in blocks of 256) 18.2 -> 16.2 us in a stream of calls; 3x3 64 -> 64 channels
-// (36864 weights, 576 a row) 27.1 -> 33.2: too few blocks, each reading too much.
+// A layer sampled by a launch of its own needs no exponent pass before it (a launch of about 2.3 us on the host) where a
+// block holds whole rows and their windows are its own (norm == 1), or where the layer is so small that every block can
+// look at all of it.  us per sampling with its matrix product (16 rows) or 3x3 layer (14x14) in a stream of calls, two
+// launches / one:
+//   one window:      256x64 16.2 / 14.0, 128x128 16.1 / 13.9, 256x128 16.0 / 13.8, 64x256 16.0 / 14.0, 128x256 16.1 / 14.0, all
+//                    bound by the host; on the device 9.2 / 9.2, 9.0 / 9.1, 9.3 / 13.3, 9.1 / 9.2, 9.4 / 13.5: at 32768 weights
+//                    the device has caught up with the host.  3x3 64->64 channels (36864 weights, 576 a row) 27.1 / 33.2.
+//   window per row:  a block takes a whole row, so rows of more than about 1536 weights need rows for two blocks per SM, or, with
+//                    taps, for one.  148x1536 16.3 / 13.9, 256x1536 19.5 / 16.8, 64x2048 16.1 / 13.8, 148x2048 15.9 / 18.3,
+//                    256x2048 20.0 / 21.6, 400x2048 25.6 / 21.9; 10x4096 16.2 / 20.5, 148x4096 20.2 / 30.4, 256x4096
+//                    30.5 / 35.3, 400x4096 37.4 / 36.3, 592x4096 37.2 / 35.7; 3x3 256->64 20.9 / 19.6, 256->256 23.3 / 21.7,
+//                    400->32 26.6 / 28.0, 400->256 37.2 / 33.6.
 bool fused_sampling(const psb_weights* wt) {
-  return wt->cfg.norm ? wt->d <= 4096u : wt->d <= 256u && (uint64_t)wt->shape.out_ch * wt->d <= 32768u;
+  const uint32_t d = wt->d, rows = wt->shape.out_ch;
+  if (!wt->cfg.norm) return d <= 256u && (uint64_t)rows * d <= 32768u;
+  const bool taps = wt->shape.kh * wt->shape.kw > 1u;
+  return d <= (rows >= (taps ? 1u : 2u) * kSms ? 4096u : taps ? 2304u : rows <= 64u ? 2048u : 1536u);
 }
 
 enum class SampleLaunch { kBatch, kTwoPass, kFused };

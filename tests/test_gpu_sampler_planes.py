@@ -116,3 +116,30 @@ def test_few_locations_at_odd_addresses(oracle):
         assert ctx.device_status() == 0 and np.array_equal(got, acc)
     wt.free()
     ctx.close()
+
+
+@pytest.mark.parametrize("case", [
+    # (norm, rows, channels, filter size, launches): both sides of the lines of the sampling without an exponent pass
+    (0, 128, 256, 1, 1), (0, 129, 256, 1, 2), (0, 3, 257, 1, 2), (1, 9, 1536, 1, 1), (1, 65, 1537, 1, 2), (1, 64, 2048, 1, 1),
+    (1, 64, 2049, 1, 2), (1, 295, 1537, 1, 2), (1, 296, 1537, 1, 1), (1, 147, 256, 3, 1), (1, 147, 257, 3, 2), (1, 148, 257, 3, 1),
+    (1, 296, 4096, 1, 1), (1, 296, 4097, 1, 2),
+])
+def test_windows_found_by_the_sampler_or_by_a_pass_of_their_own(case, oracle):
+    import torch
+
+    import paper_1904_02205_b200 as psb
+
+    norm, O, C, K, launches = case
+    ctx = psb.Context(0)
+    rng = np.random.default_rng(O + C)
+    w = rng.normal(0, 0.1, size=(O, C, K, K)).astype(np.float32)
+    w *= np.exp2(rng.integers(-3, 4, size=(O, 1, 1, 1))).astype(np.float32)
+    before = ctx.launch_count()
+    wt = ctx.sample_weights(torch.from_numpy(w).to(ctx.device), seed=3, layer_id=2, level_mask=8, norm=norm)
+    assert ctx.launch_count() - before == launches
+    W, eb, _ = oracle.sample_level(w, 3, 2, 3, norm=norm)
+    got, base = ctx.weights_export(wt, 3)
+    assert np.array_equal(got.cpu().numpy().astype(np.int64), W) and np.array_equal(base.cpu().numpy(), eb)
+    assert ctx.device_status() == 0
+    wt.free()
+    ctx.close()
