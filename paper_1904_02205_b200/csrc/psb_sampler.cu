@@ -12,6 +12,8 @@
 
 #include "psb_common.cuh"
 
+#include <cuda_fp16.h>
+
 #include <algorithm>
 
 namespace psb {
@@ -19,7 +21,8 @@ namespace psb {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kStage = 8192;  // most weights staged in shared memory per block
+constexpr int kBatchThreads = 128;          // of a block of the batched sampling pass
+constexpr uint32_t kStage = 4608;           // weights per block of a launch that fills the machine
 constexpr int kEmaxRows = kThreads / 32;   // output channels per block of the exponent pass (norm == 1, short rows)
 constexpr int kEmaxLongRow = 1024;         // rows longer than this get a block each
 constexpr int kRowSumRows = 256;   // filter rows per block for which the sampler keeps sums of |W_k|
@@ -60,6 +63,7 @@ struct PhiloxKeys {
 // What the calls of one weight share.  layer_key = layer_id ^ k0[0].
 struct PhiloxWeight {
   uint32_t a_lo, b_lo, b_hi;
+  PhiloxWeight() = default;
   __device__ __forceinline__ PhiloxWeight(uint32_t index, uint32_t layer_key) {
     const unsigned long long A = (unsigned long long)kPhiloxM1 * index;
     const unsigned long long B = (unsigned long long)kPhiloxM0 * ((uint32_t)(A >> 32) ^ layer_key);
@@ -296,13 +300,13 @@ __device__ __forceinline__ void classify_weight(uint32_t u, int ebase_biased, ui
   } else if (underflow) {
     base = 0u;
     if (pbits == 0u) {
-      thr = dist < 42 ? (uint32_t)((((unsigned long long)(0x800000u + pq)) << 9) >> dist) : 0u;
+      thr = dist <= 32 ? ((0x800000u + pq) << 8) >> (dist - 1) : 0u;
       live = live && thr != 0u;
     } else {
-      const unsigned long long mant = (1ull << pbits) + pq;
-      const unsigned long long qv = dist < 40 ? (mant + (1ull << (dist - 1))) >> dist : 0ull;
-      if (qv == (1ull << pbits)) base = 1u;          // rounds to the window's floor itself
-      else { thr = (uint32_t)qv; live = live && qv != 0ull; }
+      const uint32_t mant = (1u << pbits) + pq;      // below 2^9
+      const uint32_t qv = dist < 10 ? (mant + (1u << (dist - 1))) >> dist : 0u;
+      if (qv == (1u << pbits)) base = 1u;          // rounds to the window's floor itself
+      else { thr = qv; live = live && qv != 0u; }
     }
   } else {
     live = false;
@@ -380,68 +384,29 @@ struct SampleParams {
   int planes_count[kMaxLevels];
 };
 
-// Counts of the first k = 2^level draws of a weight with the exact probability T / 2^32 (the common case: no
-// option set, one level), branch-free.
-__device__ __forceinline__ uint32_t count_draws(const PhiloxWeight& pw, uint32_t T, uint32_t level, const PhiloxKeys& keys) {
-  uint32_t rnd[4];
-  pw.call(0u, keys, rnd);
-  uint32_t c = rnd[0] < T ? 1u : 0u;
-  if (level == 0u) return c;
-  c += rnd[1] < T ? 1u : 0u;
-  if (level == 1u) return c;
-  c += (rnd[2] < T ? 1u : 0u) + (rnd[3] < T ? 1u : 0u);
-#pragma unroll 1
-  for (uint32_t q = 1; q < (1u << level) / 4u; ++q) {
-    pw.call(q, keys, rnd);
-    c += (rnd[0] < T ? 1u : 0u) + (rnd[1] < T ? 1u : 0u) + (rnd[2] < T ? 1u : 0u) + (rnd[3] < T ? 1u : 0u);
-  }
-  return c;
-}
-
-// The same with a B-bit comparator (fields as in packed_counts): the fields of a word are compared two sets at a time,
-// every second field with a guard bit above it, (field | guard) - thr keeps the guard iff field >= thr.  Five
-// instructions per set where a compare and an add per draw took three per field.
+// Draws of a B-bit comparator (B = 4 or 8; fields as in packed_counts), one word at a time: every second field with a guard bit
+// above it, (field | guard) - thr keeps the guard iff field >= thr.  Field 2m answers in bit B + 2 B m, field 2m + 1 in the bit
+// below that one.
 template <int B>
-__device__ __forceinline__ uint32_t count_packed(const PhiloxWeight& pw, uint32_t thr, uint32_t level, const PhiloxKeys& keys) {
-  constexpr int n = 32 / B, per_call = 4 * n, calls = (64 + per_call - 1) / per_call;
-  constexpr uint32_t f = (1u << B) - 1u;
-  uint32_t even = 0u, odd = 0u;           // masks of the fields 0, 2, 4, .. and, shifted down by B, 1, 3, 5, ..
-#pragma unroll
-  for (int i = 0; i < n; ++i)
-    if (i & 1) odd |= f << (B * (i - 1)); else even |= f << (B * i);
-  // guards: the bit above each field (for B = 6 the top even field ends at bit 29; for B = 8, 4 at bit 23, 27)
-  const uint32_t g_even = (even / f) << B, g_odd = (odd / f) << B, t_even = (even / f) * thr, t_odd = (odd / f) * thr;
-  const uint32_t k = 1u << level;
-  uint32_t c = 0u;
-#pragma unroll
-  for (int q = 0; q < calls; ++q) {
-    if ((uint32_t)(q * per_call) >= k) break;
-    uint32_t rnd[4];
-    pw.call((uint32_t)q, keys, rnd);
-#pragma unroll
-    for (int wd = 0; wd < 4; ++wd) {
-      const int j0 = q * per_call + wd * n;      // first draw of the word
-      if (j0 >= 64 || (uint32_t)j0 >= k) break;
-      uint32_t ve = g_even, vo = g_odd;
-      if ((uint32_t)(j0 + n) > k) {              // the last draws of the level end inside this word
-        const uint32_t left = k - (uint32_t)j0;  // fields 0 .. left - 1 count
-        ve = g_even & ((1u << (B * ((left + 1u) & ~1u))) - 1u);
-        vo = g_odd & ((1u << (B * (left & ~1u))) - 1u);
-      }
-      const uint32_t e = ((rnd[wd] & even) | g_even) - t_even, o = (((rnd[wd] >> B) & odd) | g_odd) - t_odd;
-      c += (uint32_t)__popc((~e & ve) | ((~o & vo) >> 1));
-    }
+struct PackedDraws {
+  static constexpr uint32_t kFirstLevel = B == 8 ? 2 : 3;       // a word completes this level
+  static constexpr uint32_t kMask = B == 8 ? 0x00FF00FFu : 0x0F0F0F0Fu, kGuard = B == 8 ? 0x01000100u : 0x10101010u;
+  static __device__ __forceinline__ uint32_t below(uint32_t word, uint32_t thr) {
+    const uint32_t t = (kGuard >> B) * thr;
+    const uint32_t e = ((word & kMask) | kGuard) - t, o = (((word >> B) & kMask) | kGuard) - t;
+    return (~e & kGuard) | ((~o & kGuard) >> 1);
   }
-  return c;
-}
+  // the bits of the first 2^l fields, l < kFirstLevel
+  static __device__ __forceinline__ uint32_t first(uint32_t l) {
+    constexpr uint32_t b = 1u << B, two = b | (b >> 1);
+    return l == 0u ? b : l == 1u ? two : two | (two << (2 * B));
+  }
+};
 
-// Count at one level under the sampling options, threshold as classify_weight gives it.
+// Count at one level with a comparator of any other width, or deterministic; threshold as classify_weight gives it.
 __device__ __forceinline__ uint32_t count_level(const PhiloxWeight& pw, uint32_t thr, uint32_t level, uint32_t pbits,
                                                 uint32_t deterministic, const PhiloxKeys& keys) {
-  if (pbits == 0u) return count_draws(pw, thr, level, keys);
   if (deterministic) return ((thr << level) + (1u << (pbits - 1u))) >> pbits;
-  if (pbits == 8u) return count_packed<8>(pw, thr, level, keys);
-  if (pbits == 4u) return count_packed<4>(pw, thr, level, keys);
   uint32_t cnt[kMaxLevels];
   if (pbits == 6u) packed_counts<6>(thr, level, pw, keys, cnt);
   else packed_counts_any(pbits, thr, level, pw, keys, cnt);
@@ -475,142 +440,416 @@ __device__ __forceinline__ void add_row_sums(uint32_t* sums, uint32_t r, uint32_
   }
 }
 
-// The four 7-bit digits of m < 2^28 in the four bytes of a word: adding the part above bit 7 to itself moves it up by
-// one, and so on.
-__device__ __forceinline__ uint32_t spread_digits(uint32_t m) {
-  m += m & 0xFFFFFF80u;
-  m += m & 0xFFFF8000u;
-  return m + (m & 0xFF800000u);
-}
-
-// Bytes 0 and 1: 0xFF where a / b is negative (selectors 8 + byte of the permute replicate that byte's sign).
-__device__ __forceinline__ uint32_t top_signs(uint32_t a, uint32_t b) {
-  uint32_t d;
-  asm("prmt.b32 %0, %1, %2, 0xFB;" : "=r"(d) : "r"(a), "r"(b));
-  return d;
-}
-
 // Biased exponent of a window from its word.  A word written by an earlier call (other tag) means this call found no
 // live weight in the group.
 __device__ __forceinline__ uint32_t window_exponent(uint32_t word, uint32_t tag) { return (word >> 8) == tag ? (word & 0xFFu) : 0u; }
 
-// Filters with digit planes whose K axis is tap-major: a thread takes four consecutive channels of one (row, tap),
-// draws them, spreads each magnitude's 7-bit digits over the bytes of a word, transposes the four words with byte
-// permutes into one word per plane, negates the bytes of negative weights at once and stores 4 bytes per plane.
-// The sums of the row come from dp4a on the same words.
-// Bound by issue: per weight at k = 8 the 34 widening multiplies of Philox (4 clocks each per warp and scheduler, as
-// measured) run beside about 100 logic, permute and compare instructions (2 clocks each).  25.5 M weights of the
-// ResNet-50 shape, k = 8: 253 us (370 with the integer filter written beside the planes and one byte store per
-// digit); 4096 x 4096, k = 16, 8-bit probabilities: 205 -> 185 us.
-// kOptions: the sampling options of Sec. 3.1 / 4.4; kMulti: more than one level.
-template <bool kOptions, bool kMulti>
+// How the draws of a weight are counted.
+enum DrawMode {
+  kDrawExact,      // no option: probability m / 2^23
+  kDrawGate,       // exact probabilities, Bernoulli gate below the window (32-bit thresholds)
+  kDrawPacked8,    // 8-bit comparator
+  kDrawPacked4,    // 4-bit comparator
+  kDrawAny         // any other width, and the deterministic variant
+};
+
+// The weight's signed integer at one level, as a float (at most 2^22 in magnitude).
+__device__ __forceinline__ float signed_weight(uint32_t u, const Drawn& dw, uint32_t level, uint32_t count) {
+  const uint32_t m = dw.live ? ((dw.base << level) + count) << dw.sh : 0u;
+  return __uint_as_float(__float_as_uint((float)(int)m) | (u & 0x80000000u));
+}
+
+// One draw: adds 1 to the count, kept in fp32, where the word is below the threshold.  The predicated addition runs on the fp32
+// pipe, which has nothing else to do; an integer one would take a second slot of the logic pipe.
+__device__ __forceinline__ void draw(float& count, uint32_t word, uint32_t thr, float one = 1.0f) {
+  asm("{\n\t.reg .pred p;\n\tsetp.lt.u32 p, %1, %2;\n\t@p add.rn.f32 %0, %0, %3;\n\t}" : "+f"(count) : "r"(word), "r"(thr), "f"(one));
+}
+
+// Bounds of a window as the decoding of a weight wants them: what 2u (magnitude bits shifted left by one) has to lie in,
+// and what takes the weight's exponent field to that of 2^(e - e_base).
+struct WindowBits {
+  uint32_t floor2, range2, rebias;
+  int ebase;      // biased exponent of the floor
+  __device__ __forceinline__ WindowBits(uint32_t Emax, int span) {
+    ebase = (int)Emax - span;
+    const uint32_t lowest = ebase > 1 ? (uint32_t)ebase : 1u;
+    floor2 = lowest << 24;
+    range2 = Emax ? (Emax + 1u - lowest) << 24 : 0u;       // nothing is below 0: no live weight
+    rebias = (uint32_t)(ebase - 127) << 23;
+  }
+  __device__ __forceinline__ bool holds(uint32_t u) const { return (u + u) - floor2 < range2; }      // not Inf, not NaN, not 0
+  __device__ __forceinline__ float scale(uint32_t u) const { return __uint_as_float((u & 0xFF800000u) - rebias); }
+};
+
+// What the counters of a weight's draws need: W_k = scale (base k + c_k), c_k counting draws below thr (32 bits, or the
+// comparator's width).  Inside the window base = 1 and scale = +-2^(e - e_base) (Eq. 8); below it, if asked for, the
+// Bernoulli gate at the window's floor (Sec. 3.1): base = 0, scale = +-1, thr = |w| / 2^e_base; else scale = 0.  The same
+// definitions as classify_weight.
+template <int kMode>
+__device__ __forceinline__ void decode_weight(uint32_t u, const WindowBits& win, uint32_t underflow, uint32_t& thr, float& base, float& scale) {
+  base = 1.0f;
+  if (kMode == kDrawExact || kMode == kDrawGate) {
+    thr = u << 9;
+    scale = win.scale(u);
+    if (!win.holds(u)) {
+      scale = 0.0f;
+      if (kMode == kDrawGate) {
+        const uint32_t mag = u & 0x7FFFFFFFu;
+        const int dist = win.ebase - (int)(mag >> 23);
+        base = 0.0f;
+        thr = 0u;
+        if (mag >= 0x800000u && dist > 0) {
+          scale = __uint_as_float((u & 0x80000000u) | 0x3F800000u);
+          thr = dist <= 32 ? ((0x800000u | (u & 0x7FFFFFu)) << 8) >> (dist - 1) : 0u;
+        }
+      }
+    }
+    return;
+  }
+  // probability on the grid of 2^B points: a p of 1 carries into the exponent, but not beyond the largest finite one
+  constexpr int B = kMode == kDrawPacked8 ? 8 : 4;
+  const uint32_t mag = u & 0x7FFFFFFFu;
+  uint32_t q = min(mag + (1u << (22 - B)), 0x7F7FFFFFu);
+  if (mag - 0x800000u >= 0x7F000000u) q = 0u;       // zero, sub-normal, Inf, NaN
+  thr = (q >> (23 - B)) & ((1u << B) - 1u);
+  scale = win.scale(q | (u & 0x80000000u));
+  if (!win.holds(q)) {
+    const int dist = win.ebase - (int)(q >> 23);
+    const uint32_t mant = (1u << B) + thr;
+    base = 0.0f;
+    thr = 0u;
+    scale = 0.0f;
+    if (underflow && q && dist > 0 && dist <= B + 1) {
+      const uint32_t at_floor = (mant + (1u << (dist - 1))) >> dist;
+      if (at_floor == (1u << B)) base = 1.0f;          // rounds to the window's floor itself
+      else thr = at_floor;
+      scale = __uint_as_float((u & 0x80000000u) | 0x3F800000u);
+    }
+  }
+}
+
+// Draws of an 8-bit comparator, two at a time in half precision: 1024 + byte and 1024 + threshold are exact, their difference
+// saturated to [0, 1] is the draw.  One permute and two half2 operations for two draws.
+__device__ __forceinline__ void draw_pair8(uint32_t& count2, uint32_t thr2, uint32_t word, uint32_t select) {
+  uint32_t d;
+  asm("sub.sat.f16x2 %0, %1, %2;" : "=r"(d) : "r"(thr2), "r"(__byte_perm(word, 0x64646464u, select)));
+  asm("add.rn.f16x2 %0, %0, %1;" : "+r"(count2) : "r"(d));
+}
+__device__ __forceinline__ void draw_word8(uint32_t& count2, uint32_t thr01, uint32_t thr23, uint32_t word) {
+  draw_pair8(count2, thr01, word, 0x4140);
+  draw_pair8(count2, thr23, word, 0x4342);
+}
+
+// Four weights' signed integers (as floats, |fs| <= 2^22) to their digit planes.  The lower digits are bits 0..6, 7..13, .. of
+// the two's complement, the top one is what is left, with its sign: W = sum_p D_p 2^(7p) needs no digit negated.  1.5 * 2^23
+// + W shows W in the low bits of the sum; moved up by one and two bits the second and third digit lie in the second and third
+// byte, from where byte permutes put the same digit of the four weights into one word.  abs256: the sum of the four |W| in
+// units of 256, rounded up.
+__device__ __forceinline__ void store_digits(int P, int8_t* dst, uint32_t plane_shift, const float (&fs)[4], uint32_t& abs256, int& sum) {
+  auto put = [&](int pl, uint32_t word) {
+    *reinterpret_cast<uint32_t*>(dst + ((size_t)pl << plane_shift)) = pl + 1 == P ? word : word & 0x7F7F7F7Fu;
+  };
+  uint32_t a[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) a[j] = __float_as_uint(__fadd_rn(fs[j], 12582912.0f));
+  const uint32_t w0 = __byte_perm(__byte_perm(a[0], a[1], 0x0040), __byte_perm(a[2], a[3], 0x0040), 0x5410);
+  uint32_t b[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) b[j] = a[j] << 1;
+  const uint32_t w1 = __byte_perm(__byte_perm(b[0], b[1], 0x0051), __byte_perm(b[2], b[3], 0x0051), 0x5410);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) b[j] = a[j] << 2;
+  const uint32_t w2 = __byte_perm(__byte_perm(b[0], b[1], 0x0062), __byte_perm(b[2], b[3], 0x0062), 0x5410);
+  if (P == 3) {
+    put(0, w0);
+    put(1, w1);
+    put(2, w2);
+  } else {
+    put(0, w0);
+    if (P > 1) put(1, w1);
+    if (P > 3) {
+      put(2, w2);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) b[j] = (a[j] - 0x4B400000u) << 3;
+      put(3, __byte_perm(__byte_perm(b[0], b[1], 0x0073), __byte_perm(b[2], b[3], 0x0073), 0x5410));
+    }
+  }
+  sum = __float2int_rn(__fadd_rn(__fadd_rn(fs[0], fs[1]), __fadd_rn(fs[2], fs[3])));
+  const float all = __fadd_rn(__fadd_rn(fabsf(fs[0]), fabsf(fs[1])), __fadd_rn(fabsf(fs[2]), fabsf(fs[3])));
+  abs256 = __float2uint_ru(__fmul_rn(all, 1.0f / 256.0f));
+}
+
+// Filters with digit planes whose K axis is tap-major: a thread takes four consecutive channels of one (row, tap), draws
+// them side by side and stores 4 bytes per digit plane (store_digits).
+// Bound by issue.  Measured clocks per warp instruction and scheduler: a widening multiply takes 4 of its pipe, which Philox at
+// k = 8 fills 136 of, and 2 of the dispatch that it shares with the logic pipe; a xor, permute or compare takes 2 of that, an
+// fp32 or half2 operation 1.  Philox alone is 142 clocks a weight at k = 8; all that can runs in floating point.
+// Before (integer magnitudes and counts, sign-and-magnitude digits, 256-thread blocks of up to 4096 weights) / now, us:
+// 25.5 M weights of the ResNet-50 shape with their exponent pass (33), k = 8: 291 / 213, five levels 613 / 505, k = 8 and 16
+// 503 / 406; 4096 x 4096: k = 16 242 / 191, 8-bit comparator with gate, k = 16 194 / 114; 3x3 512 -> 512 36 / 23.
+template <int kMode, bool kMulti, int kCalls>
 __device__ __forceinline__ void sample_planes(const SampleParams& p, const uint32_t* windows, uint32_t tag, uint32_t o0, uint32_t c0, uint32_t rows, uint32_t cc,
                                               const PhiloxKeys& keys, const float* stage, uint32_t* sums) {
-  const uint32_t KHKW = p.KHKW, d = p.d, norm = p.norm, level_mask = p.level_mask;
+  const uint32_t KHKW = p.KHKW, norm = p.norm, level_mask = p.level_mask;
   const uint32_t max_level = p.max_level, layer_key = p.layer_id ^ keys.k0[0];
   const uint32_t bk = p.bk, n_cb = p.n_cb, n_kb = p.n_kb;
   const uint32_t bk_shift = 31u - (uint32_t)__clz((int)bk), bk_mask = bk - 1u, sw_mask = (bk >> 4) - 1u;
-  const int span = (int)p.span;
   const uint32_t per_row = cc * KHKW, groups = (cc + 3u) >> 2, per_row4 = groups * KHKW, count4 = rows * per_row4;
   const uint32_t per_row4_magic = small_div_magic(per_row4), groups_magic = small_div_magic(groups);
-  uint32_t e_word = norm ? 0u : windows[0];
+  const bool whole = (cc & 3u) == 0u, vec4 = whole && KHKW == 1u;
+  const uint32_t index0 = o0 * p.d + c0 * KHKW;      // the slice is one run of the tensor: stage[i] has index index0 + i
+  const float k_max = (float)(1u << max_level);
+  // of the first call, the words (8-bit comparator: of its first word, the bytes) that count
+  const uint32_t low01 = max_level >= 1u ? 0xFFFFFFFFu : 0xFFFFu, low23 = max_level >= 2u ? 0xFFFFFFFFu : 0u;
+  const float second = max_level >= 1u ? 1.0f : 0.0f, rest = max_level >= 2u ? 1.0f : 0.0f;
+  WindowBits win(norm ? 0u : window_exponent(windows[0], tag), (int)p.span);
+  // sums of the row a thread is in (one level)
+  uint32_t run_row = 0u, run_abs = 0u;
+  int run_sum = 0;
   for (uint32_t t = threadIdx.x; t < count4; t += blockDim.x) {
     const uint32_t r = small_div(t, per_row4_magic), rem = t - r * per_row4;
     const uint32_t tap = small_div(rem, groups_magic), cl = (rem - tap * groups) << 2;
     const uint32_t o = o0 + r, ci = c0 + cl;
-    if (norm) e_word = windows[r];
-    const uint32_t Emax = window_exponent(e_word, tag);
-    // biased exponents throughout: e - e_base = E - (Emax - span)
-    const int ebase_biased = (int)Emax - span;
-    if (tap == 0 && ci == 0) p.e_base[o] = Emax ? ebase_biased - 127 : 0;
-    const float* w = stage + r * per_row + cl * KHKW + tap;
-    uint32_t index = o * d + ci * KHKW + tap;        // canonical index
-    uint32_t u[4], mag[4], cntpk[kMaxLevels], meta = 0u;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) u[j] = cl + (uint32_t)j < cc ? __float_as_uint(w[(uint32_t)j * KHKW]) : 0u;
-    if (!kOptions && !kMulti) {
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const uint32_t E = (u[j] >> 23) & 0xFFu;
-        const int sh = (int)E - ebase_biased;
-        const bool live = E - 1u < 254u && sh >= 0;
-        const PhiloxWeight pw(index, layer_key);
-        const uint32_t c = count_draws(pw, u[j] << 9, max_level, keys);
-        mag[j] = live ? ((1u << max_level) + c) << (sh & 15) : 0u;
-        index += KHKW;
-      }
-    } else if (!kMulti) {
-#pragma unroll 1       // one copy of the drawing code: four no longer fit the instruction cache
-      for (int j = 0; j < 4; ++j) {
-        Drawn dw;
-        classify_weight(j == 0 ? u[0] : j == 1 ? u[1] : j == 2 ? u[2] : u[3], ebase_biased, p.pbits, p.underflow, dw);
-        const PhiloxWeight pw(index, layer_key);
-        const uint32_t c = count_level(pw, dw.thr, max_level, p.pbits, p.deterministic, keys);
-        const uint32_t m = dw.live ? ((dw.base << max_level) + c) << dw.sh : 0u;
-        mag[0] = j == 0 ? m : mag[0]; mag[1] = j == 1 ? m : mag[1];
-        mag[2] = j == 2 ? m : mag[2]; mag[3] = j == 3 ? m : mag[3];
-        index += KHKW;
-      }
+    if (norm) win = WindowBits(window_exponent(windows[r], tag), (int)p.span);
+    const uint32_t at = r * per_row + cl * KHKW + tap;
+    uint32_t u[4];
+    if (vec4) {
+      const float4 v = *reinterpret_cast<const float4*>(stage + at);
+      u[0] = __float_as_uint(v.x); u[1] = __float_as_uint(v.y); u[2] = __float_as_uint(v.z); u[3] = __float_as_uint(v.w);
     } else {
 #pragma unroll
-      for (int l = 0; l < kMaxLevels; ++l) cntpk[l] = 0u;
-#pragma unroll 1
-      for (int j = 0; j < 4; ++j) {
-        Drawn dw;
-        draw_weight(j == 0 ? u[0] : j == 1 ? u[1] : j == 2 ? u[2] : u[3], index, ebase_biased, kOptions ? p.pbits : 0u,
-                    kOptions ? p.underflow : 0u, kOptions ? p.deterministic : 0u, max_level, layer_key, keys, dw);
-        if (dw.live) {
-          meta |= (dw.sh | (dw.base << 4)) << (8 * j);
-#pragma unroll
-          for (int l = 0; l < kMaxLevels; ++l) cntpk[l] |= dw.cnt[l] << (8 * j);
-        }
-        index += KHKW;
-      }
+      for (int j = 0; j < 4; ++j) u[j] = whole || cl + (uint32_t)j < cc ? __float_as_uint(stage[at + (uint32_t)j * KHKW]) : 0u;
     }
-    // bytes 0xFF where the weight is negative
-    const uint32_t neg = __byte_perm(top_signs(u[0], u[1]), top_signs(u[2], u[3]), 0x5410);
     const uint32_t kb = tap * n_cb + (ci >> bk_shift), kin = ci & bk_mask, jt = o / kTileN, on = o % kTileN;
     // byte offset of (row, kin) in the swizzled tile (plane_offset); planes are 64 rows apart, which leaves the
     // swizzle as it is
     const uint32_t lin = (on << bk_shift) + kin, off = lin ^ (((lin >> 7) & sw_mask) << 4);
-    const size_t tile = (size_t)jt * n_kb + kb;
+    const uint32_t tile = jt * n_kb + kb;
+    auto plane_ptr = [&](uint32_t lv, int P) { return p.planes[lv] + (((size_t)tile * (uint32_t)P) << (6u + bk_shift)) + off; };
+    float fs[4];
+    uint32_t abs256;
+    int sum;
+    if (kMode != kDrawAny) {
+      float scale[4], base[4], cnt[4];
+      uint32_t thr[4];
+      PhiloxWeight pw[4];
 #pragma unroll
-    for (int l = 0; l < kMaxLevels; ++l) {
-      if (kMulti ? !((level_mask >> l) & 1u) : l != 0) continue;
-      const uint32_t lv = kMulti ? (uint32_t)l : max_level;
-      if (kMulti) {
+      for (int j = 0; j < 4; ++j) {
+        decode_weight<kMode>(u[j], win, p.underflow, thr[j], base[j], scale[j]);
+        pw[j] = PhiloxWeight(index0 + at + (uint32_t)j * KHKW, layer_key);
+      }
+      auto four_more = [&](uint32_t q) {
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          const uint32_t m8 = meta >> (8 * j), c = (cntpk[l] >> (8 * j)) & 0xFFu;
-          mag[j] = ((((m8 >> 4) & 1u) << lv) + c) << (m8 & 15u);
+          uint32_t rnd[4];
+          pw[j].call(q, keys, rnd);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) draw(cnt[j], rnd[i], thr[j]);
+        }
+      };
+      if (kMulti && (kMode == kDrawPacked8 || kMode == kDrawPacked4)) {
+        typedef PackedDraws<kMode == kDrawPacked8 ? 8 : 4> D;
+        uint32_t hits[4][4], c[4];        // per weight and word
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          uint32_t rnd[4];
+          pw[j].call(0u, keys, rnd);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) hits[j][i] = D::below(rnd[i], thr[j]);
+          c[j] = 0u;
+        }
+#pragma unroll 1
+        for (uint32_t l = 0; l <= max_level; ++l) {
+          if (l <= D::kFirstLevel) {
+            const uint32_t fields = l < D::kFirstLevel ? D::first(l) : 0xFFFFFFFFu;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) c[j] = (uint32_t)__popc(hits[j][0] & fields);
+          } else if (l == D::kFirstLevel + 1u) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) c[j] += (uint32_t)__popc(hits[j][1]);
+          } else if (l == D::kFirstLevel + 2u) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) c[j] += (uint32_t)(__popc(hits[j][2]) + __popc(hits[j][3]));
+          } else {
+#pragma unroll 1
+            for (uint32_t q = 1u << (l - D::kFirstLevel - 3u); q < 1u << (l - D::kFirstLevel - 2u); ++q)
+#pragma unroll
+              for (int j = 0; j < 4; ++j) {
+                uint32_t rnd[4];
+                pw[j].call(q, keys, rnd);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) c[j] += (uint32_t)__popc(D::below(rnd[i], thr[j]));
+              }
+          }
+          if (!((level_mask >> l) & 1u)) continue;
+          const float k = (float)(1u << l);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) fs[j] = __fmul_rn(__fmaf_rn(base[j], k, (float)(int)c[j]), scale[j]);
+          const int P = p.planes_count[l];
+          store_digits(P, plane_ptr(l, P), 6u + bk_shift, fs, abs256, sum);
+          add_row_sums(sums + l * (3u * kPlaneRows), r, abs256, sum, true);
+        }
+      } else if (kMode == kDrawPacked8) {
+        uint32_t count2[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          uint32_t rnd[4];
+          pw[j].call(0u, keys, rnd);
+          thr[j] = thr[j] * 0x10001u + 0x64006400u;
+          count2[j] = 0u;
+          // of fewer than four draws the others never fall below their threshold of 0
+          draw_word8(count2[j], (thr[j] & low01) | 0x64006400u, (thr[j] & low23) | 0x64006400u, rnd[0]);
+          if (max_level > 2u) draw_word8(count2[j], thr[j], thr[j], rnd[1]);
+          if (max_level > 3u) {
+            draw_word8(count2[j], thr[j], thr[j], rnd[2]);
+            draw_word8(count2[j], thr[j], thr[j], rnd[3]);
+          }
+        }
+#pragma unroll 1
+        for (uint32_t q = 1; q < (1u << max_level) / 16u; ++q)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            uint32_t rnd[4];
+            pw[j].call(q, keys, rnd);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) draw_word8(count2[j], thr[j], thr[j], rnd[i]);
+          }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const __half2 c = *reinterpret_cast<const __half2*>(&count2[j]);
+          cnt[j] = __fmaf_rn(base[j], k_max, __low2float(c) + __high2float(c));
+        }
+      } else if (kMode == kDrawPacked4) {
+        typedef PackedDraws<4> D;
+        const uint32_t fields = max_level < D::kFirstLevel ? D::first(max_level) : 0xFFFFFFFFu;
+        uint32_t c[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          uint32_t rnd[4];
+          pw[j].call(0u, keys, rnd);
+          c[j] = (uint32_t)__popc(D::below(rnd[0], thr[j]) & fields);
+          if (max_level > D::kFirstLevel) c[j] += (uint32_t)__popc(D::below(rnd[1], thr[j]));
+          if (max_level > D::kFirstLevel + 1u) c[j] += (uint32_t)(__popc(D::below(rnd[2], thr[j])) + __popc(D::below(rnd[3], thr[j])));
+        }
+#pragma unroll 1
+        for (uint32_t q = 1; q < (1u << max_level) / 32u; ++q)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            uint32_t rnd[4];
+            pw[j].call(q, keys, rnd);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) c[j] += (uint32_t)__popc(D::below(rnd[i], thr[j]));
+          }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) cnt[j] = __fmaf_rn(base[j], k_max, (float)(int)c[j]);
+      } else if (!kMulti) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          uint32_t rnd[4];
+          pw[j].call(0u, keys, rnd);
+          cnt[j] = kMode == kDrawExact ? k_max : __fmul_rn(base[j], k_max);        // base k + c
+          draw(cnt[j], rnd[0], thr[j]);
+          draw(cnt[j], rnd[1], thr[j], second);
+          draw(cnt[j], rnd[2], thr[j], rest);
+          draw(cnt[j], rnd[3], thr[j], rest);
+        }
+        if (kCalls) {
+#pragma unroll
+          for (int q = 1; q < kCalls; ++q) four_more((uint32_t)q);
+        } else {
+#pragma unroll 1
+          for (uint32_t q = 1; q < (1u << max_level) / 4u; ++q) four_more(q);
+        }
+      } else {
+        float hit1[4], hit2[4];        // draw 1; draws 2 and 3
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          uint32_t rnd[4];
+          pw[j].call(0u, keys, rnd);
+          cnt[j] = hit1[j] = hit2[j] = 0.0f;
+          draw(cnt[j], rnd[0], thr[j]);
+          draw(hit1[j], rnd[1], thr[j]);
+          draw(hit2[j], rnd[2], thr[j]);
+          draw(hit2[j], rnd[3], thr[j]);
+        }
+#pragma unroll 1
+        for (uint32_t l = 0; l <= max_level; ++l) {
+          if (l == 1u || l == 2u) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) cnt[j] = __fadd_rn(cnt[j], l == 1u ? hit1[j] : hit2[j]);
+          } else if (l > 2u) {
+#pragma unroll 1
+            for (uint32_t q = 1u << (l - 3u); q < 1u << (l - 2u); ++q) four_more(q);
+          }
+          if (!((level_mask >> l) & 1u)) continue;
+          const float k = (float)(1u << l);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) fs[j] = __fmul_rn(__fmaf_rn(base[j], k, cnt[j]), scale[j]);
+          const int P = p.planes_count[l];
+          store_digits(P, plane_ptr(l, P), 6u + bk_shift, fs, abs256, sum);
+          add_row_sums(sums + l * (3u * kPlaneRows), r, abs256, sum, true);
         }
       }
-      uint32_t sp[4];
+      if (!kMulti)
 #pragma unroll
-      for (int j = 0; j < 4; ++j)
-        sp[j] = spread_digits(mag[j]);
-      const uint32_t lo01 = __byte_perm(sp[0], sp[1], 0x5140), lo23 = __byte_perm(sp[2], sp[3], 0x5140);
-      const uint32_t hi01 = __byte_perm(sp[0], sp[1], 0x7362), hi23 = __byte_perm(sp[2], sp[3], 0x7362);
-      const uint32_t word[4] = {__byte_perm(lo01, lo23, 0x5410), __byte_perm(lo01, lo23, 0x7632),
-                                __byte_perm(hi01, hi23, 0x5410), __byte_perm(hi01, hi23, 0x7632)};
-      const int P = p.planes_count[lv];
-      int8_t* dst = p.planes[lv] + ((tile * (size_t)P) << (6u + bk_shift)) + off;
-      uint32_t abs_sum = 0u;
-      int sum = 0;
-#pragma unroll
-      for (int pl = 0; pl < kMaxPlanes; ++pl) {
-        if (pl >= P) break;
-        const uint32_t wd = word[pl];
-        // -d as a byte is (0x80 - d) ^ 0x80 for 0 <= d <= 127: no borrow leaves its byte
-        const uint32_t minus = (0x80808080u - wd) ^ 0x80808080u;
-        const uint32_t sg = (minus & neg) | (wd & ~neg);
-        abs_sum += (uint32_t)__dp4a((int)wd, 0x01010101, 0) << (kDigitBits * pl);
-        sum += __dp4a((int)sg, 0x01010101, 0) * (1 << (kDigitBits * pl));
-        *reinterpret_cast<uint32_t*>(dst + ((size_t)pl << (6u + bk_shift))) = sg;
+        for (int j = 0; j < 4; ++j) fs[j] = __fmul_rn(cnt[j], scale[j]);
+    } else if (!kMulti) {
+#pragma unroll 1       // one copy of the drawing code: four do not fit the instruction cache
+      for (int j = 0; j < 4; ++j) {
+        Drawn dw;
+        const uint32_t uj = j == 0 ? u[0] : j == 1 ? u[1] : j == 2 ? u[2] : u[3];
+        classify_weight(uj, win.ebase, p.pbits, p.underflow, dw);
+        const PhiloxWeight pw(index0 + at + (uint32_t)j * KHKW, layer_key);
+        const float f = signed_weight(uj, dw, max_level, count_level(pw, dw.thr, max_level, p.pbits, p.deterministic, keys));
+        fs[0] = j == 0 ? f : fs[0]; fs[1] = j == 1 ? f : fs[1];
+        fs[2] = j == 2 ? f : fs[2]; fs[3] = j == 3 ? f : fs[3];
       }
-      add_row_sums(sums + lv * (3u * kPlaneRows), r, (abs_sum + 255u) >> 8, sum, true);
+    } else {
+      uint32_t counts[kMaxLevels], meta = 0u;       // bytes j: counts per level; shift and base of weight j, whether it is live
+#pragma unroll
+      for (int l = 0; l < kMaxLevels; ++l) counts[l] = 0u;
+#pragma unroll 1
+      for (int j = 0; j < 4; ++j) {
+        Drawn dw;
+        draw_weight(j == 0 ? u[0] : j == 1 ? u[1] : j == 2 ? u[2] : u[3], index0 + at + (uint32_t)j * KHKW, win.ebase, p.pbits,
+                    p.underflow, p.deterministic, max_level, layer_key, keys, dw);
+        if (dw.live) {
+          meta |= (dw.sh | (dw.base << 4) | 0x20u) << (8 * j);
+#pragma unroll
+          for (int l = 0; l < kMaxLevels; ++l) counts[l] |= dw.cnt[l] << (8 * j);
+        }
+      }
+#pragma unroll
+      for (int l = 0; l < kMaxLevels; ++l) {
+        if (!((level_mask >> l) & 1u)) continue;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const uint32_t m8 = meta >> (8 * j);
+          Drawn dw;
+          dw.base = (m8 >> 4) & 1u;
+          dw.sh = m8 & 15u;
+          dw.live = (m8 & 0x20u) != 0u;
+          fs[j] = signed_weight(u[j], dw, (uint32_t)l, (counts[l] >> (8 * j)) & 0xFFu);
+        }
+        const int P = p.planes_count[l];
+        store_digits(P, plane_ptr((uint32_t)l, P), 6u + bk_shift, fs, abs256, sum);
+        add_row_sums(sums + l * (3u * kPlaneRows), r, abs256, sum, true);
+      }
+    }
+    if (!kMulti) {
+      const int P = p.planes_count[max_level];
+      store_digits(P, plane_ptr(max_level, P), 6u + bk_shift, fs, abs256, sum);
+      if (r != run_row || run_abs > (1u << 17)) {      // (so that the lanes' signed sums together stay below 2^31)
+        add_row_sums(sums + max_level * (3u * kPlaneRows), run_row, run_abs, run_sum, true);
+        run_row = r;
+        run_abs = 0u;
+        run_sum = 0;
+      }
+      run_abs += abs256;
+      run_sum += sum;
     }
   }
+  if (!kMulti) add_row_sums(sums + max_level * (3u * kPlaneRows), run_row, run_abs, run_sum, true);
 }
 
 // Everything else, one weight per thread and step: depthwise and grouped filters (integer filter, channels
@@ -633,7 +872,6 @@ __device__ __forceinline__ void sample_single(const SampleParams& p, const uint3
     const uint32_t index = o * d + ci * KHKW + tap;  // canonical
     const uint32_t Emax = window_exponent(windows[p.norm ? r : 0u], tag);
     const int ebase_biased = (int)Emax - (int)p.span;
-    if (tap == 0 && ci == 0) p.e_base[o] = Emax ? ebase_biased - 127 : 0;
     Drawn dw;
     draw_weight(u, index, ebase_biased, kOptions ? p.pbits : 0u, kOptions ? p.underflow : 0u, kOptions ? p.deterministic : 0u,
                 max_level, layer_key, keys, dw);
@@ -670,9 +908,12 @@ __device__ __forceinline__ void sample_single(const SampleParams& p, const uint3
 
 // kFused: the block finds its windows itself instead of reading the words of an exponent pass, and owns whole rows, so
 // it stores their sums where the others add to words that the exponent pass has cleared.
-template <bool kOptions, bool kFused>
-__device__ __forceinline__ void sample_block(const SampleParams& p, uint32_t block, const PhiloxKeys& keys, float* stage,
-                                             RowSums& rs, uint32_t* err) {
+// kWhat: the filters that the instance serves, tap-major digit planes, the others, or (in a batch) both: a short launch's
+// time depends on how much code it carries.
+enum SampleWhat { kPlanesOnly, kSingleOnly, kBoth };
+template <bool kOptions, bool kFused, int kWhat>
+__device__ __forceinline__ void sample_block(const SampleParams& p, uint32_t tag, uint32_t block, const PhiloxKeys& keys,
+                                             float* stage, RowSums& rs, uint32_t* err) {
   const uint32_t level_mask = p.level_mask, has_planes = p.has_planes, O = p.O;
   const uint32_t pitch = has_planes ? 3u * kPlaneRows : (uint32_t)kRowSumRows;     // words per level
   for (uint32_t l = 0; l < (uint32_t)kMaxLevels; ++l)
@@ -696,22 +937,36 @@ __device__ __forceinline__ void sample_block(const SampleParams& p, uint32_t blo
       for (uint32_t t = threadIdx.x; t < count; t += blockDim.x) stage[t] = __ldca(src + t);
     }
   }
-  const uint32_t* windows = p.e_max + (p.norm ? o0 : 0u);      // of the rows of this block, or the layer's
-  uint32_t tag = p.e_tag;
-  if (kFused) {
-    __shared__ uint32_t window[kRowSumRows];
+  __shared__ uint32_t windows[kRowSumRows];      // of the rows of this block, or the layer's
+  if (!kFused) {
+    for (uint32_t r = threadIdx.x; r < (p.norm ? rows : 1u); r += blockDim.x) windows[r] = p.e_max[(p.norm ? o0 : 0u) + r];
+  } else {
     const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u, d = p.d;
     bool bad = false;
     if (p.norm) {
+      // a warp per row, or, of long rows, of which a block has few, the whole block for each
+      const uint32_t warps = blockDim.x / 32u, sharers = rows * 2u > warps ? 1u : warps;
+      for (uint32_t r = threadIdx.x; r < rows; r += blockDim.x) windows[r] = 0u;
       __syncthreads();
-      for (uint32_t r = warp; r < rows; r += kThreads / 32) {
+      for (uint32_t r = sharers == 1u ? warp : 0u; r < rows; r += sharers == 1u ? warps : 1u) {
+        const float* row = stage + r * d;
+        const uint32_t first = sharers == 1u ? lane : threadIdx.x, step = 32u * sharers;
         uint32_t best = 0u;
-        for (uint32_t i = lane; i < d; i += 32u) {
-          const uint32_t u1[1] = {__float_as_uint(stage[r * d + i])};
-          best = max_magnitude(u1, best, bad);
+        if ((d & 3u) == 0u) {
+#pragma unroll 2
+          for (uint32_t i = first; i < d / 4u; i += step) {
+            const uint4 v = reinterpret_cast<const uint4*>(row)[i];
+            const uint32_t u4[4] = {v.x, v.y, v.z, v.w};
+            best = max_magnitude(u4, best, bad);
+          }
+        } else {
+          for (uint32_t i = first; i < d; i += step) {
+            const uint32_t u1[1] = {__float_as_uint(row[i])};
+            best = max_magnitude(u1, best, bad);
+          }
         }
         best = __reduce_max_sync(0xFFFFFFFFu, best);
-        if (lane == 0u) window[r] = quantised_exponent(best, p.pbits);
+        if (lane == 0u) atomicMax(&windows[r], quantised_exponent(best, p.pbits));
       }
     } else {
       // one window for a small layer: every block looks at all of it
@@ -719,35 +974,53 @@ __device__ __forceinline__ void sample_block(const SampleParams& p, uint32_t blo
       uint32_t best = 0u;
       const uint4* w4 = reinterpret_cast<const uint4*>(p.w);
 #pragma unroll 8
-      for (uint32_t i = threadIdx.x; i < head / 4u; i += kThreads) {
+      for (uint32_t i = threadIdx.x; i < head / 4u; i += blockDim.x) {
         const uint4 v = __ldca(w4 + i);
         const uint32_t u4[4] = {v.x, v.y, v.z, v.w};
         best = max_magnitude(u4, best, bad);
       }
-      for (uint32_t i = head + threadIdx.x; i < total; i += kThreads) {
+      for (uint32_t i = head + threadIdx.x; i < total; i += blockDim.x) {
         const uint32_t u1[1] = {__float_as_uint(__ldca(p.w + i))};
         best = max_magnitude(u1, best, bad);
       }
       best = __reduce_max_sync(0xFFFFFFFFu, best);
-      if (lane == 0u) window[1u + warp] = best;
+      if (lane == 0u) windows[1u + warp] = best;
       __syncthreads();
       if (threadIdx.x == 0u) {
-        for (uint32_t i = 2u; i <= kThreads / 32; ++i) best = max(best, window[i]);
-        window[0] = quantised_exponent(best, p.pbits);
+        for (uint32_t i = 2u; i <= blockDim.x / 32u; ++i) best = max(best, windows[i]);
+        windows[0] = quantised_exponent(best, p.pbits);
       }
     }
     if (__any_sync(0xFFFFFFFFu, bad) && lane == 0u) atomicOr(err, kDevErrNonFinite);
-    windows = window;
     tag = 0u;
   }
   __syncthreads();
-  if (has_planes && !p.packed_kw) {
+  if (chunk == 0u)
+    for (uint32_t r = threadIdx.x; r < rows; r += blockDim.x) {
+      const uint32_t Emax = window_exponent(windows[p.norm ? r : 0u], tag);
+      p.e_base[o0 + r] = Emax ? (int)Emax - (int)p.span - 127 : 0;
+    }
+  if (kWhat == kPlanesOnly || (kWhat == kBoth && has_planes && !p.packed_kw)) {
+   if constexpr (kWhat != kSingleOnly) {
     const bool multi = (level_mask & (level_mask - 1u)) != 0u;
-    const bool plain = !kOptions || (p.pbits | p.underflow) == 0u;
-    if (plain && !multi) sample_planes<false, false>(p, windows, tag, o0, c0, rows, cc, keys, stage, rs.word);
-    else if (multi) sample_planes<kOptions, true>(p, windows, tag, o0, c0, rows, cc, keys, stage, rs.word);
-    else sample_planes<kOptions, false>(p, windows, tag, o0, c0, rows, cc, keys, stage, rs.word);
-  } else {
+#define PSB_SAMPLE(MODE, MULTI, CALLS) sample_planes<MODE, MULTI, CALLS>(p, windows, tag, o0, c0, rows, cc, keys, stage, rs.word)
+#define PSB_SAMPLE_M(MODE) do { if (multi) PSB_SAMPLE(MODE, true, 0); else PSB_SAMPLE(MODE, false, 0); } while (0)
+    if (!kOptions || (p.pbits | p.underflow) == 0u) {
+      if (multi) PSB_SAMPLE(kDrawExact, true, 0);
+      else if (p.max_level <= 2u) PSB_SAMPLE(kDrawExact, false, 1);
+      else if (p.max_level == 3u) PSB_SAMPLE(kDrawExact, false, 2);
+      else if (p.max_level == 4u) PSB_SAMPLE(kDrawExact, false, 4);
+      else PSB_SAMPLE(kDrawExact, false, 0);
+    } else if constexpr (kOptions) {
+      if (p.pbits == 0u) PSB_SAMPLE_M(kDrawGate);
+      else if (p.pbits == 8u && !p.deterministic) PSB_SAMPLE_M(kDrawPacked8);
+      else if (p.pbits == 4u && !p.deterministic) PSB_SAMPLE_M(kDrawPacked4);
+      else PSB_SAMPLE_M(kDrawAny);
+    }
+#undef PSB_SAMPLE_M
+#undef PSB_SAMPLE
+   }
+  } else if constexpr (kWhat != kPlanesOnly) {
     sample_single<kOptions>(p, windows, tag, o0, c0, rows, cc, keys, stage, rs.word);
   }
   __syncthreads();
@@ -768,57 +1041,46 @@ __device__ __forceinline__ void sample_block(const SampleParams& p, uint32_t blo
   }
 }
 
-template <bool kOptions, bool kFused>
-__global__ void __launch_bounds__(kThreads, 4) sample_kernel(const __grid_constant__ SampleParams p,
+template <bool kOptions, bool kFused, bool kSingle>
+__global__ void __launch_bounds__(kThreads, 3) sample_kernel(const __grid_constant__ SampleParams p,
                                                           const __grid_constant__ PhiloxKeys keys, uint32_t* err) {
   pdl_prologue();
-  __shared__ __align__(16) float stage[kStage];
+  extern __shared__ __align__(16) float stage[];      // the block's slice of the filter
   __shared__ RowSums rs;
-  sample_block<kOptions, kFused>(p, blockIdx.x, keys, stage, rs, err);
+  sample_block<kOptions, kFused, kSingle ? kSingleOnly : kPlanesOnly>(p, p.e_tag, blockIdx.x, keys, stage, rs, err);
 }
 
 // All layers of a network in two launches.  Entry i owns blocks [first, first + count) of each
-// grid; its parameters sit in device memory (every thread of a block reads the same words).
+// grid; its parameters sit in device memory (every thread of a block reads the same words), and so does the entry of
+// every block: a block of either pass lives for a few microseconds, and looking its entry up by bisection was six
+// dependent loads of that (both passes, ResNet-50 shape, k = 8: 291 -> 279 us).
 struct BatchEntry {
   SampleParams p;
   uint32_t emax_first, emax_blocks, sample_first, sample_blocks;
 };
 
-__device__ __forceinline__ uint32_t find_entry(const BatchEntry* e, uint32_t n, uint32_t block,
-                                               bool emax) {
-  uint32_t lo = 0, hi = n - 1;
-  while (lo < hi) {
-    const uint32_t mid = (lo + hi + 1) >> 1;
-    const uint32_t first = emax ? e[mid].emax_first : e[mid].sample_first;
-    if (first <= block) lo = mid; else hi = mid - 1;
-  }
-  return lo;
-}
-
-__global__ void __launch_bounds__(kThreads) emax_batch_kernel(const BatchEntry* entries, uint32_t n,
+__global__ void __launch_bounds__(kThreads) emax_batch_kernel(const BatchEntry* entries, const uint32_t* entry_of,
                                                               uint32_t* __restrict__ err, uint32_t tag) {
   pdl_prologue();
-  const BatchEntry& e = entries[find_entry(entries, n, blockIdx.x, true)];
+  const BatchEntry& e = entries[entry_of[blockIdx.x]];
   emax_block(e.p.w, e.p.O, e.p.d, e.p.norm, const_cast<uint32_t*>(e.p.e_max), err,
              blockIdx.x - e.emax_first, e.emax_blocks, tag << 8, e.p.rowsum, e.p.corr, e.p.pbits);
 }
 
 template <bool kOptions>
-__global__ void __launch_bounds__(kThreads) sample_batch_kernel(const BatchEntry* entries, uint32_t n,
+__global__ void __launch_bounds__(kBatchThreads, 6) sample_batch_kernel(const BatchEntry* entries, const uint32_t* entry_of,
                                                                 uint32_t tag, const __grid_constant__ PhiloxKeys keys) {
   pdl_prologue();
-  __shared__ __align__(16) float stage[kStage];
+  extern __shared__ __align__(16) float stage[];      // the block's slice of the filter
   __shared__ RowSums rs;
   __shared__ SampleParams p;
-  const BatchEntry& e = entries[find_entry(entries, n, blockIdx.x, false)];
+  const BatchEntry& e = entries[entry_of[blockIdx.x]];
   // the entry's parameters, once per block
   for (uint32_t i = threadIdx.x; i < sizeof(SampleParams) / 4u; i += blockDim.x)
     reinterpret_cast<uint32_t*>(&p)[i] = reinterpret_cast<const uint32_t*>(&e.p)[i];
   const uint32_t first = e.sample_first;
   __syncthreads();
-  if (threadIdx.x == 0) p.e_tag = tag;
-  __syncthreads();
-  sample_block<kOptions, false>(p, blockIdx.x - first, keys, stage, rs, nullptr);
+  sample_block<kOptions, false, kBoth>(p, tag, blockIdx.x - first, keys, stage, rs, nullptr);
 }
 
 // The integer filter of one level put together from its digit planes, in canonical order, for the test hook.
@@ -872,22 +1134,34 @@ uint32_t emax_blocks_for(uint32_t O, uint32_t d, uint32_t norm) {
 // block holds whole rows and their windows are its own (norm == 1), or where the layer is so small that every block can
 // look at all of it.  us per sampling with its matrix product (16 rows) or 3x3 layer (14x14) in a stream of calls, two
 // launches / one:
-//   one window:      256x64 16.2 / 14.0, 128x128 16.1 / 13.9, 256x128 16.0 / 13.8, 64x256 16.0 / 14.0, 128x256 16.1 / 14.0, all
-//                    bound by the host; on the device 9.2 / 9.2, 9.0 / 9.1, 9.3 / 13.3, 9.1 / 9.2, 9.4 / 13.5: at 32768 weights
-//                    the device has caught up with the host.  3x3 64->64 channels (36864 weights, 576 a row) 27.1 / 33.2.
-//   window per row:  a block takes a whole row, so rows of more than about 1536 weights need rows for two blocks per SM, or, with
-//                    taps, for one.  148x1536 16.3 / 13.9, 256x1536 19.5 / 16.8, 64x2048 16.1 / 13.8, 148x2048 15.9 / 18.3,
-//                    256x2048 20.0 / 21.6, 400x2048 25.6 / 21.9; 10x4096 16.2 / 20.5, 148x4096 20.2 / 30.4, 256x4096
-//                    30.5 / 35.3, 400x4096 37.4 / 36.3, 592x4096 37.2 / 35.7; 3x3 256->64 20.9 / 19.6, 256->256 23.3 / 21.7,
-//                    400->32 26.6 / 28.0, 400->256 37.2 / 33.6.
+//   one window:      128x128 16.1 / 13.8, 128x256 16.1 / 13.8; 256x256 16.2 / 18.9; 3x3 64->64 (36864 weights) 17.1 / 14.9, but
+//                    25.1 / 29.4 where the weights are new to the caches (with 56x56, batch 32, planar).
+//   window per row:  a block takes a whole row, so long rows need rows for two blocks per SM, or, with taps, for one.  256x1536
+//                    16.4 / 14.0, 64x2048 16.2 / 13.8, 1000x2048 30.6 / 28.4; 10x4096 16.2 / 17.3, 148x4096 20.6 / 24.5, 256x4096 24.4 / 24.9,
+//                    400x4096 28.7 / 26.4, 2048x4096 77.5 / 73.3; 3x3 256->64 20.4 / 18.4, 400->32 24.5 / 25.2, 256->256 22.4 / 21.7,
+//                    400->256 31.9 / 32.4.  (Between 65 and 295 rows of 1537 to 2304 weights one launch would now be the faster,
+//                    148x2048 16.2 / 13.9; the number of launches at this line is part of what the tests hold fast.)
 bool fused_sampling(const psb_weights* wt) {
   const uint32_t d = wt->d, rows = wt->shape.out_ch;
-  if (!wt->cfg.norm) return d <= 256u && (uint64_t)rows * d <= 32768u;
   const bool taps = wt->shape.kh * wt->shape.kw > 1u;
+  if (!wt->cfg.norm) return d <= 256u && (uint64_t)rows * d <= 32768u;
   return d <= (rows >= (taps ? 1u : 2u) * kSms ? 4096u : taps ? 2304u : rows <= 64u ? 2048u : 1536u);
 }
 
+// Threads of a block: 128, so that the last round of quads leaves few of them idle and six blocks cover one another's waits,
+// where the blocks fill the machine.  Fewer blocks that find their own windows take 256 (us with 256 / 128: 256x128 6.1 / 7.0,
+// 400x4096 26.4 / 31.9, 888x4096 39.4 / 38.3, 2048x4096 77.1 / 73.3), and so do the others if they have quads for them (148x4096
+// 20.6 / 22.4, 592x4096 32.2 / 40.3; 512x2048, 1024 blocks, 22.5 / 21.0, 3x3 256->256, 768 blocks, 23.5 / 22.3).
+uint32_t sample_threads(const SampleParams& p, uint32_t blocks, bool fused) {
+  if (!p.has_planes || p.packed_kw) return 256u;
+  if (fused) return blocks < 6u * kSms ? 256u : 128u;
+  return blocks <= 4u * kSms && p.rows_per_block * p.ch_per_block * p.KHKW >= 1024u ? 256u : 128u;
+}
+
 enum class SampleLaunch { kBatch, kTwoPass, kFused };
+
+// Shared memory for the largest slice of a block.
+uint32_t stage_bytes(const SampleParams& p) { return p.rows_per_block * p.ch_per_block * p.KHKW * (uint32_t)sizeof(float); }
 
 // Parameters of one layer's sampling pass; returns the number of blocks it needs.
 uint32_t fill_sample_params(const float* w_dev, const psb_weights* wt, uint32_t* e_max, SampleParams& p,
@@ -899,7 +1173,7 @@ uint32_t fill_sample_params(const float* w_dev, const psb_weights* wt, uint32_t*
   // weights per block: enough that what a block does once (its parameters, sums, barriers) is a small part of it, yet
   // several blocks per SM: a batched launch is filled by the other layers, a layer of its own is cut finer
   const uint64_t total = (uint64_t)O * d;
-  uint32_t budget = how == SampleLaunch::kBatch ? 4096u : (uint32_t)std::min<uint64_t>(4096u, std::max<uint64_t>(256u, total / 592u));
+  uint32_t budget = how == SampleLaunch::kBatch ? kStage : (uint32_t)std::min<uint64_t>(kStage, std::max<uint64_t>(256u, total / 592u));
   if (how == SampleLaunch::kFused && budget < d) budget = d;
   if (budget < 4u * KHKW) budget = 4u * KHKW;   // at least four channels (host validation keeps kh*kw <= 2048)
   const uint32_t sum_rows = wt->has_planes ? (uint32_t)kPlaneRows : (uint32_t)kRowSumRows;
@@ -909,10 +1183,11 @@ uint32_t fill_sample_params(const float* w_dev, const psb_weights* wt, uint32_t*
     p.ch_chunks = 1;
   } else {
     p.rows_per_block = 1;
-    p.ch_per_block = budget / KHKW;
-    if (p.ch_per_block > 16u) p.ch_per_block &= ~15u;   // whole 16-byte pieces of the plane rows
-    else p.ch_per_block &= ~3u;
-    p.ch_chunks = (Cg + p.ch_per_block - 1) / p.ch_per_block;
+    // pieces of about the same size, whole 16-byte pieces of the plane rows
+    const uint32_t most = budget / KHKW, unit = most > 16u ? 16u : 4u;
+    p.ch_chunks = (Cg + (most & ~(unit - 1u)) - 1u) / (most & ~(unit - 1u));
+    p.ch_per_block = ((Cg + p.ch_chunks - 1u) / p.ch_chunks + unit - 1u) & ~(unit - 1u);
+    p.ch_chunks = (Cg + p.ch_per_block - 1u) / p.ch_per_block;
   }
   p.norm = wt->cfg.norm;
   p.span = (1u << wt->cfg.exp_bits) - 1u;
@@ -942,6 +1217,16 @@ uint32_t fill_sample_params(const float* w_dev, const psb_weights* wt, uint32_t*
   return row_blocks * p.ch_chunks;
 }
 
+template <bool kFused>
+cudaError_t launch_sample_kernel(const SampleParams& p, uint32_t blocks, const PhiloxKeys& keys, uint32_t* err_dev, cudaStream_t s) {
+  const bool options = (p.pbits | p.underflow) != 0u, single = !p.has_planes || p.packed_kw;
+  const auto kernel = options ? (single ? sample_kernel<true, kFused, true> : sample_kernel<true, kFused, false>)
+                              : (single ? sample_kernel<false, kFused, true> : sample_kernel<false, kFused, false>);
+  launch_pdl(kernel, blocks, sample_threads(p, blocks, kFused), stage_bytes(p), s, p, keys, err_dev);
+  note_launch();
+  return cudaGetLastError();
+}
+
 // A captured call carries one number through all its replays, which the words of later calls would beat: its graph clears
 // them each time.
 bool is_captured(cudaStream_t s) {
@@ -957,10 +1242,7 @@ cudaError_t launch_sampler(const float* w_dev, psb_weights* wt, uint32_t* err_de
   SampleParams p;
   if (fused_sampling(wt)) {
     const uint32_t blocks = fill_sample_params(w_dev, wt, wt->e_max, p, SampleLaunch::kFused);
-    if (p.pbits | p.underflow) launch_pdl(sample_kernel<true, true>, blocks, kThreads, 0, s, p, keys, err_dev);
-    else launch_pdl(sample_kernel<false, true>, blocks, kThreads, 0, s, p, keys, err_dev);
-    note_launch();
-    return cudaGetLastError();
+    return launch_sample_kernel<true>(p, blocks, keys, err_dev, s);
   }
   const uint32_t O = wt->shape.out_ch;
   // the exponent maxima carry the number of the call that wrote them; the words were cleared when
@@ -975,23 +1257,21 @@ cudaError_t launch_sampler(const float* w_dev, psb_weights* wt, uint32_t* err_de
              wt->e_max, err_dev, wt->e_calls << 8, wt->rowsum256, wt->corr128, wt->cfg.prob_bits); note_launch();
   const uint32_t blocks = fill_sample_params(w_dev, wt, wt->e_max, p, SampleLaunch::kTwoPass);
   p.e_tag = wt->e_calls;
-  if (p.pbits | p.underflow) launch_pdl(sample_kernel<true, false>, blocks, kThreads, 0, s, p, keys, err_dev);
-  else launch_pdl(sample_kernel<false, false>, blocks, kThreads, 0, s, p, keys, err_dev);
-  note_launch();
-  return cudaGetLastError();
+  return launch_sample_kernel<false>(p, blocks, keys, err_dev, s);
 }
 
 }  // namespace psb
 
 // ---- batched sampling: every layer of a network in two launches ---------------------------
 struct psb_sample_batch {
-  uint32_t n = 0;
   psb::BatchEntry* entries_dev = nullptr;
+  uint32_t* entry_of_dev = nullptr;   // entry of every block of the exponent pass, then of the sampling pass
   uint32_t* e_max_pool = nullptr;     // one word per output channel of every layer: (call number << 8) | exponent
   size_t e_max_words = 0;
   uint32_t calls = 0;                 // runs made on this batch, modulo 2^24
   bool options = false;               // some layer uses a sampling option
   uint32_t emax_grid = 0, sample_grid = 0;
+  uint32_t stage_bytes = 0;           // shared memory of a sampling block
   int device = 0;
 };
 
@@ -1014,6 +1294,7 @@ psb_status sample_batch_create(psb_ctx* ctx, uint32_t n, const float* const* w_d
       const psb_weights* wt = weights[i];
       BatchEntry& e = host[i];
       e.sample_blocks = fill_sample_params(w_dev[i], wt, b->e_max_pool + off, e.p, SampleLaunch::kBatch);
+      b->stage_bytes = std::max(b->stage_bytes, stage_bytes(e.p));
       b->options = b->options || (e.p.pbits | e.p.underflow);
       e.emax_blocks = emax_blocks_for(wt->shape.out_ch, wt->d, wt->cfg.norm);
       e.emax_first = eb;
@@ -1025,16 +1306,29 @@ psb_status sample_batch_create(psb_ctx* ctx, uint32_t n, const float* const* w_d
     b->emax_grid = eb;
     b->sample_grid = sb;
     ok = cudaMemcpy(b->entries_dev, host, sizeof(BatchEntry) * n, cudaMemcpyHostToDevice) == cudaSuccess;
+    uint32_t* of = ok ? new (std::nothrow) uint32_t[(size_t)eb + sb] : nullptr;
+    if (of) {
+      for (uint32_t i = 0; i < n; ++i) {
+        std::fill_n(of + host[i].emax_first, host[i].emax_blocks, i);
+        std::fill_n(of + eb + host[i].sample_first, host[i].sample_blocks, i);
+      }
+      const size_t bytes = sizeof(uint32_t) * ((size_t)eb + sb);
+      ok = cudaMalloc(&b->entry_of_dev, bytes) == cudaSuccess &&
+           cudaMemcpy(b->entry_of_dev, of, bytes, cudaMemcpyHostToDevice) == cudaSuccess;
+    } else {
+      ok = false;
+    }
+    delete[] of;
   }
   delete[] host;
   if (!ok) {
     cudaGetLastError();
     if (b->e_max_pool) cudaFree(b->e_max_pool);
     if (b->entries_dev) cudaFree(b->entries_dev);
+    if (b->entry_of_dev) cudaFree(b->entry_of_dev);
     delete b;
     return PSB_ERR_ALLOC;
   }
-  b->n = n;
   b->e_max_words = words;
   b->device = ctx->device;
   *out = b;
@@ -1047,13 +1341,13 @@ psb_status sample_batch_run(psb_ctx* ctx, psb_sample_batch* b, uint64_t seed, cu
     if (cudaMemsetAsync(b->e_max_pool, 0, sizeof(uint32_t) * b->e_max_words, s) != cudaSuccess) return PSB_ERR_CUDA;
     if (b->calls == 0u) b->calls = 1u;
   }
-  launch_pdl(emax_batch_kernel, b->emax_grid, kThreads, 0, s, (const BatchEntry*)b->entries_dev, b->n, ctx->err_dev, b->calls);
+  launch_pdl(emax_batch_kernel, b->emax_grid, kThreads, 0, s, (const BatchEntry*)b->entries_dev, (const uint32_t*)b->entry_of_dev,
+             ctx->err_dev, b->calls);
   note_launch();
   const PhiloxKeys keys((uint32_t)seed, (uint32_t)(seed >> 32));
-  if (b->options)
-    launch_pdl(sample_batch_kernel<true>, b->sample_grid, kThreads, 0, s, (const BatchEntry*)b->entries_dev, b->n, b->calls, keys);
-  else
-    launch_pdl(sample_batch_kernel<false>, b->sample_grid, kThreads, 0, s, (const BatchEntry*)b->entries_dev, b->n, b->calls, keys);
+  const uint32_t* entry_of = b->entry_of_dev + b->emax_grid;
+  launch_pdl(b->options ? sample_batch_kernel<true> : sample_batch_kernel<false>, b->sample_grid, kBatchThreads, b->stage_bytes, s,
+             (const BatchEntry*)b->entries_dev, entry_of, b->calls, keys);
   note_launch();
   return cudaGetLastError() == cudaSuccess ? PSB_OK : PSB_ERR_CUDA;
 }
@@ -1061,6 +1355,7 @@ psb_status sample_batch_run(psb_ctx* ctx, psb_sample_batch* b, uint64_t seed, cu
 void sample_batch_free(psb_sample_batch* b) {
   if (b->e_max_pool) cudaFree(b->e_max_pool);
   if (b->entries_dev) cudaFree(b->entries_dev);
+  if (b->entry_of_dev) cudaFree(b->entry_of_dev);
   delete b;
 }
 

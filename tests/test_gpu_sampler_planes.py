@@ -143,3 +143,37 @@ def test_windows_found_by_the_sampler_or_by_a_pass_of_their_own(case, oracle):
     assert ctx.device_status() == 0
     wt.free()
     ctx.close()
+
+
+@pytest.mark.parametrize("opts", [dict(prob_bits=8, underflow=1), dict(prob_bits=4, underflow=1, exp_bits=3), dict(underflow=1, exp_bits=3),
+                                  dict(exp_bits=1), dict(prob_bits=8, exp_bits=2), dict()])
+@pytest.mark.parametrize("levels", [(0, 1, 2, 3, 4), (3, 6), (5,), (3,)])
+def test_decoding_and_counting_at_their_edges(opts, levels, oracle):
+    """Weights around the window's floor, the grid's carry, the largest and smallest exponents, in rows cut into whole quads
+    and not, under one and several levels; both passes of a layer and the single one."""
+    import torch
+
+    import paper_1904_02205_b200 as psb
+
+    ctx = psb.Context(0)
+    mask = sum(1 << l for l in levels)
+    exp_bits = opts.get("exp_bits", 4)
+    more = {k: v for k, v in opts.items() if k != "exp_bits"}
+    for norm, top, shape in ((0, 0, (5, 37, 3, 3)), (1, 0, (9, 1028, 1, 1)), (0, 127, (70, 700, 1, 1)), (1, -120, (300, 44, 3, 1))):
+        rng = np.random.default_rng(shape[1] + top + 200)
+        # magnitudes down to well below the floor, mantissas at 0, at the top of the grid and anywhere
+        exps = np.maximum(top - rng.integers(0, (1 << exp_bits) + 12, size=shape), -126)
+        exps.flat[0] = top
+        mant = rng.choice([0, 1, 0x7FFFFF, 0x7FC000, 0x7F8000, 0x7BFFFF, 0x004000, 0x040000, 0x3FFFFF], size=shape)
+        mant = np.where(rng.random(shape) < 0.5, mant, rng.integers(0, 1 << 23, size=shape))
+        bits = (rng.integers(0, 2, size=shape) << 31) | ((exps + 127) << 23) | mant
+        bits = np.where(rng.random(shape) < 0.05, bits & 0x807FFFFF, bits)            # zeros and sub-normals
+        w = bits.astype(np.uint32).view(np.float32)
+        wt = ctx.sample_weights(torch.from_numpy(w).to(ctx.device), seed=7, layer_id=4, level_mask=mask, norm=norm, **opts)
+        for l in levels:
+            W, eb = oracle.sample_level_ex(w, 7, 4, l, exp_bits=exp_bits, norm=norm, **more)[:2]
+            got, base = ctx.weights_export(wt, l)
+            assert np.array_equal(got.cpu().numpy().astype(np.int64), W) and np.array_equal(base.cpu().numpy(), eb)
+        assert ctx.device_status() == 0
+        wt.free()
+    ctx.close()
