@@ -83,6 +83,7 @@ struct TensorParams {
   uint32_t resident_bytes;
   const uint32_t* rowsum256;   // [level][O] row sums of |W_k| in units of 256 (rounded up), or null
   uint32_t amax;        // largest activation magnitude the caller vouches for
+  uint32_t mid;         // 1: two digit planes fit 32 bits together (kRecMid)
   const long long* corr[kMaxLevels];  // per-channel integer addend, or null
   const int8_t* planes_ptr[kMaxLevels];  // digit planes: [o_tile][K block][P * 64 rows][BK], pre-swizzled tiles
   // Band mode (stride-1 filters with taps, one channel block, resident planes): a tile is 128
@@ -329,12 +330,34 @@ struct SharedCtl {
 //        largest row sum of |W_k|, the caller vouches for the largest activation): the planes are
 //        recombined in 32 bits (wrap-around in the partial sums is harmless) and one conversion
 //        instruction rounds to nearest even, as the 64-bit conversion would.  Otherwise 64-bit
-//        recombination plus the per-channel integer addend, converted in two exact halves.
+//        recombination plus the per-channel integer addend, converted in two exact halves.  Between the two (Recombine).
 //   y = fma(a, sc, bias); optional shortcut fma on a byte converted by the conversion unit.
 //   t = y * inv_step, clamped above in fp32; cvt.rni (round half to even, saturating) gives the
 //   integer; cvt.pack.sat packs two integers at a time into bytes, saturating to the byte's range.
 //   FAST_U8: unsigned codes whose lower bound is 0 (the ReLU, if any, folded into it): the byte
 //   saturation is the lower clamp.  Otherwise both clamps are applied in fp32 first.
+// How the plane sums of a layer become its accumulators' floats.
+//   kRec32:    in 32 bits, see above.  kRec32Add: plus an integer addend per channel (x - 128 fed for unsigned x).
+//   kRecMid:   three planes whose lower two fit 32 bits together (the host knows: 16383 x channels and taps x largest byte fed).
+//              With t = v0 + 2^7 v1 the accumulator is 2^14 (v2 + (t >> 14)) + (t mod 2^14), the upper part below 2^24 in
+//              magnitude: both parts are exact floats and one fma rounds their sum.  2^23 + the lower part is a bit
+//              pattern, and the 2^23 is taken off the upper part, as 512.  kRecMidAdd: plus an addend per channel, split alike.
+//   kRec64:    everything else.
+// An output costs a warp about 12 clocks of dispatch beside this; in 32 bits it adds 5, kRecMid 9, in 64 bits 23 (two 64-bit
+// multiply-adds, the addend's 64 bits, two conversions).  Maps of five levels, ResNet-50 shape,
+// batch 128: 4753 -> 4645 us; MobileNet-v2 shape, 8 bits, batch 64: 1042 -> 1013.
+enum Recombine { kRec64, kRec32, kRec32Add, kRecMid, kRecMidAdd };
+__host__ __device__ constexpr bool folds_all(int W) { return W == kRec32 || W == kRec32Add; }
+__host__ __device__ constexpr bool is_mid(int W) { return W == kRecMid || W == kRecMidAdd; }
+__host__ __device__ constexpr bool has_addend(int W) { return W == kRec32Add || W == kRecMidAdd || W == kRec64; }
+
+// A channel's addend as the output loop of the kind wants it in its eight bytes: 64 bits, or two words.
+template <int W>
+__device__ __forceinline__ long long addend_words(long long c) {
+  if (W == kRecMidAdd) return (long long)(((unsigned long long)(uint32_t)((int)(c >> 14) - 512) << 32) | (uint32_t)(c & 0x3FFF));
+  return c;
+}
+
 struct EpiConst {
   float res_scale, inv_step, lo_f, hi_f;   // lo_f already holds the relu (see the epilogue set-up)
   uint32_t out_signed;
@@ -353,7 +376,7 @@ __device__ __forceinline__ uint32_t pack_sat_s8(int a, int b, uint32_t c) {
 }
 
 // RES: 0 no shortcut, 1 unsigned shortcut bytes, 2 signed ones.
-template <int P, bool W32, int RES, bool FAST_U8>
+template <int P, int W, int RES, bool FAST_U8>
 __device__ __forceinline__ uint4 chunk_math(const uint32_t (&v)[P][16], const uint4& r4, const float2* scb,
                                             const long long* corr, const EpiConst& c) {
   const uint32_t rw[4] = {r4.x, r4.y, r4.z, r4.w};
@@ -366,11 +389,22 @@ __device__ __forceinline__ uint4 chunk_math(const uint32_t (&v)[P][16], const ui
     for (int e = 0; e < 4; ++e) {
       const int j = 4 * g + e;
       float af;
-      if (W32) {
+      if (folds_all(W)) {
         int acc = (int)v[0][j];
 #pragma unroll
         for (int pl = 1; pl < P; ++pl) acc += (int)v[pl][j] << (kDigitBits * pl);
+        if (W == kRec32Add) acc += reinterpret_cast<const int2*>(corr)[j].x;
         af = __int2float_rn(acc);
+      } else if (is_mid(W)) {          // v[0] = v0 + 2^7 v1 (load_chunk)
+        constexpr int top = P > 2 ? 2 : 0;
+        int t = (int)v[0][j], hi = (int)v[top][j] - 512;
+        if (W == kRecMidAdd) {
+          const int2 c2 = reinterpret_cast<const int2*>(corr)[j];
+          t += c2.x;
+          hi = (int)v[top][j] + c2.y;
+        }
+        hi += t >> 14;
+        af = __fmaf_rn(__int2float_rn(hi), 16384.0f, __uint_as_float(((uint32_t)t & 0x3FFFu) | 0x4B000000u));
       } else {
         long long acc = (long long)(int)v[0][j];
 #pragma unroll
@@ -488,9 +522,17 @@ __device__ __noinline__ void store_narrow16(uint8_t* base, long long off, uint32
 // folded as they arrive (v0 + 2^7 v1 + ..., what chunk_math computes first anyway): 32 registers at the
 // peak instead of 16 P, which is what the loop around it was spilling.  The folded planes are left as
 // literal zeros, so the arithmetic after them drops out.
-template <int P, bool W32>
+template <int P, int W>
 __device__ __forceinline__ void load_chunk(uint32_t taddr, uint32_t (&v)[P][16]) {
-  if (P >= 3 && W32) {
+  if (P >= 3 && is_mid(W)) {
+    tc_ld16(taddr, v[0]);
+    tc_ld16(taddr + kTileN, v[1]);
+    tc_wait_ld();
+    tc_ld16(taddr + 2 * kTileN, v[2]);
+#pragma unroll
+    for (int j = 0; j < 16; ++j) v[0][j] = (uint32_t)((int)v[0][j] + ((int)v[1][j] << kDigitBits));
+    tc_wait_ld();
+  } else if (P >= 3 && folds_all(W)) {
     tc_ld16(taddr, v[0]);
     tc_ld16(taddr + kTileN, v[1]);
     tc_wait_ld();
@@ -529,9 +571,10 @@ __device__ __noinline__ void epilogue_chunk_q(uint32_t taddr, bool valid, uint8_
                                               uint32_t unit, uint32_t count, const float2* scb, const long long* corr,
                                               const int32_t* corr32, EpiConst c) {
   uint32_t v[P][16];
-  load_chunk<P, W32>(taddr, v);
+  constexpr int W = W32 ? kRec32 : kRec64;
+  load_chunk<P, W>(taddr, v);
   if (W32 && corr32) add_corr32(corr32, v[0]);
-  const uint4 q = chunk_math<P, W32, RES, false>(v, r4, scb, corr, c);
+  const uint4 q = chunk_math<P, W, RES, false>(v, r4, scb, corr, c);
   if (unit < 8u) store_narrow16(q_out, valid ? (long long)off : -1ll, unit, count, q);
   else if (valid) store_row16(q_out + off, q, unit == 16u, count >= 16u);
 }
@@ -698,12 +741,12 @@ struct RowMapSorted {
 // buffer back at once (the MMA of the tile after next can start), then do the arithmetic and
 // the store.  Shortcut bytes are fetched one tile ahead.  RM maps the rows of a tile to output
 // locations (plain tiles or band mode).  Returns true if a wait timed out.
-template <int P, bool W32, int RES, bool FAST_U8, typename RM>
+template <int P, int W, int RES, bool FAST_U8, typename RM>
 __device__ __noinline__ bool epilogue_uniform(const TensorParams& p, SharedCtl* ctl, uint32_t tmem_base,
                                               uint32_t ew, uint32_t lane, EpiConst c) {
   constexpr bool HAS_RES = RES != 0;
   // every instance of this loop gets its own instance of the out-of-line planar helpers (see load_planar16)
-  constexpr int TAG = (((P * 2 + (W32 ? 1 : 0)) * 3 + RES) * 2 + (FAST_U8 ? 1 : 0)) * 2 + RM::kTag;
+  constexpr int TAG = (((P * 5 + W) * 3 + RES) * 2 + (FAST_U8 ? 1 : 0)) * 3 + RM::kTag;
   const ConvArgs& a = p.a;
   const uint32_t quarter = ew & 3u, sub = ew >> 2;
   const uint32_t row = quarter * 32u + lane;
@@ -790,10 +833,10 @@ __device__ __noinline__ bool epilogue_uniform(const TensorParams& p, SharedCtl* 
         if (o < a.O) {
           sb.x = ldexpf(a.scale[o], a.e_base[o] - (int)l);
           sb.y = a.bias[o];
-          if (use_corr) cr = p.corr[l][o];
+          if (has_addend(W) && use_corr) cr = p.corr[l][o];
         }
         ctl->scb[ew][lane] = sb;
-        ctl->corr[ew][lane] = cr;
+        if (has_addend(W)) ctl->corr[ew][lane] = addend_words<W>(cr);
       }
       cur_o_tile = kSorted ? o_tile * 8u + l : o_tile;
       __syncwarp();
@@ -815,7 +858,7 @@ __device__ __noinline__ bool epilogue_uniform(const TensorParams& p, SharedCtl* 
     uint32_t v[P][16];
     if (active) {
       const uint32_t taddr = tmem_base + buf * kTmemBufStride + ((quarter * 32u) << 16) + sub * 16u;
-      load_chunk<P, W32>(taddr, v);
+      load_chunk<P, W>(taddr, v);
     }
     // the chunk is in registers: give the accumulator buffer back before doing the arithmetic
     tc_fence_before();
@@ -830,7 +873,7 @@ __device__ __noinline__ bool epilogue_uniform(const TensorParams& p, SharedCtl* 
       }
     }
     if (active && row_valid) {
-      const uint4 q16 = chunk_math<P, W32, RES, FAST_U8>(v, r_cur, scb, corr, c);
+      const uint4 q16 = chunk_math<P, W, RES, FAST_U8>(v, r_cur, scb, corr, c);
       uint8_t* dst = q_base + rm.offset(m, o_base);
       if (planar) store_planar16<TAG>(dst, ohow, rm.O - o_base, q16);
       else store_row16(dst, q16, vec16, o_base + 16u <= rm.O);
@@ -863,7 +906,7 @@ __device__ __forceinline__ void load_folded(uint32_t taddr, uint32_t (&a)[1][16]
 // buffer of its parity, a warp taking 32 rows x 32 channels, so that the bookkeeping of a tile is spent on twice as many
 // outputs.  1x1 64 -> 256 channels @56 with a shortcut, batch 64: 55.4 -> 40.3 us (staged without the groups 48.4; 17.7 us
 // at memory rate).
-template <int P, bool W32, int RES, bool FAST_U8>
+template <int P, int W, int RES, bool FAST_U8>
 __device__ __noinline__ bool epilogue_staged(const TensorParams& p, SharedCtl* ctl, uint32_t tmem_base, uint32_t slots_addr,
                                              uint32_t ew, uint32_t lane, EpiConst c) {
   const ConvArgs& a = p.a;
@@ -897,10 +940,10 @@ __device__ __noinline__ bool epilogue_staged(const TensorParams& p, SharedCtl* c
       if (o < O) {
         sb.x = ldexpf(a.scale[o], a.e_base[o] - (int)l);
         sb.y = a.bias[o];
-        if (use_corr) cr = p.corr[l][o];
+        if (has_addend(W) && use_corr) cr = p.corr[l][o];
       }
       ctl->scb[ew][lane] = sb;
-      if (!W32) ctl->corr[ew][lane] = cr;
+      if (has_addend(W)) ctl->corr[ew][lane] = addend_words<W>(cr);
       cur_o_tile = o_tile;
       __syncwarp();
     }
@@ -921,7 +964,7 @@ __device__ __noinline__ bool epilogue_staged(const TensorParams& p, SharedCtl* c
     auto store = [&](uint32_t at, uint4 q) {
       asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(q.x), "r"(q.y), "r"(q.z), "r"(q.w) : "memory");
     };
-    if (W32) {
+    if (folds_all(W)) {
       uint32_t a0[1][16], a1[1][16];
       if (active) {
         load_folded<P>(taddr, a0);
@@ -931,20 +974,20 @@ __device__ __noinline__ bool epilogue_staged(const TensorParams& p, SharedCtl* c
       ok = mbar_wait(ready0 + 8u * slot, (n >> 1) & 1u, abort, 32);
       if (__any_sync(0xFFFFFFFFu, !ok)) return true;
       if (active) {
-        store(addr + piece[0], chunk_math<1, true, RES, FAST_U8>(a0, shortcut(addr + piece[0]), scb, corr, c));
-        store(addr + piece[1], chunk_math<1, true, RES, FAST_U8>(a1, shortcut(addr + piece[1]), scb + 16, corr + 16, c));
+        store(addr + piece[0], chunk_math<1, W, RES, FAST_U8>(a0, shortcut(addr + piece[0]), scb, corr, c));
+        store(addr + piece[1], chunk_math<1, W, RES, FAST_U8>(a1, shortcut(addr + piece[1]), scb + 16, corr + 16, c));
       }
     } else {
       ok = mbar_wait(ready0 + 8u * slot, (n >> 1) & 1u, abort, 32);
       if (__any_sync(0xFFFFFFFFu, !ok)) return true;
       uint32_t v[P][16];
       if (active) {
-        load_chunk<P, false>(taddr, v);
-        store(addr + piece[0], chunk_math<P, false, RES, FAST_U8>(v, shortcut(addr + piece[0]), scb, corr, c));
-        load_chunk<P, false>(taddr + 16u, v);
+        load_chunk<P, W>(taddr, v);
+        store(addr + piece[0], chunk_math<P, W, RES, FAST_U8>(v, shortcut(addr + piece[0]), scb, corr, c));
+        load_chunk<P, W>(taddr + 16u, v);
       }
       release();
-      if (active) store(addr + piece[1], chunk_math<P, false, RES, FAST_U8>(v, shortcut(addr + piece[1]), scb + 16, corr + 16, c));
+      if (active) store(addr + piece[1], chunk_math<P, W, RES, FAST_U8>(v, shortcut(addr + piece[1]), scb + 16, corr + 16, c));
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncwarp();
@@ -961,7 +1004,7 @@ __device__ __noinline__ bool epilogue_staged(const TensorParams& p, SharedCtl* c
 // by the instructions of the 64-bit recombination and by L2 sectors; with a row per lane, every load and store touched 32
 // lines for 16 bytes each (ResNet-50 shape, batch 128, maps of five levels: 5401 -> 4853 us, layers with a shortcut and
 // without; its attention mode, batch 32 in the second pass: 3109 -> 2980 us).
-template <int P, bool W32, int RES, bool FAST_U8>
+template <int P, int W, int RES, bool FAST_U8>
 __device__ __noinline__ bool epilogue_sorted(const TensorParams& p, SharedCtl* ctl, uint32_t tmem_base, uint32_t slots_addr,
                                              uint32_t ew, uint32_t lane, EpiConst c) {
   const ConvArgs& a = p.a;
@@ -1042,10 +1085,10 @@ __device__ __noinline__ bool epilogue_sorted(const TensorParams& p, SharedCtl* c
       if (o < O) {
         sb.x = ldexpf(a.scale[o], a.e_base[o] - (int)l);
         sb.y = a.bias[o];
-        if (use_corr) cr = p.corr[l][o];
+        if (has_addend(W) && use_corr) cr = p.corr[l][o];
       }
       ctl->scb[ew][lane] = sb;
-      if (!W32) ctl->corr[ew][lane] = cr;
+      if (has_addend(W)) ctl->corr[ew][lane] = addend_words<W>(cr);
       cur_key = o_tile * 8u + l;
       __syncwarp();
     }
@@ -1075,7 +1118,7 @@ __device__ __noinline__ bool epilogue_sorted(const TensorParams& p, SharedCtl* c
       asm volatile("cp.async.wait_group 1;" ::: "memory");       // this tile's
       __syncwarp();
     };
-    if (W32) {
+    if (folds_all(W)) {
       uint32_t a0[1][16], a1[1][16];
       if (active) {
         load_folded<P>(taddr, a0);
@@ -1084,19 +1127,19 @@ __device__ __noinline__ bool epilogue_sorted(const TensorParams& p, SharedCtl* c
       release();
       arrive_shortcut();
       if (active) {
-        put(slot_addr + own[0], chunk_math<1, true, RES, FAST_U8>(a0, shortcut(slot_addr + own[0]), scb, corr, c));
-        put(slot_addr + own[1], chunk_math<1, true, RES, FAST_U8>(a1, shortcut(slot_addr + own[1]), scb + 16, corr + 16, c));
+        put(slot_addr + own[0], chunk_math<1, W, RES, FAST_U8>(a0, shortcut(slot_addr + own[0]), scb, corr, c));
+        put(slot_addr + own[1], chunk_math<1, W, RES, FAST_U8>(a1, shortcut(slot_addr + own[1]), scb + 16, corr + 16, c));
       }
     } else {
       arrive_shortcut();
       uint32_t v[P][16];
       if (active) {
-        load_chunk<P, false>(taddr, v);
-        put(slot_addr + own[0], chunk_math<P, false, RES, FAST_U8>(v, shortcut(slot_addr + own[0]), scb, corr, c));
-        load_chunk<P, false>(taddr + 16u, v);
+        load_chunk<P, W>(taddr, v);
+        put(slot_addr + own[0], chunk_math<P, W, RES, FAST_U8>(v, shortcut(slot_addr + own[0]), scb, corr, c));
+        load_chunk<P, W>(taddr + 16u, v);
       }
       release();
-      if (active) put(slot_addr + own[1], chunk_math<P, false, RES, FAST_U8>(v, shortcut(slot_addr + own[1]), scb + 16, corr + 16, c));
+      if (active) put(slot_addr + own[1], chunk_math<P, W, RES, FAST_U8>(v, shortcut(slot_addr + own[1]), scb + 16, corr + 16, c));
     }
     __syncwarp();
 #pragma unroll
@@ -1146,38 +1189,52 @@ __device__ __noinline__ bool io_role(const TensorParams& p, const TmapSet& maps,
 }
 
 // Run-time options of the uniform output stage -> template instance.
-template <int P, bool W32, int RES, bool kSorted>
+struct EpiChoice {
+  bool fast_u8;
+  uint32_t res;       // 0 no shortcut, 1 unsigned, 2 signed bytes
+  int rec;            // Recombine
+};
+template <int P, int W, int RES, bool kSorted>
 __device__ __forceinline__ bool uniform_dispatch_tail(const TensorParams& p, SharedCtl* ctl, uint32_t tmem_base,
                                                       uint32_t slots_addr, uint32_t ew, uint32_t lane, const EpiConst& c,
                                                       bool fast_u8) {
+  // band mode and staged outputs never meet flipped activations, and so no addend
+  constexpr bool kFlipped = W == kRec32Add || W == kRecMidAdd;
   if constexpr (kSorted) {
     if (p.staged)
-      return fast_u8 ? epilogue_sorted<P, W32, RES, true>(p, ctl, tmem_base, slots_addr, ew, lane, c)
-                     : epilogue_sorted<P, W32, RES, false>(p, ctl, tmem_base, slots_addr, ew, lane, c);
-    return fast_u8 ? epilogue_uniform<P, W32, RES, true, RowMapSorted>(p, ctl, tmem_base, ew, lane, c)
-                   : epilogue_uniform<P, W32, RES, false, RowMapSorted>(p, ctl, tmem_base, ew, lane, c);
+      return fast_u8 ? epilogue_sorted<P, W, RES, true>(p, ctl, tmem_base, slots_addr, ew, lane, c)
+                     : epilogue_sorted<P, W, RES, false>(p, ctl, tmem_base, slots_addr, ew, lane, c);
+    return fast_u8 ? epilogue_uniform<P, W, RES, true, RowMapSorted>(p, ctl, tmem_base, ew, lane, c)
+                   : epilogue_uniform<P, W, RES, false, RowMapSorted>(p, ctl, tmem_base, ew, lane, c);
   }
-  if (RES && p.staged)
-    return fast_u8 ? epilogue_staged<P, W32, RES ? RES : 1, true>(p, ctl, tmem_base, slots_addr, ew, lane, c)
-                   : epilogue_staged<P, W32, RES ? RES : 1, false>(p, ctl, tmem_base, slots_addr, ew, lane, c);
-  if (p.band)
-    return fast_u8 ? epilogue_uniform<P, W32, RES, true, RowMapBand>(p, ctl, tmem_base, ew, lane, c)
-                   : epilogue_uniform<P, W32, RES, false, RowMapBand>(p, ctl, tmem_base, ew, lane, c);
-  return fast_u8 ? epilogue_uniform<P, W32, RES, true, RowMap>(p, ctl, tmem_base, ew, lane, c)
-                 : epilogue_uniform<P, W32, RES, false, RowMap>(p, ctl, tmem_base, ew, lane, c);
+  if constexpr (!kFlipped) {
+    if (RES && p.staged)
+      return fast_u8 ? epilogue_staged<P, W, RES ? RES : 1, true>(p, ctl, tmem_base, slots_addr, ew, lane, c)
+                     : epilogue_staged<P, W, RES ? RES : 1, false>(p, ctl, tmem_base, slots_addr, ew, lane, c);
+    if (p.band)
+      return fast_u8 ? epilogue_uniform<P, W, RES, true, RowMapBand>(p, ctl, tmem_base, ew, lane, c)
+                     : epilogue_uniform<P, W, RES, false, RowMapBand>(p, ctl, tmem_base, ew, lane, c);
+  }
+  return fast_u8 ? epilogue_uniform<P, W, RES, true, RowMap>(p, ctl, tmem_base, ew, lane, c)
+                 : epilogue_uniform<P, W, RES, false, RowMap>(p, ctl, tmem_base, ew, lane, c);
+}
+template <int P, int W, bool kSorted>
+__device__ __forceinline__ bool uniform_dispatch_res(const TensorParams& p, SharedCtl* ctl, uint32_t tmem_base, uint32_t slots_addr,
+                                                     uint32_t ew, uint32_t lane, const EpiConst& c, const EpiChoice& how) {
+  if (how.res == 0u) return uniform_dispatch_tail<P, W, 0, kSorted>(p, ctl, tmem_base, slots_addr, ew, lane, c, how.fast_u8);
+  if (how.res == 1u) return uniform_dispatch_tail<P, W, 1, kSorted>(p, ctl, tmem_base, slots_addr, ew, lane, c, how.fast_u8);
+  return uniform_dispatch_tail<P, W, 2, kSorted>(p, ctl, tmem_base, slots_addr, ew, lane, c, how.fast_u8);
 }
 template <int P, bool kSorted>
 __device__ __forceinline__ bool uniform_dispatch(const TensorParams& p, SharedCtl* ctl, uint32_t tmem_base, uint32_t slots_addr,
-                                                 uint32_t ew, uint32_t lane, const EpiConst& c, bool fast_u8,
-                                                 bool w32, uint32_t res) {
-  if (w32) {
-    if (res == 0u) return uniform_dispatch_tail<P, true, 0, kSorted>(p, ctl, tmem_base, slots_addr, ew, lane, c, fast_u8);
-    if (res == 1u) return uniform_dispatch_tail<P, true, 1, kSorted>(p, ctl, tmem_base, slots_addr, ew, lane, c, fast_u8);
-    return uniform_dispatch_tail<P, true, 2, kSorted>(p, ctl, tmem_base, slots_addr, ew, lane, c, fast_u8);
+                                                 uint32_t ew, uint32_t lane, const EpiConst& c, const EpiChoice& how) {
+  if (how.rec == kRec32) return uniform_dispatch_res<P, kRec32, kSorted>(p, ctl, tmem_base, slots_addr, ew, lane, c, how);
+  if constexpr (P == 3) {
+    if (how.rec == kRec32Add) return uniform_dispatch_res<P, kRec32Add, kSorted>(p, ctl, tmem_base, slots_addr, ew, lane, c, how);
+    if (how.rec == kRecMid) return uniform_dispatch_res<P, kRecMid, kSorted>(p, ctl, tmem_base, slots_addr, ew, lane, c, how);
+    if (how.rec == kRecMidAdd) return uniform_dispatch_res<P, kRecMidAdd, kSorted>(p, ctl, tmem_base, slots_addr, ew, lane, c, how);
   }
-  if (res == 0u) return uniform_dispatch_tail<P, false, 0, kSorted>(p, ctl, tmem_base, slots_addr, ew, lane, c, fast_u8);
-  if (res == 1u) return uniform_dispatch_tail<P, false, 1, kSorted>(p, ctl, tmem_base, slots_addr, ew, lane, c, fast_u8);
-  return uniform_dispatch_tail<P, false, 2, kSorted>(p, ctl, tmem_base, slots_addr, ew, lane, c, fast_u8);
+  return uniform_dispatch_res<P, kRec64, kSorted>(p, ctl, tmem_base, slots_addr, ew, lane, c, how);
 }
 
 // All lanes of the warp wait together; false when a wait ran out.
@@ -1567,17 +1624,22 @@ psb_mma_kernel(const __grid_constant__ TmapSet maps, const __grid_constant__ Ten
     const uint32_t bounded = a.kmap ? a.level_mask : 1u << a.uniform_log2k;
     find_row_maxima(p, ctl, kKind != kGeneralOutputs || q_only ? bounded : 0u);
     if constexpr (kKind != kGeneralOutputs) {
-      // (an integer addend takes the 64-bit loop here: a branch for it in the 32-bit one cost every layer 1 %)
-      bool w32 = p.corr[(uint32_t)__ffs((int)(a.level_mask & 0x7Fu)) - 1u] == nullptr;
+      const bool addend = p.corr[(uint32_t)__ffs((int)(a.level_mask & 0x7Fu)) - 1u] != nullptr;
+      bool w32 = true;
       if (kSorted) {         // every level a tile may have must fit
         for (uint32_t lv = 0; lv < (uint32_t)kMaxLevels; ++lv)
           if ((a.level_mask >> lv) & 1u) w32 = fits_32_bits(p, ctl, lv) && w32;
       } else {
-        w32 = fits_32_bits(p, ctl, a.uniform_log2k) && w32;
+        w32 = fits_32_bits(p, ctl, a.uniform_log2k);
       }
-      if (P0 == 4u) failed = uniform_dispatch<4, kSorted>(p, ctl, tmem_base, slots_addr, ew, lane, ec, fast_u8, w32, res_kind);
-      else if (P0 == 3u) failed = uniform_dispatch<3, kSorted>(p, ctl, tmem_base, slots_addr, ew, lane, ec, fast_u8, w32, res_kind);
-      else failed = uniform_dispatch<2, kSorted>(p, ctl, tmem_base, slots_addr, ew, lane, ec, fast_u8, w32, res_kind);
+      EpiChoice how;
+      how.fast_u8 = fast_u8;
+      how.res = res_kind;
+      how.rec = w32 ? (addend ? kRec32Add : kRec32) : !p.mid ? kRec64 : addend ? kRecMidAdd : kRecMid;
+      if (P0 != 3u && how.rec != kRec32) how.rec = kRec64;
+      if (P0 == 4u) failed = uniform_dispatch<4, kSorted>(p, ctl, tmem_base, slots_addr, ew, lane, ec, how);
+      else if (P0 == 3u) failed = uniform_dispatch<3, kSorted>(p, ctl, tmem_base, slots_addr, ew, lane, ec, how);
+      else failed = uniform_dispatch<2, kSorted>(p, ctl, tmem_base, slots_addr, ew, lane, ec, how);
     } else {
       // general loop: per-location draw counts, any outputs and layouts, ragged channel counts
       const float2* scb = ctl->scb[ew];

@@ -183,6 +183,8 @@ psb_status launch_tensor(psb_ctx* ctx, const psb_weights* wt, const ConvArgs& a,
   for (int l = 0; l < kMaxLevels; ++l) p.corr[l] = add_corr128 && wt->level[l].planes ? wt->corr128 + (size_t)l * a.O : nullptr;
   p.rowsum256 = wt->rowsum256;
   p.amax = amax;
+  // the lower two digits of a weight are at most 16383 together; the bytes fed are at most 128 where an offset is taken off
+  p.mid = (uint64_t)wt->d * (add_corr128 ? 128u : amax) * 16383ull + 16383ull < (1ull << 31) ? 1u : 0u;
   const CUtensorMapSwizzle swz = swizzle_for(bk);
   EncodeTiledFn enc_tiled = (EncodeTiledFn)ctx->encode_tiled;
   EncodeIm2colFn enc_im2col = (EncodeIm2colFn)ctx->encode_im2col;

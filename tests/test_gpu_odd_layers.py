@@ -240,3 +240,55 @@ def test_line_between_the_paths(case, oracle):
     compare(g, oracle_layer(oracle, *args), list(levels or (3,)))
     assert g["path"] == (psb.PSB_PATH_TENSOR if tensor else psb.PSB_PATH_SHIFT_ADD)
     ctx.close()
+
+
+@pytest.mark.parametrize("case", [
+    # (channels, largest byte, signed input, shortcut, draw-count map): sums whose lower two planes fit 32 bits, at the limit
+    # (16383 x channels x byte just below 2^31) and just beyond it, with and without an addend, and sums that fit as a whole
+    (1024, 255, False, False, False), (1040, 255, False, False, False), (1024, 255, False, True, True), (1024, 127, True, True, False),
+    (8736, 15, False, False, False), (8752, 15, False, True, False), (960, 255, False, True, False), (8736, 15, False, True, True),
+    (16, 255, False, True, False), (16, 255, False, False, True), (1040, 255, False, True, True),
+])
+def test_large_sums_are_rounded_once(case, oracle):
+    """Accumulators near 2^36 that differ by a few units in the last place of their fp32 value: codes show each of them."""
+    import torch
+
+    import paper_1904_02205_b200 as psb
+
+    C, amax, signed, shortcut, with_map = case
+    ctx = psb.Context(0)
+    rng = np.random.default_rng(C + amax)
+    O, H, W = 80, 15, 20
+    # a third of the weights small: their activations vary, the others' do not
+    small = rng.random(C) < 0.34
+    small[0] = False
+    exps = np.where(small, rng.integers(-15, -6, size=(O, C)), rng.integers(-2, 1, size=(O, C)))
+    exps[:, 0] = 0
+    w = (np.exp2(exps) * (1.0 + rng.random((O, C)))).astype(np.float32).reshape(O, C, 1, 1)
+    dt = np.int8 if signed else np.uint8
+    x = np.where(small, rng.integers(0, amax + 1, size=(1, H, W, C)), amax).astype(dt)
+    res = rng.integers(0, 4, size=(1, H, W, O)).astype(np.uint8) if shortcut else None
+    levels = (2, 4) if with_map else (4,)
+    kmap = rng.choice(levels, size=(1, H, W)).astype(np.uint8) if with_map else None
+    Ws = {l: oracle.sample_level(w, 3, 0, l)[0] for l in levels}
+    eb = oracle.sample_level(w, 3, 0, 4)[1]
+    g = oracle.geom(x.shape, oracle.NHWC, oracle.S8 if signed else oracle.U8, w.shape, 1, 1, 0)
+    acc = oracle.conv_acc(x, g, Ws, kmap=kmap, uniform_log2k=4)
+    scale = np.exp2(4.0 - eb.astype(np.float64)).astype(np.float32)
+    mid = np.median(acc.reshape(-1, O) if kmap is None else acc.reshape(-1, O)[kmap.ravel() == 4], axis=0)
+    bias = (-mid.astype(np.float32)).astype(np.float32)
+    step = max(1.0, float(np.exp2(np.floor(np.log2(mid.max())) - 23)))
+    inv_step = np.float32(1.0 / step)
+    _, q = oracle.epilogue(acc, g, scale, bias, eb, False, inv_step, -128, 127, kmap=kmap, uniform_log2k=4, residual=res,
+                           residual_scale=np.float32(step))
+    assert len(np.unique(q)) > 50
+    cu = lambda a: None if a is None else torch.from_numpy(a).to(ctx.device)
+    wt = ctx.sample_weights(cu(w), seed=3, layer_id=0, level_mask=sum(1 << l for l in levels))
+    ctx.set_sample_map(cu(kmap), 4)
+    got = ctx.conv2d(wt, cu(x), psb.PSB_LAYOUT_NHWC, 1, 0, cu(scale), cu(bias), False, float(inv_step), -128, 127, out_dtype=psb.PSB_DT_S8,
+                     residual=cu(res), residual_scale=step, in_max=amax, path=psb.PSB_PATH_TENSOR, want=("q",))["q"]
+    assert ctx.device_status() == 0
+    assert np.array_equal(got.cpu().numpy().astype(np.int32), q)
+    ctx.set_sample_map(None, 4)
+    wt.free()
+    ctx.close()
