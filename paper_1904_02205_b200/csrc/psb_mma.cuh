@@ -83,6 +83,7 @@ struct TensorParams {
   uint32_t resident_bytes;
   const uint32_t* rowsum256;   // [level][O] row sums of |W_k| in units of 256 (rounded up), or null
   uint32_t amax;        // largest activation magnitude the caller vouches for
+  uint32_t real_slots;  // 1: real-valued rows pass through shared memory (epilogue_chunk_real), 2 KB per epilogue warp
   uint32_t mid;         // 1: two digit planes fit 32 bits together (kRecMid)
   const long long* corr[kMaxLevels];  // per-channel integer addend, or null
   const int8_t* planes_ptr[kMaxLevels];  // digit planes: [o_tile][K block][P * 64 rows][BK], pre-swizzled tiles
@@ -628,6 +629,125 @@ __device__ __noinline__ void epilogue_chunk(const TensorParams& p, uint32_t tadd
     *reinterpret_cast<uint4*>((uint8_t*)a.q_out + (size_t)m * a.O + o_base) = make_uint4(qw[0], qw[1], qw[2], qw[3]);
 }
 
+// Real-valued outputs, codes beside them if wanted, any layout and channel count: 16 channels of one location per lane, the same
+// arithmetic as dequant() and requant() (the clamp to whole numbers before the rounding instead of after it).  Channels-last rows
+// of whole 16-byte pieces pass through a slot of the warp's own in shared memory, so that four lanes store the 64 bytes of
+// a row together (a row per lane touches 32 cache lines per instruction).
+// us, one output at a time in a rolled loop / so, codes and fp32: 3x3 64->64 @56 batch 32 142 / 27.7 (codes only 11.8), 3x3
+// stride 2 120->544 @89 batch 26 519 / 161, 1x1 336->176 planar 38 / 16; fp32 alone, 2048->1000 features, 512 rows 25 / 11.
+struct RealOut {
+  float* f32;
+  uint8_t* q;            // or null
+  const uint8_t* res;    // or null
+  uint32_t O, ohow, slot;
+  bool planar, vec, relu, res_signed;
+  float res_scale, inv_step, lo, hi;
+  __device__ __forceinline__ RealOut(const TensorParams& p, uint32_t warp_slot) {
+    const ConvArgs& a = p.a;
+    f32 = a.f32_out; q = (uint8_t*)a.q_out; res = (const uint8_t*)a.residual;
+    O = a.O; ohow = a.OH * a.OW; slot = warp_slot;
+    planar = a.out_nchw != 0u; vec = p.real_slots != 0u; relu = a.relu != 0u; res_signed = a.residual_dtype == PSB_DT_S8;
+    res_scale = a.residual_scale; inv_step = a.inv_step; lo = (float)a.qmin; hi = (float)a.qmax;
+  }
+  __device__ __forceinline__ size_t offset(uint32_t m, uint32_t o_base) const {
+    if (!planar) return (size_t)m * O + o_base;
+    const uint32_t n = m / ohow;
+    return ((size_t)n * O + o_base) * ohow + (m - n * ohow);
+  }
+};
+
+// The shortcut bytes of a lane's 16 channels.
+__device__ __forceinline__ void load_real_shortcut(const RealOut& r, size_t at, uint32_t count, uint32_t (&rw)[4]) {
+#pragma unroll
+  for (int g = 0; g < 4; ++g) {
+    rw[g] = 0u;
+    if ((uint32_t)(4 * g) >= count) break;
+    if (r.vec) {
+      rw[g] = *reinterpret_cast<const uint32_t*>(r.res + at + 4 * g);
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if ((uint32_t)(4 * g + e) < count) rw[g] |= (uint32_t)r.res[at + (size_t)(4 * g + e) * (r.planar ? r.ohow : 1u)] << (8 * e);
+    }
+  }
+}
+
+template <int P, int W>
+__device__ __forceinline__ void store_real(const RealOut& r, const uint32_t (&v)[P][16], const uint32_t (&rw)[4], uint32_t o_base, uint32_t m,
+                                           bool valid, const float2* scb, const long long* corr) {
+  const uint32_t count = min(16u, r.O - o_base), lane = threadIdx.x & 31u;
+  const size_t at = r.offset(m, o_base), step = r.planar ? r.ohow : 1u;
+#pragma unroll
+  for (int g = 0; g < 4; ++g) {
+    if ((uint32_t)(4 * g) >= count) break;
+    float y[4];
+    uint32_t code = 0u;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int j = 4 * g + e;
+      float af;
+      if (is_mid(W)) {
+        const int2 c2 = reinterpret_cast<const int2*>(corr)[j];
+        const int t = (int)v[0][j] + c2.x;
+        af = __fmaf_rn(__int2float_rn((int)v[P > 2 ? 2 : 0][j] + (t >> 14) + c2.y), 16384.0f,
+                       __uint_as_float(((uint32_t)t & 0x3FFFu) | 0x4B000000u));
+      } else {
+        long long acc = (long long)(int)v[0][j] + corr[j];
+#pragma unroll
+        for (int pl = 1; pl < P; ++pl) acc += (long long)(int)v[pl][j] * (long long)(1 << (kDigitBits * pl));
+        af = __ll2float_rn(acc);
+      }
+      const float2 sb = scb[j];
+      y[e] = __fmaf_rn(af, sb.x, sb.y);
+      if (r.res) {
+        const uint32_t rb = (rw[g] >> (8 * e)) & 0xFFu;
+        y[e] = __fmaf_rn(r.res_signed ? (float)(int)(signed char)rb : (float)rb, r.res_scale, y[e]);
+      }
+      if (r.relu) y[e] = fmaxf(y[e], 0.0f);
+      code |= ((uint32_t)__float2int_rn(fminf(fmaxf(__fmul_rn(y[e], r.inv_step), r.lo), r.hi)) & 0xFFu) << (8 * e);
+    }
+    if (r.vec) {
+      // pieces permuted by the row, against bank conflicts both ways
+      asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(r.slot + lane * 64u + (((uint32_t)g ^ (lane >> 1)) & 3u) * 16u),
+                   "f"(y[0]), "f"(y[1]), "f"(y[2]), "f"(y[3]) : "memory");
+      if (r.q && valid) *reinterpret_cast<uint32_t*>(r.q + at + 4 * g) = code;
+    } else if (valid) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if ((uint32_t)(4 * g + e) < count) {
+          r.f32[at + (size_t)(4 * g + e) * step] = y[e];
+          if (r.q) r.q[at + (size_t)(4 * g + e) * step] = (uint8_t)(code >> (8 * e));
+        }
+    }
+  }
+  if (r.vec) {
+    __syncwarp();
+    const uint32_t piece = lane & 3u;
+#pragma unroll
+    for (uint32_t i = 0; i < 4u; ++i) {
+      const uint32_t row = 8u * i + (lane >> 2);
+      const uint32_t mm = __shfl_sync(0xFFFFFFFFu, m, (int)row);
+      const int ok = __shfl_sync(0xFFFFFFFFu, valid ? 1 : 0, (int)row);
+      float4 y;
+      asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(y.x), "=f"(y.y), "=f"(y.z), "=f"(y.w)
+                   : "r"(r.slot + row * 64u + ((piece ^ (row >> 1)) & 3u) * 16u) : "memory");
+      if (ok && piece * 4u < count) *reinterpret_cast<float4*>(r.f32 + (size_t)mm * r.O + o_base + piece * 4u) = y;
+    }
+    __syncwarp();
+  }
+}
+
+// One chunk of the general loop (draw-count maps).
+template <int P, int W>
+__device__ __noinline__ void epilogue_chunk_real(const TensorParams& p, uint32_t taddr, uint32_t slot, uint32_t o_base, uint32_t m,
+                                                 bool valid, const float2* scb, const long long* corr) {
+  const RealOut r(p, slot);
+  uint32_t v[P][16], rw[4] = {0u, 0u, 0u, 0u};
+  load_chunk<P, W>(taddr, v);
+  if (r.res && valid) load_real_shortcut(r, r.offset(m, o_base), min(16u, r.O - o_base), rw);
+  store_real<P, W>(r, v, rw, o_base, m, valid, scb, corr);
+}
+
 // True when the layer takes the specialised epilogue loop below.
 __host__ __device__ __forceinline__ bool uniform_epilogue(const TensorParams& p) {
   const ConvArgs& a = p.a;
@@ -878,6 +998,59 @@ __device__ __noinline__ bool epilogue_uniform(const TensorParams& p, SharedCtl* 
       if (planar) store_planar16<TAG>(dst, ohow, rm.O - o_base, q16);
       else store_row16(dst, q16, vec16, o_base + 16u <= rm.O);
     }
+    ++pass;
+  }
+  return false;
+}
+
+// The loop for real-valued outputs under one draw count: as epilogue_uniform, the accumulator handed back before the arithmetic.
+template <int P, int W>
+__device__ __noinline__ bool epilogue_real(const TensorParams& p, SharedCtl* ctl, uint32_t tmem_base, uint32_t slots_addr,
+                                           uint32_t ew, uint32_t lane) {
+  const ConvArgs& a = p.a;
+  const RealOut r(p, slots_addr + ew * 2048u);
+  const uint32_t quarter = ew & 3u, sub = ew >> 2, row = quarter * 32u + lane, l = a.uniform_log2k, M = p.M;
+  const bool use_corr = p.corr[l] != nullptr;
+  WaitCtl* abort = &ctl->wait;
+  const float2* scb = ctl->scb[ew];
+  const long long* corr = ctl->corr[ew];
+  TileIter ti;
+  ti.init(p);
+  uint32_t pass = 0, cur_o_tile = 0xFFFFFFFFu;
+  while (ti.valid()) {
+    const uint32_t m = ti.m_tile * kTileM + row, o_tile = ti.o_tile, o_base = o_tile * kTileN + sub * 16u;
+    const bool valid = m < M, active = o_base < r.O;
+    ti.next();
+    if (o_tile != cur_o_tile) {
+      // per-channel constants of this channel tile: the warp keeps its own copy of its 16 channels
+      __syncwarp();
+      if (lane < 16u) {
+        const uint32_t o = o_base + lane;
+        float2 sb = make_float2(0.f, 0.f);
+        long long cr = 0;
+        if (o < r.O) {
+          sb.x = ldexpf(a.scale[o], a.e_base[o] - (int)l);
+          sb.y = a.bias[o];
+          if (use_corr) cr = p.corr[l][o];
+        }
+        ctl->scb[ew][lane] = sb;
+        ctl->corr[ew][lane] = addend_words<W>(cr);
+      }
+      cur_o_tile = o_tile;
+      __syncwarp();
+    }
+    uint32_t rw[4] = {0u, 0u, 0u, 0u};
+    if (r.res && valid && active) load_real_shortcut(r, r.offset(m, o_base), min(16u, r.O - o_base), rw);
+    const uint32_t buf = pass & 1u, aph = (pass >> 1) & 1u;
+    const bool ok = mbar_wait(smem_u32(&ctl->acc_full[buf]), aph, abort, 32);
+    if (__any_sync(0xFFFFFFFFu, !ok)) return true;
+    tc_fence_after();
+    uint32_t v[P][16];
+    if (active) load_chunk<P, W>(tmem_base + buf * kTmemBufStride + ((quarter * 32u) << 16) + sub * 16u, v);
+    tc_fence_before();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(smem_u32(&ctl->acc_empty[buf]));
+    if (active) store_real<P, W>(r, v, rw, o_base, m, valid, scb, corr);
     ++pass;
   }
   return false;
@@ -1442,7 +1615,7 @@ psb_mma_kernel(const __grid_constant__ TmapSet maps, const __grid_constant__ Ten
   const uint32_t stage_bytes = p.band ? p.band_bytes : sub_bytes * p.group;
   // staged outputs: kIoSlots tiles between the ring and the control block
   const uint32_t slots_addr = smem_u32(ring) + p.stages * stage_bytes;
-  SharedCtl* ctl = reinterpret_cast<SharedCtl*>(ring + (size_t)p.stages * stage_bytes + (p.staged ? kIoSlots * kIoTileBytes : 0u));
+  SharedCtl* ctl = reinterpret_cast<SharedCtl*>(ring + (size_t)p.stages * stage_bytes + (p.staged | p.real_slots ? kIoSlots * kIoTileBytes : 0u));
 
   const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u;
   const uint32_t k_iters = p.a.KH * p.a.KW * p.n_cb;
@@ -1645,12 +1818,22 @@ psb_mma_kernel(const __grid_constant__ TmapSet maps, const __grid_constant__ Ten
       const float2* scb = ctl->scb[ew];
       const long long* corr = ctl->corr[ew];
       uint32_t pass = 0, cur_key = 0xFFFFFFFFu;
+      const bool real = a.f32_out && !a.acc_out;
+      bool done = false;
+      if (real && !a.kmap) {
+        done = true;
+        if (P0 == 4u) failed = epilogue_real<4, kRec64>(p, ctl, tmem_base, slots_addr, ew, lane);
+        else if (P0 == 3u && p.mid) failed = epilogue_real<3, kRecMidAdd>(p, ctl, tmem_base, slots_addr, ew, lane);
+        else if (P0 == 3u) failed = epilogue_real<3, kRec64>(p, ctl, tmem_base, slots_addr, ew, lane);
+        else if (P0 == 2u) failed = epilogue_real<2, kRec64>(p, ctl, tmem_base, slots_addr, ew, lane);
+        else failed = epilogue_real<1, kRec64>(p, ctl, tmem_base, slots_addr, ew, lane);
+      }
       uint32_t w32_levels = 0;      // levels whose accumulators are known to fit 32 bits
       if (q_only)
         for (uint32_t l = 0; l < (uint32_t)kMaxLevels; ++l)
           if (((a.level_mask >> l) & 1u) && fits_32_bits(p, ctl, l)) w32_levels |= 1u << l;
       TileIter ti;
-      for (ti.init(p); !failed && ti.valid(); ti.next()) {
+      for (ti.init(p); !done && !failed && ti.valid(); ti.next()) {
         const uint32_t m0 = ti.m_tile * kTileM, o_tile = ti.o_tile;
         const uint32_t levels = tile_levels(p, ti.m_tile) & a.level_mask;
         uint32_t m = m0 + row;
@@ -1688,7 +1871,7 @@ psb_mma_kernel(const __grid_constant__ TmapSet maps, const __grid_constant__ Ten
                 if (use_corr) cr = p.corr[l][o];
               }
               ctl->scb[ew][lane] = sb;
-              ctl->corr[ew][lane] = cr;
+              ctl->corr[ew][lane] = real && p.mid && P == 3u ? addend_words<kRecMidAdd>(cr) : cr;
               ctl->corr32[ew][lane] = (int32_t)cr;
             }
             cur_key = key;
@@ -1720,7 +1903,18 @@ psb_mma_kernel(const __grid_constant__ TmapSet maps, const __grid_constant__ Ten
             } else {
               const uint32_t ohow = a.OH * a.OW;
               const uint32_t n = in_range ? m / ohow : 0u, pix = in_range ? m % ohow : 0u;
-              switch (P) {
+              const uint32_t slot = slots_addr + ew * 2048u;
+              if (real) {
+                switch (P) {
+                  case 1: epilogue_chunk_real<1, kRec64>(p, taddr, slot, o_base, m, valid, scb, corr); break;
+                  case 2: epilogue_chunk_real<2, kRec64>(p, taddr, slot, o_base, m, valid, scb, corr); break;
+                  case 3:
+                    if (p.mid) epilogue_chunk_real<3, kRecMidAdd>(p, taddr, slot, o_base, m, valid, scb, corr);
+                    else epilogue_chunk_real<3, kRec64>(p, taddr, slot, o_base, m, valid, scb, corr);
+                    break;
+                  default: epilogue_chunk_real<4, kRec64>(p, taddr, slot, o_base, m, valid, scb, corr); break;
+                }
+              } else switch (P) {
                 case 1: epilogue_chunk<1>(p, taddr, o_base, m, valid, n, pix, scb, corr, use_corr); break;
                 case 2: epilogue_chunk<2>(p, taddr, o_base, m, valid, n, pix, scb, corr, use_corr); break;
                 case 3: epilogue_chunk<3>(p, taddr, o_base, m, valid, n, pix, scb, corr, use_corr); break;

@@ -152,10 +152,15 @@ psb_status launch_tensor(psb_ctx* ctx, const psb_weights* wt, const ConvArgs& a,
   // they lie anywhere, and no role but the output stage takes part, so flipped activations are served too.
   p.staged = (uniform_epilogue(p) && !p.band && !a.out_nchw && p.unit == 16u && (a.kmap || (a.residual && !flip)) &&
               (uint64_t)p.m_tiles * p.o_tiles >= kStagedMinTiles * (uint64_t)ctx->sm_count) ? 1u : 0u;
-  const size_t io_bytes = p.staged ? (size_t)kIoSlots * kIoTileBytes : 0u;
+  const uint32_t sub_bytes = p.stage_bytes_a + (p.resident ? 0u : p.stage_bytes_b_max);
+  // real-valued rows use the same region, 2 KB for each epilogue warp, where four stages still fit
+  static_assert(kIoSlots * kIoTileBytes == kEpilogueWarps * 2048u, "one region serves both");
+  p.real_slots = (a.f32_out && !a.acc_out && !a.out_nchw && (a.O & 3u) == 0u && !((uintptr_t)a.f32_out & 15u) &&
+                  !(((uintptr_t)a.q_out | (uintptr_t)a.residual) & 3u) &&
+                  (kSmemBudget - ctl_bytes - p.resident_bytes - kIoSlots * kIoTileBytes) / sub_bytes >= 4u) ? 1u : 0u;
+  const size_t io_bytes = p.staged | p.real_slots ? (size_t)kIoSlots * kIoTileBytes : 0u;
   // K blocks are handed over in groups: every barrier round trip costs the issuing thread a
   // few hundred cycles, so a stage should carry about eight MMAs (M=128, N=P*64, K=32 each)
-  const uint32_t sub_bytes = p.stage_bytes_a + (p.resident ? 0u : p.stage_bytes_b_max);
   const size_t avail = kSmemBudget - ctl_bytes - p.resident_bytes - io_bytes;
   uint32_t group = 8u / (bk / 32u);
   if (group < 1) group = 1;

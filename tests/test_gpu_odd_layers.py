@@ -292,3 +292,36 @@ def test_large_sums_are_rounded_once(case, oracle):
     ctx.set_sample_map(None, 4)
     wt.free()
     ctx.close()
+
+
+@pytest.mark.parametrize("want", [("q", "f32"), ("f32",)])
+@pytest.mark.parametrize("case", CASES + [
+    (3, 128, 12, 11, 192, 3, 1, 1, 1, np.uint8, 15, np.uint8, None),      # whole 16-byte pieces, streamed planes
+    (2, 64, 13, 11, 68, 1, 1, 0, 1, np.uint8, 127, np.int8, None),        # rows of 16 bytes of fp32, 4 of codes
+    (2, 64, 13, 11, 80, 3, 2, 1, 1, np.int8, 127, None, (0, 2, 4)),       # a draw-count map
+    (2, 96, 9, 14, 64, 1, 1, 0, 1, np.uint8, 255, np.uint8, (6, 2)),      # levels of three and of four planes
+    (2, 160, 20, 11, 48, 3, 1, 1, 0, np.uint8, 15, np.uint8, None),       # planar
+    (2, 3, 21, 19, 36, 7, 2, 3, 1, np.uint8, 255, None, None),            # flat K axis
+])
+def test_real_valued_outputs(case, want, oracle):
+    import paper_1904_02205_b200 as psb
+
+    N, C, H, W, O, K, stride, pad, layout, dtype, top, res_dtype, levels = case
+    ctx = psb.Context(0)
+    rng = np.random.default_rng(C * 11 + O)
+    w = rng.normal(0, np.sqrt(2.0 / (C * K * K)), size=(O, C, K, K)).astype(np.float32)
+    x = rng.integers(0 if dtype == np.uint8 else -top, top + 1, size=(N, C, H, W) if layout == 0 else (N, H, W, C)).astype(dtype)
+    oh, ow = (H + 2 * pad - K) // stride + 1, (W + 2 * pad - K) // stride + 1
+    res = None
+    if res_dtype is not None:
+        lo = 0 if res_dtype == np.uint8 else -128
+        res = rng.integers(lo, lo + 256, size=(N, O, oh, ow) if layout == 0 else (N, oh, ow, O)).astype(res_dtype)
+    kmap = None if levels is None else rng.choice(levels, size=(N, oh, ow)).astype(np.uint8)
+    for relu, qmin, qmax, dt in ((True, 0, 255, psb.PSB_DT_U8), (False, -100, 90, psb.PSB_DT_S8)):
+        args = (w, x, layout, 1, stride, pad, 5, 3, list(levels or (3,)), kmap, 3, rng.uniform(0.5, 1.5, O).astype(np.float32),
+                rng.normal(0, 0.5, O).astype(np.float32), relu, np.float32(0.02), qmin, qmax)
+        o = oracle_layer(oracle, *args, residual=res, res_scale=np.float32(0.3))
+        g = gpu_layer(psb, ctx, *args, dt, residual=res, res_scale=np.float32(0.3), in_max=top, path=psb.PSB_PATH_TENSOR, want=want)
+        compare(g, o, list(levels or (3,)))
+        assert np.array_equal(g["f32"], o["f32"])       # rounded operations only, in the same order
+    ctx.close()
