@@ -1371,8 +1371,9 @@ template <int P, int W, int RES, bool kSorted>
 __device__ __forceinline__ bool uniform_dispatch_tail(const TensorParams& p, SharedCtl* ctl, uint32_t tmem_base,
                                                       uint32_t slots_addr, uint32_t ew, uint32_t lane, const EpiConst& c,
                                                       bool fast_u8) {
-  // band mode and staged outputs never meet flipped activations, and so no addend
-  constexpr bool kFlipped = W == kRec32Add || W == kRecMidAdd;
+  // An addend comes with flipped activations, which are never in band mode and never staged in tile order, or with the gathered
+  // rows of a flat K axis, which are never in band mode but may be staged.
+  constexpr bool kAddend = W == kRec32Add || W == kRecMidAdd;
   if constexpr (kSorted) {
     if (p.staged)
       return fast_u8 ? epilogue_sorted<P, W, RES, true>(p, ctl, tmem_base, slots_addr, ew, lane, c)
@@ -1380,10 +1381,10 @@ __device__ __forceinline__ bool uniform_dispatch_tail(const TensorParams& p, Sha
     return fast_u8 ? epilogue_uniform<P, W, RES, true, RowMapSorted>(p, ctl, tmem_base, ew, lane, c)
                    : epilogue_uniform<P, W, RES, false, RowMapSorted>(p, ctl, tmem_base, ew, lane, c);
   }
-  if constexpr (!kFlipped) {
-    if (RES && p.staged)
-      return fast_u8 ? epilogue_staged<P, W, RES ? RES : 1, true>(p, ctl, tmem_base, slots_addr, ew, lane, c)
-                     : epilogue_staged<P, W, RES ? RES : 1, false>(p, ctl, tmem_base, slots_addr, ew, lane, c);
+  if (RES && p.staged)
+    return fast_u8 ? epilogue_staged<P, W, RES ? RES : 1, true>(p, ctl, tmem_base, slots_addr, ew, lane, c)
+                   : epilogue_staged<P, W, RES ? RES : 1, false>(p, ctl, tmem_base, slots_addr, ew, lane, c);
+  if constexpr (!kAddend) {
     if (p.band)
       return fast_u8 ? epilogue_uniform<P, W, RES, true, RowMapBand>(p, ctl, tmem_base, ew, lane, c)
                      : epilogue_uniform<P, W, RES, false, RowMapBand>(p, ctl, tmem_base, ew, lane, c);

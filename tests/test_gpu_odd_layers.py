@@ -113,6 +113,54 @@ def test_shortcut_tiles_through_shared_memory(case, signed_out, oracle):
 
 
 @pytest.mark.parametrize("case", [
+    # (N, C, H, W, O, K, stride, shortcut dtype, exp_bits, log2k, largest byte, sums that fit 32 bits), each with and without an
+    # addend where the bytes are unsigned, three planes, then two and four
+    (19, 3, 112, 111, 64, 7, 2, np.uint8, 4, 3, 255, False), (19, 3, 112, 111, 64, 7, 2, np.int8, 4, 0, 255, True),
+    (13, 12, 40, 39, 144, 3, 1, np.int8, 4, 4, 255, False), (13, 12, 40, 39, 144, 3, 1, np.uint8, 4, 1, 15, True),
+    (13, 12, 40, 39, 144, 3, 1, np.uint8, 4, 3, -127, True), (13, 12, 40, 39, 144, 5, 1, np.uint8, 4, 4, -127, False),
+    (13, 12, 40, 39, 144, 3, 1, np.uint8, 3, 2, 255, True), (19, 3, 112, 111, 64, 7, 2, np.uint8, 4, 6, 255, False),
+])
+@pytest.mark.parametrize("signed_out", [False, True])
+def test_shortcut_of_a_flat_k_axis(case, signed_out, oracle):
+    """Filters with fewer than 16 input channels, a shortcut, and enough tiles for the staged output stage."""
+    import torch
+
+    import paper_1904_02205_b200 as psb
+
+    N, C, H, W, O, K, stride, res_dtype, exp_bits, log2k, top, fits = case
+    oh, ow = (H + 2 * (K // 2) - K) // stride + 1, (W + 2 * (K // 2) - K) // stride + 1
+    assert -(-N * oh * ow // 128) * -(-O // 64) >= 3 * 148 and O % 16 == 0
+    ctx = psb.Context(0)
+    rng = np.random.default_rng(O + H + log2k)
+    w = rng.normal(0, np.sqrt(2.0 / (C * K * K)), size=(O, C, K, K)).astype(np.float32)
+    x = rng.integers(min(top, 0), abs(top) + 1, size=(N, H, W, C)).astype(np.uint8 if top > 0 else np.int8)
+    lo = 0 if res_dtype == np.uint8 else -128
+    res = rng.integers(lo, lo + 256, size=(N, oh, ow, O)).astype(res_dtype)
+    scale, bias = rng.uniform(0.5, 1.5, O).astype(np.float32), rng.normal(0, 0.5, O).astype(np.float32)
+    # the output stage's bound: row sums of |W| in units of 256, each contribution rounded up
+    sums = np.abs(oracle.sample_level(w, 5, 3, log2k, exp_bits=exp_bits)[0].astype(np.int64)).reshape(O, -1)
+    assert (int((-(-sums // 256)).sum(1).max()) * 256 * abs(top) < 1 << 31) == fits
+    assert fits or int(sums.sum(1).max()) * abs(top) >= 1 << 31
+    dev = lambda t: torch.from_numpy(t).to(ctx.device)
+    wt = ctx.sample_weights(dev(w), seed=5, layer_id=3, level_mask=1 << log2k, exp_bits=exp_bits)
+    ctx.set_sample_map(None, log2k)
+    qmin, qmax = (-100, 101) if signed_out else (0, 255)
+    inv_step = np.float32(32.0 / abs(top))
+    q = ctx.conv2d(wt, dev(x), psb.PSB_LAYOUT_NHWC, stride, K // 2, dev(scale), dev(bias), not signed_out, inv_step, qmin, qmax,
+                   out_dtype=psb.PSB_DT_S8 if signed_out else psb.PSB_DT_U8, residual=dev(res), residual_scale=0.3, in_max=abs(top),
+                   path=psb.PSB_PATH_TENSOR)["q"].cpu().numpy()
+    assert ctx.device_status() == 0
+    # first and last image against the oracle
+    for n in (0, N - 1):
+        o = oracle_layer(oracle, w, x[n:n + 1], 1, 1, stride, K // 2, 5, 3, [log2k], None, log2k, scale, bias, not signed_out, inv_step,
+                         qmin, qmax, residual=res[n:n + 1], res_scale=np.float32(0.3), exp_bits=exp_bits)
+        assert np.array_equal(q[n:n + 1].astype(np.int32), o["q"])
+        assert len(np.unique(q[n])) > 50
+    wt.free()
+    ctx.close()
+
+
+@pytest.mark.parametrize("case", [
     # (N, C, H, W, stride, dtype, shortcut dtype or None): odd channel counts, one row or column, long strips, wide sums
     (2, 37, 9, 11, 1, np.uint8, None), (1, 5, 7, 1, 2, np.int8, None), (3, 64, 1, 13, 1, np.uint8, np.int8),
     (1, 8, 61, 9, 1, np.int8, np.uint8), (2, 12, 64, 33, 2, np.uint8, None), (130, 48, 14, 15, 1, np.uint8, None),
