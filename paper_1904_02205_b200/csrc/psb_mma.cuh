@@ -1598,13 +1598,14 @@ __device__ __forceinline__ bool flip_role(const TensorParams& p, SharedCtl* ctl,
 }
 
 // kKind: which output stage the instance carries, the loops for the common case (uniform_epilogue), for one draw count or
-// for rows sorted by level, or the general one; the host picks the instance, so that none drags the others' code and
-// registers along (sorted rows in an instance of their own: ResNet-50 shape, batch 64, one draw count 1659 -> 1645 us).
-constexpr int kOneLevel = 0, kSortedRows = 1, kGeneralOutputs = 2;
+// for rows sorted by level, the one for real-valued outputs (with or without codes beside them), or the general one; the host
+// picks the instance, so that none drags the others' code and registers along (sorted rows in an instance of their own:
+// ResNet-50 shape, batch 64, one draw count 1659 -> 1645 us).
+constexpr int kOneLevel = 0, kSortedRows = 1, kGeneralOutputs = 2, kRealOutputs = 3;
 template <int BK, int kKind>
 __global__ void __launch_bounds__(kThreadsTensor, 1)
 psb_mma_kernel(const __grid_constant__ TmapSet maps, const __grid_constant__ TensorParams p) {
-  constexpr bool kSorted = kKind == kSortedRows;
+  constexpr bool kSorted = kKind == kSortedRows, kReal = kKind == kRealOutputs, kCodes = kKind == kOneLevel || kSorted;
   extern __shared__ uint8_t smem_raw[];
   // stage buffers need 1024-byte alignment for the 128-byte swizzle pattern
   uint8_t* smem = reinterpret_cast<uint8_t*>(((uintptr_t)smem_raw + 1023u) & ~(uintptr_t)1023u);
@@ -1792,12 +1793,11 @@ psb_mma_kernel(const __grid_constant__ TmapSet maps, const __grid_constant__ Ten
                   bar);
       }
     }
-    // (real-valued outputs and accumulators are always recombined in 64 bits: 1x1 32 -> 110 channels with a map of five levels,
-    // codes and fp32 wanted, 38.8 -> 37.5 us without the look-ups; no level instead of a branch around the call, with which
-    // 3x3 100 -> 150 channels, codes only, took 49.3 us and not 48.4)
+    // (accumulators are always recombined in 64 bits, real-valued outputs as the host knows beforehand (p.mid); no level instead
+    // of a branch around the call, with which 3x3 100 -> 150 channels, codes only, took 49.3 us and not 48.4)
     const uint32_t bounded = a.kmap ? a.level_mask : 1u << a.uniform_log2k;
-    find_row_maxima(p, ctl, kKind != kGeneralOutputs || q_only ? bounded : 0u);
-    if constexpr (kKind != kGeneralOutputs) {
+    if constexpr (!kReal) find_row_maxima(p, ctl, kCodes || q_only ? bounded : 0u);
+    if constexpr (kCodes) {
       const bool addend = p.corr[(uint32_t)__ffs((int)(a.level_mask & 0x7Fu)) - 1u] != nullptr;
       bool w32 = true;
       if (kSorted) {         // every level a tile may have must fit
@@ -1819,9 +1819,8 @@ psb_mma_kernel(const __grid_constant__ TmapSet maps, const __grid_constant__ Ten
       const float2* scb = ctl->scb[ew];
       const long long* corr = ctl->corr[ew];
       uint32_t pass = 0, cur_key = 0xFFFFFFFFu;
-      const bool real = a.f32_out && !a.acc_out;
       bool done = false;
-      if (real && !a.kmap) {
+      if constexpr (kReal) if (!a.kmap) {
         done = true;
         if (P0 == 4u) failed = epilogue_real<4, kRec64>(p, ctl, tmem_base, slots_addr, ew, lane);
         else if (P0 == 3u && p.mid) failed = epilogue_real<3, kRecMidAdd>(p, ctl, tmem_base, slots_addr, ew, lane);
@@ -1830,7 +1829,7 @@ psb_mma_kernel(const __grid_constant__ TmapSet maps, const __grid_constant__ Ten
         else failed = epilogue_real<1, kRec64>(p, ctl, tmem_base, slots_addr, ew, lane);
       }
       uint32_t w32_levels = 0;      // levels whose accumulators are known to fit 32 bits
-      if (q_only)
+      if (!kReal && q_only)
         for (uint32_t l = 0; l < (uint32_t)kMaxLevels; ++l)
           if (((a.level_mask >> l) & 1u) && fits_32_bits(p, ctl, l)) w32_levels |= 1u << l;
       TileIter ti;
@@ -1849,7 +1848,7 @@ psb_mma_kernel(const __grid_constant__ TmapSet maps, const __grid_constant__ Ten
         const uint32_t o_base = o_tile * kTileN + sub * 16u;
         const size_t oidx = (size_t)m * a.O + o_base;
         const uint32_t unit = p.unit, count = o_base < a.O ? a.O - o_base : 0u;
-        const bool fast = q_only && !a.out_nchw && o_base < a.O;
+        const bool fast = !kReal && q_only && !a.out_nchw && o_base < a.O;
         uint4 r4 = make_uint4(0, 0, 0, 0);
         if (fast && a.residual && in_range) r4 = unit < 8u ? load_narrow16((const uint8_t*)a.residual + oidx, unit, count)
                     : load_row16((const uint8_t*)a.residual + oidx, unit == 16u, count >= 16u);
@@ -1872,7 +1871,7 @@ psb_mma_kernel(const __grid_constant__ TmapSet maps, const __grid_constant__ Ten
                 if (use_corr) cr = p.corr[l][o];
               }
               ctl->scb[ew][lane] = sb;
-              ctl->corr[ew][lane] = real && p.mid && P == 3u ? addend_words<kRecMidAdd>(cr) : cr;
+              ctl->corr[ew][lane] = kReal && p.mid && P == 3u ? addend_words<kRecMidAdd>(cr) : cr;
               ctl->corr32[ew][lane] = (int32_t)cr;
             }
             cur_key = key;
@@ -1885,7 +1884,18 @@ psb_mma_kernel(const __grid_constant__ TmapSet maps, const __grid_constant__ Ten
           const uint32_t taddr = tmem_base + buf * kTmemBufStride + ((quarter * 32u) << 16) + sub * 16u;
           const bool valid = in_range && my_level == l;
           if (o_base < a.O) {
-            if (fast) {
+            if constexpr (kReal) {
+              const uint32_t slot = slots_addr + ew * 2048u;
+              switch (P) {
+                case 1: epilogue_chunk_real<1, kRec64>(p, taddr, slot, o_base, m, valid, scb, corr); break;
+                case 2: epilogue_chunk_real<2, kRec64>(p, taddr, slot, o_base, m, valid, scb, corr); break;
+                case 3:
+                  if (p.mid) epilogue_chunk_real<3, kRecMidAdd>(p, taddr, slot, o_base, m, valid, scb, corr);
+                  else epilogue_chunk_real<3, kRec64>(p, taddr, slot, o_base, m, valid, scb, corr);
+                  break;
+                default: epilogue_chunk_real<4, kRec64>(p, taddr, slot, o_base, m, valid, scb, corr); break;
+              }
+            } else if (fast) {
               const bool w32 = ((w32_levels >> l) & 1u) != 0u;
 #define PSB_EPI(PV, WV, RV) epilogue_chunk_q<PV, WV, RV>(taddr, valid, (uint8_t*)a.q_out, oidx, r4, unit, count, scb, corr, \
                                                          use_corr ? ctl->corr32[ew] : nullptr, ec)
@@ -1904,18 +1914,7 @@ psb_mma_kernel(const __grid_constant__ TmapSet maps, const __grid_constant__ Ten
             } else {
               const uint32_t ohow = a.OH * a.OW;
               const uint32_t n = in_range ? m / ohow : 0u, pix = in_range ? m % ohow : 0u;
-              const uint32_t slot = slots_addr + ew * 2048u;
-              if (real) {
-                switch (P) {
-                  case 1: epilogue_chunk_real<1, kRec64>(p, taddr, slot, o_base, m, valid, scb, corr); break;
-                  case 2: epilogue_chunk_real<2, kRec64>(p, taddr, slot, o_base, m, valid, scb, corr); break;
-                  case 3:
-                    if (p.mid) epilogue_chunk_real<3, kRecMidAdd>(p, taddr, slot, o_base, m, valid, scb, corr);
-                    else epilogue_chunk_real<3, kRec64>(p, taddr, slot, o_base, m, valid, scb, corr);
-                    break;
-                  default: epilogue_chunk_real<4, kRec64>(p, taddr, slot, o_base, m, valid, scb, corr); break;
-                }
-              } else switch (P) {
+              switch (P) {
                 case 1: epilogue_chunk<1>(p, taddr, o_base, m, valid, n, pix, scb, corr, use_corr); break;
                 case 2: epilogue_chunk<2>(p, taddr, o_base, m, valid, n, pix, scb, corr, use_corr); break;
                 case 3: epilogue_chunk<3>(p, taddr, o_base, m, valid, n, pix, scb, corr, use_corr); break;

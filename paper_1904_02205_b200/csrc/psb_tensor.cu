@@ -250,7 +250,8 @@ psb_status launch_tensor(psb_ctx* ctx, const psb_weights* wt, const ConvArgs& a,
   cfg.stream = s;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  const int kind = !uniform_epilogue(p) ? kGeneralOutputs : a.kmap ? kSortedRows : kOneLevel;
+  const int kind = uniform_epilogue(p) ? (a.kmap ? kSortedRows : kOneLevel)
+                                       : a.f32_out && !a.acc_out ? kRealOutputs : kGeneralOutputs;
   const bool timed = ctx->time_contraction && ctx->t_begin[0] && ctx->timed_launches < psb_ctx::kTimedLaunches;
   if (timed) cudaEventRecord(ctx->t_begin[ctx->timed_launches], s);
   e = bk == 128 ? launch_mma_kernel<128>(cfg, maps, p, ctx->device, kind)
