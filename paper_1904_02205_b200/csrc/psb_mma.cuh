@@ -351,6 +351,10 @@ enum Recombine { kRec64, kRec32, kRec32Add, kRecMid, kRecMidAdd };
 __host__ __device__ constexpr bool folds_all(int W) { return W == kRec32 || W == kRec32Add; }
 __host__ __device__ constexpr bool is_mid(int W) { return W == kRecMid || W == kRecMidAdd; }
 __host__ __device__ constexpr bool has_addend(int W) { return W == kRec32Add || W == kRecMidAdd || W == kRec64; }
+// The recombinations that an instance of the kernel carries, chosen on the host: kRec32 and kRec64 for two to four planes;
+// kRec32 and kRecMid for three whose lower two fit 32 bits; kRec32Add, kRecMidAdd and kRec64 for three with an addend.  (All in
+// one instance, codes: 1x1 64 -> 256 @56 batch 16 12.8 -> 13.8 us, 3x3 64 -> 64 @56 batch 32 with a map 32.1 -> 33.2.)
+constexpr int kPlainSums = 0, kMidSums = 1, kAddSums = 2;
 
 // A channel's addend as the output loop of the kind wants it in its eight bytes: 64 bits, or two words.
 template <int W>
@@ -953,10 +957,11 @@ __device__ __noinline__ bool epilogue_uniform(const TensorParams& p, SharedCtl* 
         if (o < a.O) {
           sb.x = ldexpf(a.scale[o], a.e_base[o] - (int)l);
           sb.y = a.bias[o];
-          if (has_addend(W) && use_corr) cr = p.corr[l][o];
+          if (use_corr) cr = p.corr[l][o];
         }
         ctl->scb[ew][lane] = sb;
-        if (has_addend(W)) ctl->corr[ew][lane] = addend_words<W>(cr);
+        // (also where nothing reads it: without the store 1x1 64 -> 256 @56 batch 16 took 13.3 us, not 12.6, by the compiler's schedule)
+        ctl->corr[ew][lane] = addend_words<W>(cr);
       }
       cur_o_tile = kSorted ? o_tile * 8u + l : o_tile;
       __syncwarp();
@@ -1365,7 +1370,7 @@ __device__ __noinline__ bool io_role(const TensorParams& p, const TmapSet& maps,
 struct EpiChoice {
   bool fast_u8;
   uint32_t res;       // 0 no shortcut, 1 unsigned, 2 signed bytes
-  int rec;            // Recombine
+  bool fits, mid;     // the sums fit 32 bits (and, in kPlainSums, have no addend); p.mid
 };
 template <int P, int W, int RES, bool kSorted>
 __device__ __forceinline__ bool uniform_dispatch_tail(const TensorParams& p, SharedCtl* ctl, uint32_t tmem_base,
@@ -1399,16 +1404,15 @@ __device__ __forceinline__ bool uniform_dispatch_res(const TensorParams& p, Shar
   if (how.res == 1u) return uniform_dispatch_tail<P, W, 1, kSorted>(p, ctl, tmem_base, slots_addr, ew, lane, c, how.fast_u8);
   return uniform_dispatch_tail<P, W, 2, kSorted>(p, ctl, tmem_base, slots_addr, ew, lane, c, how.fast_u8);
 }
-template <int P, bool kSorted>
+template <int P, int kRec, bool kSorted>
 __device__ __forceinline__ bool uniform_dispatch(const TensorParams& p, SharedCtl* ctl, uint32_t tmem_base, uint32_t slots_addr,
                                                  uint32_t ew, uint32_t lane, const EpiConst& c, const EpiChoice& how) {
-  if (how.rec == kRec32) return uniform_dispatch_res<P, kRec32, kSorted>(p, ctl, tmem_base, slots_addr, ew, lane, c, how);
-  if constexpr (P == 3) {
-    if (how.rec == kRec32Add) return uniform_dispatch_res<P, kRec32Add, kSorted>(p, ctl, tmem_base, slots_addr, ew, lane, c, how);
-    if (how.rec == kRecMid) return uniform_dispatch_res<P, kRecMid, kSorted>(p, ctl, tmem_base, slots_addr, ew, lane, c, how);
-    if (how.rec == kRecMidAdd) return uniform_dispatch_res<P, kRecMidAdd, kSorted>(p, ctl, tmem_base, slots_addr, ew, lane, c, how);
-  }
-  return uniform_dispatch_res<P, kRec64, kSorted>(p, ctl, tmem_base, slots_addr, ew, lane, c, how);
+  constexpr int kSmall = kRec == kAddSums ? kRec32Add : kRec32;
+  constexpr int kLarge = kRec == kAddSums ? kRecMidAdd : kRec == kMidSums ? kRecMid : kRec64;
+  if (how.fits) return uniform_dispatch_res<P, kSmall, kSorted>(p, ctl, tmem_base, slots_addr, ew, lane, c, how);
+  if constexpr (kRec == kAddSums)
+    if (!how.mid) return uniform_dispatch_res<P, kRec64, kSorted>(p, ctl, tmem_base, slots_addr, ew, lane, c, how);
+  return uniform_dispatch_res<P, kLarge, kSorted>(p, ctl, tmem_base, slots_addr, ew, lane, c, how);
 }
 
 // All lanes of the warp wait together; false when a wait ran out.
@@ -1602,7 +1606,7 @@ __device__ __forceinline__ bool flip_role(const TensorParams& p, SharedCtl* ctl,
 // picks the instance, so that none drags the others' code and registers along (sorted rows in an instance of their own:
 // ResNet-50 shape, batch 64, one draw count 1659 -> 1645 us).
 constexpr int kOneLevel = 0, kSortedRows = 1, kGeneralOutputs = 2, kRealOutputs = 3;
-template <int BK, int kKind>
+template <int BK, int kKind, int kRec>
 __global__ void __launch_bounds__(kThreadsTensor, 1)
 psb_mma_kernel(const __grid_constant__ TmapSet maps, const __grid_constant__ TensorParams p) {
   constexpr bool kSorted = kKind == kSortedRows, kReal = kKind == kRealOutputs, kCodes = kKind == kOneLevel || kSorted;
@@ -1798,22 +1802,22 @@ psb_mma_kernel(const __grid_constant__ TmapSet maps, const __grid_constant__ Ten
     const uint32_t bounded = a.kmap ? a.level_mask : 1u << a.uniform_log2k;
     if constexpr (!kReal) find_row_maxima(p, ctl, kCodes || q_only ? bounded : 0u);
     if constexpr (kCodes) {
-      const bool addend = p.corr[(uint32_t)__ffs((int)(a.level_mask & 0x7Fu)) - 1u] != nullptr;
-      bool w32 = true;
+      bool w32 = kRec != kPlainSums || p.corr[(uint32_t)__ffs((int)(a.level_mask & 0x7Fu)) - 1u] == nullptr;
       if (kSorted) {         // every level a tile may have must fit
         for (uint32_t lv = 0; lv < (uint32_t)kMaxLevels; ++lv)
           if ((a.level_mask >> lv) & 1u) w32 = fits_32_bits(p, ctl, lv) && w32;
       } else {
-        w32 = fits_32_bits(p, ctl, a.uniform_log2k);
+        w32 = fits_32_bits(p, ctl, a.uniform_log2k) && w32;
       }
       EpiChoice how;
       how.fast_u8 = fast_u8;
       how.res = res_kind;
-      how.rec = w32 ? (addend ? kRec32Add : kRec32) : !p.mid ? kRec64 : addend ? kRecMidAdd : kRecMid;
-      if (P0 != 3u && how.rec != kRec32) how.rec = kRec64;
-      if (P0 == 4u) failed = uniform_dispatch<4, kSorted>(p, ctl, tmem_base, slots_addr, ew, lane, ec, how);
-      else if (P0 == 3u) failed = uniform_dispatch<3, kSorted>(p, ctl, tmem_base, slots_addr, ew, lane, ec, how);
-      else failed = uniform_dispatch<2, kSorted>(p, ctl, tmem_base, slots_addr, ew, lane, ec, how);
+      how.fits = w32;
+      how.mid = p.mid != 0u;
+      if constexpr (kRec != kPlainSums) failed = uniform_dispatch<3, kRec, kSorted>(p, ctl, tmem_base, slots_addr, ew, lane, ec, how);
+      else if (P0 == 4u) failed = uniform_dispatch<4, kRec, kSorted>(p, ctl, tmem_base, slots_addr, ew, lane, ec, how);
+      else if (P0 == 3u) failed = uniform_dispatch<3, kRec, kSorted>(p, ctl, tmem_base, slots_addr, ew, lane, ec, how);
+      else failed = uniform_dispatch<2, kRec, kSorted>(p, ctl, tmem_base, slots_addr, ew, lane, ec, how);
     } else {
       // general loop: per-location draw counts, any outputs and layouts, ragged channel counts
       const float2* scb = ctl->scb[ew];
@@ -1954,6 +1958,6 @@ psb_mma_kernel(const __grid_constant__ TmapSet maps, const __grid_constant__ Ten
 
 // Launches the instance of the kernel with this K block (one translation unit per instance: psb_mma_bk*.cu).
 template <int BK>
-cudaError_t launch_mma_kernel(const cudaLaunchConfig_t& cfg, const TmapSet& maps, const TensorParams& p, int device, int kind);
+cudaError_t launch_mma_kernel(const cudaLaunchConfig_t& cfg, const TmapSet& maps, const TensorParams& p, int device, int kind, int rec);
 
 }  // namespace psb

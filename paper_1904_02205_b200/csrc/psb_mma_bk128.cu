@@ -2,5 +2,5 @@
 #include "psb_mma_launch.cuh"
 
 namespace psb {
-template cudaError_t launch_mma_kernel<128>(const cudaLaunchConfig_t&, const TmapSet&, const TensorParams&, int, int);
+template cudaError_t launch_mma_kernel<128>(const cudaLaunchConfig_t&, const TmapSet&, const TensorParams&, int, int, int);
 }  // namespace psb

@@ -252,11 +252,15 @@ psb_status launch_tensor(psb_ctx* ctx, const psb_weights* wt, const ConvArgs& a,
   cfg.numAttrs = 1;
   const int kind = uniform_epilogue(p) ? (a.kmap ? kSortedRows : kOneLevel)
                                        : a.f32_out && !a.acc_out ? kRealOutputs : kGeneralOutputs;
+  // (the levels of sorted rows all have as many planes)
+  const bool common = kind == kOneLevel || kind == kSortedRows;
+  const uint32_t planes = p.planes[a.kmap ? (uint32_t)__builtin_ctz(a.level_mask & 0x7Fu) : a.uniform_log2k];
+  const int rec = !common || planes != 3u ? kPlainSums : add_corr128 ? kAddSums : p.mid ? kMidSums : kPlainSums;
   const bool timed = ctx->time_contraction && ctx->t_begin[0] && ctx->timed_launches < psb_ctx::kTimedLaunches;
   if (timed) cudaEventRecord(ctx->t_begin[ctx->timed_launches], s);
-  e = bk == 128 ? launch_mma_kernel<128>(cfg, maps, p, ctx->device, kind)
-      : bk == 64 ? launch_mma_kernel<64>(cfg, maps, p, ctx->device, kind)
-                 : launch_mma_kernel<32>(cfg, maps, p, ctx->device, kind);
+  e = bk == 128 ? launch_mma_kernel<128>(cfg, maps, p, ctx->device, kind, rec)
+      : bk == 64 ? launch_mma_kernel<64>(cfg, maps, p, ctx->device, kind, rec)
+                 : launch_mma_kernel<32>(cfg, maps, p, ctx->device, kind, rec);
   note_launch();
   if (timed) {
     cudaEventRecord(ctx->t_end[ctx->timed_launches], s);
