@@ -1009,8 +1009,10 @@ __device__ __noinline__ bool epilogue_uniform(const TensorParams& p, SharedCtl* 
 }
 
 // The loop for real-valued outputs under one draw count: as epilogue_uniform, the accumulator handed back before the arithmetic.
+// Inlined into its instance: out of line, four planes spill 552 bytes and not 196 (1x1 64 -> 256 @56 batch 16 planar, k = 64,
+// 54.0 -> 38.0 us).
 template <int P, int W>
-__device__ __noinline__ bool epilogue_real(const TensorParams& p, SharedCtl* ctl, uint32_t tmem_base, uint32_t slots_addr,
+__device__ __forceinline__ bool epilogue_real(const TensorParams& p, SharedCtl* ctl, uint32_t tmem_base, uint32_t slots_addr,
                                            uint32_t ew, uint32_t lane) {
   const ConvArgs& a = p.a;
   const RealOut r(p, slots_addr + ew * 2048u);
@@ -1602,14 +1604,15 @@ __device__ __forceinline__ bool flip_role(const TensorParams& p, SharedCtl* ctl,
 }
 
 // kKind: which output stage the instance carries, the loops for the common case (uniform_epilogue), for one draw count or
-// for rows sorted by level, the one for real-valued outputs (with or without codes beside them), or the general one; the host
-// picks the instance, so that none drags the others' code and registers along (sorted rows in an instance of their own:
-// ResNet-50 shape, batch 64, one draw count 1659 -> 1645 us).
-constexpr int kOneLevel = 0, kSortedRows = 1, kGeneralOutputs = 2, kRealOutputs = 3;
+// for rows sorted by level, those for real-valued outputs (with or without codes beside them), for one draw count or for sorted
+// rows, or the general one; the host picks the instance, so that none drags the others' code and registers along (sorted rows
+// in an instance of their own: ResNet-50 shape, batch 64, one draw count 1659 -> 1645 us; real-valued outputs out of the general
+// instance: accumulators of 3x3 64 -> 64 on 81 locations 23.2 -> 19.9 us).
+constexpr int kOneLevel = 0, kSortedRows = 1, kGeneralOutputs = 2, kRealOutputs = 3, kRealSorted = 4;
 template <int BK, int kKind, int kRec>
 __global__ void __launch_bounds__(kThreadsTensor, 1)
 psb_mma_kernel(const __grid_constant__ TmapSet maps, const __grid_constant__ TensorParams p) {
-  constexpr bool kSorted = kKind == kSortedRows, kReal = kKind == kRealOutputs, kCodes = kKind == kOneLevel || kSorted;
+  constexpr bool kSorted = kKind == kSortedRows, kReal = kKind == kRealOutputs || kKind == kRealSorted, kCodes = kKind == kOneLevel || kSorted;
   extern __shared__ uint8_t smem_raw[];
   // stage buffers need 1024-byte alignment for the 128-byte swizzle pattern
   uint8_t* smem = reinterpret_cast<uint8_t*>(((uintptr_t)smem_raw + 1023u) & ~(uintptr_t)1023u);
@@ -1818,26 +1821,23 @@ psb_mma_kernel(const __grid_constant__ TmapSet maps, const __grid_constant__ Ten
       else if (P0 == 4u) failed = uniform_dispatch<4, kRec, kSorted>(p, ctl, tmem_base, slots_addr, ew, lane, ec, how);
       else if (P0 == 3u) failed = uniform_dispatch<3, kRec, kSorted>(p, ctl, tmem_base, slots_addr, ew, lane, ec, how);
       else failed = uniform_dispatch<2, kRec, kSorted>(p, ctl, tmem_base, slots_addr, ew, lane, ec, how);
+    } else if constexpr (kKind == kRealOutputs) {
+      if (P0 == 4u) failed = epilogue_real<4, kRec64>(p, ctl, tmem_base, slots_addr, ew, lane);
+      else if (P0 == 3u && p.mid) failed = epilogue_real<3, kRecMidAdd>(p, ctl, tmem_base, slots_addr, ew, lane);
+      else if (P0 == 3u) failed = epilogue_real<3, kRec64>(p, ctl, tmem_base, slots_addr, ew, lane);
+      else if (P0 == 2u) failed = epilogue_real<2, kRec64>(p, ctl, tmem_base, slots_addr, ew, lane);
+      else failed = epilogue_real<1, kRec64>(p, ctl, tmem_base, slots_addr, ew, lane);
     } else {
       // general loop: per-location draw counts, any outputs and layouts, ragged channel counts
       const float2* scb = ctl->scb[ew];
       const long long* corr = ctl->corr[ew];
       uint32_t pass = 0, cur_key = 0xFFFFFFFFu;
-      bool done = false;
-      if constexpr (kReal) if (!a.kmap) {
-        done = true;
-        if (P0 == 4u) failed = epilogue_real<4, kRec64>(p, ctl, tmem_base, slots_addr, ew, lane);
-        else if (P0 == 3u && p.mid) failed = epilogue_real<3, kRecMidAdd>(p, ctl, tmem_base, slots_addr, ew, lane);
-        else if (P0 == 3u) failed = epilogue_real<3, kRec64>(p, ctl, tmem_base, slots_addr, ew, lane);
-        else if (P0 == 2u) failed = epilogue_real<2, kRec64>(p, ctl, tmem_base, slots_addr, ew, lane);
-        else failed = epilogue_real<1, kRec64>(p, ctl, tmem_base, slots_addr, ew, lane);
-      }
       uint32_t w32_levels = 0;      // levels whose accumulators are known to fit 32 bits
       if (!kReal && q_only)
         for (uint32_t l = 0; l < (uint32_t)kMaxLevels; ++l)
           if (((a.level_mask >> l) & 1u) && fits_32_bits(p, ctl, l)) w32_levels |= 1u << l;
       TileIter ti;
-      for (ti.init(p); !done && !failed && ti.valid(); ti.next()) {
+      for (ti.init(p); !failed && ti.valid(); ti.next()) {
         const uint32_t m0 = ti.m_tile * kTileM, o_tile = ti.o_tile;
         const uint32_t levels = tile_levels(p, ti.m_tile) & a.level_mask;
         uint32_t m = m0 + row;

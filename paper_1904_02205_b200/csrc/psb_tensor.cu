@@ -251,7 +251,7 @@ psb_status launch_tensor(psb_ctx* ctx, const psb_weights* wt, const ConvArgs& a,
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   const int kind = uniform_epilogue(p) ? (a.kmap ? kSortedRows : kOneLevel)
-                                       : a.f32_out && !a.acc_out ? kRealOutputs : kGeneralOutputs;
+                                       : !a.f32_out || a.acc_out ? kGeneralOutputs : a.kmap ? kRealSorted : kRealOutputs;
   // (the levels of sorted rows all have as many planes)
   const bool common = kind == kOneLevel || kind == kSortedRows;
   const uint32_t planes = p.planes[a.kmap ? (uint32_t)__builtin_ctz(a.level_mask & 0x7Fu) : a.uniform_log2k];
