@@ -403,19 +403,28 @@ struct PackedDraws {
   }
 };
 
-// Count at one level with a comparator of any other width, or deterministic; threshold as classify_weight gives it.
-__device__ __forceinline__ uint32_t count_level(const PhiloxWeight& pw, uint32_t thr, uint32_t level, uint32_t pbits,
-                                                uint32_t deterministic, const PhiloxKeys& keys) {
-  if (deterministic) return ((thr << level) + (1u << (pbits - 1u))) >> pbits;
-  uint32_t cnt[kMaxLevels];
-  if (pbits == 6u) packed_counts<6>(thr, level, pw, keys, cnt);
-  else packed_counts_any(pbits, thr, level, pw, keys, cnt);
-  uint32_t c = cnt[0];
-#pragma unroll
-  for (int l = 1; l < kMaxLevels; ++l)
-    if ((uint32_t)l == level) c = cnt[l];
-  return c;
-}
+// The same for any width b of 1..8, known at run time: n = 32 / b fields in a word, of which the last even one may end short of
+// the top (b = 6); field 2m answers in bit b + 2 b m, field 2m + 1 in the bit below that one.
+struct PackedDrawsAny {
+  uint32_t b, n, even, guard_even, guard_odd, ones;       // ones: bit 0 of every even field
+  __device__ __forceinline__ explicit PackedDrawsAny(uint32_t width) : b(width), n(32u / width) {
+    ones = 0u;
+    for (uint32_t f = 0; f < n; f += 2u) ones |= 1u << (f * b);
+    even = ones * ((1u << b) - 1u);
+    guard_even = ones << b;
+    guard_odd = n & 1u ? guard_even & ((1u << ((n - 1u) * b)) - 1u) : guard_even;
+  }
+  __device__ __forceinline__ uint32_t below(uint32_t word, uint32_t thr) const {
+    const uint32_t t = ones * thr;
+    const uint32_t e = ((word & even) | guard_even) - t, o = (((word >> b) & even) | guard_even) - t;
+    return (~e & guard_even) | ((~o & guard_odd) >> 1);
+  }
+  // the bits of the first `left` fields, left < n
+  __device__ __forceinline__ uint32_t first(uint32_t left) const {
+    const uint32_t e = (1u << (b * ((left + 1u) & ~1u))) - 1u, o = (1u << (b * (left & ~1u))) - 1u;
+    return (guard_even & e) | ((guard_odd & o) >> 1);
+  }
+};
 
 // Row sums of a block's slice, kept in shared memory and added to the layer's words at the end: the sum of |W_k| in
 // units of 256 (each contribution rounded up) bounds the accumulators; the signed sum, as hi * 4096 + lo, is what an
@@ -453,12 +462,6 @@ enum DrawMode {
   kDrawAny         // any other width, and the deterministic variant
 };
 
-// The weight's signed integer at one level, as a float (at most 2^22 in magnitude).
-__device__ __forceinline__ float signed_weight(uint32_t u, const Drawn& dw, uint32_t level, uint32_t count) {
-  const uint32_t m = dw.live ? ((dw.base << level) + count) << dw.sh : 0u;
-  return __uint_as_float(__float_as_uint((float)(int)m) | (u & 0x80000000u));
-}
-
 // One draw: adds 1 to the count, kept in fp32, where the word is below the threshold.  The predicated addition runs on the fp32
 // pipe, which has nothing else to do; an integer one would take a second slot of the logic pipe.
 __device__ __forceinline__ void draw(float& count, uint32_t word, uint32_t thr, float one = 1.0f) {
@@ -486,7 +489,7 @@ struct WindowBits {
 // Bernoulli gate at the window's floor (Sec. 3.1): base = 0, scale = +-1, thr = |w| / 2^e_base; else scale = 0.  The same
 // definitions as classify_weight.
 template <int kMode>
-__device__ __forceinline__ void decode_weight(uint32_t u, const WindowBits& win, uint32_t underflow, uint32_t& thr, float& base, float& scale) {
+__device__ __forceinline__ void decode_weight(uint32_t u, const WindowBits& win, uint32_t underflow, uint32_t pbits, uint32_t& thr, float& base, float& scale) {
   base = 1.0f;
   if (kMode == kDrawExact || kMode == kDrawGate) {
     thr = u << 9;
@@ -507,7 +510,7 @@ __device__ __forceinline__ void decode_weight(uint32_t u, const WindowBits& win,
     return;
   }
   // probability on the grid of 2^B points: a p of 1 carries into the exponent, but not beyond the largest finite one
-  constexpr int B = kMode == kDrawPacked8 ? 8 : 4;
+  const int B = kMode == kDrawPacked8 ? 8 : kMode == kDrawPacked4 ? 4 : (int)pbits;
   const uint32_t mag = u & 0x7FFFFFFFu;
   uint32_t q = min(mag + (1u << (22 - B)), 0x7F7FFFFFu);
   if (mag - 0x800000u >= 0x7F000000u) q = 0u;       // zero, sub-normal, Inf, NaN
@@ -603,6 +606,7 @@ __device__ __forceinline__ void sample_planes(const SampleParams& p, const uint3
   const uint32_t low01 = max_level >= 1u ? 0xFFFFFFFFu : 0xFFFFu, low23 = max_level >= 2u ? 0xFFFFFFFFu : 0u;
   const float second = max_level >= 1u ? 1.0f : 0.0f, rest = max_level >= 2u ? 1.0f : 0.0f;
   WindowBits win(norm ? 0u : window_exponent(windows[0], tag), (int)p.span);
+  const PackedDrawsAny any(kMode == kDrawAny && !p.deterministic ? p.pbits : 8u);
   // sums of the row a thread is in (one level)
   uint32_t run_row = 0u, run_abs = 0u;
   int run_sum = 0;
@@ -629,213 +633,233 @@ __device__ __forceinline__ void sample_planes(const SampleParams& p, const uint3
     float fs[4];
     uint32_t abs256;
     int sum;
-    if (kMode != kDrawAny) {
-      float scale[4], base[4], cnt[4];
-      uint32_t thr[4];
-      PhiloxWeight pw[4];
+    float scale[4], base[4], cnt[4];
+    uint32_t thr[4];
+    PhiloxWeight pw[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      decode_weight<kMode>(u[j], win, p.underflow, p.pbits, thr[j], base[j], scale[j]);
+      if (kMode != kDrawAny) pw[j] = PhiloxWeight(index0 + at + (uint32_t)j * KHKW, layer_key);
+    }
+    auto four_more = [&](uint32_t q) {
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        decode_weight<kMode>(u[j], win, p.underflow, thr[j], base[j], scale[j]);
-        pw[j] = PhiloxWeight(index0 + at + (uint32_t)j * KHKW, layer_key);
+        uint32_t rnd[4];
+        pw[j].call(q, keys, rnd);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) draw(cnt[j], rnd[i], thr[j]);
       }
-      auto four_more = [&](uint32_t q) {
+    };
+    if (kMode == kDrawAny) {
+      // Word by word, the fields of a word all at once; a level may end inside a word.  us, field by field and weight by weight / so:
+      // 25.5 M weights of the ResNet-50 shape with their exponent pass, 1 bit 1620 / 244, 3 bits, five levels 969 / 418, 6 bits,
+      // k = 64 649 / 576, deterministic, five levels 397 / 293; MobileNet-v2 shape, 7 bits, k = 64 231 / 104; 3x3 64->64, 1 bit 18.6 / 7.5.
+      uint32_t c[4] = {0u, 0u, 0u, 0u}, l = 0u;
+      auto complete = [&](const uint32_t (&count)[4]) {
+        const float k = (float)(1u << l);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) fs[j] = __fmul_rn(__fmaf_rn(base[j], k, (float)(int)count[j]), scale[j]);
+        if (kMulti) {
+          const int P = p.planes_count[l];
+          store_digits(P, plane_ptr(l, P), 6u + bk_shift, fs, abs256, sum);
+          add_row_sums(sums + l * (3u * kPlaneRows), r, abs256, sum, true);
+        }
+      };
+      if (p.deterministic) {
+#pragma unroll 1
+        for (l = kMulti ? 0u : max_level; l <= max_level; ++l) {
+          if (!((level_mask >> l) & 1u)) continue;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) c[j] = ((thr[j] << l) + (1u << (p.pbits - 1u))) >> p.pbits;
+          complete(c);
+        }
+      } else {
+        const uint32_t n = any.n;
+        uint32_t drawn = 0u, todo = level_mask;
+        l = (uint32_t)__ffs((int)todo) - 1u;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) pw[j] = PhiloxWeight(index0 + at + (uint32_t)j * KHKW, layer_key);
+#pragma unroll 1
+        for (uint32_t q = 0; todo; ++q) {
+          uint32_t hits[4][4];        // per weight and word; the word at hand comes first
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            uint32_t rnd[4];
+            pw[j].call(q, keys, rnd);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) hits[j][i] = any.below(rnd[i], thr[j]);
+          }
+          if ((1u << l) > drawn + 4u * n) {        // no level ends in this call
+#pragma unroll
+            for (int j = 0; j < 4; ++j) c[j] += (uint32_t)(__popc(hits[j][0]) + __popc(hits[j][1]) + __popc(hits[j][2]) + __popc(hits[j][3]));
+            drawn += 4u * n;
+            continue;
+          }
+#pragma unroll 1
+          for (int w = 0; w < 4 && todo; ++w, drawn += n) {
+            while (todo && (1u << l) <= drawn + n) {
+              const uint32_t left = (1u << l) - drawn, fields = left < n ? any.first(left) : 0xFFFFFFFFu;
+              uint32_t count[4];
+#pragma unroll
+              for (int j = 0; j < 4; ++j) count[j] = c[j] + (uint32_t)__popc(hits[j][0] & fields);
+              complete(count);
+              todo &= todo - 1u;
+              l = (uint32_t)__ffs((int)todo) - 1u;
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              c[j] += (uint32_t)__popc(hits[j][0]);
+              hits[j][0] = hits[j][1]; hits[j][1] = hits[j][2]; hits[j][2] = hits[j][3];
+            }
+          }
+        }
+      }
+    } else if (kMulti && (kMode == kDrawPacked8 || kMode == kDrawPacked4)) {
+      typedef PackedDraws<kMode == kDrawPacked8 ? 8 : 4> D;
+      uint32_t hits[4][4], c[4];        // per weight and word
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        uint32_t rnd[4];
+        pw[j].call(0u, keys, rnd);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) hits[j][i] = D::below(rnd[i], thr[j]);
+        c[j] = 0u;
+      }
+#pragma unroll 1
+      for (uint32_t l = 0; l <= max_level; ++l) {
+        if (l <= D::kFirstLevel) {
+          const uint32_t fields = l < D::kFirstLevel ? D::first(l) : 0xFFFFFFFFu;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) c[j] = (uint32_t)__popc(hits[j][0] & fields);
+        } else if (l == D::kFirstLevel + 1u) {
+#pragma unroll
+          for (int j = 0; j < 4; ++j) c[j] += (uint32_t)__popc(hits[j][1]);
+        } else if (l == D::kFirstLevel + 2u) {
+#pragma unroll
+          for (int j = 0; j < 4; ++j) c[j] += (uint32_t)(__popc(hits[j][2]) + __popc(hits[j][3]));
+        } else {
+#pragma unroll 1
+          for (uint32_t q = 1u << (l - D::kFirstLevel - 3u); q < 1u << (l - D::kFirstLevel - 2u); ++q)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              uint32_t rnd[4];
+              pw[j].call(q, keys, rnd);
+#pragma unroll
+              for (int i = 0; i < 4; ++i) c[j] += (uint32_t)__popc(D::below(rnd[i], thr[j]));
+            }
+        }
+        if (!((level_mask >> l) & 1u)) continue;
+        const float k = (float)(1u << l);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) fs[j] = __fmul_rn(__fmaf_rn(base[j], k, (float)(int)c[j]), scale[j]);
+        const int P = p.planes_count[l];
+        store_digits(P, plane_ptr(l, P), 6u + bk_shift, fs, abs256, sum);
+        add_row_sums(sums + l * (3u * kPlaneRows), r, abs256, sum, true);
+      }
+    } else if (kMode == kDrawPacked8) {
+      uint32_t count2[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        uint32_t rnd[4];
+        pw[j].call(0u, keys, rnd);
+        thr[j] = thr[j] * 0x10001u + 0x64006400u;
+        count2[j] = 0u;
+        // of fewer than four draws the others never fall below their threshold of 0
+        draw_word8(count2[j], (thr[j] & low01) | 0x64006400u, (thr[j] & low23) | 0x64006400u, rnd[0]);
+        if (max_level > 2u) draw_word8(count2[j], thr[j], thr[j], rnd[1]);
+        if (max_level > 3u) {
+          draw_word8(count2[j], thr[j], thr[j], rnd[2]);
+          draw_word8(count2[j], thr[j], thr[j], rnd[3]);
+        }
+      }
+#pragma unroll 1
+      for (uint32_t q = 1; q < (1u << max_level) / 16u; ++q)
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           uint32_t rnd[4];
           pw[j].call(q, keys, rnd);
 #pragma unroll
-          for (int i = 0; i < 4; ++i) draw(cnt[j], rnd[i], thr[j]);
+          for (int i = 0; i < 4; ++i) draw_word8(count2[j], thr[j], thr[j], rnd[i]);
         }
-      };
-      if (kMulti && (kMode == kDrawPacked8 || kMode == kDrawPacked4)) {
-        typedef PackedDraws<kMode == kDrawPacked8 ? 8 : 4> D;
-        uint32_t hits[4][4], c[4];        // per weight and word
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          uint32_t rnd[4];
-          pw[j].call(0u, keys, rnd);
-#pragma unroll
-          for (int i = 0; i < 4; ++i) hits[j][i] = D::below(rnd[i], thr[j]);
-          c[j] = 0u;
-        }
-#pragma unroll 1
-        for (uint32_t l = 0; l <= max_level; ++l) {
-          if (l <= D::kFirstLevel) {
-            const uint32_t fields = l < D::kFirstLevel ? D::first(l) : 0xFFFFFFFFu;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) c[j] = (uint32_t)__popc(hits[j][0] & fields);
-          } else if (l == D::kFirstLevel + 1u) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) c[j] += (uint32_t)__popc(hits[j][1]);
-          } else if (l == D::kFirstLevel + 2u) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) c[j] += (uint32_t)(__popc(hits[j][2]) + __popc(hits[j][3]));
-          } else {
-#pragma unroll 1
-            for (uint32_t q = 1u << (l - D::kFirstLevel - 3u); q < 1u << (l - D::kFirstLevel - 2u); ++q)
-#pragma unroll
-              for (int j = 0; j < 4; ++j) {
-                uint32_t rnd[4];
-                pw[j].call(q, keys, rnd);
-#pragma unroll
-                for (int i = 0; i < 4; ++i) c[j] += (uint32_t)__popc(D::below(rnd[i], thr[j]));
-              }
-          }
-          if (!((level_mask >> l) & 1u)) continue;
-          const float k = (float)(1u << l);
-#pragma unroll
-          for (int j = 0; j < 4; ++j) fs[j] = __fmul_rn(__fmaf_rn(base[j], k, (float)(int)c[j]), scale[j]);
-          const int P = p.planes_count[l];
-          store_digits(P, plane_ptr(l, P), 6u + bk_shift, fs, abs256, sum);
-          add_row_sums(sums + l * (3u * kPlaneRows), r, abs256, sum, true);
-        }
-      } else if (kMode == kDrawPacked8) {
-        uint32_t count2[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          uint32_t rnd[4];
-          pw[j].call(0u, keys, rnd);
-          thr[j] = thr[j] * 0x10001u + 0x64006400u;
-          count2[j] = 0u;
-          // of fewer than four draws the others never fall below their threshold of 0
-          draw_word8(count2[j], (thr[j] & low01) | 0x64006400u, (thr[j] & low23) | 0x64006400u, rnd[0]);
-          if (max_level > 2u) draw_word8(count2[j], thr[j], thr[j], rnd[1]);
-          if (max_level > 3u) {
-            draw_word8(count2[j], thr[j], thr[j], rnd[2]);
-            draw_word8(count2[j], thr[j], thr[j], rnd[3]);
-          }
-        }
-#pragma unroll 1
-        for (uint32_t q = 1; q < (1u << max_level) / 16u; ++q)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            uint32_t rnd[4];
-            pw[j].call(q, keys, rnd);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) draw_word8(count2[j], thr[j], thr[j], rnd[i]);
-          }
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const __half2 c = *reinterpret_cast<const __half2*>(&count2[j]);
-          cnt[j] = __fmaf_rn(base[j], k_max, __low2float(c) + __high2float(c));
-        }
-      } else if (kMode == kDrawPacked4) {
-        typedef PackedDraws<4> D;
-        const uint32_t fields = max_level < D::kFirstLevel ? D::first(max_level) : 0xFFFFFFFFu;
-        uint32_t c[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          uint32_t rnd[4];
-          pw[j].call(0u, keys, rnd);
-          c[j] = (uint32_t)__popc(D::below(rnd[0], thr[j]) & fields);
-          if (max_level > D::kFirstLevel) c[j] += (uint32_t)__popc(D::below(rnd[1], thr[j]));
-          if (max_level > D::kFirstLevel + 1u) c[j] += (uint32_t)(__popc(D::below(rnd[2], thr[j])) + __popc(D::below(rnd[3], thr[j])));
-        }
-#pragma unroll 1
-        for (uint32_t q = 1; q < (1u << max_level) / 32u; ++q)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            uint32_t rnd[4];
-            pw[j].call(q, keys, rnd);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) c[j] += (uint32_t)__popc(D::below(rnd[i], thr[j]));
-          }
-#pragma unroll
-        for (int j = 0; j < 4; ++j) cnt[j] = __fmaf_rn(base[j], k_max, (float)(int)c[j]);
-      } else if (!kMulti) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          uint32_t rnd[4];
-          pw[j].call(0u, keys, rnd);
-          cnt[j] = kMode == kDrawExact ? k_max : __fmul_rn(base[j], k_max);        // base k + c
-          draw(cnt[j], rnd[0], thr[j]);
-          draw(cnt[j], rnd[1], thr[j], second);
-          draw(cnt[j], rnd[2], thr[j], rest);
-          draw(cnt[j], rnd[3], thr[j], rest);
-        }
-        if (kCalls) {
-#pragma unroll
-          for (int q = 1; q < kCalls; ++q) four_more((uint32_t)q);
-        } else {
-#pragma unroll 1
-          for (uint32_t q = 1; q < (1u << max_level) / 4u; ++q) four_more(q);
-        }
-      } else {
-        float hit1[4], hit2[4];        // draw 1; draws 2 and 3
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          uint32_t rnd[4];
-          pw[j].call(0u, keys, rnd);
-          cnt[j] = hit1[j] = hit2[j] = 0.0f;
-          draw(cnt[j], rnd[0], thr[j]);
-          draw(hit1[j], rnd[1], thr[j]);
-          draw(hit2[j], rnd[2], thr[j]);
-          draw(hit2[j], rnd[3], thr[j]);
-        }
-#pragma unroll 1
-        for (uint32_t l = 0; l <= max_level; ++l) {
-          if (l == 1u || l == 2u) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) cnt[j] = __fadd_rn(cnt[j], l == 1u ? hit1[j] : hit2[j]);
-          } else if (l > 2u) {
-#pragma unroll 1
-            for (uint32_t q = 1u << (l - 3u); q < 1u << (l - 2u); ++q) four_more(q);
-          }
-          if (!((level_mask >> l) & 1u)) continue;
-          const float k = (float)(1u << l);
-#pragma unroll
-          for (int j = 0; j < 4; ++j) fs[j] = __fmul_rn(__fmaf_rn(base[j], k, cnt[j]), scale[j]);
-          const int P = p.planes_count[l];
-          store_digits(P, plane_ptr(l, P), 6u + bk_shift, fs, abs256, sum);
-          add_row_sums(sums + l * (3u * kPlaneRows), r, abs256, sum, true);
-        }
-      }
-      if (!kMulti)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) fs[j] = __fmul_rn(cnt[j], scale[j]);
-    } else if (!kMulti) {
-#pragma unroll 1       // one copy of the drawing code: four do not fit the instruction cache
       for (int j = 0; j < 4; ++j) {
-        Drawn dw;
-        const uint32_t uj = j == 0 ? u[0] : j == 1 ? u[1] : j == 2 ? u[2] : u[3];
-        classify_weight(uj, win.ebase, p.pbits, p.underflow, dw);
-        const PhiloxWeight pw(index0 + at + (uint32_t)j * KHKW, layer_key);
-        const float f = signed_weight(uj, dw, max_level, count_level(pw, dw.thr, max_level, p.pbits, p.deterministic, keys));
-        fs[0] = j == 0 ? f : fs[0]; fs[1] = j == 1 ? f : fs[1];
-        fs[2] = j == 2 ? f : fs[2]; fs[3] = j == 3 ? f : fs[3];
+        const __half2 c = *reinterpret_cast<const __half2*>(&count2[j]);
+        cnt[j] = __fmaf_rn(base[j], k_max, __low2float(c) + __high2float(c));
+      }
+    } else if (kMode == kDrawPacked4) {
+      typedef PackedDraws<4> D;
+      const uint32_t fields = max_level < D::kFirstLevel ? D::first(max_level) : 0xFFFFFFFFu;
+      uint32_t c[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        uint32_t rnd[4];
+        pw[j].call(0u, keys, rnd);
+        c[j] = (uint32_t)__popc(D::below(rnd[0], thr[j]) & fields);
+        if (max_level > D::kFirstLevel) c[j] += (uint32_t)__popc(D::below(rnd[1], thr[j]));
+        if (max_level > D::kFirstLevel + 1u) c[j] += (uint32_t)(__popc(D::below(rnd[2], thr[j])) + __popc(D::below(rnd[3], thr[j])));
+      }
+#pragma unroll 1
+      for (uint32_t q = 1; q < (1u << max_level) / 32u; ++q)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          uint32_t rnd[4];
+          pw[j].call(q, keys, rnd);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) c[j] += (uint32_t)__popc(D::below(rnd[i], thr[j]));
+        }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) cnt[j] = __fmaf_rn(base[j], k_max, (float)(int)c[j]);
+    } else if (!kMulti) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        uint32_t rnd[4];
+        pw[j].call(0u, keys, rnd);
+        cnt[j] = kMode == kDrawExact ? k_max : __fmul_rn(base[j], k_max);        // base k + c
+        draw(cnt[j], rnd[0], thr[j]);
+        draw(cnt[j], rnd[1], thr[j], second);
+        draw(cnt[j], rnd[2], thr[j], rest);
+        draw(cnt[j], rnd[3], thr[j], rest);
+      }
+      if (kCalls) {
+#pragma unroll
+        for (int q = 1; q < kCalls; ++q) four_more((uint32_t)q);
+      } else {
+#pragma unroll 1
+        for (uint32_t q = 1; q < (1u << max_level) / 4u; ++q) four_more(q);
       }
     } else {
-      uint32_t counts[kMaxLevels], meta = 0u;       // bytes j: counts per level; shift and base of weight j, whether it is live
+      float hit1[4], hit2[4];        // draw 1; draws 2 and 3
 #pragma unroll
-      for (int l = 0; l < kMaxLevels; ++l) counts[l] = 0u;
-#pragma unroll 1
       for (int j = 0; j < 4; ++j) {
-        Drawn dw;
-        draw_weight(j == 0 ? u[0] : j == 1 ? u[1] : j == 2 ? u[2] : u[3], index0 + at + (uint32_t)j * KHKW, win.ebase, p.pbits,
-                    p.underflow, p.deterministic, max_level, layer_key, keys, dw);
-        if (dw.live) {
-          meta |= (dw.sh | (dw.base << 4) | 0x20u) << (8 * j);
-#pragma unroll
-          for (int l = 0; l < kMaxLevels; ++l) counts[l] |= dw.cnt[l] << (8 * j);
-        }
+        uint32_t rnd[4];
+        pw[j].call(0u, keys, rnd);
+        cnt[j] = hit1[j] = hit2[j] = 0.0f;
+        draw(cnt[j], rnd[0], thr[j]);
+        draw(hit1[j], rnd[1], thr[j]);
+        draw(hit2[j], rnd[2], thr[j]);
+        draw(hit2[j], rnd[3], thr[j]);
       }
+#pragma unroll 1
+      for (uint32_t l = 0; l <= max_level; ++l) {
+        if (l == 1u || l == 2u) {
 #pragma unroll
-      for (int l = 0; l < kMaxLevels; ++l) {
-        if (!((level_mask >> l) & 1u)) continue;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const uint32_t m8 = meta >> (8 * j);
-          Drawn dw;
-          dw.base = (m8 >> 4) & 1u;
-          dw.sh = m8 & 15u;
-          dw.live = (m8 & 0x20u) != 0u;
-          fs[j] = signed_weight(u[j], dw, (uint32_t)l, (counts[l] >> (8 * j)) & 0xFFu);
+          for (int j = 0; j < 4; ++j) cnt[j] = __fadd_rn(cnt[j], l == 1u ? hit1[j] : hit2[j]);
+        } else if (l > 2u) {
+#pragma unroll 1
+          for (uint32_t q = 1u << (l - 3u); q < 1u << (l - 2u); ++q) four_more(q);
         }
+        if (!((level_mask >> l) & 1u)) continue;
+        const float k = (float)(1u << l);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) fs[j] = __fmul_rn(__fmaf_rn(base[j], k, cnt[j]), scale[j]);
         const int P = p.planes_count[l];
-        store_digits(P, plane_ptr((uint32_t)l, P), 6u + bk_shift, fs, abs256, sum);
+        store_digits(P, plane_ptr(l, P), 6u + bk_shift, fs, abs256, sum);
         add_row_sums(sums + l * (3u * kPlaneRows), r, abs256, sum, true);
       }
     }
+    if (!kMulti && kMode != kDrawAny)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) fs[j] = __fmul_rn(cnt[j], scale[j]);
     if (!kMulti) {
       const int P = p.planes_count[max_level];
       store_digits(P, plane_ptr(max_level, P), 6u + bk_shift, fs, abs256, sum);
@@ -910,8 +934,12 @@ __device__ __forceinline__ void sample_single(const SampleParams& p, const uint3
 // it stores their sums where the others add to words that the exponent pass has cleared.
 // kWhat: the filters that the instance serves, tap-major digit planes, the others, or (in a batch) both: a short launch's
 // time depends on how much code it carries.
+// Comparators that kDrawAny serves.
+__host__ __device__ inline bool other_options(const SampleParams& p) { return p.deterministic || (p.pbits != 0u && p.pbits != 4u && p.pbits != 8u); }
+
+enum SampleOptions { kNoOptions, kCommonOptions, kOtherOptions, kAllOptions };
 enum SampleWhat { kPlanesOnly, kSingleOnly, kBoth };
-template <bool kOptions, bool kFused, int kWhat>
+template <int kOptions, bool kFused, int kWhat>
 __device__ __forceinline__ void sample_block(const SampleParams& p, uint32_t tag, uint32_t block, const PhiloxKeys& keys,
                                              float* stage, RowSums& rs, uint32_t* err) {
   const uint32_t level_mask = p.level_mask, has_planes = p.has_planes, O = p.O;
@@ -1005,23 +1033,26 @@ __device__ __forceinline__ void sample_block(const SampleParams& p, uint32_t tag
     const bool multi = (level_mask & (level_mask - 1u)) != 0u;
 #define PSB_SAMPLE(MODE, MULTI, CALLS) sample_planes<MODE, MULTI, CALLS>(p, windows, tag, o0, c0, rows, cc, keys, stage, rs.word)
 #define PSB_SAMPLE_M(MODE) do { if (multi) PSB_SAMPLE(MODE, true, 0); else PSB_SAMPLE(MODE, false, 0); } while (0)
-    if (!kOptions || (p.pbits | p.underflow) == 0u) {
-      if (multi) PSB_SAMPLE(kDrawExact, true, 0);
-      else if (p.max_level <= 2u) PSB_SAMPLE(kDrawExact, false, 1);
-      else if (p.max_level == 3u) PSB_SAMPLE(kDrawExact, false, 2);
-      else if (p.max_level == 4u) PSB_SAMPLE(kDrawExact, false, 4);
-      else PSB_SAMPLE(kDrawExact, false, 0);
-    } else if constexpr (kOptions) {
+    if (kOptions == kNoOptions || (kOptions == kAllOptions && (p.pbits | p.underflow) == 0u)) {
+      if constexpr (kOptions == kNoOptions || kOptions == kAllOptions) {
+        if (multi) PSB_SAMPLE(kDrawExact, true, 0);
+        else if (p.max_level <= 2u) PSB_SAMPLE(kDrawExact, false, 1);
+        else if (p.max_level == 3u) PSB_SAMPLE(kDrawExact, false, 2);
+        else if (p.max_level == 4u) PSB_SAMPLE(kDrawExact, false, 4);
+        else PSB_SAMPLE(kDrawExact, false, 0);
+      }
+    } else if (kOptions == kOtherOptions || (kOptions == kAllOptions && other_options(p))) {
+      if constexpr (kOptions >= kOtherOptions) PSB_SAMPLE_M(kDrawAny);
+    } else if constexpr (kOptions != kNoOptions && kOptions != kOtherOptions) {
       if (p.pbits == 0u) PSB_SAMPLE_M(kDrawGate);
-      else if (p.pbits == 8u && !p.deterministic) PSB_SAMPLE_M(kDrawPacked8);
-      else if (p.pbits == 4u && !p.deterministic) PSB_SAMPLE_M(kDrawPacked4);
-      else PSB_SAMPLE_M(kDrawAny);
+      else if (p.pbits == 8u) PSB_SAMPLE_M(kDrawPacked8);
+      else PSB_SAMPLE_M(kDrawPacked4);
     }
 #undef PSB_SAMPLE_M
 #undef PSB_SAMPLE
    }
   } else if constexpr (kWhat != kPlanesOnly) {
-    sample_single<kOptions>(p, windows, tag, o0, c0, rows, cc, keys, stage, rs.word);
+    sample_single<kOptions != kNoOptions>(p, windows, tag, o0, c0, rows, cc, keys, stage, rs.word);
   }
   __syncthreads();
   for (uint32_t l = 0; l < (uint32_t)kMaxLevels; ++l) {
@@ -1041,7 +1072,7 @@ __device__ __forceinline__ void sample_block(const SampleParams& p, uint32_t tag
   }
 }
 
-template <bool kOptions, bool kFused, bool kSingle>
+template <int kOptions, bool kFused, bool kSingle>
 __global__ void __launch_bounds__(kThreads, 3) sample_kernel(const __grid_constant__ SampleParams p,
                                                           const __grid_constant__ PhiloxKeys keys, uint32_t* err) {
   pdl_prologue();
@@ -1067,7 +1098,7 @@ __global__ void __launch_bounds__(kThreads) emax_batch_kernel(const BatchEntry* 
              blockIdx.x - e.emax_first, e.emax_blocks, tag << 8, e.p.rowsum, e.p.corr, e.p.pbits);
 }
 
-template <bool kOptions>
+template <int kOptions>
 __global__ void __launch_bounds__(kBatchThreads, 6) sample_batch_kernel(const BatchEntry* entries, const uint32_t* entry_of,
                                                                 uint32_t tag, const __grid_constant__ PhiloxKeys keys) {
   pdl_prologue();
@@ -1220,8 +1251,9 @@ uint32_t fill_sample_params(const float* w_dev, const psb_weights* wt, uint32_t*
 template <bool kFused>
 cudaError_t launch_sample_kernel(const SampleParams& p, uint32_t blocks, const PhiloxKeys& keys, uint32_t* err_dev, cudaStream_t s) {
   const bool options = (p.pbits | p.underflow) != 0u, single = !p.has_planes || p.packed_kw;
-  const auto kernel = options ? (single ? sample_kernel<true, kFused, true> : sample_kernel<true, kFused, false>)
-                              : (single ? sample_kernel<false, kFused, true> : sample_kernel<false, kFused, false>);
+  const auto kernel = single    ? (options ? sample_kernel<kCommonOptions, kFused, true> : sample_kernel<kNoOptions, kFused, true>)
+                      : !options ? sample_kernel<kNoOptions, kFused, false>
+                                 : other_options(p) ? sample_kernel<kOtherOptions, kFused, false> : sample_kernel<kCommonOptions, kFused, false>;
   launch_pdl(kernel, blocks, sample_threads(p, blocks, kFused), stage_bytes(p), s, p, keys, err_dev);
   note_launch();
   return cudaGetLastError();
@@ -1346,7 +1378,7 @@ psb_status sample_batch_run(psb_ctx* ctx, psb_sample_batch* b, uint64_t seed, cu
   note_launch();
   const PhiloxKeys keys((uint32_t)seed, (uint32_t)(seed >> 32));
   const uint32_t* entry_of = b->entry_of_dev + b->emax_grid;
-  launch_pdl(b->options ? sample_batch_kernel<true> : sample_batch_kernel<false>, b->sample_grid, kBatchThreads, b->stage_bytes, s,
+  launch_pdl(b->options ? sample_batch_kernel<kAllOptions> : sample_batch_kernel<kNoOptions>, b->sample_grid, kBatchThreads, b->stage_bytes, s,
              (const BatchEntry*)b->entries_dev, entry_of, b->calls, keys);
   note_launch();
   return cudaGetLastError() == cudaSuccess ? PSB_OK : PSB_ERR_CUDA;

@@ -177,3 +177,11 @@ def test_decoding_and_counting_at_their_edges(opts, levels, oracle):
         assert ctx.device_status() == 0
         wt.free()
     ctx.close()
+
+
+@pytest.mark.parametrize("opts", [dict(prob_bits=b, underflow=b % 2, exp_bits=4 - b % 3) for b in (1, 2, 3, 5, 6, 7)] +
+                         [dict(prob_bits=3, deterministic=1, underflow=1), dict(prob_bits=8, deterministic=1), dict(prob_bits=4, deterministic=1, exp_bits=3)])
+@pytest.mark.parametrize("levels", [(0, 1, 2, 3, 4, 5, 6), (1, 5), (6,), (4,), (0,)])
+def test_comparators_of_other_widths(opts, levels, oracle):
+    """Widths whose words end inside a level (3, 5, 6 bits) and at one, one level and several; no draws at all."""
+    test_decoding_and_counting_at_their_edges(opts, levels, oracle)
