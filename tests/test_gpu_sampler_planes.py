@@ -185,3 +185,13 @@ def test_decoding_and_counting_at_their_edges(opts, levels, oracle):
 def test_comparators_of_other_widths(opts, levels, oracle):
     """Widths whose words end inside a level (3, 5, 6 bits) and at one, one level and several; no draws at all."""
     test_decoding_and_counting_at_their_edges(opts, levels, oracle)
+
+
+@pytest.mark.parametrize("case", [
+    # (rows, channels, filter size): one to six rows in a block of eight warps, one to four in a block of four, which share them out;
+    # tap-major planes, then flat K axes
+    (40, 300, 1), (1300, 160, 1), (2000, 160, 1), (2500, 160, 1), (3100, 160, 1), (30, 20, 3), (1000, 2400, 1), (1900, 2100, 1),
+    (4600, 1000, 1), (40, 3, 7), (64, 12, 5), (2400, 15, 3),
+])
+def test_windows_of_rows_that_warps_share(case, oracle):
+    test_windows_found_by_the_sampler_or_by_a_pass_of_their_own((1, *case, 1), oracle)
