@@ -878,7 +878,9 @@ __device__ __forceinline__ void sample_planes(const SampleParams& p, const uint3
 
 // Everything else, one weight per thread and step: depthwise and grouped filters (integer filter, channels
 // innermost, for the CUDA-core kernels) and flat K axes (few input channels).
-template <bool kOptions>
+// kOwnBases: launches of such a layer alone take the bases along here and read the windows of an exponent pass where they are;
+// passed through shared memory and stored apart, depthwise 3x3 on 960 channels took 4.9 us and not 4.7, 5x5 12->128 7.5 and not 7.1.
+template <bool kOptions, bool kOwnBases>
 __device__ __forceinline__ void sample_single(const SampleParams& p, const uint32_t* windows, uint32_t tag, uint32_t o0,
                                               uint32_t c0, uint32_t rows, uint32_t cc, const PhiloxKeys& keys, const float* stage,
                                               uint32_t* sums) {
@@ -896,6 +898,7 @@ __device__ __forceinline__ void sample_single(const SampleParams& p, const uint3
     const uint32_t index = o * d + ci * KHKW + tap;  // canonical
     const uint32_t Emax = window_exponent(windows[p.norm ? r : 0u], tag);
     const int ebase_biased = (int)Emax - (int)p.span;
+    if (kOwnBases && tap == 0u && ci == 0u) p.e_base[o] = Emax ? ebase_biased - 127 : 0;
     Drawn dw;
     draw_weight(u, index, ebase_biased, kOptions ? p.pbits : 0u, kOptions ? p.underflow : 0u, kOptions ? p.deterministic : 0u,
                 max_level, layer_key, keys, dw);
@@ -965,8 +968,11 @@ __device__ __forceinline__ void sample_block(const SampleParams& p, uint32_t tag
       for (uint32_t t = threadIdx.x; t < count; t += blockDim.x) stage[t] = __ldca(src + t);
     }
   }
-  __shared__ uint32_t windows[kRowSumRows];      // of the rows of this block, or the layer's
-  if (!kFused) {
+  __shared__ uint32_t found[kRowSumRows];      // of the rows of this block, or the layer's
+  uint32_t* windows = found;
+  if (!kFused && kWhat == kSingleOnly) {
+    windows = const_cast<uint32_t*>(p.e_max) + (p.norm ? o0 : 0u);
+  } else if (!kFused) {
     for (uint32_t r = threadIdx.x; r < (p.norm ? rows : 1u); r += blockDim.x) windows[r] = p.e_max[(p.norm ? o0 : 0u) + r];
   } else {
     const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u, d = p.d;
@@ -1005,17 +1011,17 @@ __device__ __forceinline__ void sample_block(const SampleParams& p, uint32_t tag
         }
       }
     } else {
-      // one window for a small layer: every block looks at all of it
+      // one window for a small layer: every block, of kThreads threads, looks at all of it
       const uint32_t total = O * d, head = (((uintptr_t)p.w) & 15u) == 0u ? total & ~3u : 0u;
       uint32_t best = 0u;
       const uint4* w4 = reinterpret_cast<const uint4*>(p.w);
 #pragma unroll 8
-      for (uint32_t i = threadIdx.x; i < head / 4u; i += blockDim.x) {
+      for (uint32_t i = threadIdx.x; i < head / 4u; i += (uint32_t)kThreads) {
         const uint4 v = __ldca(w4 + i);
         const uint32_t u4[4] = {v.x, v.y, v.z, v.w};
         best = max_magnitude(u4, best, bad);
       }
-      for (uint32_t i = head + threadIdx.x; i < total; i += blockDim.x) {
+      for (uint32_t i = head + threadIdx.x; i < total; i += (uint32_t)kThreads) {
         const uint32_t u1[1] = {__float_as_uint(__ldca(p.w + i))};
         best = max_magnitude(u1, best, bad);
       }
@@ -1023,7 +1029,7 @@ __device__ __forceinline__ void sample_block(const SampleParams& p, uint32_t tag
       if (lane == 0u) windows[1u + warp] = best;
       __syncthreads();
       if (threadIdx.x == 0u) {
-        for (uint32_t i = 2u; i <= blockDim.x / 32u; ++i) best = max(best, windows[i]);
+        for (uint32_t i = 2u; i <= (uint32_t)kThreads / 32u; ++i) best = max(best, windows[i]);
         windows[0] = quantised_exponent(best, p.pbits);
       }
     }
@@ -1031,7 +1037,7 @@ __device__ __forceinline__ void sample_block(const SampleParams& p, uint32_t tag
     tag = 0u;
   }
   __syncthreads();
-  if (chunk == 0u)
+  if (kWhat != kSingleOnly && chunk == 0u)
     for (uint32_t r = threadIdx.x; r < rows; r += blockDim.x) {
       const uint32_t Emax = window_exponent(windows[p.norm ? r : 0u], tag);
       p.e_base[o0 + r] = Emax ? (int)Emax - (int)p.span - 127 : 0;
@@ -1060,7 +1066,7 @@ __device__ __forceinline__ void sample_block(const SampleParams& p, uint32_t tag
 #undef PSB_SAMPLE
    }
   } else if constexpr (kWhat != kPlanesOnly) {
-    sample_single<kOptions != kNoOptions>(p, windows, tag, o0, c0, rows, cc, keys, stage, rs.word);
+    sample_single<kOptions != kNoOptions, kWhat == kSingleOnly>(p, windows, tag, o0, c0, rows, cc, keys, stage, rs.word);
   }
   __syncthreads();
   for (uint32_t l = 0; l < (uint32_t)kMaxLevels; ++l) {
@@ -1193,7 +1199,7 @@ bool fused_sampling(const psb_weights* wt) {
 // 20.6 / 22.4, 592x4096 32.2 / 40.3; 512x2048, 1024 blocks, 22.5 / 21.0, 3x3 256->256, 768 blocks, 23.5 / 22.3).
 uint32_t sample_threads(const SampleParams& p, uint32_t blocks, bool fused) {
   if (!p.has_planes || p.packed_kw) return 256u;
-  if (fused) return blocks < 6u * kSms ? 256u : 128u;
+  if (fused) return !p.norm || blocks < 6u * kSms ? 256u : 128u;
   return blocks <= 4u * kSms && p.rows_per_block * p.ch_per_block * p.KHKW >= 1024u ? 256u : 128u;
 }
 
