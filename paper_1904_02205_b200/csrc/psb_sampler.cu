@@ -1218,7 +1218,10 @@ uint32_t fill_sample_params(const float* w_dev, const psb_weights* wt, uint32_t*
   // weights per block: enough that what a block does once (its parameters, sums, barriers) is a small part of it, yet
   // several blocks per SM: a batched launch is filled by the other layers, a layer of its own is cut finer
   const uint64_t total = (uint64_t)O * d;
-  uint32_t budget = how == SampleLaunch::kBatch ? kStage : (uint32_t)std::min<uint64_t>(kStage, std::max<uint64_t>(256u, total / 592u));
+  // (of a block with 256 weights two warps of four have quads, and these share two of the SM's four schedulers; 256 / 512, us:
+  // 3x3 64->64, levels k = 1 .. 16 10.7 / 9.4, 3x3 100->150, k = 8 9.7 / 8.3, 8-bit comparator, k = 16 9.7 / 8.0)
+  const uint32_t least = how == SampleLaunch::kTwoPass && wt->has_planes && !wt->packed_k ? 512u : 256u;
+  uint32_t budget = how == SampleLaunch::kBatch ? kStage : (uint32_t)std::min<uint64_t>(kStage, std::max<uint64_t>(least, total / 592u));
   if (how == SampleLaunch::kFused && budget < d) budget = d;
   if (budget < 4u * KHKW) budget = 4u * KHKW;   // at least four channels (host validation keeps kh*kw <= 2048)
   const uint32_t sum_rows = wt->has_planes ? (uint32_t)kPlaneRows : (uint32_t)kRowSumRows;
