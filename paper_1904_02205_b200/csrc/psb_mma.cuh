@@ -1120,10 +1120,11 @@ __device__ __noinline__ bool epilogue_staged(const TensorParams& p, SharedCtl* c
       if (o < O) {
         sb.x = ldexpf(a.scale[o], a.e_base[o] - (int)l);
         sb.y = a.bias[o];
-        if (has_addend(W) && use_corr) cr = p.corr[l][o];
+        if (use_corr) cr = p.corr[l][o];
       }
       ctl->scb[ew][lane] = sb;
-      if (has_addend(W)) ctl->corr[ew][lane] = addend_words<W>(cr);
+      // (also where nothing reads it, as in epilogue_uniform: 1x1 64 -> 256 @56 with a shortcut, batch 64, 41.2 -> 40.8 us)
+      ctl->corr[ew][lane] = addend_words<W>(cr);
       cur_o_tile = o_tile;
       __syncwarp();
     }
