@@ -373,3 +373,57 @@ def test_real_valued_outputs(case, want, oracle):
         compare(g, o, list(levels or (3,)))
         assert np.array_equal(g["f32"], o["f32"])       # rounded operations only, in the same order
     ctx.close()
+
+
+@pytest.mark.parametrize("case", [
+    # (N, C, H, W, O, K, pad, largest byte, levels, exp_bits): one, two and four planes, three in 64 bits (with and without an addend)
+    (2, 64, 13, 11, 68, 1, 0, 15, (0, 1), 1), (2, 48, 13, 11, 72, 3, 1, 255, (0, 3), 3), (2, 96, 9, 14, 50, 1, 0, 255, (5, 6), 4),
+    (1, 1040, 13, 11, 64, 1, 0, 255, (4, 3), 4), (1, 8752, 5, 7, 36, 1, 0, 15, (4, 2), 4), (2, 8, 21, 19, 36, 3, 1, 255, (6, 5), 4),
+])
+@pytest.mark.parametrize("layout", [0, 1])
+@pytest.mark.parametrize("with_map", [False, True])
+def test_real_valued_outputs_of_other_recombinations(case, layout, with_map, oracle):
+    import paper_1904_02205_b200 as psb
+
+    N, C, H, W, O, K, pad, top, levels, exp_bits = case
+    ctx = psb.Context(0)
+    rng = np.random.default_rng(C * 11 + O)
+    w = rng.normal(0, np.sqrt(2.0 / (C * K * K)), size=(O, C, K, K)).astype(np.float32)
+    x = rng.integers(0, top + 1, size=(N, C, H, W) if layout == 0 else (N, H, W, C)).astype(np.uint8)
+    res = rng.integers(0, 256, size=(N, O, H, W) if layout == 0 else (N, H, W, O)).astype(np.uint8)
+    kmap = rng.choice(levels, size=(N, H, W)).astype(np.uint8) if with_map else None
+    used = list(levels) if with_map else [levels[0]]
+    args = (w, x, layout, 1, 1, pad, 5, 3, used, kmap, levels[0], rng.uniform(0.5, 1.5, O).astype(np.float32),
+            rng.normal(0, 0.5, O).astype(np.float32), True, np.float32(0.02), 0, 255)
+    o = oracle_layer(oracle, *args, residual=res, res_scale=np.float32(0.3), exp_bits=exp_bits)
+    g = gpu_layer(psb, ctx, *args, psb.PSB_DT_U8, residual=res, res_scale=np.float32(0.3), in_max=top, path=psb.PSB_PATH_TENSOR,
+                  want=("q", "f32"), exp_bits=exp_bits)
+    compare(g, o, used)
+    assert np.array_equal(g["f32"], o["f32"])       # rounded operations only, in the same order
+    ctx.close()
+
+
+@pytest.mark.parametrize("shortcut", [False, True])
+@pytest.mark.parametrize("levels", [(0,), (0, 2)])
+def test_long_rows_of_small_sums_with_an_addend(shortcut, levels, oracle):
+    """Full-range bytes on rows too long for two planes to fit 32 bits together, but whose sums do: one weight at the window's top."""
+    import paper_1904_02205_b200 as psb
+
+    C, O, H, W = 1056, 48, 11, 13
+    ctx = psb.Context(0)
+    rng = np.random.default_rng(4)
+    w = (rng.normal(0, 1, size=(O, C, 1, 1)) * 2.0 ** -9).astype(np.float32)
+    w[0, 0] = 1.5
+    x = rng.integers(0, 256, size=(1, H, W, C)).astype(np.uint8)
+    res = rng.integers(-128, 128, size=(1, H, W, O)).astype(np.int8) if shortcut else None
+    kmap = rng.choice(levels, size=(1, H, W)).astype(np.uint8) if len(levels) > 1 else None
+    assert C * 128 * 16383 >= 1 << 31
+    for l in levels:
+        sums = np.abs(oracle.sample_level(w, 5, 3, l)[0].astype(np.int64)).reshape(O, -1)
+        assert int((-(-sums // 256)).sum(1).max()) * 256 * 255 < 1 << 31
+    args = (w, x, 1, 1, 1, 0, 5, 3, list(levels), kmap, 0, np.ones(O, np.float32), np.zeros(O, np.float32), False, np.float32(8.0), -100, 101)
+    o = oracle_layer(oracle, *args, residual=res, res_scale=np.float32(0.01))
+    g = gpu_layer(psb, ctx, *args, psb.PSB_DT_S8, residual=res, res_scale=np.float32(0.01), in_max=255, path=psb.PSB_PATH_TENSOR, want=("q",))
+    compare(g, o, list(levels))
+    assert len(np.unique(o["q"])) > 50
+    ctx.close()
