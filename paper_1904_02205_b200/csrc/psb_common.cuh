@@ -47,7 +47,9 @@ __host__ __device__ inline uint32_t plane_offset(uint32_t row, uint32_t kin, uin
 
 struct LevelStore {
   int32_t* wint = nullptr;  // [O][KH][KW][Cg]  signed integer filter, channels innermost (filters without planes)
-  int8_t* planes = nullptr; // [O_tiles][K blocks][P * kTileN rows][bk bytes]  signed 7-bit digits: every
+  int8_t* planes = nullptr; // [O_tiles][K blocks][P * kTileN rows][bk bytes]  signed 7-bit digits, all but the top one in
+                            // -127 .. 127, the top one in -64 .. 64: of the two's complement where the K axis is tap-major
+                            // (lower digits 0 .. 127), of the magnitude with the weight's sign where it is flat.  Every
                             // (channel tile, K block) operand tile is contiguous and already in the
                             // swizzled order the MMA reads from shared memory (plane_offset below)
   int planes_count = 0;

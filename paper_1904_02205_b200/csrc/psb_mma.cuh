@@ -7,7 +7,7 @@
 // tcgen05.mma (kind::i8, s8 x s8 -> s32) of shape 128 x (P*64) x 32 multiplies an
 // activation tile with all planes of 64 output channels at once; each plane owns
 // 64 accumulator columns in tensor memory (TMEM) and the epilogue recombines them
-// in 64-bit integers, which makes the result exact.
+// exactly (Recombine).
 //
 // Structure of one CTA (one per SM, persistent over tiles):
 //   warps 0-1 producers (one thread each, taking the stages in turns): TMA loads of the activation tile (im2col mode for
@@ -343,7 +343,7 @@ struct SharedCtl {
 //              With t = v0 + 2^7 v1 the accumulator is 2^14 (v2 + (t >> 14)) + (t mod 2^14), the upper part below 2^24 in
 //              magnitude: both parts are exact floats and one fma rounds their sum.  2^23 + the lower part is a bit
 //              pattern, and the 2^23 is taken off the upper part, as 512.  kRecMidAdd: plus an addend per channel, split alike.
-//   kRec64:    everything else.
+//   kRec64:    everything else.  (Of the networks' layers the classifier of the MobileNet-v2 shape, 1280 inputs with bytes to 255.)
 // An output costs a warp about 12 clocks of dispatch beside this; in 32 bits it adds 5, kRecMid 9, in 64 bits 23 (two 64-bit
 // multiply-adds, the addend's 64 bits, two conversions).  Maps of five levels, ResNet-50 shape,
 // batch 128: 4753 -> 4645 us; MobileNet-v2 shape, 8 bits, batch 64: 1042 -> 1013.
@@ -584,7 +584,8 @@ __device__ __noinline__ void epilogue_chunk_q(uint32_t taddr, bool valid, uint8_
   else if (valid) store_row16(q_out + off, q, unit == 16u, count >= 16u);
 }
 
-// General output stage: any combination of outputs, layouts, ragged channel counts.
+// General output stage: accumulators with any other outputs beside them, and codes that no other loop takes; any layout and
+// channel count.
 template <int P>
 __device__ __noinline__ void epilogue_chunk(const TensorParams& p, uint32_t taddr, uint32_t o_base,
                                             uint32_t m, bool valid, uint32_t n, uint32_t pix,
@@ -1182,8 +1183,7 @@ __device__ __noinline__ bool epilogue_staged(const TensorParams& p, SharedCtl* c
 // two groups of warps of epilogue_staged, but the rows of a tile lie anywhere in the tensors, so every warp moves its own
 // 32 rows x 32 bytes, two lanes per row (whole sectors, 16 cache lines per instruction instead of 32): the shortcut of its
 // next tile into a slot of its own by asynchronous copies, the codes from the slot to the tensor.  Bound
-// by the instructions of the 64-bit recombination and by L2 sectors; with a row per lane, every load and store touched 32
-// lines for 16 bytes each (ResNet-50 shape, batch 128, maps of five levels: 5401 -> 4853 us, layers with a shortcut and
+// by instruction issue and by L2 sectors; with a row per lane, every load and store touched 32 lines for 16 bytes each (ResNet-50 shape, batch 128, maps of five levels: 5401 -> 4853 us, layers with a shortcut and
 // without; its attention mode, batch 32 in the second pass: 3109 -> 2980 us).
 template <int P, int W, int RES, bool FAST_U8>
 __device__ __noinline__ bool epilogue_sorted(const TensorParams& p, SharedCtl* ctl, uint32_t tmem_base, uint32_t slots_addr,

@@ -1184,7 +1184,7 @@ uint32_t emax_blocks_for(uint32_t O, uint32_t d, uint32_t norm) {
 //   window per row:  a block takes a whole row, so long rows need rows for two blocks per SM, or, with taps, for one.  256x1536
 //                    16.4 / 14.0, 64x2048 16.2 / 13.8, 1000x2048 30.6 / 28.4; 10x4096 16.2 / 17.3, 148x4096 20.6 / 24.5, 256x4096 24.4 / 24.9,
 //                    400x4096 28.7 / 26.4, 2048x4096 77.5 / 73.3; 3x3 256->64 20.4 / 18.4, 400->32 24.5 / 25.2, 256->256 22.4 / 21.7,
-//                    400->256 31.9 / 32.4.  (Between 65 and 295 rows of 1537 to 2304 weights one launch would now be the faster,
+//                    400->256 31.9 / 32.4 (the wrong side of the line by 0.5).  (Between 65 and 295 rows of 1537 to 2304 weights one launch would now be the faster,
 //                    148x2048 16.2 / 13.9; the number of launches at this line is part of what the tests hold fast.)
 bool fused_sampling(const psb_weights* wt) {
   const uint32_t d = wt->d, rows = wt->shape.out_ch;
