@@ -1208,20 +1208,20 @@ enum class SampleLaunch { kBatch, kTwoPass, kFused };
 // Shared memory for the largest slice of a block.
 uint32_t stage_bytes(const SampleParams& p) { return p.rows_per_block * p.ch_per_block * p.KHKW * (uint32_t)sizeof(float); }
 
-// Parameters of one layer's sampling pass; returns the number of blocks it needs.
+// Parameters of one layer's sampling pass in a launch over `launch_weights` weights; returns the number of blocks it needs.
 uint32_t fill_sample_params(const float* w_dev, const psb_weights* wt, uint32_t* e_max, SampleParams& p,
-                            SampleLaunch how) {
+                            SampleLaunch how, uint64_t launch_weights) {
   const psb_wshape& sh = wt->shape;
   const uint32_t O = sh.out_ch, Cg = sh.in_ch_per_group, KHKW = sh.kh * sh.kw, d = wt->d;
   p.w = w_dev;
   p.O = O; p.Cg = Cg; p.KHKW = KHKW; p.d = d;
-  // weights per block: enough that what a block does once (its parameters, sums, barriers) is a small part of it, yet
-  // several blocks per SM: a batched launch is filled by the other layers, a layer of its own is cut finer
-  const uint64_t total = (uint64_t)O * d;
-  // (of a block with 256 weights two warps of four have quads, and these share two of the SM's four schedulers; 256 / 512, us:
-  // 3x3 64->64, levels k = 1 .. 16 10.7 / 9.4, 3x3 100->150, k = 8 9.7 / 8.3, 8-bit comparator, k = 16 9.7 / 8.0)
-  const uint32_t least = how == SampleLaunch::kTwoPass && wt->has_planes && !wt->packed_k ? 512u : 256u;
-  uint32_t budget = how == SampleLaunch::kBatch ? kStage : (uint32_t)std::min<uint64_t>(kStage, std::max<uint64_t>(least, total / 592u));
+  // weights per block: enough that what a block does once (its parameters, sums, barriers) is a small part of it, yet four blocks
+  // per SM of the launch, which is all layers of a batch (13 layers, 38 k weights, k = 1 and 16, with blocks of 4608 / so, us:
+  // 23.6 and 28.7 / 8.5 and 9.2).  (Of a block with 256 weights two warps of four have quads, and these share two of the SM's four
+  // schedulers; 256 / 512, us: 3x3 64->64, levels k = 1 .. 16 10.7 / 9.4, 3x3 100->150, k = 8 9.7 / 8.3, 8-bit comparator, k = 16
+  // 9.7 / 8.0.)
+  const uint32_t least = how != SampleLaunch::kFused && wt->has_planes && !wt->packed_k ? 512u : 256u;
+  uint32_t budget = (uint32_t)std::min<uint64_t>(kStage, std::max<uint64_t>(least, launch_weights / 592u));
   if (how == SampleLaunch::kFused && budget < d) budget = d;
   if (budget < 4u * KHKW) budget = 4u * KHKW;   // at least four channels (host validation keeps kh*kw <= 2048)
   const uint32_t sum_rows = wt->has_planes ? (uint32_t)kPlaneRows : (uint32_t)kRowSumRows;
@@ -1290,7 +1290,7 @@ cudaError_t launch_sampler(const float* w_dev, psb_weights* wt, uint32_t* err_de
   const PhiloxKeys keys((uint32_t)wt->cfg.seed, (uint32_t)(wt->cfg.seed >> 32));
   SampleParams p;
   if (fused_sampling(wt)) {
-    const uint32_t blocks = fill_sample_params(w_dev, wt, wt->e_max, p, SampleLaunch::kFused);
+    const uint32_t blocks = fill_sample_params(w_dev, wt, wt->e_max, p, SampleLaunch::kFused, (uint64_t)wt->shape.out_ch * wt->d);
     return launch_sample_kernel<true>(p, blocks, keys, err_dev, s);
   }
   const uint32_t O = wt->shape.out_ch;
@@ -1304,7 +1304,7 @@ cudaError_t launch_sampler(const float* w_dev, psb_weights* wt, uint32_t* err_de
   }
   launch_pdl(emax_kernel, emax_blocks_for(O, wt->d, wt->cfg.norm), kThreads, 0, s, w_dev, O, wt->d, wt->cfg.norm,
              wt->e_max, err_dev, wt->e_calls << 8, wt->rowsum256, wt->corr128, wt->cfg.prob_bits); note_launch();
-  const uint32_t blocks = fill_sample_params(w_dev, wt, wt->e_max, p, SampleLaunch::kTwoPass);
+  const uint32_t blocks = fill_sample_params(w_dev, wt, wt->e_max, p, SampleLaunch::kTwoPass, (uint64_t)wt->shape.out_ch * wt->d);
   p.e_tag = wt->e_calls;
   return launch_sample_kernel<false>(p, blocks, keys, err_dev, s);
 }
@@ -1332,7 +1332,11 @@ psb_status sample_batch_create(psb_ctx* ctx, uint32_t n, const float* const* w_d
   BatchEntry* host = new (std::nothrow) BatchEntry[n];
   if (!b || !host) { delete b; delete[] host; return PSB_ERR_ALLOC; }
   size_t words = 0;
-  for (uint32_t i = 0; i < n; ++i) words += weights[i]->shape.out_ch;
+  uint64_t total = 0;
+  for (uint32_t i = 0; i < n; ++i) {
+    words += weights[i]->shape.out_ch;
+    total += (uint64_t)weights[i]->shape.out_ch * weights[i]->d;
+  }
   bool ok = cudaMalloc(&b->e_max_pool, sizeof(uint32_t) * words) == cudaSuccess &&
             cudaMemset(b->e_max_pool, 0, sizeof(uint32_t) * words) == cudaSuccess &&
             cudaMalloc(&b->entries_dev, sizeof(BatchEntry) * n) == cudaSuccess;
@@ -1342,7 +1346,7 @@ psb_status sample_batch_create(psb_ctx* ctx, uint32_t n, const float* const* w_d
     for (uint32_t i = 0; i < n; ++i) {
       const psb_weights* wt = weights[i];
       BatchEntry& e = host[i];
-      e.sample_blocks = fill_sample_params(w_dev[i], wt, b->e_max_pool + off, e.p, SampleLaunch::kBatch);
+      e.sample_blocks = fill_sample_params(w_dev[i], wt, b->e_max_pool + off, e.p, SampleLaunch::kBatch, total);
       b->stage_bytes = std::max(b->stage_bytes, stage_bytes(e.p));
       b->options = b->options || (e.p.pbits | e.p.underflow);
       e.emax_blocks = emax_blocks_for(wt->shape.out_ch, wt->d, wt->cfg.norm);

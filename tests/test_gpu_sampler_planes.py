@@ -195,3 +195,34 @@ def test_comparators_of_other_widths(opts, levels, oracle):
 ])
 def test_windows_of_rows_that_warps_share(case, oracle):
     test_windows_found_by_the_sampler_or_by_a_pass_of_their_own((1, *case, 1), oracle)
+
+
+@pytest.mark.parametrize("scale", [1, 3, 9])
+@pytest.mark.parametrize("opts", [dict(), dict(norm=1, prob_bits=5, underflow=1), dict(prob_bits=8)])
+def test_batches_of_any_size(scale, opts, oracle):
+    """The blocks of a batch are cut by the weights of all its layers: 22 thousand, 142 thousand and 1.1 million here, every kind of filter
+    among them, rows that no block holds as a whole and rows that many fit into one."""
+    import torch
+
+    import paper_1904_02205_b200 as psb
+
+    ctx = psb.Context(0)
+    rng = np.random.default_rng(scale)
+    shapes = [((24 * scale, 3, 7, 7), 1), ((32 * scale, 1, 3, 3), 32 * scale), ((16 * scale, 70 * scale, 3, 3), 1), ((33, 17 * scale, 1, 1), 1),
+              ((64 * scale, 48 * scale, 1, 1), 1), ((24, 6, 3, 3), 4), ((10, 300 * scale, 1, 1), 1), ((150, 4, 1, 1), 1)]
+    ws = [(rng.normal(0, 0.1, size=s) * np.exp2(rng.integers(-3, 4, size=(s[0], 1, 1, 1)))).astype(np.float32) for s, _ in shapes]
+    dev = [torch.from_numpy(w).to(ctx.device) for w in ws]
+    hs = [ctx.sample_weights(d, groups=g, seed=1, layer_id=i, level_mask=0b1001, **opts) for i, (d, (_, g)) in enumerate(zip(dev, shapes))]
+    batch = ctx.sample_batch_create(dev, hs)
+    for seed in (7, 8):
+        ctx.sample_batch_run(batch, seed)
+        for i, (w, h) in enumerate(zip(ws, hs)):
+            for level in (0, 3):
+                W, eb = oracle.sample_level_ex(w, seed, i, level, **opts)[:2]
+                got, base = ctx.weights_export(h, level)
+                assert np.array_equal(got.cpu().numpy().astype(np.int64), W) and np.array_equal(base.cpu().numpy(), eb), (i, level)
+    assert ctx.device_status() == 0
+    ctx.sample_batch_free(batch)
+    for h in hs:
+        h.free()
+    ctx.close()
